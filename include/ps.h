@@ -410,8 +410,8 @@ int ps_eval_compact_noalloc(ps_ctx* ctx, const ps_space* space, uint64_t first, 
  * data_offset: theta0[units*h], then the inputs x[accum][D][b][h], then the
  * targets y[accum][D][b][h].  A case with D outside 1..4, a code above 624 or
  * data outside [0, data_len) gets a zero result and makes ps_status return
- * PS_E_DEVICE; nothing is read or written out of bounds.  The call may grow the
- * context's scratch (a workspace per case).  Ranges of the shape: see its
+ * PS_E_DEVICE; nothing is read or written out of bounds.  A case's states
+ * live on the SM that runs it; no scratch is used.  Ranges of the shape: see its
  * comments; outside them PS_E_RANGE. */
 typedef struct {
   uint32_t units, h, b;          /* layers 1..8, parameters per layer 1..32, samples per device and micro-batch 1..4 */

@@ -636,10 +636,7 @@ int ps_verify_batch(ps_ctx* ctx, const ps_verify_shape* shape, const ps_verify_c
   if (n == 0) return PS_OK;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return PS_E_CUDA;
-  rc = ensure_scratch(ctx, sizeof(double) * verify_workspace_doubles(s) * (size_t)n);
-  if (rc != PS_OK) return rc;
-  CUDA_OK(launch_verify(s, d_cases, n, d_data, data_len, static_cast<double*>(ctx->scratch), d_theta_out, d_out,
-                        ctx->d_status, ctx->stream));
+  CUDA_OK(launch_verify(s, d_cases, n, d_data, data_len, d_theta_out, d_out, ctx->d_status, ctx->stream));
   return enqueue_status_copy(ctx);
 }
 

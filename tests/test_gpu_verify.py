@@ -74,6 +74,25 @@ def test_verifier_equals_simulator_and_rules(ctx, ps, units, h, b, accum, nbuf):
     assert n_match == 475 + 3 * 171
 
 
+@pytest.mark.parametrize("units,h,b,accum,steps", [(1, 1, 1, 1, 1), (8, 32, 4, 4, 2), (1, 17, 1, 2, 2), (5, 16, 4, 1, 2),
+                                                  (3, 17, 4, 1, 2), (8, 3, 2, 2, 16)])
+def test_verifier_at_the_edges_of_its_block_shapes(ctx, ps, units, h, b, accum, steps):
+    """The smallest and the largest shape, and columns on both sides of a block's threads; every activation mode."""
+    data, offsets, parts = problems(units, h, b, accum, seed=31 * units + h)
+    codes = sorted({(37 * k + 125 * a) % 625 for k in range(5) for a in range(5)} | {0, 32, 156, 57, 249, 375 + 31})
+    cases = np.array([(c, D, offsets[D]) for D in (1, 2, 3, 4) for c in codes], dtype=ps.VERIFY_CASE_DTYPE)
+    got, theta = ctx.verify_batch(dict(units=units, h=h, b=b, accum=accum, steps=steps), cases, data, want_theta=True)
+    for k, c in enumerate(cases):
+        D, code = int(c["D"]), int(c["code"])
+        want = sim.simulate_problem(units, h, b, D, code, *parts[D], steps=steps)
+        g = got[k]
+        assert bool(g["match"]) == want["match"], (code, D)
+        assert (int(g["mem"]), int(g["comm"]), int(g["host"])) == (want["mem"], want["comm"], want["host"]), (code, D)
+        if want["theta"] is not None:
+            # (a step changes a parameter by at most lr; sums of up to 64 samples in another order: 64 ulp of that)
+            assert np.allclose(theta[k], want["theta"], rtol=1e-12, atol=1e-14), (code, D)
+
+
 def test_verifier_reports_bad_cases_without_touching_memory(ctx, ps):
     data, offsets, _ = problems(2, 4, 2, 1, seed=3)
     cases = np.zeros(4, dtype=ps.VERIFY_CASE_DTYPE)
