@@ -94,8 +94,8 @@ enum { PS_REDUCE_PARETO = 0, PS_REDUCE_TOPK = 1 };
 
 #define PS_NO_LIMIT UINT64_MAX
 #define PS_TOPK_MAX 64           /* largest max_entries of a top-k sweep            */
-#define PS_FRONTIER_FAST 128     /* a model whose frontier (or the part of it one warp of the
-                                    sweep finds) is longer is reduced by a slow exact path */
+#define PS_FRONTIER_FAST 128     /* a model whose frontier is longer (here or at a stage of its
+                                    reduction) is reduced by a slow exact path             */
 
 /* ------------------------------------------------------------------ types */
 typedef struct ps_ctx ps_ctx;     /* opaque: device, borrowed stream, scratch memory      */
@@ -257,8 +257,7 @@ int ps_eval_batch(ps_ctx* ctx, const ps_space* space, uint64_t first, uint64_t c
  * next ps_status return PS_E_TRUNCATED once (a notice: the head of the frontier
  * was written and later calls are not affected).  Frontiers of any length are
  * exact; one longer than PS_FRONTIER_FAST is computed by a slow path (one pass
- * over the model's points per entry).  n_caps <= 8.  The call may grow the
- * context's scratch (one partial list per warp of the sweep). */
+ * over the model's points per entry).  n_caps <= 8.  No scratch is used. */
 int ps_sweep_pareto(ps_ctx* ctx, const ps_space* space, const ps_filter* filter,
                     const uint64_t* caps_bytes /* host */, uint32_t n_caps, uint32_t reduce_kind,
                     uint32_t max_entries, ps_front_entry* d_out, uint32_t* d_counts);
