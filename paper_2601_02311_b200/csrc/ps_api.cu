@@ -65,15 +65,17 @@ bool shape_in_range(const ps_model_shape& s, u32 tp_coll, u32 accum = 1) {
 
 // whether every byte count of a (Theta, Omega, G) triple of this model -- device
 // bytes (at most wsum * (P + 2 unit)), host bytes (at most (2 accum + 1) * wsum * P)
-// and data-axis volume (at most (4 accum + 1) * wsum * P) -- stays below 2^53
-bool shape_is_small(const ps_model_shape& s, u32 accum) {
+// and volume (data axis: at most (4 accum + 1) * wsum * P, with several copies of every
+// shard 6 wsum * P more; tensor and pipeline axes as in shape_in_range) -- stays below 2^53
+bool shape_is_small(const ps_model_shape& s, u32 tp_coll, u32 accum, u32 copies) {
   typedef unsigned __int128 u128;
   const u128 H = s.hidden;
   const u128 P = s.param_elems_override ? (u128)s.param_elems_override
                                         : 12 * (u128)s.layers * H * H + (u128)s.vocab * H;
   const u128 unit = s.unit_from_shape ? 12 * H * H : 0;
   const u128 wsum = (u128)s.w_param + s.w_grad + s.w_opt;
-  return (4 * (u128)accum + 1) * wsum * (P + 2 * unit) < ((u128)1 << 53);
+  const u128 axes = ((u128)s.layers * 2 * tp_coll * s.w_act + 2 * s.w_act) * s.seq * s.micro_batch * H * accum;
+  return (4 * (u128)accum + 1 + (copies > 1 ? 6 : 0)) * wsum * (P + 2 * unit) + axes < ((u128)1 << 53);
 }
 
 int ensure_scratch(ps_ctx* ctx, size_t bytes) {
@@ -101,22 +103,6 @@ constexpr u32 KNOWN_FLAGS = (PS_F_PAPER_PRICED << 1) - 1u;
 int enqueue_status_copy(ps_ctx* ctx) {
   CUDA_OK(cudaMemcpyAsync(ctx->h_status, ctx->d_status, sizeof(u32), cudaMemcpyDeviceToHost, ctx->stream));
   return PS_OK;
-}
-
-u32 pick_chunks(const ps_ctx* ctx, const ps_space* sp, int kind, bool many) {
-  // Blocks per model.  Every extra block of a model builds its lists from
-  // scratch -- a top-k block takes every survivor as a candidate until it has
-  // found its own first k -- so only as many as fill the GPU once (top-k) or
-  // twice (Pareto, whose blocks are fewer and longer).
-  const u64 waves = kind == PS_REDUCE_PARETO ? 2 : 1;
-  const u64 target = (u64)ctx->sm_count * sweep_blocks_per_sm(kind, many) * waves;
-  u64 c = (target + sp->dev.n_models / 2) / sp->dev.n_models;       // to the nearest: one block too few is cheaper than a second list
-  if (c < 1) c = 1;
-  if (c > SWEEP_MAX_CHUNKS) c = SWEEP_MAX_CHUNKS;
-  const u64 by_units = (sp->dev.n_facts + sweep_warps(kind, many) - 1) / sweep_warps(kind, many);   // a unit per warp at least
-  if (c > by_units) c = by_units;
-  if (c < 1) c = 1;
-  return (u32)c;
 }
 
 }  // namespace
@@ -332,7 +318,7 @@ int ps_space_set_models(ps_space* sp, const ps_model_shape* models, uint32_t n_m
   u32 all_small = 1;
   for (u32 i = 0; i < n_models; ++i) {
     if (!shape_in_range(models[i], sp->dev.tp_coll, sp->dev.accum)) return PS_E_RANGE;
-    if (!shape_is_small(models[i], sp->dev.accum)) all_small = 0;
+    if (!shape_is_small(models[i], sp->dev.tp_coll, sp->dev.accum, sp->dev.repl)) all_small = 0;
   }
   sp->dev.all_small = all_small;
   sweep_order(sp, models, n_models);
@@ -476,63 +462,22 @@ int ps_sweep_pareto(ps_ctx* ctx, const ps_space* sp, const ps_filter* filter,
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return PS_E_CUDA;
 
-  // top-k over a table of many models, in the fast case (powers of two, byte counts exact in a
-  // double, every capacity below 2^53, nothing skipped): smaller blocks
-  bool many = reduce_kind == PS_REDUCE_TOPK && !filter->skip_rejected && sp->dev.all_pow2 && sp->dev.all_small &&
-              sp->dev.repl == 1 &&
-              (u64)sp->dev.n_models >= (u64)SWEEP_TOPK_MANY_WAVES * ctx->sm_count * SWEEP_BLOCKS_TOPK_MANY;
-  for (u32 c = 0; c < n_caps; ++c) many = many && caps_bytes[c] < ((u64)1 << 53) - 1;
-  const u32 n_chunks = pick_chunks(ctx, sp, (int)reduce_kind, many);
-  const size_t slots = (size_t)sp->dev.n_models * n_chunks * sweep_warps((int)reduce_kind, many);   // one list per warp
-  const size_t partial_bytes = slots * SWEEP_LIST_CAP * sizeof(PartialEntry);
-  const size_t lengths_bytes = (slots * sizeof(uint2) + 15) & ~size_t(15);
-  rc = ensure_scratch(ctx, partial_bytes + lengths_bytes + sizeof(u32) * (size_t)sp->dev.n_models);
-  if (rc != PS_OK) return rc;
   SweepArgs s;
   memset(&s, 0, sizeof(s));
+  for (u32 c = 0; c < n_caps; ++c) {
+    s.caps[c] = caps_bytes[c];
+    s.cap_max = std::max(s.cap_max, s.caps[c]);
+  }
   s.host_cap = filter->host_cap;
   s.require_flags = filter->require_flags & ~(u32)PS_F_FEASIBLE;
   s.comm_kind = filter->comm_kind;
-  s.k_keep = reduce_kind == PS_REDUCE_TOPK ? max_entries : 0;
+  s.n_caps = n_caps;
+  s.max_entries = max_entries;
   s.skip_rejected = filter->skip_rejected ? 1u : 0u;
-  s.many_models = many ? 1u : 0u;
-  s.partial = static_cast<PartialEntry*>(ctx->scratch);
-  s.partial_n = reinterpret_cast<uint2*>(static_cast<char*>(ctx->scratch) + partial_bytes);
+  s.out = d_out;
+  s.counts = d_counts;
   s.status = ctx->d_status;
-  MergeArgs m;
-  memset(&m, 0, sizeof(m));
-  m.partial = s.partial;
-  m.partial_n = s.partial_n;
-  m.n_lists = n_chunks * sweep_warps((int)reduce_kind, many);
-  m.host_cap = filter->host_cap;
-  m.require_flags = s.require_flags;
-  m.n_caps_total = n_caps;
-  m.max_entries = max_entries;
-  m.k_keep = s.k_keep;
-  m.comm_kind = filter->comm_kind;
-  m.out = d_out;
-  m.counts = d_counts;
-  m.slow_path = reinterpret_cast<u32*>(static_cast<char*>(ctx->scratch) + partial_bytes + lengths_bytes);
-  m.status = ctx->d_status;
-  if (reduce_kind == PS_REDUCE_PARETO) {
-    u64 cap_max = 0;
-    for (u32 c = 0; c < n_caps; ++c) { m.caps[c] = caps_bytes[c]; if (caps_bytes[c] > cap_max) cap_max = caps_bytes[c]; }
-    s.cap_max = cap_max;
-    m.cap_max = cap_max;
-    m.n_caps = n_caps;
-    CUDA_OK(launch_sweep(PS_REDUCE_PARETO, sp->dev, s, n_chunks, ctx->stream));
-    CUDA_OK(launch_sweep_merge(PS_REDUCE_PARETO, sp->dev, m, ctx->stream));
-  } else {
-    for (u32 c = 0; c < n_caps; ++c) {
-      s.cap_max = caps_bytes[c];
-      m.caps[0] = caps_bytes[c];
-      m.n_caps = 1;
-      m.cap_index = c;
-      m.cap_max = caps_bytes[c];
-      CUDA_OK(launch_sweep(PS_REDUCE_TOPK, sp->dev, s, n_chunks, ctx->stream));
-      CUDA_OK(launch_sweep_merge(PS_REDUCE_TOPK, sp->dev, m, ctx->stream));
-    }
-  }
+  CUDA_OK(launch_sweep((int)reduce_kind, sp->dev, s, ctx->sm_count, ctx->stream));
   return enqueue_status_copy(ctx);
 }
 

@@ -48,9 +48,8 @@ struct SpaceDev {
   u32 accum;          // micro-batches per step (gradient accumulation), >= 1
   u32 repl;           // copies of every shard (k-way replication of the sharded modes), >= 1
   u32 all_pow2;       // 1 if every device count of the space is a power of two (then every T, K, D is)
-  u32 all_small;      // 1 if for every model (4 accum + 1) (w_T + w_O + w_G) (P + 2 unit) < 2^53: the device
-                      // bytes, host bytes and data-axis volume of a (Theta, Omega, G) triple are then
-                      // exact in a double
+  u32 all_small;      // 1 if for every model the device bytes, host bytes and volume of a (Theta, Omega, G)
+                      // triple are below 2^53: exact in a double
 };
 
 enum : u32 {
@@ -327,12 +326,10 @@ __device__ __forceinline__ u32 point_flags(u32 th, u32 om, u32 gr, u32 ac, bool 
 // loading offloaded Theta, moving activations to the host and back, tensor- and
 // pipeline-axis traffic) is counted accum times, what happens once per step
 // (synchronising gradients, the update and what it moves) once.
-__device__ __forceinline__ PointOut eval_point(const ModelRec& r, const Fact& f, u32 v, u32 tau,
-                                               u32 th, u32 om, u32 gr, u32 ac, u32 tp_max_valid,
-                                               u32 tp_coll, bool axis_form, u32 sstar_units = 1,
-                                               u32 accum = 1, u32 repl = 1) {
-  UnitBase b = unit_base(r, f, tp_max_valid, axis_form, repl);
-  ActBase a = act_base(r, f, v, tau, b.G);
+// from the quantities of its factorisation and activation variant
+__device__ __forceinline__ PointOut eval_point_from(const ModelRec& r, const Fact& f, const UnitBase& b, const ActBase& a,
+                                                    u32 tau, u32 th, u32 om, u32 gr, u32 ac, u32 tp_coll,
+                                                    u32 sstar_units, u32 accum) {
   PointOut o;
   o.mem = r.wT * mu_elems(th, b.E2, b.sh, b.u, sstar_units) + r.wO * mu_elems(om, b.E2, b.sh, b.u, sstar_units) +
           r.wG * mu_elems(gr, b.E2, b.sh, b.u, sstar_units) + mu_elems(ac, a.EA, a.shA, a.uA, sstar_units);
@@ -356,6 +353,13 @@ __device__ __forceinline__ PointOut eval_point(const ModelRec& r, const Fact& f,
            (gr == PS_MODE_O ? 2 * b.sh * r.wG : 0) + (ac == PS_MODE_O ? 2 * a.EA * accum : 0);
   o.flags = point_flags(th, om, gr, ac, b.d1, b.cv, ext == 0);
   return o;
+}
+__device__ __forceinline__ PointOut eval_point(const ModelRec& r, const Fact& f, u32 v, u32 tau,
+                                               u32 th, u32 om, u32 gr, u32 ac, u32 tp_max_valid,
+                                               u32 tp_coll, bool axis_form, u32 sstar_units = 1,
+                                               u32 accum = 1, u32 repl = 1) {
+  const UnitBase b = unit_base(r, f, tp_max_valid, axis_form, repl);
+  return eval_point_from(r, f, b, act_base(r, f, v, tau, b.G), tau, th, om, gr, ac, tp_coll, sstar_units, accum);
 }
 
 // ---------------------------------------------------------------- filters on (Theta, Omega, G) triples

@@ -34,93 +34,24 @@ struct ps_space {
 };
 
 // ---- sweep
-// Block shapes of the sweep: warps per block and the resident blocks per SM the
-// kernel is compiled for (which sets its register budget).  The top-k sweep is
-// fastest with eight blocks of three warps (24 warps of 80 registers; 1184 resident
-// blocks, so that a thousand models run as one wave): few and long lists per model.
-// The Pareto sweep is fastest with four blocks of four warps (16 warps of 128
-// registers): since its reduction pass became short, what it gains from registers
-// outweighs what larger blocks gain from sharing a coarse staircase (2 x 10 warps of
-// 96 registers: +6 %; 2 x 8: +2.5 %; 3 x 5, 8 x 2, 1 x 16: +3 to +10 %).
-#ifndef SWEEP_WARPS_TOPK
-#define SWEEP_WARPS_TOPK 3
-#endif
-#ifndef SWEEP_BLOCKS_TOPK
-#define SWEEP_BLOCKS_TOPK 8
-#endif
-#ifndef SWEEP_WARPS_PARETO
-#define SWEEP_WARPS_PARETO 4
-#endif
-#ifndef SWEEP_BLOCKS_PARETO
-#define SWEEP_BLOCKS_PARETO 4
-#endif
-// A table of many models (at least SWEEP_TOPK_MANY_WAVES full waves of the smaller blocks) is
-// swept for top-k with blocks of two warps, nine resident per SM: -3.7 % on four thousand
-// models; on a thousand models the GPU is then short of warps (+10 %), so those keep three.
-// Compiled for the fast case without skipping only (see launch_sweep_t).
-#ifndef SWEEP_WARPS_TOPK_MANY
-#define SWEEP_WARPS_TOPK_MANY 2
-#endif
-#ifndef SWEEP_BLOCKS_TOPK_MANY
-#define SWEEP_BLOCKS_TOPK_MANY 9
-#endif
-#ifndef SWEEP_TOPK_MANY_WAVES
-#define SWEEP_TOPK_MANY_WAVES 2
-#endif
-static inline int sweep_warps(int kind, bool many = false) {
-  return kind == PS_REDUCE_PARETO ? SWEEP_WARPS_PARETO : (many ? SWEEP_WARPS_TOPK_MANY : SWEEP_WARPS_TOPK);
-}
-static inline int sweep_blocks_per_sm(int kind, bool many = false) {
-  return kind == PS_REDUCE_PARETO ? SWEEP_BLOCKS_PARETO : (many ? SWEEP_BLOCKS_TOPK_MANY : SWEEP_BLOCKS_TOPK);
-}
-#define SWEEP_LIST_CAP 128        /* entries of a warp's list and of a block's partial list */
-#define SWEEP_MAX_CHUNKS 16       /* blocks per model                                        */
-#define MERGE_CAP (5 * SWEEP_LIST_CAP)    /* entries the merge kernel combines at a time: what it
-                                     has kept plus as many of the warps' lists as fit      */
+#define SWEEP_MAX_WARPS 16        /* warps of a block at most */
 #define PS_MAX_CAPS 8
 
-struct PartialEntry {
-  u64 a, b;   // Pareto: (mem, comm); top-k: (comm, mem)
-  u32 i;      // point index within the model
-  u32 pad;
-};
-
 struct SweepArgs {
-  u64 cap_max;          // survivors need mem <= cap_max
+  u64 caps[PS_MAX_CAPS];
+  u64 cap_max;          // the largest of them
   u64 host_cap;
   u32 require_flags;    // without PS_F_FEASIBLE
   u32 comm_kind;
-  u32 k_keep;           // top-k: entries kept
+  u32 n_caps;
+  u32 max_entries;      // entries of an output row; top-k: entries kept
   u32 skip_rejected;    // do not evaluate factorisations whose composition bits miss a required flag
-  u32 many_models;      // top-k: the blocks of two warps (the host has checked that the fast case applies)
-  u32 pad;
-  PartialEntry* partial;   // [n_models * n_chunks * warps][SWEEP_LIST_CAP]: one list per warp
-  uint2* partial_n;        // [n_models * n_chunks * warps]: (entries, survivors)
-  u32* status;
-};
-
-struct MergeArgs {
-  const PartialEntry* partial;
-  const uint2* partial_n;
-  u64 caps[PS_MAX_CAPS];
-  u64 cap_max, host_cap;  // the filter again, for the slow exact path
-  u32 require_flags;
-  u32 n_lists;          // partial lists per model: blocks per model x warps per block
-  u32 n_caps;           // capacities this launch emits
-  u32 n_caps_total;     // capacities of the output layout
-  u32 cap_index;        // top-k: which capacity this launch is for
-  u32 max_entries;
-  u32 k_keep;
-  u32 comm_kind;
   ps_front_entry* out;
   u32* counts;
-  u32* slow_path;       // Pareto, [n_models]: set by the merge for a model whose frontier outgrew the lists
   u32* status;
 };
 
-cudaError_t launch_sweep(int kind, const SpaceDev& sp, const SweepArgs& a, u32 n_chunks,
-                         cudaStream_t stream);
-cudaError_t launch_sweep_merge(int kind, const SpaceDev& sp, const MergeArgs& a, cudaStream_t stream);
+cudaError_t launch_sweep(int kind, const SpaceDev& sp, const SweepArgs& a, int sm_count, cudaStream_t stream);
 
 // ---- batch evaluation
 /* Block shape of the window kernels: four resident blocks of four warps (128 registers a thread
