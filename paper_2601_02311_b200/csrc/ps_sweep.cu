@@ -29,10 +29,10 @@
 //
 // What bounds it: the fp64 pipe and the issue slots of the screening (a compare per point;
 // 64 a clock and SM).  4096 models of the stress configuration, 6.96e9 points: top-k 1.94 ->
-// 0.93 ms, Pareto 2.37 -> 0.97 ms against a sweep whose warps took a unit each (the set-up
+// 0.79 ms, Pareto 2.37 -> 0.85 ms against a sweep whose warps took a unit each (the set-up
 // of a unit paid by a whole warp, candidates inserted one by one into a sorted list per
 // warp, the lists merged by a second kernel); 1024 models skipping rejected factorisations
-// 0.41 -> 0.16 ms.
+// 0.41 -> 0.10 ms.  The screening alone takes 0.52 and 0.58 ms of the former two.
 #include <type_traits>
 #include "ps_device.cuh"
 #include "ps_internal.h"
@@ -45,13 +45,14 @@ constexpr u64 U64MAX = ~0ull;
 constexpr int SEG = 1024;                  // units of a segment
 constexpr int CELLS = 512;                 // cells of the histogram
 constexpr int CAND_CAP = 512;              // candidates the block's buffer holds
-constexpr int KEEP_CAP = PS_FRONTIER_FAST; // Pareto: frontier entries the buffer may keep after a cut
+constexpr int KEEP_CAP = PS_FRONTIER_FAST; // Pareto: frontier entries that can be emitted from the buffer
 constexpr int HIT_CAP = 256;               // top-k: (unit, triple, tensor-axis variant) hits the block holds
 constexpr int MAX_TRIPLES = 125;
 constexpr u32 NO_CODE = 0xffffffffu;       // an empty entry
 constexpr u32 ALL_STEPS = 0xffffffffu;
-// a step of the second pass appends at most four entries a lane, a hit becomes at most ten points
-static_assert(CAND_CAP - KEEP_CAP >= 128 && HIT_CAP >= 128 && CAND_CAP - PS_TOPK_MAX >= 320,
+constexpr int STEP_CAP = 128;              // entries that a step of the second pass appends at most: four a lane
+// (a hit becomes at most ten points)
+static_assert(PS_TOPK_MAX <= KEEP_CAP && HIT_CAP >= STEP_CAP && CAND_CAP - PS_TOPK_MAX >= 320,
               "what a step brings fits an emptied buffer");
 
 struct Key {
@@ -84,7 +85,8 @@ struct __align__(16) Triple {
   u64 k[4];             // ka, kb, kc and kh, as the screening's type
   u64 kx;               // kx, the same
   u32 allowed;          // allowed activation digits: bits 0..4, 8..12, 16..20 for the three CLS_* of a unit;
-                        // bits 24.. reductions to shards (2 bits) and all-reduces (1 bit) beyond kx * x (copies)
+                        // bits 24.. reductions to shards (2 bits) and all-reduces (1 bit) beyond kx * x, where
+                        // shards have copies
   u32 pad;
 };
 
@@ -100,20 +102,34 @@ __device__ __forceinline__ int cell_of(double m) {
   return max((__double2hiint(m) >> 17) - (1023 << 3) + 1, 0);
 }
 
+// what decides whether one triple dominates another (see dominated)
+struct Rank {
+  u32 bytes;            // ka, ka + kb, kc, a byte each
+  u32 volume;           // kx, kh
+  u32 allowed;          // as in Triple
+};
+
 struct BlockShared {
   ModelRec rec;
   Triple tri[MAX_TRIPLES];
+  unsigned char allowed[3][MAX_TRIPLES + 3];   // allowed activation digits of a triple for the three CLS_* of a unit
   u64 state[2][5][4];                      // Theta, Omega: the coefficients of E, s, u and the host coefficient, by digit
   u64 cell[CELLS];                         // the histogram
   u64 cand_a[CAND_CAP], cand_b[CAND_CAP];  // the buffer: Pareto (mem, comm), top-k (comm, mem)
   u32 cand_i[CAND_CAP];
+  unsigned char place[CAND_CAP];           // candidates that stay
+  u64 sorted_a[KEEP_CAP], sorted_b[KEEP_CAP];
+  u32 sorted_i[KEEP_CAP];
+  int kept;
   u64 hit_comm[HIT_CAP];
   u32 hit[HIT_CAP];
   u32 flags[SEG / 32];                     // units of the segment with survivors
   u16 heavy[SEG];                          // the same as a list
-  u32 n_heavy, next1, next2, n_cand, n_hits, full, limit_cell, survivors;
-  u64 warp_min[SWEEP_MAX_WARPS];
-  int warp_sum[SWEEP_MAX_WARPS];
+  u32 least_cell[SEG];                     // top-k: the lowest cell that a survivor of a listed unit falls into
+  unsigned char live[MAX_TRIPLES + 3];     // the triples the passes walk
+  Rank rank[MAX_TRIPLES];
+  unsigned char alive[MAX_TRIPLES + 3];
+  u32 n_live, n_heavy, next1, next2, n_cand, n_hits, full, limit_cell, survivors;
 };
 
 // ------------------------------------------------------------------ small arithmetic
@@ -201,9 +217,10 @@ struct LaneUnit {
 };
 
 // ------------------------------------------------------------------ screening
-// Whether any of four variants of an activation digit survives: one compare per point, its
-// result chained through the next one's input predicate.
-__device__ __forceinline__ void any_digit(u32& any, double m, const double* b, u32 allowed_bit) {
+// Whether any of four variants of an activation digit fits: one compare per point, its
+// result chained through the next one's input predicate; BIT joins `fit` if one does.
+template <u32 BIT>
+__device__ __forceinline__ void any_variant(u32& fit, double m, const double* b) {
   asm("{\n\t"
       ".reg .pred p;\n\t"
       "setp.lt.f64 p, %1, %2;\n\t"
@@ -212,12 +229,28 @@ __device__ __forceinline__ void any_digit(u32& any, double m, const double* b, u
       "setp.lt.or.f64 p, %1, %5, p;\n\t"
       "@p or.b32 %0, %0, %6;\n\t"
       "}"
-      : "+r"(any)
-      : "d"(m), "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]), "r"(allowed_bit));
+      : "+r"(fit)
+      : "d"(m), "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]), "n"(BIT));
 }
-__device__ __forceinline__ void any_digit(u32& any, u64 m, const u64* b, u32 allowed_bit) {
+template <u32 BIT>
+__device__ __forceinline__ void any_variant(u32& fit, u64 m, const u64* b) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) any |= (m < b[q]) ? allowed_bit : 0u;
+  for (int q = 0; q < 4; ++q) fit |= (m < b[q]) ? BIT : 0u;
+}
+template <int D, int NM, typename T, bool HOST_LIMITED>
+__device__ __forceinline__ void fitting_digits(u32& fit, const LaneUnit<NM, T, HOST_LIMITED>& lu, u32 modemap, T m, T h,
+                                               T cap_room) {
+  if constexpr (D < NM) {
+    if (digit_mode(modemap, D) == PS_MODE_O) {
+      // the four variants have the same bytes: one capacity compare, and the host bytes of each
+      u32 with_host = HOST_LIMITED ? 0u : 1u << D;
+      if (HOST_LIMITED) any_variant<1u << D>(with_host, h, lu.host_bound);
+      fit |= m < cap_room ? with_host : 0u;
+    } else {
+      any_variant<1u << D>(fit, m, lu.bound[D]);
+    }
+    fitting_digits<D + 1>(fit, lu, modemap, m, h, cap_room);
+  }
 }
 
 // Does any point of the lane's unit whose (Theta, Omega) pair lies in [p0, p1) survive?
@@ -225,6 +258,7 @@ template <int NM, typename T, bool HOST_LIMITED>
 __device__ __forceinline__ u32 screen_pairs(const BlockShared& sh, const LaneUnit<NM, T, HOST_LIMITED>& lu, u32 modemap,
                                             T cap_room, T host_room, u32 p0, u32 p1) {
   u32 any = 0;
+  const unsigned char* allowed_of = sh.allowed[lu.shift >> 3];
 #pragma unroll 1
   for (u32 p = p0; p < p1; ++p) {
     const u32 th = p / NM, om = p - th * NM;
@@ -236,115 +270,40 @@ __device__ __forceinline__ u32 screen_pairs(const BlockShared& sh, const LaneUni
 #pragma unroll
     for (int gr = 0; gr < NM; ++gr) {
       const T m = to_mem + lu.gr_mem[gr];
-      u32 allowed = (sh.tri[th + NM * om + NM * NM * gr].allowed >> lu.shift) & lu.allowed;
       T h = to_host;
-      if (HOST_LIMITED) {
-        if (digit_mode(modemap, gr) == PS_MODE_O) h += lu.gr_host;
-        if (!(h < host_room)) allowed = 0;               // the triple's own host bytes against the budget
-      }
-#pragma unroll
-      for (int d = 0; d < NM; ++d) {
-        if (digit_mode(modemap, d) == PS_MODE_O) {
-          // the four variants have the same bytes: one capacity compare, then the host bytes of each
-          u32 fits = HOST_LIMITED ? 0u : allowed;
-          if (HOST_LIMITED) any_digit(fits, h, lu.host_bound, allowed);
-          any |= (m < cap_room) ? fits & (1u << d) : 0u;
-        } else {
-          any_digit(any, m, lu.bound[d], allowed & (1u << d));
-        }
-      }
+      if (HOST_LIMITED && digit_mode(modemap, gr) == PS_MODE_O) h += lu.gr_host;
+      u32 fit = 0;                                       // digits with a point that fits, whatever its flags
+      fitting_digits<0>(fit, lu, modemap, m, h, cap_room);
+      if (HOST_LIMITED) fit = h < host_room ? fit : 0u;  // the triple's own host bytes against the budget
+      any |= fit & allowed_of[th + NM * om + NM * NM * gr];
     }
   }
-  return any;
+  return any & lu.allowed;
+}
+
+// Pareto: the classes of units in which triple t can never add to a frontier because triple
+// a has, in every unit, a point with no more bytes, volume and host bytes wherever t has one
+// -- and fewer bytes, or a smaller index for the same pair.  (E >= s >= 1: bytes are compared
+// as ka (E - s) + (ka + kb) s + kc u.)  Bits 0, 8 and 16 for the three CLS_*.
+__device__ __forceinline__ u32 dominated(const Rank& t, const Rank& a, bool a_first) {
+  const bool less = (a.bytes & 0xff00u) < (t.bytes & 0xff00u);
+  const u32 copies_t = t.allowed >> 24, copies_a = a.allowed >> 24;
+  if (__vcmpgtu4(a.bytes, t.bytes) | __vcmpgtu2(a.volume, t.volume)) return 0;
+  if (!(less || a_first) || (copies_a & 3u) > (copies_t & 3u) || (copies_a & 4u) > (copies_t & 4u)) return 0;
+  const u32 misses = t.allowed & ~a.allowed & 0x1f1f1fu; // digits that t may use and a may not
+  return __vcmpeq4(misses, 0u) & 0x010101u;
 }
 
 // ------------------------------------------------------------------ the buffer
-// exclusive prefix minimum / prefix sum over the threads of a block
-__device__ __forceinline__ u64 block_excl_min(u64 mine, u64* warp_min, int tid) {
-  const int lane = tid & 31, warp = tid >> 5;
-  u64 incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const u64 up = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl = min(incl, up);
-  }
-  u64 excl = __shfl_up_sync(0xffffffffu, incl, 1);
-  if (lane == 0) excl = U64MAX;
-  if (lane == 31) warp_min[warp] = incl;
-  __syncthreads();
-  for (int w = 0; w < warp; ++w) excl = min(excl, warp_min[w]);
-  __syncthreads();
-  return excl;
-}
-__device__ __forceinline__ int block_excl_sum(int mine, int* warp_sum, int tid, int warps, int* total) {
-  const int lane = tid & 31, warp = tid >> 5;
-  int incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int up = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += up;
-  }
-  if (lane == 31) warp_sum[warp] = incl;
-  __syncthreads();
-  int before = 0, all = 0;
-  for (int w = 0; w < warps; ++w) {
-    if (w < warp) before += warp_sum[w];
-    all += warp_sum[w];
-  }
-  __syncthreads();
-  *total = all;
-  return before + incl - mine;
-}
-
-// Sort the block's n candidates and keep those that matter, sorted, at the front; returns
-// how many stay.  Pareto: keys (mem, comm, idx), kept if the communication is below that of
-// everything before.  Top-k: keys (comm, mem, idx), the k smallest.  (Empty slots hold the
-// largest key and fall out.)  Every thread of the block takes part.
-//
-// Usually the candidates are about as many as the threads: then every thread ranks its own
-// against all others (broadcast reads, no barrier in the loop), else a bitonic sort.
-template <int KIND>
-__device__ __noinline__ int cut_buffer(BlockShared& sh, int n, int k_keep) {
+// The block's n candidates, sorted by key (a bitonic network over shared memory).
+__device__ __noinline__ void sort_candidates(BlockShared& sh, int n) {
   const int tid = threadIdx.x, threads = blockDim.x;
   u64* const a = sh.cand_a;
   u64* const b = sh.cand_b;
   u32* const ix = sh.cand_i;
-  __syncthreads();
-  if (n <= threads) {
-    const Key e{tid < n ? a[tid] : U64MAX, tid < n ? b[tid] : U64MAX, tid < n ? ix[tid] : 0xffffffffu};
-    bool keep = tid < n && e.a != U64MAX;
-    int rank = 0, total;
-    if (KIND == PS_REDUCE_PARETO) {
-      if (keep) {
-#pragma unroll 4
-        for (int q = 0; q < n; ++q) {
-          const u64 oa = a[q], ob = b[q];
-          if (oa <= e.a && ob <= e.b && (oa != e.a || ob != e.b || ix[q] < e.i)) keep = false;
-        }
-      }
-      // (what stays is few: only it is ranked, by its bytes, which are distinct)
-      __syncthreads();
-      const int at = block_excl_sum(keep ? 1 : 0, sh.warp_sum, tid, threads >> 5, &total);
-      if (keep) a[at] = e.a;
-      __syncthreads();
-      if (keep)
-        for (int q = 0; q < total; ++q) rank += a[q] < e.a ? 1 : 0;
-      __syncthreads();
-    } else {
-      if (keep) {
-#pragma unroll 4
-        for (int q = 0; q < n; ++q) rank += key_less(Key{a[q], b[q], ix[q]}, e) ? 1 : 0;
-      }
-      keep = keep && rank < k_keep;
-      total = __syncthreads_count(keep);
-    }
-    if (keep) { a[rank] = e.a; b[rank] = e.b; ix[rank] = e.i; }
-    __syncthreads();
-    return total;
-  }
   int size = 32;
   while (size < n) size <<= 1;
-  for (int p = n + tid; p < size; p += threads) { a[p] = U64MAX; b[p] = U64MAX; ix[p] = 0xffffffffu; }
+  for (int p = n + tid; p < size; p += threads) { a[p] = U64MAX; b[p] = U64MAX; ix[p] = NO_CODE; }
   for (int k = 2; k <= size; k <<= 1)
     for (int j = k >> 1; j > 0; j >>= 1) {
       __syncthreads();
@@ -358,30 +317,115 @@ __device__ __noinline__ int cut_buffer(BlockShared& sh, int n, int k_keep) {
       }
     }
   __syncthreads();
-  int kept = 0;
-  if (KIND == PS_REDUCE_TOPK) {
-    for (int p = tid; p < min(n, k_keep); p += threads) kept += a[p] != U64MAX ? 1 : 0;
-    int total;
-    block_excl_sum(kept, sh.warp_sum, tid, threads >> 5, &total);
-    return total;
-  }
-  u64 least = U64MAX;                      // of everything before this stretch
-  for (int base = 0; base < n; base += threads) {
-    const int p = base + tid;
-    const Key e{p < n ? a[p] : U64MAX, p < n ? b[p] : U64MAX, p < n ? ix[p] : 0u};
-    const u64 before = min(least, block_excl_min(e.b, sh.warp_min, tid));
-    const bool keep = p < n && e.b < before;
-    int total;
-    const int at = block_excl_sum(keep ? 1 : 0, sh.warp_sum, tid, threads >> 5, &total);
-    // (the places written lie before the stretch just read; its end is read by everyone first)
-    if (tid == threads - 1) sh.warp_min[0] = min(before, e.b);
-    if (keep) { a[kept + at] = e.a; b[kept + at] = e.b; ix[kept + at] = e.i; }
+}
+
+// Up to this many candidates every thread tests its own against all others (no barrier in
+// the loop); more are sorted, whose work grows more slowly.  With 64 instead the zoo's
+// frontiers take 0.110 ms instead of 0.100; without the sort top-k of the stress
+// configuration takes 0.90 ms instead of 0.79.
+constexpr int PAIRWISE = 128;
+
+// Pareto, without regard to indices: drops the candidates that another one beats strictly;
+// returns how many are left (equal pairs all stay).
+__device__ __noinline__ int drop_dominated(BlockShared& sh, int n) {
+  const int tid = threadIdx.x, lane = tid & 31, threads = blockDim.x;
+  __syncthreads();
+  const bool pairwise = n <= PAIRWISE;
+  if (pairwise) {
+    for (int p = tid; p < n; p += threads) {
+      const u64 a = sh.cand_a[p], b = sh.cand_b[p];
+      bool keep = a != U64MAX;
+#pragma unroll 4
+      for (int q = 0; q < n; ++q) {
+        const u64 oa = sh.cand_a[q], ob = sh.cand_b[q];
+        if (oa <= a && ob <= b && (oa < a || ob < b)) keep = false;
+      }
+      sh.place[p] = keep ? 1 : 0;
+    }
     __syncthreads();
-    least = sh.warp_min[0];
-    __syncthreads();
-    kept += total;
+  } else {
+    sort_candidates(sh, n);
   }
-  return kept;
+  if (tid < 32) {                                        // closed up by one warp, 32 at a time
+    int left = 0;
+    u64 least = U64MAX, least_at = 0;                    // the least communication before these 32, and the bytes it came with
+    for (int base = 0; base < n; base += 32) {
+      const int p = base + lane;
+      const u64 a = p < n ? sh.cand_a[p] : U64MAX, b = p < n ? sh.cand_b[p] : U64MAX;
+      const u32 code = p < n ? sh.cand_i[p] : NO_CODE;
+      bool keep;
+      if (pairwise) {
+        keep = p < n && sh.place[p] != 0;
+      } else {
+        // in the order of (bytes, communication) a candidate stays if nothing before it has
+        // as little communication, or only its own pair
+        u64 m = b, at = a;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const u64 mu = __shfl_up_sync(0xffffffffu, m, o), au = __shfl_up_sync(0xffffffffu, at, o);
+          if (lane >= o && mu <= m) { m = mu; at = au; }
+        }
+        if (least <= m) { m = least; at = least_at; }
+        keep = a != U64MAX && m == b && at == a;         // (m: the least up to here, earliest first)
+        least = __shfl_sync(0xffffffffu, m, 31);
+        least_at = __shfl_sync(0xffffffffu, at, 31);
+      }
+      const u32 votes = __ballot_sync(0xffffffffu, keep);
+      if (keep) {
+        const int to = left + __popc(votes & ((1u << lane) - 1u));
+        sh.cand_a[to] = a; sh.cand_b[to] = b; sh.cand_i[to] = code;
+      }
+      left += __popc(votes);
+      __syncwarp();
+    }
+    if (lane == 0) sh.kept = left;
+  }
+  __syncthreads();
+  return sh.kept;
+}
+
+// The n candidates sorted by key, without those of a pair that a smaller index has (Pareto,
+// where no strict domination is left), or the k smallest of them (top-k).  Returns how many
+// stay; more than KEEP_CAP are not all written.
+template <int KIND>
+__device__ __noinline__ int rank_candidates(BlockShared& sh, int n, int k_keep) {
+  constexpr bool PARETO = KIND == PS_REDUCE_PARETO;
+  const int tid = threadIdx.x, threads = blockDim.x;
+  __syncthreads();
+  if (!PARETO && n > PAIRWISE) {
+    sort_candidates(sh, n);
+    return min(n, k_keep);
+  }
+  if (tid == 0) sh.kept = 0;
+  if (PARETO)
+    for (int p = tid; p < n; p += threads) {
+      const u64 a = sh.cand_a[p];
+      const u32 ix = sh.cand_i[p];
+      bool keep = true;
+      for (int q = 0; q < n; ++q)
+        if (sh.cand_a[q] == a && sh.cand_i[q] < ix) keep = false;
+      sh.place[p] = keep ? 1 : 0;
+    }
+  __syncthreads();
+  for (int p = tid; p < n; p += threads) {
+    const Key e{sh.cand_a[p], sh.cand_b[p], sh.cand_i[p]};
+    if (PARETO && sh.place[p] == 0) continue;
+    int rank = 0;
+#pragma unroll 4
+    for (int q = 0; q < n; ++q) {
+      if (PARETO) rank += (sh.place[q] != 0 && sh.cand_a[q] < e.a) ? 1 : 0;
+      else rank += key_less(Key{sh.cand_a[q], sh.cand_b[q], sh.cand_i[q]}, e) ? 1 : 0;
+    }
+    if (PARETO) atomicAdd(&sh.kept, 1);
+    if (rank < KEEP_CAP) { sh.sorted_a[rank] = e.a; sh.sorted_b[rank] = e.b; sh.sorted_i[rank] = e.i; }
+  }
+  __syncthreads();
+  const int stay = PARETO ? sh.kept : min(n, k_keep);
+  for (int p = tid; p < min(stay, KEEP_CAP); p += threads) {
+    sh.cand_a[p] = sh.sorted_a[p]; sh.cand_b[p] = sh.sorted_b[p]; sh.cand_i[p] = sh.sorted_i[p];
+  }
+  __syncthreads();
+  return stay;
 }
 
 // ------------------------------------------------------------------ candidates to points
@@ -420,16 +464,14 @@ __device__ __forceinline__ void points_of(const SpaceDev& sp, const BlockShared&
   }
 }
 
-// Pareto: the buffer's entries from n_resolved on get the index of their point, the smallest
-// with the entry's bytes
+// Pareto: the buffer's n entries get the index of their point, the smallest with the entry's
+// bytes
 template <int NM>
-__device__ __noinline__ void resolve_candidates(const SpaceDev& sp, BlockShared& sh, int n_resolved, u32 modemap,
-                                                u64 cap_x, u64 host_x) {
+__device__ __noinline__ void resolve_candidates(const SpaceDev& sp, BlockShared& sh, int n, u32 modemap, u64 cap_x,
+                                                u64 host_x) {
   __syncthreads();
-  const int n = min((int)sh.n_cand, CAND_CAP);
-  for (int p = n_resolved + (int)threadIdx.x; p < n; p += blockDim.x) {
+  for (int p = threadIdx.x; p < n; p += blockDim.x) {
     const u32 code = sh.cand_i[p];
-    if (code == NO_CODE) continue;
     const u64 want = sh.cand_a[p];
     points_of<NM>(sp, sh, code, modemap, cap_x, host_x, [&](u64 m, u32 idx) {
       if (m == want) sh.cand_i[p] = idx;
@@ -609,6 +651,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
       if (gr == PS_MODE_M) { cg += on_shard ? 1 : 2; if (on_shard) n2 += 1; else n3 += 1; }
       if (gr == PS_MODE_O) { cg += 1; n2 += 1; }
     }
+    if (sp.repl == 1) n2 = n3 = 0;           // (x2 and x3 are zero)
     const u32 a_many = allowed_act_digits(triple_bits(th, om, gr, CLS_SHARDED), req, all, own, is_o, not_mo);
     const u32 a_one = allowed_act_digits(triple_bits(th, om, gr, CLS_ONE_DEVICE), req, all, all, is_o, not_mo);
     const u32 a_copies = allowed_act_digits(triple_bits(th, om, gr, CLS_ALL_COPIES), req, all, all, is_o, not_mo);
@@ -617,6 +660,10 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     tr.kx = bits<T>(as<T>(ct * rec.wT + co * rec.wO + cg * rec.wG));
     tr.allowed = a_many | (a_one << 8) | (a_copies << 16) | (n2 << 24) | (n3 << 26);
     tr.pad = 0;
+    sh.rank[t] = Rank{a | ((a + b) << 8) | (c << 16), (ct * rec.wT + co * rec.wO + cg * rec.wG) | (h << 16), tr.allowed};
+    sh.allowed[CLS_SHARDED][t] = (unsigned char)a_many;
+    sh.allowed[CLS_ONE_DEVICE][t] = (unsigned char)a_one;
+    sh.allowed[CLS_ALL_COPIES][t] = (unsigned char)a_copies;
   }
   for (int t = tid; t < 2 * NM; t += threads) {
     const u32 st = t / NM, d = t % NM, mode = digit_mode(modemap, d), w = st == 0 ? rec.wT : rec.wO;
@@ -626,10 +673,41 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     for (int j = 0; j < 4; ++j) sh.state[st][d][j] = bits<T>(as<T>(k[j]));
   }
 
+  // ---- the triples that the passes walk: those that the flags allow; for Pareto only those
+  // that no triple differing in one mode dominates (55 of 95 with valid points required)
+  __syncthreads();
+  for (int t = tid; t < N3; t += threads) {
+    const Rank own = sh.rank[t];
+    // (0x01 in the byte of a class with allowed digits)
+    u32 used = __vcmpgtu4(own.allowed & 0x1f1f1fu, 0u) & 0x010101u;
+    if (PARETO) {
+      const int digit[3] = {t % NM, (t / NM) % NM, t / N2}, weight[3] = {1, NM, N2};
+#pragma unroll
+      for (int st = 0; st < 3; ++st)
+#pragma unroll
+        for (int k = 1; k < (NM > 1 ? NM : 0); ++k) {
+          const int d = digit[st] + k < NM ? digit[st] + k : digit[st] + k - NM;
+          used &= ~dominated(own, sh.rank[t + (d - digit[st]) * weight[st]], d < digit[st]);
+        }
+    }
+    sh.alive[t] = used != 0;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    u32 n = 0;
+    for (int base = 0; base < N3; base += 32) {
+      const int t = base + lane;
+      const bool live = t < N3 && sh.alive[t] != 0;
+      const u32 votes = __ballot_sync(0xffffffffu, live);
+      if (live) sh.live[n + __popc(votes & ((1u << lane) - 1u))] = (unsigned char)t;
+      n += __popc(votes);
+    }
+    if (lane == 0) sh.n_live = n;
+  }
+
   Key threshold{U64MAX, U64MAX, 0xffffffffu};        // top-k: nothing at or above it is wanted
   u32 survivors = 0;
   bool overflowed = false;                           // the same for every thread
-  int n_resolved = 0;                                // Pareto: candidates whose indices are known
   const bool skip = args.skip_rejected && req_cv != 0;
 
   for (u32 seg = 0; seg < sp.n_facts; seg += SEG) {
@@ -673,13 +751,22 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
       if (lane == 31) sh.n_heavy = incl;
     }
     __syncthreads();
-    const u32 n_heavy = sh.n_heavy, heavy_batches = (n_heavy + 31) / 32;
-    if (n_heavy == 0) continue;
+    const u32 n_live = sh.n_live;
+    u32 n_heavy = sh.n_heavy;
+    if (n_heavy == 0 || n_live == 0) continue;
+    if (!PARETO)
+      for (u32 k = tid; k < n_heavy; k += threads) sh.least_cell[k] = CELLS;
 
     // ---- the two passes.  An item is a batch of 32 listed units and a part of the triples.
-    const u32 parts = min(max((u32)warps / heavy_batches, 1u), (u32)N2), n_items = heavy_batches * parts;
-    // walks an item's triples from triple `from` on; returns the one at which the buffer was
-    // full, or none
+    u32 parts, n_items;
+    auto deal = [&]() {
+      const u32 batches = (n_heavy + 31) / 32;
+      parts = min(max((u32)warps / batches, 1u), (n_live + 1) / 2);
+      n_items = batches * parts;
+    };
+    deal();
+    // walks an item's triples from place `from` of the list on; returns the place at which the
+    // buffer was full, or none
     auto walk = [&](auto second, u32 item, u32 from) -> u32 {
       constexpr bool SECOND = decltype(second)::value;
       const u32 b = item / parts, part = item - b * parts, k = b * 32 + lane;
@@ -698,16 +785,17 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
         act[tau] = cap_room;
       }
       u32 set = 0;                                   // the allowed digits act[] is for
-      const u32 t_end = (part + 1) * N3 / parts;
+      const u32 t_end = (part + 1) * n_live / parts;
+      u32 lowest = CELLS;                            // top-k, first pass: the lowest cell of a survivor
       // Two triples at a time, all four candidates side by side and one vote for them: what
       // a step waits for (table loads, dependent fp64 operations, votes) is waited for once.
 #pragma unroll 1
-      for (u32 t0 = max(part * N3 / parts, from); t0 < t_end; t0 += 2) {
+      for (u32 t0 = max(part * n_live / parts, from); t0 < t_end; t0 += 2) {
         T m[2], c[2], h[2], act_of_set[2][2];
         u32 allowed[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-          const Triple& tr = sh.tri[min(t0 + j, t_end - 1)];
+          const Triple& tr = sh.tri[sh.live[min(t0 + j, t_end - 1)]];
           allowed[j] = t0 + j < t_end ? (tr.allowed >> lu.shift) & lu.allowed : 0u;
           m[j] = mul_add(lu.E, from_bits<T>(tr.k[0]), mul_add(lu.s, from_bits<T>(tr.k[1]),
                  mul_add(lu.u, from_bits<T>(tr.k[2]), T(0))));
@@ -735,8 +823,9 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
                 }
             }
             survivors += (u32)(n0 + n1);
-            if (n0 != 0.0f) atomicAdd(reinterpret_cast<u32*>(&sh.cell[cell_of(c[j] + axis[0])]), (u32)n0);
-            if (n1 != 0.0f) atomicAdd(reinterpret_cast<u32*>(&sh.cell[cell_of(c[j] + axis[1])]), (u32)n1);
+            const int cell0 = cell_of(c[j] + axis[0]), cell1 = cell_of(c[j] + axis[1]);
+            if (n0 != 0.0f) { atomicAdd(reinterpret_cast<u32*>(&sh.cell[cell0]), (u32)n0); lowest = min(lowest, (u32)cell0); }
+            if (n1 != 0.0f) { atomicAdd(reinterpret_cast<u32*>(&sh.cell[cell1]), (u32)n1); lowest = min(lowest, (u32)cell1); }
           }
           continue;
         }
@@ -807,7 +896,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
           for (int w = 0; w < 4; ++w)
             if (cand[w]) {
               if (at < limit) {
-                const u32 code = room ? (unit << 8) | ((t0 + (w >> 1)) << 1) | (w & 1) : NO_CODE;
+                const u32 code = room ? (unit << 8) | ((u32)sh.live[min(t0 + (w >> 1), t_end - 1)] << 1) | (w & 1) : NO_CODE;
                 if (PARETO) {
                   sh.cand_a[at] = room ? (u64)mem[w] : U64MAX; sh.cand_b[at] = room ? (u64)comm[w] : U64MAX; sh.cand_i[at] = code;
                 } else {
@@ -819,6 +908,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
           if (!room) return t0;
         }
       }
+      if (!PARETO && !SECOND && lowest < CELLS) atomicMin(&sh.least_cell[k], lowest);
       return ALL_STEPS;
     };
 
@@ -862,9 +952,27 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
           while ((run += (u32)sh.cell[lane * PER + q]) < args.max_entries) ++q;
           sh.limit_cell = lane * PER + q;
         }
+        // and only the units with a survivor that low are walked again
+        __syncwarp();
+        const u32 limit = sh.limit_cell;
+        u32 n = 0;
+        for (u32 base = 0; base < n_heavy; base += 32) {
+          const bool again = base + lane < n_heavy && sh.least_cell[base + lane] <= limit;
+          const u16 p = sh.heavy[min(base + lane, n_heavy - 1)];
+          const u32 votes = __ballot_sync(0xffffffffu, again);
+          if (again) sh.heavy[n + __popc(votes & ((1u << lane) - 1u))] = p;
+          n += __popc(votes);
+          __syncwarp();
+        }
+        if (lane == 0) sh.n_heavy = n;
       }
     }
     __syncthreads();
+    if (!PARETO) {
+      n_heavy = sh.n_heavy;
+      if (n_heavy == 0) continue;
+      deal();
+    }
     u32 item = ALL_STEPS, from = 0;                  // the warp's item in hand and the triple to resume at
     for (;;) {
       if (tid == 0) { sh.full = 0; sh.n_hits = 0; }
@@ -888,19 +996,17 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
       const bool full = sh.full != 0;
       if (PARETO) {
         if (!full) break;
-        resolve_candidates<NM>(sp, sh, n_resolved, modemap, cap_x, host_x);
-        const int n = cut_buffer<KIND>(sh, min((int)sh.n_cand, CAND_CAP), 0);
-        if (n > KEEP_CAP) { overflowed = true; break; }
+        const int n = drop_dominated(sh, min((int)sh.n_cand, CAND_CAP));
+        if (n > CAND_CAP - STEP_CAP) { overflowed = true; break; }
         __syncthreads();
         if (tid == 0) sh.n_cand = (u32)n;
-        n_resolved = n;
       } else {
         // the hits' points, as many hits at a time as surely fit
         const u32 n_hits = min(sh.n_hits, (u32)HIT_CAP);
         for (u32 base = 0; base < n_hits;) {
           u32 room = (CAND_CAP - sh.n_cand) / (2 * NM);
           if (room < min(n_hits - base, 32u)) {
-            const int n = cut_buffer<KIND>(sh, (int)sh.n_cand, (int)args.max_entries);
+            const int n = rank_candidates<KIND>(sh, (int)sh.n_cand, (int)args.max_entries);
             if (n == (int)args.max_entries) threshold = Key{sh.cand_a[n - 1], sh.cand_b[n - 1], sh.cand_i[n - 1]};
             __syncthreads();
             if (tid == 0) sh.n_cand = (u32)n;
@@ -925,12 +1031,14 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
   int n_list = 0;
   if (!overflowed) {
     if (PARETO) {
-      resolve_candidates<NM>(sp, sh, n_resolved, modemap, cap_x, host_x);
+      n_list = drop_dominated(sh, (int)sh.n_cand);
+      resolve_candidates<NM>(sp, sh, n_list, modemap, cap_x, host_x);
+      n_list = rank_candidates<KIND>(sh, n_list, 0);
     } else {
       for (int o = 16; o > 0; o >>= 1) survivors += __shfl_xor_sync(0xffffffffu, survivors, o);
       if (lane == 0 && survivors) atomicAdd(&sh.survivors, survivors);
+      n_list = rank_candidates<KIND>(sh, (int)sh.n_cand, (int)args.max_entries);
     }
-    n_list = cut_buffer<KIND>(sh, (int)sh.n_cand, (int)args.max_entries);
     overflowed = PARETO && n_list > KEEP_CAP;
     __syncthreads();
   }
