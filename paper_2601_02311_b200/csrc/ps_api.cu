@@ -90,20 +90,21 @@ int ensure_scratch(ps_ctx* ctx, size_t bytes) {
   return PS_OK;
 }
 
-// a kernel-reported problem seen by an earlier status copy
+// ST_* bits of the problems that kernels have reported
+u32 reported(const ps_ctx* ctx) {
+  u32 st = 0;
+  for (u32 b = 0; b < 8; ++b)
+    if (ctx->h->status[b]) st |= 1u << b;
+  return st;
+}
+
+// a problem that a kernel has reported by now
 int pending_device_error(ps_ctx* ctx) {
-  const u32 st = *ctx->h_status & ~(u32)ST_TRUNCATED;     // a truncated frontier blocks nothing
-  if (st) return PS_E_DEVICE;
-  return PS_OK;
+  return reported(ctx) & ~(u32)ST_TRUNCATED ? PS_E_DEVICE : PS_OK;     // a truncated frontier blocks nothing
 }
 
 // flag bits a filter may require
 constexpr u32 KNOWN_FLAGS = (PS_F_PAPER_PRICED << 1) - 1u;
-
-int enqueue_status_copy(ps_ctx* ctx) {
-  CUDA_OK(cudaMemcpyAsync(ctx->h_status, ctx->d_status, sizeof(u32), cudaMemcpyDeviceToHost, ctx->stream));
-  return PS_OK;
-}
 
 }  // namespace
 
@@ -140,19 +141,19 @@ int ps_create(ps_ctx** out, int device, void* cuda_stream) {
   ctx->stream = static_cast<cudaStream_t>(cuda_stream);
   ctx->scratch = nullptr;
   ctx->scratch_bytes = 0;
-  ctx->d_status = nullptr;
-  ctx->h_status = nullptr;
+  ctx->d_lengths = nullptr;
+  ctx->h = nullptr;
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { delete ctx; return PS_E_CUDA; }
   ctx->sm_count = prop.multiProcessorCount;
   ctx->compact_calls = 0;
-  if (cudaMalloc(&ctx->d_status, 4 * sizeof(u32)) != cudaSuccess ||
-      cudaMallocHost(&ctx->h_status, sizeof(u32)) != cudaSuccess ||
-      cudaMemsetAsync(ctx->d_status, 0, 4 * sizeof(u32), ctx->stream) != cudaSuccess) {
+  if (cudaMalloc(&ctx->d_lengths, 2 * sizeof(u32)) != cudaSuccess ||
+      cudaHostAlloc(reinterpret_cast<void**>(&ctx->h), sizeof(HostWords), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess ||
+      cudaMemsetAsync(ctx->d_lengths, 0, 2 * sizeof(u32), ctx->stream) != cudaSuccess) {
     ps_destroy(ctx);
     return PS_E_CUDA;
   }
-  *ctx->h_status = 0;
+  for (volatile u32& w : ctx->h->status) w = 0;
   if (ensure_scratch(ctx, size_t(8) << 20) != PS_OK) { ps_destroy(ctx); return PS_E_CUDA; }
   *out = ctx;
   return PS_OK;
@@ -163,8 +164,8 @@ void ps_destroy(ps_ctx* ctx) {
   DeviceGuard guard(ctx->device);
   cudaStreamSynchronize(ctx->stream);
   if (ctx->scratch) cudaFree(ctx->scratch);
-  if (ctx->d_status) cudaFree(ctx->d_status);
-  if (ctx->h_status) cudaFreeHost(ctx->h_status);
+  if (ctx->d_lengths) cudaFree(ctx->d_lengths);
+  if (ctx->h) cudaFreeHost(ctx->h);
   delete ctx;
 }
 
@@ -172,16 +173,48 @@ int ps_status(ps_ctx* ctx) {
   if (!ctx) return PS_E_NULLPTR;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return PS_E_CUDA;
-  CUDA_OK(cudaMemcpyAsync(ctx->h_status, ctx->d_status, sizeof(u32), cudaMemcpyDeviceToHost, ctx->stream));
   CUDA_OK(cudaStreamSynchronize(ctx->stream));
   int rc = pending_device_error(ctx);
-  if (rc == PS_OK && (*ctx->h_status & ST_TRUNCATED)) rc = PS_E_TRUNCATED;
-  if (rc != PS_OK) {
-    *ctx->h_status = 0;
-    CUDA_OK(cudaMemsetAsync(ctx->d_status, 0, sizeof(u32), ctx->stream));
-    CUDA_OK(cudaStreamSynchronize(ctx->stream));
-  }
+  if (rc == PS_OK && (reported(ctx) & ST_TRUNCATED)) rc = PS_E_TRUNCATED;
+  if (rc != PS_OK)
+    for (volatile u32& w : ctx->h->status) w = 0;
   return rc;
+}
+
+// The order in which the sweeps' blocks take the models: most expected work first, so
+// that the blocks still running when the grid runs out are short ones.  A sweep block's
+// duration grows with the number of factorisations that pass the composition tests for
+// its model (T divides the heads, K divides the layers, T within the valid tensor
+// degree): only those have survivors under a filter that requires a valid composition,
+// and a unit with survivors costs several times one without.  The count is a sum over
+// the distinct (T, K) pairs of the space, weighted by how many device counts have them.
+static void sweep_degrees(ps_space* sp) {        // T -> (K, number of factorisations)
+  auto& by_t = sp->degrees;
+  for (const Fact& f : sp->facts) {
+    if (f.T > sp->dev.tp_max_valid) continue;
+    auto t = std::find_if(by_t.begin(), by_t.end(), [&](const auto& e) { return e.first == f.T; });
+    if (t == by_t.end()) { by_t.push_back({f.T, {}}); t = by_t.end() - 1; }
+    auto k = std::find_if(t->second.begin(), t->second.end(), [&](const auto& e) { return e.first == f.K; });
+    if (k == t->second.end()) t->second.push_back({f.K, 1u}); else ++k->second;
+  }
+}
+static void sweep_order(ps_space* sp, const ps_model_shape* models, u32 n_models) {
+  std::vector<u32> work(n_models, 0);
+  for (u32 i = 0; i < n_models; ++i)
+    for (const auto& t : sp->degrees) {
+      if (models[i].heads % t.first) continue;
+      for (const auto& k : t.second)
+        if (models[i].layers % k.first == 0) work[i] += k.second;
+    }
+  sp->order.resize(n_models);
+  for (u32 i = 0; i < n_models; ++i) sp->order[i] = i;
+  // (among models with the same count the smaller first: more of its points fit a capacity)
+  std::stable_sort(sp->order.begin(), sp->order.end(), [&](u32 a, u32 b) {
+    if (work[a] != work[b]) return work[a] > work[b];
+    const u64 pa = (u64)models[a].layers * models[a].hidden * models[a].hidden;
+    const u64 pb = (u64)models[b].layers * models[b].hidden * models[b].hidden;
+    return pa < pb;
+  });
 }
 
 // ------------------------------------------------------------------ space
@@ -271,45 +304,12 @@ int ps_space_create(ps_ctx* ctx, const ps_space_desc* desc, ps_space** out) {
   d.recs = sp->d_recs;
   d.facts = sp->d_facts;
   d.order = sp->d_order;
+  sweep_degrees(sp);
   int rc = ps_space_set_models(sp, desc->models, desc->n_models);
   if (rc == PS_OK && cudaStreamSynchronize(ctx->stream) != cudaSuccess) rc = PS_E_CUDA;
   if (rc != PS_OK) { ps_space_destroy(sp); return rc; }
   *out = sp;
   return PS_OK;
-}
-
-// The order in which the sweeps' blocks take the models: most expected work first, so
-// that the blocks still running when the grid runs out are short ones.  A sweep block's
-// duration grows with the number of factorisations that pass the composition tests for
-// its model (T divides the heads, K divides the layers, T within the valid tensor
-// degree): only those have survivors under a filter that requires a valid composition,
-// and a unit with survivors costs several times one without.  The count is a sum over
-// the distinct (T, K) pairs of the space, weighted by how many device counts have them.
-static void sweep_order(ps_space* sp, const ps_model_shape* models, u32 n_models) {
-  std::vector<std::pair<u32, std::vector<std::pair<u32, u32>>>> by_t;   // T -> (K, number of factorisations)
-  for (const Fact& f : sp->facts) {
-    if (f.T > sp->dev.tp_max_valid) continue;
-    auto t = std::find_if(by_t.begin(), by_t.end(), [&](const auto& e) { return e.first == f.T; });
-    if (t == by_t.end()) { by_t.push_back({f.T, {}}); t = by_t.end() - 1; }
-    auto k = std::find_if(t->second.begin(), t->second.end(), [&](const auto& e) { return e.first == f.K; });
-    if (k == t->second.end()) t->second.push_back({f.K, 1u}); else ++k->second;
-  }
-  std::vector<u32> work(n_models, 0);
-  for (u32 i = 0; i < n_models; ++i)
-    for (const auto& t : by_t) {
-      if (models[i].heads % t.first) continue;
-      for (const auto& k : t.second)
-        if (models[i].layers % k.first == 0) work[i] += k.second;
-    }
-  sp->order.resize(n_models);
-  for (u32 i = 0; i < n_models; ++i) sp->order[i] = i;
-  // (among models with the same count the smaller first: more of its points fit a capacity)
-  std::stable_sort(sp->order.begin(), sp->order.end(), [&](u32 a, u32 b) {
-    if (work[a] != work[b]) return work[a] > work[b];
-    const u64 pa = (u64)models[a].layers * models[a].hidden * models[a].hidden;
-    const u64 pb = (u64)models[b].layers * models[b].hidden * models[b].hidden;
-    return pa < pb;
-  });
 }
 
 int ps_space_set_models(ps_space* sp, const ps_model_shape* models, uint32_t n_models) {
@@ -321,15 +321,25 @@ int ps_space_set_models(ps_space* sp, const ps_model_shape* models, uint32_t n_m
     if (!shape_is_small(models[i], sp->dev.tp_coll, sp->dev.accum, sp->dev.repl)) all_small = 0;
   }
   sp->dev.all_small = all_small;
-  sweep_order(sp, models, n_models);
   ps_ctx* ctx = sp->ctx;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return PS_E_CUDA;
-  CUDA_OK(cudaMemcpyAsync(sp->d_order, sp->order.data(), sizeof(u32) * (size_t)n_models, cudaMemcpyHostToDevice,
-                          ctx->stream));
+  // (blocks of a table that fits the GPU at once all start together: any order will do,
+  // and the one that is there stays)
+  const bool by_work = n_models > (u32)ctx->sm_count;
+  if (by_work || sp->order.empty()) {
+    if (by_work) {
+      sweep_order(sp, models, n_models);
+    } else {
+      sp->order.resize(n_models);
+      for (u32 i = 0; i < n_models; ++i) sp->order[i] = i;
+    }
+    CUDA_OK(cudaMemcpyAsync(sp->d_order, sp->order.data(), sizeof(u32) * (size_t)n_models, cudaMemcpyHostToDevice,
+                            ctx->stream));
+  }
   CUDA_OK(cudaMemcpyAsync(sp->d_shapes, models, sizeof(ps_model_shape) * (size_t)n_models,
                           cudaMemcpyHostToDevice, ctx->stream));
-  CUDA_OK(launch_model_derive(sp->d_shapes, sp->d_recs, n_models, ctx->d_status, ctx->stream));
+  CUDA_OK(launch_model_derive(sp->d_shapes, sp->d_recs, n_models, ctx->h->status, ctx->stream));
   return PS_OK;
 }
 
@@ -338,7 +348,7 @@ int ps_space_rederive(ps_space* sp) {
   ps_ctx* ctx = sp->ctx;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return PS_E_CUDA;
-  CUDA_OK(launch_model_derive(sp->d_shapes, sp->d_recs, sp->dev.n_models, ctx->d_status, ctx->stream));
+  CUDA_OK(launch_model_derive(sp->d_shapes, sp->d_recs, sp->dev.n_models, ctx->h->status, ctx->stream));
   return PS_OK;
 }
 
@@ -416,7 +426,7 @@ int ps_eval_batch(ps_ctx* ctx, const ps_space* sp, uint64_t first, uint64_t coun
   a.out = out;
   a.idx_out = d_idx_out;
   a.n_out = d_n_out;
-  a.status = ctx->d_status;
+  a.status = ctx->h->status;
   if (!filter) {
     CUDA_OK(launch_eval_materialise(sp->dev, a, ctx->stream));
   } else {
@@ -435,15 +445,15 @@ int ps_eval_batch(ps_ctx* ctx, const ps_space* sp, uint64_t first, uint64_t coun
     a.tile_offset = reinterpret_cast<u64*>(base + 2 * cnt_bytes + 16);
     // the list's length: one of the context's two counters, zero by now (the previous
     // compaction's scan cleared it); this call's scan clears the other
-    a.n_nonempty = ctx->d_status + 2 + (ctx->compact_calls & 1u);
-    a.n_nonempty_other = ctx->d_status + 2 + ((ctx->compact_calls + 1) & 1u);
+    a.n_nonempty = ctx->d_lengths + (ctx->compact_calls & 1u);
+    a.n_nonempty_other = ctx->d_lengths + ((ctx->compact_calls + 1) & 1u);
     ++ctx->compact_calls;
     eval_plan_runs(a);
     CUDA_OK(launch_eval_count(sp->dev, a, ctx->stream));
     CUDA_OK(launch_tile_scan(a, ctx->stream));
     CUDA_OK(launch_eval_write(sp->dev, a, ctx->stream));
   }
-  return enqueue_status_copy(ctx);
+  return PS_OK;
 }
 
 // ------------------------------------------------------------------ sweeps
@@ -476,9 +486,9 @@ int ps_sweep_pareto(ps_ctx* ctx, const ps_space* sp, const ps_filter* filter,
   s.skip_rejected = filter->skip_rejected ? 1u : 0u;
   s.out = d_out;
   s.counts = d_counts;
-  s.status = ctx->d_status;
+  s.status = ctx->h->status;
   CUDA_OK(launch_sweep((int)reduce_kind, sp->dev, s, ctx->sm_count, ctx->stream));
-  return enqueue_status_copy(ctx);
+  return PS_OK;
 }
 
 // ------------------------------------------------------------------ one composition
@@ -497,24 +507,18 @@ int ps_check_composition(ps_ctx* ctx, const ps_model_shape* shape, uint32_t N, u
   if (!shape_in_range(*shape, tp_coll_per_layer)) return PS_E_RANGE;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return PS_E_CUDA;
-  int rc = ensure_scratch(ctx, 1024);
-  if (rc != PS_OK) return rc;
-  char* base = static_cast<char*>(ctx->scratch);
-  ps_model_shape* d_shape = reinterpret_cast<ps_model_shape*>(base);
-  ModelRec* d_rec = reinterpret_cast<ModelRec*>(base + 256);
-  ps_front_entry* d_out = reinterpret_cast<ps_front_entry*>(base + 512);
-  CUDA_OK(cudaMemcpyAsync(d_shape, shape, sizeof(ps_model_shape), cudaMemcpyHostToDevice, ctx->stream));
-  CUDA_OK(launch_model_derive(d_shape, d_rec, 1, ctx->d_status, ctx->stream));
   // Table 2: tensor axis (S,S,S,S) or (S,S,S,R), pipeline axis (S,S,S,R); an axis
   // of degree 1 is absent.  Activation mode of the tensor axis: digit 3 of its code.
   const bool tp_form = (T == 1) || code_tp == PS_CODE_TP_SEQPAR || code_tp == PS_CODE_TP;
   const bool pp_form = (K == 1) || code_pp == PS_CODE_PP;
   const u32 tau = ((code_tp / 125) % 5 == PS_MODE_S) ? 0 : 1;
-  CUDA_OK(launch_check_point(d_rec, Fact{N, T, K, D}, act_variant, tau, code_dp, tp_max_valid,
+  // the shape travels with the launch and the answer comes back through mapped memory: one
+  // launch and one wait
+  CUDA_OK(launch_check_point(*shape, Fact{N, T, K, D}, act_variant, tau, code_dp, tp_max_valid,
                              tp_coll_per_layer, (tp_form && pp_form) ? 1 : 0, comm_kind, cap_bytes,
-                             d_out, ctx->stream));
-  CUDA_OK(cudaMemcpyAsync(h_out, d_out, sizeof(ps_front_entry), cudaMemcpyDeviceToHost, ctx->stream));
+                             &ctx->h->entry, ctx->h->status, ctx->stream));
   CUDA_OK(cudaStreamSynchronize(ctx->stream));
+  *h_out = ctx->h->entry;
   return PS_OK;
 }
 
@@ -581,8 +585,8 @@ int ps_verify_batch(ps_ctx* ctx, const ps_verify_shape* shape, const ps_verify_c
   if (n == 0) return PS_OK;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return PS_E_CUDA;
-  CUDA_OK(launch_verify(s, d_cases, n, d_data, data_len, d_theta_out, d_out, ctx->d_status, ctx->stream));
-  return enqueue_status_copy(ctx);
+  CUDA_OK(launch_verify(s, d_cases, n, d_data, data_len, d_theta_out, d_out, ctx->h->status, ctx->stream));
+  return PS_OK;
 }
 
 // ------------------------------------------------------------------ measurement

@@ -425,10 +425,12 @@ __device__ __forceinline__ LocalPoint decode_local(const SpaceDev& sp, u32 lidx)
   return p;
 }
 
-// status word bits set by kernels
+// problems that kernels report, as bits (ps_status) and each with a word of host memory that
+// the kernel sets (report): a store over the link when something is wrong, nothing otherwise
 enum : u32 {
   ST_BAD_SHAPE = 1u << 0,      // a model shape outside the supported ranges
   ST_SELF_CHECK = 1u << 2,     // an emitted entry did not re-evaluate to itself
   ST_TRUNCATED = 1u << 3,      // a frontier was longer than the caller's max_entries (a notice, not a fault)
   ST_BAD_CASE = 1u << 4        // a verifier case outside the supported ranges or the given data
 };
+__device__ __forceinline__ void report(volatile u32* status, u32 bit) { status[__ffs(bit) - 1] = 1u; }

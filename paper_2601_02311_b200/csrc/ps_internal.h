@@ -6,14 +6,19 @@
 #include "ps_device.cuh"
 
 // ---- the opaque handles of ps.h
+#include <utility>
 #include <vector>
+struct HostWords {
+  volatile u32 status[8];      // one word per ST_* bit, set by the kernel that meets the problem (report)
+  ps_front_entry entry;        // ps_check_composition's answer
+};
 struct ps_ctx {
   int device;
   cudaStream_t stream;
   void* scratch;
   size_t scratch_bytes;
-  u32* d_status;      // 16 bytes: the status word, then (at +2) the two list lengths of the compaction
-  u32* h_status;      // pinned
+  u32* d_lengths;     // the two list lengths of the compaction
+  HostWords* h;       // pinned host memory that kernels write to (nothing has to be copied back)
   u32 compact_calls;  // compactions enqueued so far (picks which list length a call uses)
   int sm_count;
 };
@@ -30,6 +35,7 @@ struct ps_space {
   Fact* d_facts;
   u32* d_order;                   // see SpaceDev::order
   std::vector<u32> order;
+  std::vector<std::pair<u32, std::vector<std::pair<u32, u32>>>> degrees;   // see sweep_order
   SpaceDev dev;
 };
 
@@ -48,7 +54,7 @@ struct SweepArgs {
   u32 skip_rejected;    // do not evaluate factorisations whose composition bits miss a required flag
   ps_front_entry* out;
   u32* counts;
-  u32* status;
+  volatile u32* status;
 };
 
 cudaError_t launch_sweep(int kind, const SpaceDev& sp, const SweepArgs& a, int sm_count, cudaStream_t stream);
@@ -87,7 +93,7 @@ struct EvalArgs {
   u32* n_nonempty_other;    // the next compaction's counter: the scan kernel clears it, so that no
                             // call needs a memset of its own (calls alternate between two counters)
   u64* tile_offset;         // [n_runs <= n_tiles] survivors of each run, then (scan) of all runs before it
-  u32* status;
+  volatile u32* status;
 };
 
 void eval_plan_runs(EvalArgs& a);   // fills n_runs, run_len from n_tiles (current device)
@@ -98,17 +104,17 @@ cudaError_t launch_eval_write(const SpaceDev& sp, const EvalArgs& a, cudaStream_
 
 // ---- small kernels
 cudaError_t launch_model_derive(const ps_model_shape* d_shapes, ModelRec* d_recs, u32 n,
-                                u32* status, cudaStream_t stream);
-cudaError_t launch_check_point(const ModelRec* d_rec, Fact f, u32 v, u32 tau, u32 code_dp,
+                                volatile u32* status, cudaStream_t stream);
+cudaError_t launch_check_point(const ps_model_shape& shape, Fact f, u32 v, u32 tau, u32 code_dp,
                                u32 tp_max_valid, u32 tp_coll, u32 axis_form, u32 comm_kind,
-                               u64 cap_bytes, ps_front_entry* d_out, cudaStream_t stream);
+                               u64 cap_bytes, ps_front_entry* out, volatile u32* status, cudaStream_t stream);
 cudaError_t launch_select(const ps_select_query* d_q, u64 n, u32 head_num, u32 head_den, u32 layer_num,
                           u32 layer_den, u32 tp_degree, ps_select_result* d_out, cudaStream_t stream);
 cudaError_t launch_int_peak(u32 blocks, u32 iters, u32* d_sink, cudaStream_t stream);
 
 // ---- brute-force verifier
 cudaError_t launch_verify(const ps_verify_shape& s, const ps_verify_case* d_cases, u64 n, const double* d_data,
-                          u64 data_len, double* d_theta_out, ps_verify_result* d_out, u32* status,
+                          u64 data_len, double* d_theta_out, ps_verify_result* d_out, volatile u32* status,
                           cudaStream_t stream);
 
 cudaError_t launch_select_compare(const SpaceDev& sp, u32 unit_begin, u32 unit_end, u32 N, u64 device_bytes, u32 fast,

@@ -10,17 +10,7 @@ namespace {
 // formula; this is the per-layer count of the selective-recomputation analysis
 // it cites for sequence parallelism): 34 S b H + 5 a S^2 b bytes stored,
 // 2 S b H with full checkpointing.
-__global__ void k_model_derive(const ps_model_shape* __restrict__ shapes, ModelRec* __restrict__ recs,
-                               u32 n, u32* status) {
-  const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  // 48-byte shape as three 16-byte loads
-  ps_model_shape s;
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(shapes + i);
-    uint4* dst = reinterpret_cast<uint4*>(&s);
-    dst[0] = __ldg(src); dst[1] = __ldg(src + 1); dst[2] = __ldg(src + 2);
-  }
+__device__ __forceinline__ ModelRec derive_record(const ps_model_shape& s, volatile u32* status) {
   bool ok = s.layers >= 1 && s.layers <= (1u << 10) && s.hidden >= 1 && s.hidden <= (1u << 16) &&
             s.heads >= 1 && s.heads <= (1u << 16) && s.vocab >= 1 && s.vocab <= (1u << 24) &&
             s.seq >= 1 && s.seq <= (1u << 17) && s.micro_batch >= 1 && s.micro_batch <= (1u << 10) &&
@@ -56,17 +46,34 @@ __global__ void k_model_derive(const ps_model_shape* __restrict__ shapes, ModelR
     // keep every later division and product harmless
     r.P = 1; r.unit = 0; r.Sbh = 1; r.L = 1; r.heads = 1;
     r.wT = r.wO = r.wG = r.wA = 1;
-    atomicOr(status, ST_BAD_SHAPE);
+    report(status, ST_BAD_SHAPE);
   }
-  recs[i] = r;
+  return r;
 }
 
-__global__ void k_check_point(const ModelRec* rec, Fact f, u32 v, u32 tau, u32 code_dp,
+__global__ void k_model_derive(const ps_model_shape* __restrict__ shapes, ModelRec* __restrict__ recs,
+                               u32 n, volatile u32* status) {
+  const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  // 48-byte shape as three 16-byte loads
+  ps_model_shape s;
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(shapes + i);
+    uint4* dst = reinterpret_cast<uint4*>(&s);
+    dst[0] = __ldg(src); dst[1] = __ldg(src + 1); dst[2] = __ldg(src + 2);
+  }
+  recs[i] = derive_record(s, status);
+}
+
+// One composition of one shape, by one thread; `out` is host memory.  A call is a launch and
+// a wait: as a copy in, two kernels and a copy back it took 28 us, so @@.
+__global__ void k_check_point(const __grid_constant__ ps_model_shape shape, Fact f, u32 v, u32 tau, u32 code_dp,
                               u32 tp_max_valid, u32 tp_coll, u32 axis_form, u32 comm_kind,
-                              u64 cap_bytes, ps_front_entry* out) {
+                              u64 cap_bytes, ps_front_entry* out, volatile u32* status) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const u32 th = code_dp % 5, om = (code_dp / 5) % 5, gr = (code_dp / 25) % 5, ac = (code_dp / 125) % 5;
-  const PointOut p = eval_point(*rec, f, v, tau, th, om, gr, ac, tp_max_valid, tp_coll, axis_form != 0);
+  const ModelRec rec = derive_record(shape, status);
+  const PointOut p = eval_point(rec, f, v, tau, th, om, gr, ac, tp_max_valid, tp_coll, axis_form != 0);
   ps_front_entry e;
   e.mem = p.mem;
   e.comm = comm_kind == PS_COMM_PAPER ? p.comm_paper : p.comm_paper + p.comm_ext;
@@ -335,17 +342,17 @@ __global__ void __launch_bounds__(256) k_int_peak(u32 iters, u32* sink) {
 
 }  // namespace
 
-cudaError_t launch_model_derive(const ps_model_shape* d_shapes, ModelRec* d_recs, u32 n, u32* status,
+cudaError_t launch_model_derive(const ps_model_shape* d_shapes, ModelRec* d_recs, u32 n, volatile u32* status,
                                 cudaStream_t stream) {
   k_model_derive<<<(n + 127) / 128, 128, 0, stream>>>(d_shapes, d_recs, n, status);
   return cudaGetLastError();
 }
 
-cudaError_t launch_check_point(const ModelRec* d_rec, Fact f, u32 v, u32 tau, u32 code_dp,
+cudaError_t launch_check_point(const ps_model_shape& shape, Fact f, u32 v, u32 tau, u32 code_dp,
                                u32 tp_max_valid, u32 tp_coll, u32 axis_form, u32 comm_kind,
-                               u64 cap_bytes, ps_front_entry* d_out, cudaStream_t stream) {
-  k_check_point<<<1, 32, 0, stream>>>(d_rec, f, v, tau, code_dp, tp_max_valid, tp_coll, axis_form,
-                                      comm_kind, cap_bytes, d_out);
+                               u64 cap_bytes, ps_front_entry* out, volatile u32* status, cudaStream_t stream) {
+  k_check_point<<<1, 32, 0, stream>>>(shape, f, v, tau, code_dp, tp_max_valid, tp_coll, axis_form,
+                                      comm_kind, cap_bytes, out, status);
   return cudaGetLastError();
 }
 

@@ -72,8 +72,8 @@ extern "C" int ps_eval_compact_noalloc(ps_ctx* ctx, const ps_space* sp, uint64_t
     return PS_E_ALIGN;
   if (filter->comm_kind > PS_COMM_PAPER_PLUS_EXT || (filter->require_flags & ~((PS_F_PAPER_PRICED << 1) - 1u)))
     return PS_E_RANGE;
-  const u32 seen = *ctx->h_status & ~(u32)ST_TRUNCATED;   // a kernel-reported problem of an earlier call
-  if (seen) return PS_E_DEVICE;
+  for (u32 b = 0; b < 8; ++b)                              // a kernel-reported problem of an earlier call
+    if (ctx->h->status[b] && (1u << b) != ST_TRUNCATED) return PS_E_DEVICE;
   CurrentDevice guard(ctx->device);
   if (!guard.ok) return PS_E_CUDA;
   if (count == 0) {
@@ -94,7 +94,7 @@ extern "C" int ps_eval_compact_noalloc(ps_ctx* ctx, const ps_space* sp, uint64_t
   a.out = out;
   a.idx_out = d_idx_out;
   a.n_out = d_n_out;
-  a.status = ctx->d_status;
+  a.status = ctx->h->status;
   a.has_filter = 1;
   a.cap_bytes = filter->cap_bytes;
   a.host_cap = filter->host_cap;
@@ -102,8 +102,8 @@ extern "C" int ps_eval_compact_noalloc(ps_ctx* ctx, const ps_space* sp, uint64_t
   unsigned char* bytes = static_cast<unsigned char*>(base);
   a.tile_count = reinterpret_cast<u32*>(bytes);
   a.nonempty = reinterpret_cast<u32*>(bytes + COUNT_BYTES);
-  a.n_nonempty = ctx->d_status + 2 + (ctx->compact_calls & 1u);          // the context's alternating list lengths
-  a.n_nonempty_other = ctx->d_status + 2 + ((ctx->compact_calls + 1) & 1u);
+  a.n_nonempty = ctx->d_lengths + (ctx->compact_calls & 1u);          // the context's alternating list lengths
+  a.n_nonempty_other = ctx->d_lengths + ((ctx->compact_calls + 1) & 1u);
   ++ctx->compact_calls;
   a.tile_offset = reinterpret_cast<u64*>(bytes + 2 * COUNT_BYTES + LENGTH_BYTES);
   eval_plan_runs(a);
@@ -116,7 +116,5 @@ extern "C" int ps_eval_compact_noalloc(ps_ctx* ctx, const ps_space* sp, uint64_t
   if (launch_eval_count(sp->dev, a, ctx->stream) != cudaSuccess) return PS_E_CUDA;
   if (launch_tile_scan(a, ctx->stream) != cudaSuccess) return PS_E_CUDA;
   if (launch_eval_write(sp->dev, a, ctx->stream) != cudaSuccess) return PS_E_CUDA;
-  if (cudaMemcpyAsync(ctx->h_status, ctx->d_status, sizeof(u32), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess)
-    return PS_E_CUDA;
   return PS_OK;
 }

@@ -569,7 +569,7 @@ __device__ __noinline__ void frontier_by_definition(const SpaceDev& sp, const Sw
     for (u64 p = found[ci] + (u64)tid; p < args.max_entries; p += threads) write_empty(out + p);
     if (tid == 0) {
       args.counts[(u64)model * args.n_caps + ci] = found[ci];
-      if (found[ci] > args.max_entries) atomicOr(args.status, ST_TRUNCATED);
+      if (found[ci] > args.max_entries) report(args.status, ST_TRUNCATED);
     }
   }
 }
@@ -1063,7 +1063,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     if (tid == 0) {
       args.counts[(u64)model * args.n_caps + ci] = PARETO ? (u32)n_cap : sh.survivors;
       // a frontier that does not fit the caller's rows: its head is written, the count is the true one
-      if (PARETO && (u32)n_cap > args.max_entries) atomicOr(args.status, ST_TRUNCATED);
+      if (PARETO && (u32)n_cap > args.max_entries) report(args.status, ST_TRUNCATED);
     }
     for (u64 p = (u64)n_cap + tid; p < args.max_entries; p += threads) write_empty(rows + (u64)ci * args.max_entries + p);
   }
@@ -1073,7 +1073,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     const u64 comm = args.comm_kind == PS_COMM_PAPER ? po.comm_paper : po.comm_paper + po.comm_ext;
     const u64 list_mem = PARETO ? sh.cand_a[p] : sh.cand_b[p];
     const u64 list_comm = PARETO ? sh.cand_b[p] : sh.cand_a[p];
-    if (po.mem != list_mem || comm != list_comm) atomicOr(args.status, ST_SELF_CHECK);
+    if (po.mem != list_mem || comm != list_comm) report(args.status, ST_SELF_CHECK);
     for (u32 ci = c_begin; ci < c_end; ++ci)
       if (!PARETO || po.mem <= args.caps[ci])
         write_entry(rows + (u64)ci * args.max_entries + p, po, comm, (u64)model * sp.ppm + lidx);

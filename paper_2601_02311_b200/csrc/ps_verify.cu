@@ -153,7 +153,7 @@ __device__ Books keep_books(const Dims& dm, int D, int pT, int pO, int pG, int p
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS) k_verify(Dims dm, const ps_verify_case* __restrict__ cases, u64 n_cases,
                                                     const double* __restrict__ data, u64 data_len,
-                                                    double* theta_out, ps_verify_result* __restrict__ out, u32* status) {
+                                                    double* theta_out, ps_verify_result* __restrict__ out, volatile u32* status) {
   extern __shared__ __align__(16) double mem[];
   const int tid = threadIdx.x;
   const int P = dm.P, h = dm.h, b = dm.b, units = dm.units, EA = dm.EA;
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(THREADS) k_verify(Dims dm, const ps_verify_cas
           ps_verify_result r;
           r.mem = 0; r.comm = 0; r.host = 0; r.match = 0; r.pad = 0; r.max_rel_err = 0.0;
           out[idx] = r;
-          atomicOr(status, ST_BAD_CASE);
+          report(status, ST_BAD_CASE);
         }
         if (theta_out) for (int e = tid; e < P; e += THREADS) theta_out[idx * (u64)P + e] = 0.0;
         continue;                                          // the same for every thread of the block
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(THREADS) k_verify(Dims dm, const ps_verify_cas
 
 template <int THREADS>
 cudaError_t launch_verify_t(const Dims& dm, const ps_verify_case* d_cases, u64 n, const double* d_data, u64 data_len,
-                            double* d_theta_out, ps_verify_result* d_out, u32* status, cudaStream_t stream) {
+                            double* d_theta_out, ps_verify_result* d_out, volatile u32* status, cudaStream_t stream) {
   const int smem = make_layout(dm.P, dm.EA).total * (int)sizeof(double);      // at most 190 KB
   cudaError_t e = cudaFuncSetAttribute(k_verify<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -460,7 +460,7 @@ cudaError_t launch_verify_t(const Dims& dm, const ps_verify_case* d_cases, u64 n
 }  // namespace
 
 cudaError_t launch_verify(const ps_verify_shape& s, const ps_verify_case* d_cases, u64 n, const double* d_data,
-                          u64 data_len, double* d_theta_out, ps_verify_result* d_out, u32* status,
+                          u64 data_len, double* d_theta_out, ps_verify_result* d_out, volatile u32* status,
                           cudaStream_t stream) {
   Dims dm;
   dm.units = (int)s.units; dm.h = (int)s.h; dm.b = (int)s.b;
