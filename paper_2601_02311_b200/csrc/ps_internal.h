@@ -6,11 +6,13 @@
 #include "ps_device.cuh"
 
 // ---- the opaque handles of ps.h
+#include <mutex>
 #include <utility>
 #include <vector>
 struct HostWords {
   volatile u32 status[8];      // one word per ST_* bit, set by the kernel that meets the problem (report)
-  ps_front_entry entry;        // ps_check_composition's answer
+  ps_front_entry entry;        // ps_check_composition's answer,
+  volatile u32 answered;       // and the number of the call that it answers
 };
 struct ps_ctx {
   int device;
@@ -19,6 +21,8 @@ struct ps_ctx {
   size_t scratch_bytes;
   u32* d_lengths;     // the two list lengths of the compaction
   HostWords* h;       // pinned host memory that kernels write to (nothing has to be copied back)
+  std::mutex* check;  // one ps_check_composition at a time uses h->entry
+  u32 checks;
   u32 compact_calls;  // compactions enqueued so far (picks which list length a call uses)
   int sm_count;
 };
@@ -107,7 +111,7 @@ cudaError_t launch_model_derive(const ps_model_shape* d_shapes, ModelRec* d_recs
                                 volatile u32* status, cudaStream_t stream);
 cudaError_t launch_check_point(const ps_model_shape& shape, Fact f, u32 v, u32 tau, u32 code_dp,
                                u32 tp_max_valid, u32 tp_coll, u32 axis_form, u32 comm_kind,
-                               u64 cap_bytes, ps_front_entry* out, volatile u32* status, cudaStream_t stream);
+                               u64 cap_bytes, HostWords* h, u32 call, cudaStream_t stream);
 cudaError_t launch_select(const ps_select_query* d_q, u64 n, u32 head_num, u32 head_den, u32 layer_num,
                           u32 layer_den, u32 tp_degree, ps_select_result* d_out, cudaStream_t stream);
 cudaError_t launch_int_peak(u32 blocks, u32 iters, u32* d_sink, cudaStream_t stream);
