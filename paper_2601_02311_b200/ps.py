@@ -34,6 +34,7 @@ COMM_PAPER, COMM_PAPER_PLUS_EXT = 0, 1
 REDUCE_PARETO, REDUCE_TOPK = 0, 1
 NO_LIMIT = (1 << 64) - 1
 TOPK_MAX = 64
+PINNED_RESULT_BYTES = 1 << 20       # a sweep's result up to this size is read back through pinned memory
 
 SELECT_QUERY_DTYPE = np.dtype([("param_elems", "<u8"), ("layer_elems", "<u8"), ("device_bytes", "<u8"),
                                ("n_devices", "<u4"), ("w_param", "u1"), ("w_grad", "u1"), ("w_opt", "u1"),
@@ -178,6 +179,11 @@ class Context:
         self._h = None
 
     __del__ = close
+
+    def on_current_stream(self) -> bool:
+        """Whether torch's current stream on the device is the one the library enqueues on."""
+        mine = self.stream.cuda_stream if self.stream is not None else 0
+        return torch.cuda.current_stream(self.device).cuda_stream == mine
 
     def status(self) -> int:
         return _lib.ps_status(self._h)
@@ -359,10 +365,13 @@ class Space:
     # ---- ps_sweep_pareto
     def sweep_into(self, filt: dict, caps, kind: int, max_entries: int, d_out: torch.Tensor,
                    d_counts: torch.Tensor):
+        self._sweep(filt, caps, kind, max_entries, d_out.data_ptr(), d_counts.data_ptr())
+
+    def _sweep(self, filt, caps, kind, max_entries, out_ptr, counts_ptr):
         caps = np.ascontiguousarray(caps, dtype=np.uint64)
         f = _mk_filter(filt)
         _check(_lib.ps_sweep_pareto(self.ctx._h, self._h, C.byref(f), caps.ctypes.data, len(caps),
-                                    kind, max_entries, _dptr(d_out), _dptr(d_counts)),
+                                    kind, max_entries, out_ptr, counts_ptr),
                "ps_sweep_pareto")
 
     def select_compare(self, n_index: int, device_bytes: int, filt: dict, d_frontier: torch.Tensor,
@@ -385,11 +394,22 @@ class Space:
 
     def sweep(self, filt: dict, caps, kind: int, max_entries: int):
         """Returns (entries[n_models, n_caps, max_entries] structured, counts[n_models, n_caps])."""
-        d_out, d_counts = self.alloc_sweep(len(caps), max_entries)
-        self.sweep_into(filt, caps, kind, max_entries, d_out, d_counts)
-        self.last_sweep_status = self.ctx.check_status(allow_truncated=True)
-        entries = d_out.cpu().numpy().view(ENTRY_DTYPE).reshape(self.n_models, len(caps), max_entries)
-        counts = d_counts.cpu().numpy().view(np.uint32).reshape(self.n_models, len(caps))
+        rows = self.n_models * len(caps)
+        at = rows * max_entries * 40                   # the counts lie behind the entries: one copy brings both
+        d_all = torch.empty(at + rows * 4, dtype=torch.uint8, device=self.ctx.torch_device)
+        base = d_all.data_ptr()
+        self._sweep(filt, caps, kind, max_entries, base, base + at)
+        if d_all.numel() <= PINNED_RESULT_BYTES and self.ctx.on_current_stream():
+            # a small result: the copy is enqueued behind the sweep and one wait covers both
+            host = torch.empty(d_all.numel(), dtype=torch.uint8, pin_memory=True)
+            host.copy_(d_all, non_blocking=True)
+            self.last_sweep_status = self.ctx.check_status(allow_truncated=True)
+        else:
+            self.last_sweep_status = self.ctx.check_status(allow_truncated=True)
+            host = d_all.cpu()
+        flat = host.numpy()
+        entries = flat[:at].view(ENTRY_DTYPE).reshape(self.n_models, len(caps), max_entries)
+        counts = flat[at:].view(np.uint32).reshape(self.n_models, len(caps))
         return entries, counts
 
 
