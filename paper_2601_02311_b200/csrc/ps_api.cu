@@ -150,9 +150,9 @@ int ps_create(ps_ctx** out, int device, void* cuda_stream) {
   if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { ps_destroy(ctx); return PS_E_CUDA; }
   ctx->sm_count = prop.multiProcessorCount;
   ctx->compact_calls = 0;
-  if (!ctx->check || cudaMalloc(&ctx->d_lengths, 2 * sizeof(u32)) != cudaSuccess ||
+  if (!ctx->check || cudaMalloc(&ctx->d_lengths, 4 * sizeof(u32)) != cudaSuccess ||
       cudaHostAlloc(reinterpret_cast<void**>(&ctx->h), sizeof(HostWords), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess ||
-      cudaMemsetAsync(ctx->d_lengths, 0, 2 * sizeof(u32), ctx->stream) != cudaSuccess) {
+      cudaMemsetAsync(ctx->d_lengths, 0, 4 * sizeof(u32), ctx->stream) != cudaSuccess) {
     ps_destroy(ctx);
     return PS_E_CUDA;
   }
@@ -440,23 +440,23 @@ int ps_eval_batch(ps_ctx* ctx, const ps_space* sp, uint64_t first, uint64_t coun
     a.cap_bytes = filter->cap_bytes;
     a.host_cap = filter->host_cap;
     a.require_flags = filter->require_flags & ~(u32)PS_F_FEASIBLE;
-    // per group a count and a place in the list of groups with survivors, the list's length,
-    // per run of groups an offset
-    const size_t cnt_bytes = (sizeof(u32) * n_groups + 15) & ~size_t(15);
-    rc = ensure_scratch(ctx, 2 * cnt_bytes + 16 + sizeof(u64) * n_groups);
+    // per group an offset and a place in the list of groups with survivors, per run of
+    // factorisations an offset
+    eval_plan_runs(sp->dev, a);
+    const size_t group_bytes = (sizeof(u32) * n_groups + 15) & ~size_t(15);
+    rc = ensure_scratch(ctx, 2 * group_bytes + sizeof(u64) * (size_t)a.n_runs);
     if (rc != PS_OK) return rc;
     char* base = static_cast<char*>(ctx->scratch);
-    a.tile_count = reinterpret_cast<u32*>(base);
-    a.nonempty = reinterpret_cast<u32*>(base + cnt_bytes);
-    a.tile_offset = reinterpret_cast<u64*>(base + 2 * cnt_bytes + 16);
+    a.group_offset = reinterpret_cast<u32*>(base);
+    a.nonempty = reinterpret_cast<u32*>(base + group_bytes);
+    a.run_offset = reinterpret_cast<u64*>(base + 2 * group_bytes);
     // the list's length: one of the context's two counters, zero by now (the previous
-    // compaction's scan cleared it); this call's scan clears the other
+    // compaction cleared it); this call clears the other
     a.n_nonempty = ctx->d_lengths + (ctx->compact_calls & 1u);
     a.n_nonempty_other = ctx->d_lengths + ((ctx->compact_calls + 1) & 1u);
     ++ctx->compact_calls;
-    eval_plan_runs(a);
+    a.blocks_done = ctx->d_lengths + 2;
     CUDA_OK(launch_eval_count(sp->dev, a, ctx->stream));
-    CUDA_OK(launch_tile_scan(a, ctx->stream));
     CUDA_OK(launch_eval_write(sp->dev, a, ctx->stream));
   }
   return PS_OK;

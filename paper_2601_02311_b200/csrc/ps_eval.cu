@@ -16,27 +16,23 @@
 // (shared -> global, asynchronous), so the warp computes the next array while
 // the previous one drains.
 //
-// Compaction is count -> scan -> write.  The count pass (k_compact_count, one
-// warp per run of up to 32 consecutive groups) never forms a point's bytes or
-// flags: like the sweeps it compares a triple's own bytes with a per-(variant,
-// digit) bound and masks the result with the digits the required flags allow.
-// It stores the survivors of each group and of each run and appends the groups
-// that have survivors to a list.  A single-block scan turns the runs' totals
-// into offsets.  The write pass takes the listed groups one per warp, evaluates
-// them and places their survivors with ballot/popc prefix sums; a group's offset
-// is its run's plus the counts of the run's earlier groups.  Output order is the
-// index order, so the result is unique.
+// Compaction is count -> write.  The count pass (k_compact_count) never forms a point's
+// bytes or flags: a lane owns a factorisation, and a point is one compare of a triple's own
+// bytes with a per-(variant, digit) bound, masked by the digits the required flags allow.
+// It leaves each group's offset in its run of factorisations, appends the groups that have
+// survivors to a list, and its last block turns the runs' totals into offsets.  The write
+// pass takes the listed groups one per warp, evaluates them and places their survivors with
+// ballot/popc prefix sums.  Output order is the index order, so the result is unique.
 #include "ps_device.cuh"
 #include "ps_internal.h"
+#include "ps_lane.cuh"
 
 namespace {
 
 // Launch shapes (blocks of four warps per SM; four are resident at a time).  Materialise is
 // fastest with about one group per warp: short-lived blocks keep the warps of an
 // SM at different stages (set-up, staging, draining stores) and the running
-// warps write neighbouring stretches of every output array.  The count pass
-// prefers long runs of groups per warp (what a model and a factorisation fix is
-// then computed once).  The write pass takes the listed groups round-robin; with
+// warps write neighbouring stretches of every output array.  The write pass takes the listed groups round-robin; with
 // many short blocks the stores of neighbouring groups are in flight together
 // (every point surviving: 0.56 of the copy bandwidth with 32 warps in the grid per
 // SM, 0.62 with 256).
@@ -46,8 +42,10 @@ namespace {
 #ifndef EVAL_GRID_PER_SM_MATERIALISE
 #define EVAL_GRID_PER_SM_MATERIALISE 128
 #endif
-#ifndef EVAL_GRID_PER_SM_COMPACT
-#define EVAL_GRID_PER_SM_COMPACT 2
+// (resident blocks of the write pass: half of 2^23 points surviving 0.067 ms with four, 0.062
+// with five, 0.071 with six, whose registers spill)
+#ifndef EVAL_MIN_BLOCKS_WRITE
+#define EVAL_MIN_BLOCKS_WRITE 5
 #endif
 #ifndef EVAL_GRID_PER_SM_WRITE
 #define EVAL_GRID_PER_SM_WRITE 64
@@ -61,12 +59,6 @@ enum : u32 {
   X_MO3 = 1u << 17,       // one of them is materialised or offloaded
   X_EXT0 = 1u << 18       // the data axis moves nothing beyond Theorem 2's terms
 };
-
-__device__ __forceinline__ u64 mad_small(u64 a, u32 k, u64 acc) {
-  u64 r = (u64)(u32)a * (u64)k + acc;
-  r += (u64)((u32)(a >> 32) * k) << 32;
-  return r;
-}
 
 // static description of a triple when the data axis has several shard positions (d1 = false)
 // or a single device (d1 = true)
@@ -154,9 +146,16 @@ __device__ __forceinline__ void warp_bulk_store(T* __restrict__ dst, const T* bu
   if (lane == 0) asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
+__device__ __forceinline__ void load_record(const SpaceDev& sp, u32 model, ModelRec& rec) {
+  const uint4* src = reinterpret_cast<const uint4*>(&sp.recs[model]);
+  uint4* dst = reinterpret_cast<uint4*>(&rec);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) dst[k] = __ldg(src + k);   // the 96-byte record, 16 bytes at a time
+}
+
 // POW2: every degree of the space is a power of two (no division is compiled in)
 template <int MODE, int NM, bool POW2>
-__global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, EvalArgs a) {
+__global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE ? EVAL_MIN_BLOCKS_WRITE : EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, EvalArgs a) {
   constexpr int N2 = NM * NM, N3 = NM * NM * NM, NC = N3 * NM;
   constexpr int R = (N3 + 31) / 32;
   // materialise: two staging buffers per warp (dynamic shared memory, none in the other modes)
@@ -216,10 +215,7 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
     const u32 v = vt / sp.nt, tau = vt - v * sp.nt;
     if (model != model_cur) {
       model_cur = model;
-      const uint4* src = reinterpret_cast<const uint4*>(&sp.recs[model]);
-      uint4* dst = reinterpret_cast<uint4*>(&rec);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) dst[k] = __ldg(src + k);   // the 96-byte record, 16 bytes at a time
+      load_record(sp, model, rec);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const u32 modes[3] = {th[r], om[r], gr[r]};
@@ -302,13 +298,8 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
     u32 n_kept = 0;
     u64 write_base = 0;
     if (MODE == MODE_WRITE) {
-      // survivors before this group = those of the runs before its run (scanned) plus
-      // those of the run's earlier groups
-      const u32 run = seg / a.run_len;
-      u64 part = 0;
-      for (u32 j = run * a.run_len + lane; j < seg; j += 32) part += a.tile_count[j];
-      for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-      write_base = a.tile_offset[run] + part;
+      // survivors before this group: those of the runs before its run, and of the run's earlier groups
+      write_base = a.run_offset[(u32)(g / sp.nvt - a.first_unit) / EVAL_RUN_UNITS] + a.group_offset[seg];
     }
 
     // flags of a point = what the triple fixes | what the digit fixes | what needs both:
@@ -363,8 +354,11 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
       continue;
     }
 
-#pragma unroll
+    // (a loop: unrolled, its registers spilled the staged path's: 2^25 points 0.191 ms instead
+    // of 0.179)
+#pragma unroll 1
     for (int d = 0; d < NM; ++d) {
+      const u64 act_d = mu_elems(digit_mode(modemap, d), ab.EA, ab.shA, ab.uA, sp.sstar_units);
       const bool d_avail = (avail >> d) & 1u, d_off = (is_o >> d) & 1u, d_notmo = (not_mo >> d) & 1u;
       const u32 fl_digit = (d_avail ? PS_F_ACT_AVAIL : 0) | (d_off ? PS_F_USES_HOST : 0);
       const u32 gi_mask = d_avail ? ~0u : 0u, priced_mask = d_notmo ? ~0u : 0u;
@@ -373,7 +367,7 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
       for (int r = 0; r < R; ++r) {
         const u32 code = lane + 32 * r + d * N3;
         const bool inside = live[r] && (whole || (code >= code_lo && code < code_hi));
-        const u64 mem = mem3[r] + act[d];
+        const u64 mem = mem3[r] + act_d;
         const u64 host = host3[r] + host_add;
         const u32 fl = fl_base[r] | fl_digit | (fl_gi[r] & gi_mask) | (fl_priced[r] & priced_mask);
         if (MODE == MODE_MATERIALISE) {
@@ -415,30 +409,56 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
   if (MODE == MODE_MATERIALISE && lane == 0) bulk_wait_all();
 }
 
-// The count pass of the compaction.  One warp per run of consecutive groups.  What
-// a factorisation fixes is computed once for its (up to four) groups: the lanes'
-// triples' own bytes and host bytes, and for every (variant, digit) the bound the
-// own bytes must stay below for the point to fit the capacity (cap + 1 - activation
-// bytes) and the host budget.  A point then costs one compare, masked by the
-// digits the required flags allow for its triple (fixed for the whole kernel).
-struct CountTables {
-  u64 bound[5][4];       // [digit][variant]
-  __align__(16) double bound_f64[5][4];   // the same as doubles (exact below 2^53), 0 for variants the space lacks
-  u64 host_bound[4];     // the triple's own host bytes must stay below this to offload activations
-};
+// ------------------------------------------------------------------ compaction: count
+// Survivors of the lane's unit among the four variants of one activation digit: a compare
+// per point on the fp64 pipe, masked by its input predicate, counted with predicated fp32
+// adds (small integers are exact).
+__device__ __forceinline__ void count_variants(float* n, double m, const double* b, u32 on) {
+  asm("{\n\t"
+      ".reg .pred q, p0, p1, p2, p3;\n\t"
+      "setp.ne.u32 q, %9, 0;\n\t"
+      "setp.lt.and.f64 p0, %4, %5, q;\n\t"
+      "setp.lt.and.f64 p1, %4, %6, q;\n\t"
+      "setp.lt.and.f64 p2, %4, %7, q;\n\t"
+      "setp.lt.and.f64 p3, %4, %8, q;\n\t"
+      "@p0 add.f32 %0, %0, 0f3F800000;\n\t"
+      "@p1 add.f32 %1, %1, 0f3F800000;\n\t"
+      "@p2 add.f32 %2, %2, 0f3F800000;\n\t"
+      "@p3 add.f32 %3, %3, 0f3F800000;\n\t"
+      "}"
+      : "+f"(n[0]), "+f"(n[1]), "+f"(n[2]), "+f"(n[3])
+      : "d"(m), "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]), "r"(on));
+}
+__device__ __forceinline__ void count_variants(float* n, u64 m, const u64* b, u32 on) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) n[q] += on != 0 && m < b[q] ? 1.0f : 0.0f;
+}
 
-template <int NM, bool POW2>
-__global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_compact_count(SpaceDev sp, EvalArgs a) {
+// bytes of a state under a mode (the same for every lane) in the lane's unit
+template <int NM, typename T, bool HOST_LIMITED>
+__device__ __forceinline__ T state_bytes(const LaneUnit<NM, T, HOST_LIMITED>& lu, u32 mode, T width, u32 sstar_units) {
+  if (mode == PS_MODE_R) return width * lu.E;
+  if (mode == PS_MODE_S) return width * lu.s;
+  if (mode == PS_MODE_SG) return width * (lu.s + as<T>(sstar_units) * lu.u);
+  if (mode == PS_MODE_M) return width * lu.u;
+  return T(0);
+}
+
+// One block per run of 32 consecutive units; a lane owns a unit, the warps share the
+// (Theta, Omega) pairs.  What bounds it: the fp64 pipe (a compare per point), and for small
+// windows the chain of a unit's set-up.  As one warp per run of groups, its lanes the
+// triples, it took 21 us for 2^25 points and was followed by a scan kernel of 3 us; like
+// this it takes 15.
+constexpr int COUNT_WARPS = 8;
+template <int NM, typename T, bool HOST_LIMITED>
+__global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev sp, EvalArgs a) {
   constexpr int N2 = NM * NM, N3 = NM * NM * NM, NC = N3 * NM;
-  constexpr int R = (N3 + 31) / 32;
-  __shared__ CountTables tables[WARPS];
-  const int lane = threadIdx.x & 31;
-  const u32 run = blockIdx.x * WARPS + (threadIdx.x >> 5);
-  if (run >= a.n_runs) return;
-  CountTables& tb = tables[threadIdx.x >> 5];
-  const u32 seg_begin = run * a.run_len;
-  const u32 seg_end = min(seg_begin + a.run_len, a.n_tiles);
-  const u32 groups_per_model = sp.n_facts * sp.nvt;
+  __shared__ unsigned char allowed_of[3][N3];
+  __shared__ u32 cnt[4][32];
+  __shared__ u64 warp_sum[COUNT_WARPS];
+  __shared__ u64 carry;
+  __shared__ u32 last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const u32 modemap = (NM == 5) ? 0x43210u : sp.modemap;
   const u32 req = a.require_flags;
   constexpr u32 CV_BITS = PS_F_CV | PS_F_T_DIV_HEADS | PS_F_K_DIV_LAYERS | PS_F_TP_LE_MAX | PS_F_AXIS_FORM;
@@ -446,7 +466,8 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_compact_count(Spac
   // capacities as exclusive bounds (memory and host bytes stay below 2^62)
   const u64 cap_x = min(a.cap_bytes, (u64)1 << 62) + 1;
   const u64 host_x = min(a.host_cap, (u64)1 << 62) + 1;
-  u32 all = (1u << NM) - 1u, own = 0, is_o = 0, not_mo = 0;
+  constexpr u32 all = (1u << NM) - 1u;
+  u32 own = 0, is_o = 0, not_mo = 0;
 #pragma unroll
   for (int d = 0; d < NM; ++d) {
     const u32 ac = digit_mode(modemap, d);
@@ -454,213 +475,145 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_compact_count(Spac
     if (ac == PS_MODE_O) is_o |= 1u << d;
     if (!in_set(SET_M_OR_O, ac)) not_mo |= 1u << d;
   }
-  // the lane's triples: modes and the activation digits the required flags allow
-  // (bits 0..4, 8..12, 16..20 for the three classes of a factorisation), fixed for the kernel
-  u32 th[R], om[R], gr[R], t_allowed[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const u32 t = lane + 32 * r;
-    const bool live = t < (u32)N3;
-    const u32 tt = live ? t : 0;
-    th[r] = digit_mode(modemap, tt % NM);
-    om[r] = digit_mode(modemap, (tt / NM) % NM);
-    gr[r] = digit_mode(modemap, tt / N2);
-    const u32 a_many = allowed_act_digits(triple_bits(th[r], om[r], gr[r], CLS_SHARDED), req, all, own, is_o, not_mo);
-    const u32 a_one = allowed_act_digits(triple_bits(th[r], om[r], gr[r], CLS_ONE_DEVICE), req, all, all, is_o, not_mo);
-    const u32 a_copies = allowed_act_digits(triple_bits(th[r], om[r], gr[r], CLS_ALL_COPIES), req, all, all, is_o, not_mo);
-    t_allowed[r] = live ? (a_many | (a_one << 8) | (a_copies << 16)) : 0;
+  if (tid < 128) cnt[warp][lane] = 0;
+  for (int t = tid; t < N3; t += COUNT_WARPS * 32) {
+    const u32 th = digit_mode(modemap, t % NM), om = digit_mode(modemap, (t / NM) % NM), gr = digit_mode(modemap, t / N2);
+    allowed_of[CLS_SHARDED][t] = (unsigned char)allowed_act_digits(triple_bits(th, om, gr, CLS_SHARDED), req, all, own, is_o, not_mo);
+    allowed_of[CLS_ONE_DEVICE][t] = (unsigned char)allowed_act_digits(triple_bits(th, om, gr, CLS_ONE_DEVICE), req, all, all, is_o, not_mo);
+    allowed_of[CLS_ALL_COPIES][t] = (unsigned char)allowed_act_digits(triple_bits(th, om, gr, CLS_ALL_COPIES), req, all, all, is_o, not_mo);
   }
-  // this lane's table entry (variant, digit)
-  const u32 tl_vt = lane / NM, tl_d = lane - tl_vt * NM;
-  const bool tl_mine = tl_vt < sp.nvt;
-  const u32 tl_v = tl_mine ? tl_vt / sp.nt : 0;
-  const u32 tl_tau = tl_mine ? tl_vt - tl_v * sp.nt : 0;
-  const u32 tl_mode = digit_mode(modemap, tl_d);
-
-  u32 model_cur = 0xffffffffu, unit_cur = 0xffffffffu;
+  // ---- the lane's unit
+  const u32 k = blockIdx.x * EVAL_RUN_UNITS + lane;
+  const bool have = k < a.n_units;
+  const u64 unit_global = a.first_unit + min(k, a.n_units - 1);
+  const u32 model = (u32)(unit_global / sp.n_facts);
   ModelRec rec;
-  u32 ka[R], kb[R], kc[R], kh[R];
-  u64 mem3[R], host3[R];
-  bool small = false;                      // the factorisation's byte counts are exact as doubles
-  u32 allowed[R];
-  u64 run_total = 0;
-  u32 with_survivors = 0;                  // bit j: group seg_begin + j has survivors
-  const u64 window_end = a.first + a.count;
-
-  // the run's first group by division, the following ones by counting up
-  u32 model, unit, vt;
-  {
-    const u64 g0 = a.first_group + seg_begin;
-    model = (u32)(g0 / groups_per_model);
-    const u32 gl = (u32)(g0 - (u64)model * groups_per_model);
-    unit = gl / sp.nvt;
-    vt = gl - unit * sp.nvt;
-  }
-  for (u32 seg = seg_begin; seg < seg_end;) {
-    const u64 g0 = a.first_group + seg;
-    if (model != model_cur) {
-      model_cur = model;
-      unit_cur = 0xffffffffu;
-      const uint4* src = reinterpret_cast<const uint4*>(&sp.recs[model]);
-      uint4* dst = reinterpret_cast<uint4*>(&rec);
+  load_record(sp, model, rec);
+  const Fact f = sp.facts[(u32)(unit_global - (u64)model * sp.n_facts)];
+  const UnitBase ub = unit_of(sp, rec, f);
+  LaneUnit<NM, T, HOST_LIMITED> lu;
+  lu.load(sp, rec, f, ub, modemap, cap_x, host_x, have && (ub.cv & req_cv) == req_cv);
+  const T host_room = as<T>(host_x);
+  const T wT = as<T>(rec.wT), wO = as<T>(rec.wO);
+  const T host_T = as<T>((2 * sp.accum + 1) * rec.wT), host_O = as<T>(2 * rec.wO);
+  const unsigned char* const allowed_here = allowed_of[lu.shift >> 3];
+  __syncthreads();
+  float n[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+  for (u32 p = warp * N2 / COUNT_WARPS; p < (warp + 1) * N2 / COUNT_WARPS; ++p) {
+    const u32 th = p / NM, om = p - th * NM, th_mode = digit_mode(modemap, th), om_mode = digit_mode(modemap, om);
+    const T to_mem = state_bytes(lu, th_mode, wT, sp.sstar_units) + state_bytes(lu, om_mode, wO, sp.sstar_units);
+    const T to_host = (th_mode == PS_MODE_O ? host_T * lu.s : T(0)) + (om_mode == PS_MODE_O ? host_O * lu.s : T(0));
 #pragma unroll
-      for (int k = 0; k < 6; ++k) dst[k] = __ldg(src + k);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const u32 modes[3] = {th[r], om[r], gr[r]};
-        const u32 width[3] = {rec.wT, rec.wO, rec.wG};
-        u32 ca = 0, cb = 0, cc = 0;
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {        // Theorem 1: R holds E, S and S* a shard, S* and M a unit
-          if (modes[s] == PS_MODE_R) ca += width[s];
-          if (in_set(SET_SHARDLIKE, modes[s])) cb += width[s];
-          if (modes[s] == PS_MODE_SG) cc += width[s] * sp.sstar_units;
-          if (modes[s] == PS_MODE_M) cc += width[s];
-        }
-        ka[r] = ca; kb[r] = cb; kc[r] = cc;
-        kh[r] = (th[r] == PS_MODE_O ? (2 * sp.accum + 1) * rec.wT : 0) + (om[r] == PS_MODE_O ? 2 * rec.wO : 0) +
-                (gr[r] == PS_MODE_O ? 2 * rec.wG : 0);
+    for (int gr = 0; gr < NM; ++gr) {
+      const T m = to_mem + lu.gr_mem[gr];
+      u32 allowed = allowed_here[th + NM * om + N2 * gr] & lu.allowed;
+      T h = to_host;
+      if (HOST_LIMITED) {
+        if (digit_mode(modemap, gr) == PS_MODE_O) h += lu.gr_host;
+        if (!(h < host_room)) allowed = 0;
       }
-    }
-    if (unit != unit_cur) {
-      unit_cur = unit;
-      const Fact f = sp.facts[unit];
-      const u32 repl = POW2 ? 1u : sp.repl;
-      const Pow2 p2 = POW2 ? pow2_of(f) : pow2_of(f, repl);
-      const UnitBase ub = POW2 ? unit_base_pow2_one_copy(rec, f, p2, sp.tp_max_valid, true)
-                          : p2.all ? unit_base_pow2(rec, f, p2, sp.tp_max_valid, true)
-                                   : unit_base(rec, f, sp.tp_max_valid, true, repl);
-      __syncwarp();                            // the previous factorisation's bounds have been read
-      if (tl_mine) {
-        const ActBase ab = POW2 ? act_base_pow2_one_copy(rec, p2, tl_v, tl_tau)
-                           : p2.all ? act_base_pow2(rec, p2, tl_v, tl_tau) : act_base(rec, f, tl_v, tl_tau, ub.G);
-        const u64 am = mu_elems(tl_mode, ab.EA, ab.shA, ab.uA, sp.sstar_units);
-        const u64 bound = am < cap_x ? cap_x - am : 0;
-        tb.bound[tl_d][tl_vt] = bound;
-        tb.bound_f64[tl_d][tl_vt] = (double)bound;
-        if (tl_d == 0) {
-          const u64 ah = 2 * ab.EA * sp.accum;  // offloaded after forward, reloaded for backward, per micro-batch
-          tb.host_bound[tl_vt] = ah < host_x ? host_x - ah : 0;
-        }
-      } else if (tl_vt < 4) {
-        tb.bound_f64[tl_d][tl_vt] = 0.0;
-        if (tl_d == 0) tb.host_bound[tl_vt] = 0;
-      }
-      __syncwarp();
-      const bool unit_ok = (ub.cv & req_cv) == req_cv;
-      const u32 shift = POW2 ? (ub.d1 ? 8u : 0u) : 8 * ub.cls;
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        mem3[r] = mad_small(ub.E2, ka[r], mad_small(ub.sh, kb[r], mad_small(ub.u, kc[r], 0)));
-        host3[r] = mad_small(ub.sh, kh[r], 0);
-        allowed[r] = (unit_ok && host3[r] < host_x) ? ((t_allowed[r] >> shift) & all) : 0;
-      }
-      // Integers below 2^53 are exact as doubles: when the capacity and every triple's bytes
-      // are that small (one test for the warp), whole factorisations are counted with
-      // compares on the fp64 pipe and predicated fp32 adds (see below).
-      small = cap_x < ((u64)1 << 53) && (u64)(rec.wT + rec.wO + rec.wG) * (ub.E2 + 2 * ub.u) < ((u64)1 << 53);
-    }
-    // the factorisation's groups inside this run: variants vt .. vt + n_here - 1
-    const u32 n_here = min(sp.nvt - vt, seg_end - seg);
-    u32 cnt[4] = {0, 0, 0, 0};             // this lane's survivors per variant
-    if (small && g0 * NC >= a.first && (g0 + n_here) * NC <= window_end) {
-      // The usual case, every group whole inside the window: all variants at once.  A
-      // triple's digit is tested for the four variants with one mask bit; a point costs a
-      // compare on the fp64 pipe and a predicated fp32 add.
-      float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
       for (int d = 0; d < NM; ++d) {
-        double bound[4];
-        {
-          const double2 b01 = *reinterpret_cast<const double2*>(&tb.bound_f64[d][0]);
-          const double2 b23 = *reinterpret_cast<const double2*>(&tb.bound_f64[d][2]);
-          bound[0] = b01.x; bound[1] = b01.y; bound[2] = b23.x; bound[3] = b23.y;
+        if (HOST_LIMITED && digit_mode(modemap, d) == PS_MODE_O) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            n[q] += ((allowed >> d) & 1u) && m < lu.bound[d][q] && h < lu.host_bound[q] ? 1.0f : 0.0f;
+        } else {
+          count_variants(n, m, lu.bound[d], allowed & (1u << d));
         }
-        const bool offload = (is_o >> d) & 1u;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const bool on = (allowed[r] >> d) & 1u;
-          const double m = (double)mem3[r];
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (on && m < bound[j] && (!offload || host3[r] < tb.host_bound[j])) c[j] += 1.0f;
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) cnt[j] = (u32)c[j];
-    } else {
-#pragma unroll 1
-      for (u32 k = 0; k < n_here; ++k) {
-        // a group at the window's edge (or byte counts beyond 2^53): only the codes inside the window
-        const u64 group_first = (g0 + k) * NC;
-        const u32 code_lo = a.first > group_first ? (u32)(a.first - group_first) : 0u;
-        const u32 code_hi = window_end < group_first + NC ? (u32)(window_end - group_first) : (u32)NC;
-        const u64 host_bound = tb.host_bound[vt + k];
-        u32 n = 0;
-#pragma unroll 1
-        for (int d = 0; d < NM; ++d) {
-          const u64 bound = tb.bound[d][vt + k];
-          const bool offload = (is_o >> d) & 1u;
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const u32 code = lane + 32 * r + d * N3;
-            const bool pass = ((allowed[r] >> d) & 1u) && mem3[r] < bound && (!offload || host3[r] < host_bound) &&
-                              code >= code_lo && code < code_hi;
-            n += pass ? 1u : 0u;
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if ((u32)j == vt + k) cnt[j] = n;
       }
     }
+  }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if ((u32)j >= vt && (u32)j < vt + n_here) {              // (the same for every lane)
-        const u32 n = __reduce_add_sync(0xffffffffu, cnt[j]);
-        const u32 at = seg + ((u32)j - vt);
-        if (lane == 0) a.tile_count[at] = n;
-        run_total += n;
-        if (n) with_survivors |= 1u << (at - seg_begin);
-      }
-    }
-    // the next factorisation, else the next model
-    seg += n_here;
-    vt = 0;
-    if (++unit == sp.n_facts) { unit = 0; ++model; }
-  }
-  if (lane == 0) a.tile_offset[run] = run_total;
-  // the groups with survivors join the write pass's list (in any order: a group's place
-  // in the output comes from the scan, not from the list)
-  const u32 n_listed = __popc(with_survivors);
-  if (n_listed) {
-    u32 base = 0;
-    if (lane == 0) base = atomicAdd(a.n_nonempty, n_listed);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if ((with_survivors >> lane) & 1u)
-      a.nonempty[base + __popc(with_survivors & ((1u << lane) - 1u))] = seg_begin + lane;
-  }
-}
-
-// exclusive prefix sum, in place, of the survivors of the count pass's runs
-// (a.tile_offset[0 .. n_runs)); the total goes to *a.n_out.  One block: there are
-// a few thousand runs, four per thread and tile.
-constexpr int SCAN_THREADS = 1024, SCAN_ITEMS = 4;
-__global__ void __launch_bounds__(SCAN_THREADS) k_tile_scan(EvalArgs a) {
-  __shared__ u64 warp_sum[32];
-  __shared__ u64 carry;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const u32 n = a.n_runs;
-  if (tid == 0) carry = 0;
+  for (int q = 0; q < 4; ++q)
+    if (n[q] != 0.0f) atomicAdd(&cnt[q][lane], (u32)n[q]);
   __syncthreads();
-  for (u32 tile = 0; tile < n; tile += SCAN_THREADS * SCAN_ITEMS) {
-    const u32 i0 = tile + SCAN_ITEMS * tid;
-    u64 c[SCAN_ITEMS];
+
+  if (warp == 0) {
+    // ---- the groups at the window's edges again, code by code (at most two groups)
+    const u64 window_end = a.first + a.count;
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+      const u64 g = side == 0 ? a.first / NC : (window_end - 1) / NC;
+      const u64 ug = g / sp.nvt, u = ug - a.first_unit;
+      if (u / EVAL_RUN_UNITS != blockIdx.x || (side == 1 && g == a.first / NC)) continue;
+      const u64 group_first = g * NC;
+      const u32 code_lo = a.first > group_first ? (u32)(a.first - group_first) : 0u;
+      const u32 code_hi = window_end < group_first + NC ? (u32)(window_end - group_first) : (u32)NC;
+      if (code_lo == 0 && code_hi == (u32)NC) continue;
+      const u32 vt = (u32)(g - ug * sp.nvt), v = vt / sp.nt, tau = vt - v * sp.nt;
+      const u32 em = (u32)(ug / sp.n_facts);
+      ModelRec er;
+      load_record(sp, em, er);
+      const Fact ef = sp.facts[(u32)(ug - (u64)em * sp.n_facts)];
+      const UnitBase eb = unit_of(sp, er, ef);
+      const ActBase ea = act_of(sp, er, ef, eb, v, tau);
+      const u32 width[3] = {er.wT, er.wO, er.wG};
+      u32 survivors = 0;
+      for (u32 code = code_lo + lane; code < code_hi; code += 32) {
+        const u32 t = code % N3, d = code / N3;
+        const u32 modes[3] = {digit_mode(modemap, t % NM), digit_mode(modemap, (t / NM) % NM), digit_mode(modemap, t / N2)};
+        const u32 ac = digit_mode(modemap, d);
+        u64 mem = mu_elems(ac, ea.EA, ea.shA, ea.uA, sp.sstar_units), host = ac == PS_MODE_O ? 2 * ea.EA * sp.accum : 0;
 #pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; ++k) c[k] = (i0 + k < n) ? a.tile_offset[i0 + k] : 0;
-    u64 mine = 0;
+        for (int st = 0; st < 3; ++st) {
+          mem += width[st] * mu_elems(modes[st], eb.E2, eb.sh, eb.u, sp.sstar_units);
+          if (modes[st] == PS_MODE_O) host += (st == 0 ? 2 * sp.accum + 1 : 2) * (u64)width[st] * eb.sh;
+        }
+        if (((allowed_of[eb.cls][t] >> d) & 1u) && (eb.cv & req_cv) == req_cv && mem < cap_x && host < host_x) ++survivors;
+      }
+      survivors = __reduce_add_sync(0xffffffffu, survivors);
+      if (lane == 0) cnt[2 * v + tau][u % EVAL_RUN_UNITS] = survivors;
+      __syncwarp();
+    }
+    // ---- offsets inside the run, and the list of groups with survivors
+    u32 mine = 0, filled = 0, c[4];
+    bool inside[4];
+    u64 at[4];
 #pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; ++k) mine += c[k];
+    for (u32 q = 0; q < 4; ++q) {
+      const u32 v = q >> 1, tau = q & 1;
+      at[q] = unit_global * sp.nvt + v * sp.nt + tau - a.first_group;      // (wraps before the window)
+      inside[q] = have && v < sp.nv && tau < sp.nt && at[q] < a.n_tiles;
+      c[q] = inside[q] ? cnt[q][lane] : 0;
+      mine += c[q];
+      filled += c[q] ? 1u : 0u;
+    }
+    u32 incl = mine, listed = filled;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u32 up = __shfl_up_sync(0xffffffffu, incl, o), up2 = __shfl_up_sync(0xffffffffu, listed, o);
+      if (lane >= o) { incl += up; listed += up2; }
+    }
+    u32 base = 0;
+    if (lane == 31 && listed) base = atomicAdd(a.n_nonempty, listed);
+    base = __shfl_sync(0xffffffffu, base, 31) + listed - filled;
+    u32 before = incl - mine;
+#pragma unroll
+    for (u32 q = 0; q < 4; ++q) {
+      if (inside[q]) a.group_offset[at[q]] = before;
+      if (c[q]) a.nonempty[base++] = (u32)at[q];
+      before += c[q];
+    }
+    if (lane == 31) a.run_offset[blockIdx.x] = incl;
+    // ---- the block that finishes last turns the runs' totals into offsets
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) last = atomicAdd(a.blocks_done, 1u) == gridDim.x - 1 ? 1u : 0u;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (tid == 0) carry = 0;
+  constexpr int SCAN_ITEMS = 4;
+  volatile u64* const runs = a.run_offset;
+  for (u64 tile = 0; tile < a.n_runs; tile += COUNT_WARPS * 32 * SCAN_ITEMS) {
+    __syncthreads();
+    const u64 i0 = tile + SCAN_ITEMS * tid;
+    u64 c[SCAN_ITEMS], mine = 0;
+#pragma unroll
+    for (int j = 0; j < SCAN_ITEMS; ++j) { c[j] = i0 + j < a.n_runs ? runs[i0 + j] : 0; mine += c[j]; }
     u64 incl = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -673,17 +626,18 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_tile_scan(EvalArgs a) {
     for (int w = 0; w < warp; ++w) before += warp_sum[w];
     u64 run = before + incl - mine;
 #pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; ++k) {
-      if (i0 + k < n) a.tile_offset[i0 + k] = run;
-      run += c[k];
+    for (int j = 0; j < SCAN_ITEMS; ++j) {
+      if (i0 + j < a.n_runs) runs[i0 + j] = run;
+      run += c[j];
     }
     __syncthreads();
-    if (tid == SCAN_THREADS - 1) carry = before + incl;
-    __syncthreads();
+    if (tid == COUNT_WARPS * 32 - 1) carry = before + incl;
   }
+  __syncthreads();
   if (tid == 0) {
     *a.n_out = carry;
     *a.n_nonempty_other = 0;      // the next compaction's list starts empty
+    *a.blocks_done = 0;
   }
 }
 
@@ -725,18 +679,10 @@ cudaError_t launch_eval_m(const SpaceDev& sp, const EvalArgs& a, cudaStream_t st
 
 }  // namespace
 
-// The count pass's runs: as many as fill the GPU with long-lived warps, but no
-// run longer than 32 groups (the write pass adds up the counts of a run's
-// earlier groups with one load per lane).
-void eval_plan_runs(EvalArgs& a) {
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const u32 target = (u32)sms * EVAL_GRID_PER_SM_COMPACT * WARPS;
-  u32 len = (a.n_tiles + target - 1) / target;
-  if (len < 1) len = 1;
-  if (len > 32) len = 32;
-  a.run_len = len;
-  a.n_runs = (a.n_tiles + len - 1) / len;
+void eval_plan_runs(const SpaceDev& sp, EvalArgs& a) {
+  a.first_unit = a.first_group / sp.nvt;
+  a.n_units = (u32)((a.first_group + a.n_tiles - 1) / sp.nvt - a.first_unit + 1);
+  a.n_runs = (a.n_units + EVAL_RUN_UNITS - 1) / EVAL_RUN_UNITS;
 }
 
 cudaError_t launch_eval_materialise(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
@@ -744,9 +690,13 @@ cudaError_t launch_eval_materialise(const SpaceDev& sp, const EvalArgs& a, cudaS
 }
 template <int NM>
 static cudaError_t launch_count_t(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
-  const unsigned blocks = (a.n_runs + WARPS - 1) / WARPS;       // a warp per run
-  if (sp.all_pow2 && sp.repl == 1) k_compact_count<NM, true><<<blocks, THREADS, 0, stream>>>(sp, a);
-  else k_compact_count<NM, false><<<blocks, THREADS, 0, stream>>>(sp, a);
+  // every byte count exact in a double
+  if (sp.all_small && a.cap_bytes < ((u64)1 << 53) - 1) {
+    if (NM < 4 || a.host_cap < ((u64)1 << 62)) k_compact_count<NM, double, true><<<a.n_runs, COUNT_WARPS * 32, 0, stream>>>(sp, a);
+    else k_compact_count<NM, double, NM < 4><<<a.n_runs, COUNT_WARPS * 32, 0, stream>>>(sp, a);
+  } else {
+    k_compact_count<NM, u64, true><<<a.n_runs, COUNT_WARPS * 32, 0, stream>>>(sp, a);
+  }
   return cudaGetLastError();
 }
 cudaError_t launch_eval_count(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
@@ -757,10 +707,6 @@ cudaError_t launch_eval_count(const SpaceDev& sp, const EvalArgs& a, cudaStream_
     case 4: return launch_count_t<4>(sp, a, stream);
     default: return launch_count_t<5>(sp, a, stream);
   }
-}
-cudaError_t launch_tile_scan(const EvalArgs& a, cudaStream_t stream) {
-  k_tile_scan<<<1, SCAN_THREADS, 0, stream>>>(a);
-  return cudaGetLastError();
 }
 cudaError_t launch_eval_write(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
   return launch_eval_m<MODE_WRITE>(sp, a, stream);

@@ -19,7 +19,7 @@ struct ps_ctx {
   cudaStream_t stream;
   void* scratch;
   size_t scratch_bytes;
-  u32* d_lengths;     // the two list lengths of the compaction
+  u32* d_lengths;     // the compaction's two list lengths and its count of finished blocks
   HostWords* h;       // pinned host memory that kernels write to (nothing has to be copied back)
   std::mutex* check;  // one ps_check_composition at a time uses h->entry
   u32 checks;
@@ -74,7 +74,7 @@ cudaError_t launch_sweep(int kind, const SpaceDev& sp, const SweepArgs& a, int s
 #ifndef EVAL_MIN_BLOCKS
 #define EVAL_MIN_BLOCKS 4
 #endif
-#define EVAL_GROUPS_PER_TILE 8    /* a tile = this many consecutive groups of n_codes points */
+#define EVAL_RUN_UNITS 32
 
 struct EvalArgs {
   u64 first, count;         // the window
@@ -87,23 +87,23 @@ struct EvalArgs {
   ps_out_soa out;
   u64* idx_out;
   u64* n_out;
-  // compaction scratch
-  // compaction: the count pass walks the groups in n_runs runs of run_len
-  // consecutive groups (one warp per run) -- set by eval_plan_runs
-  u32 n_runs, run_len;
-  u32* tile_count;          // [n_tiles] survivors of each group
+  // compaction scratch.  The window's factorisations ("units", counted through all models)
+  // are taken in runs of EVAL_RUN_UNITS, a block of the count pass each.
+  u64 first_unit;
+  u32 n_units, n_runs;
+  u32* group_offset;        // [n_tiles] survivors of the earlier groups of the group's run
   u32* nonempty;            // [n_tiles] the groups that have survivors, in any order
   u32* n_nonempty;          // how many (zero before the count pass)
-  u32* n_nonempty_other;    // the next compaction's counter: the scan kernel clears it, so that no
+  u32* n_nonempty_other;    // the next compaction's counter: cleared by the count pass, so that no
                             // call needs a memset of its own (calls alternate between two counters)
-  u64* tile_offset;         // [n_runs <= n_tiles] survivors of each run, then (scan) of all runs before it
+  u32* blocks_done;         // count pass: blocks that have finished (zero between calls)
+  u64* run_offset;          // [n_runs] survivors of each run, then of all runs before it
   volatile u32* status;
 };
 
-void eval_plan_runs(EvalArgs& a);   // fills n_runs, run_len from n_tiles (current device)
+void eval_plan_runs(const SpaceDev& sp, EvalArgs& a);   // fills first_unit, n_units, n_runs
 cudaError_t launch_eval_materialise(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream);
 cudaError_t launch_eval_count(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream);
-cudaError_t launch_tile_scan(const EvalArgs& a, cudaStream_t stream);
 cudaError_t launch_eval_write(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream);
 
 // ---- small kernels

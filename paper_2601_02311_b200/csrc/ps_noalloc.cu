@@ -1,7 +1,7 @@
 // ps_eval_compact_noalloc: the filter-and-compact path of ps_eval_batch for
-// callers that must not allocate device memory.  The per-group survivor counts
-// and the prefix sums over runs of groups live in a fixed array that is part of
-// the library image instead of in the context's growable scratch.
+// callers that must not allocate device memory.  The groups' offsets, the list of groups
+// with survivors and the prefix sums over runs of factorisations live in a fixed array that
+// is part of the library image instead of in the context's growable scratch.
 #include <cuda_runtime.h>
 #include <string.h>
 #include <mutex>
@@ -17,9 +17,9 @@ constexpr size_t LENGTH_BYTES = 256;
 constexpr size_t OFFSET_BYTES = sizeof(u64) * (size_t)PS_NOALLOC_MAX_GROUPS;
 
 // 2 MiB on every GPU that loads the library, for the life of the process:
-// [0, COUNT_BYTES) survivor count of each group, then the list of groups that
-// have survivors, its length, and the exclusive prefix sums (one per run of
-// groups, so at most one per group).
+// [0, COUNT_BYTES) offset of each group in its run, then the list of groups that have
+// survivors and the exclusive prefix sums (one per run of factorisations, so at most one
+// per group).
 static __device__ __align__(256) unsigned char g_fixed_scratch[2 * COUNT_BYTES + LENGTH_BYTES + OFFSET_BYTES];
 
 constexpr int MAX_DEVICES = 64;
@@ -100,21 +100,20 @@ extern "C" int ps_eval_compact_noalloc(ps_ctx* ctx, const ps_space* sp, uint64_t
   a.host_cap = filter->host_cap;
   a.require_flags = filter->require_flags & ~(u32)PS_F_FEASIBLE;
   unsigned char* bytes = static_cast<unsigned char*>(base);
-  a.tile_count = reinterpret_cast<u32*>(bytes);
+  eval_plan_runs(sp->dev, a);
+  a.group_offset = reinterpret_cast<u32*>(bytes);
   a.nonempty = reinterpret_cast<u32*>(bytes + COUNT_BYTES);
   a.n_nonempty = ctx->d_lengths + (ctx->compact_calls & 1u);          // the context's alternating list lengths
   a.n_nonempty_other = ctx->d_lengths + ((ctx->compact_calls + 1) & 1u);
   ++ctx->compact_calls;
-  a.tile_offset = reinterpret_cast<u64*>(bytes + 2 * COUNT_BYTES + LENGTH_BYTES);
-  eval_plan_runs(a);
-  // The array still holds the previous call's numbers.  Every word this call
-  // reads is written earlier in this call (the count pass stores a count for
-  // each group and a total for each run of groups, the scan turns the totals
-  // into offsets); the counts are cleared anyway so that a stale value can
-  // never be mistaken for a fresh one.
-  if (cudaMemsetAsync(a.tile_count, 0, sizeof(u32) * n_groups, ctx->stream) != cudaSuccess) return PS_E_CUDA;
+  a.blocks_done = ctx->d_lengths + 2;
+  a.run_offset = reinterpret_cast<u64*>(bytes + 2 * COUNT_BYTES + LENGTH_BYTES);
+  // The array still holds the previous call's numbers.  Every word this call reads is
+  // written earlier in this call (the count pass stores an offset for each group and a total
+  // for each run, its last block turns the totals into offsets); the groups' offsets are
+  // cleared anyway so that a stale value can never be mistaken for a fresh one.
+  if (cudaMemsetAsync(a.group_offset, 0, sizeof(u32) * n_groups, ctx->stream) != cudaSuccess) return PS_E_CUDA;
   if (launch_eval_count(sp->dev, a, ctx->stream) != cudaSuccess) return PS_E_CUDA;
-  if (launch_tile_scan(a, ctx->stream) != cudaSuccess) return PS_E_CUDA;
   if (launch_eval_write(sp->dev, a, ctx->stream) != cudaSuccess) return PS_E_CUDA;
   return PS_OK;
 }

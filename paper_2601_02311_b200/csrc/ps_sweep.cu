@@ -36,6 +36,7 @@
 #include <type_traits>
 #include "ps_device.cuh"
 #include "ps_internal.h"
+#include "ps_lane.cuh"
 
 namespace {
 
@@ -132,16 +133,6 @@ struct BlockShared {
   u32 n_live, n_heavy, next1, next2, n_cand, n_hits, full, limit_cell, survivors;
 };
 
-// ------------------------------------------------------------------ small arithmetic
-// a * k + acc for a 64-bit a and a small 32-bit k: two multiply-adds
-__device__ __forceinline__ u64 mad_small(u64 a, u32 k, u64 acc) {
-  u64 r = (u64)(u32)a * (u64)k + acc;
-  r += (u64)((u32)(a >> 32) * k) << 32;
-  return r;
-}
-__device__ __forceinline__ u64 mul_add(u64 a, u64 k, u64 acc) { return mad_small(a, (u32)k, acc); }
-__device__ __forceinline__ double mul_add(double a, double k, double acc) { return fma(a, k, acc); }
-
 // the composition bits of a factorisation against the required ones (ps_filter.skip_rejected:
 // a factorisation that misses one has no survivor, so it need not be evaluated)
 __device__ __forceinline__ bool unit_rejected(const SpaceDev& sp, const ModelRec& rec, u32 unit, u32 req_cv) {
@@ -153,68 +144,6 @@ __device__ __forceinline__ bool unit_rejected(const SpaceDev& sp, const ModelRec
   if (t_heads && k_layers && tp_le && whole) cv |= PS_F_CV;
   return (cv & req_cv) != req_cv;
 }
-
-// ------------------------------------------------------------------ a lane's unit
-template <typename T> __device__ __forceinline__ T as(u64 x);
-template <> __device__ __forceinline__ u64 as<u64>(u64 x) { return x; }
-template <> __device__ __forceinline__ double as<double>(u64 x) { return (double)(long long)x; }
-template <typename T> __device__ __forceinline__ u64 bits(T x);
-template <> __device__ __forceinline__ u64 bits<u64>(u64 x) { return x; }
-template <> __device__ __forceinline__ u64 bits<double>(double x) { return (u64)__double_as_longlong(x); }
-template <typename T> __device__ __forceinline__ T from_bits(u64 x);
-template <> __device__ __forceinline__ u64 from_bits<u64>(u64 x) { return x; }
-template <> __device__ __forceinline__ double from_bits<double>(u64 x) { return __longlong_as_double((long long)x); }
-
-__device__ __forceinline__ UnitBase unit_of(const SpaceDev& sp, const ModelRec& rec, const Fact& f) {
-  if (sp.all_pow2) return unit_base_pow2(rec, f, pow2_of(f, sp.repl), sp.tp_max_valid, true);
-  return unit_base(rec, f, sp.tp_max_valid, true, sp.repl);
-}
-__device__ __forceinline__ ActBase act_of(const SpaceDev& sp, const ModelRec& rec, const Fact& f, const UnitBase& ub,
-                                          u32 v, u32 tau) {
-  if (sp.all_pow2) return act_base_pow2(rec, pow2_of(f, sp.repl), v, tau);
-  return act_base(rec, f, v, tau, ub.G);
-}
-
-// A unit as a lane holds it.  T = double where every byte count and volume of the space is
-// below 2^53 (exact there), else u64.  Variants are slots q = 2 v + tau; a slot that the
-// space does not have bounds everything out.
-template <int NM, typename T, bool HOST_LIMITED>
-struct LaneUnit {
-  T E, s, u;                 // elements of a state, of its largest shard, of a reconstruction unit
-  T gr_mem[NM], gr_host;     // G's terms; only mode O has host bytes
-  // a triple whose own bytes are below bound[d][q] fits the capacity with activation digit
-  // d under variant q.  The offloaded digit keeps no activation bytes: its bound is the
-  // capacity for every variant the space has, and its host bytes have to fit too.
-  T bound[NM][4], host_bound[4];
-  u32 allowed, shift;        // digits of a triple that count for this unit: (bits >> shift) & allowed
-
-  __device__ __forceinline__ void load(const SpaceDev& sp, const ModelRec& rec, const Fact& f, const UnitBase& ub,
-                                       u32 modemap, u64 cap_x, u64 host_x, bool live) {
-    E = as<T>(ub.E2); s = as<T>(ub.sh); u = as<T>(ub.u);
-    gr_host = as<T>(mad_small(ub.sh, 2 * rec.wG, 0));
-#pragma unroll
-    for (int d = 0; d < NM; ++d)
-      gr_mem[d] = as<T>(mad_small(mu_elems(digit_mode(modemap, d), ub.E2, ub.sh, ub.u, sp.sstar_units), rec.wG, 0));
-#pragma unroll
-    for (u32 q = 0; q < 4; ++q) {
-      const u32 v = q >> 1, tau = q & 1;
-      const bool have = v < sp.nv && tau < sp.nt;
-      const ActBase ab = act_of(sp, rec, f, ub, v, tau);
-#pragma unroll
-      for (int d = 0; d < NM; ++d) {
-        const u64 am = mu_elems(digit_mode(modemap, d), ab.EA, ab.shA, ab.uA, sp.sstar_units);
-        bound[d][q] = as<T>(have && am < cap_x ? cap_x - am : 0);
-      }
-      if (HOST_LIMITED) {
-        const u64 ah = 2 * ab.EA * sp.accum;             // offload after fwd, reload for bwd, per micro-batch
-        // (rounded only above 2^53, where no host figure of the double case reaches)
-        host_bound[q] = as<T>(have && ah < host_x ? host_x - ah : 0);
-      }
-    }
-    shift = 8 * ub.cls;
-    allowed = live ? (1u << NM) - 1u : 0u;
-  }
-};
 
 // ------------------------------------------------------------------ screening
 // Whether any of four variants of an activation digit fits: one compare per point, its
