@@ -42,8 +42,9 @@ namespace {
 #ifndef EVAL_GRID_PER_SM_MATERIALISE
 #define EVAL_GRID_PER_SM_MATERIALISE 128
 #endif
-// (resident blocks of the write pass: half of 2^23 points surviving 0.067 ms with four, 0.062
-// with five, 0.071 with six, whose registers spill)
+// (resident blocks of the write pass with up to four modes: half of 2^23 points surviving
+// 0.067 ms with four, 0.062 with five, 0.071 with six, whose registers spill.  With five modes
+// five blocks spill as well: 2^24 points all surviving 0.204 ms against 0.175 with four.)
 #ifndef EVAL_MIN_BLOCKS_WRITE
 #define EVAL_MIN_BLOCKS_WRITE 5
 #endif
@@ -155,7 +156,7 @@ __device__ __forceinline__ void load_record(const SpaceDev& sp, u32 model, Model
 
 // POW2: every degree of the space is a power of two (no division is compiled in)
 template <int MODE, int NM, bool POW2>
-__global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE ? EVAL_MIN_BLOCKS_WRITE : EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, EvalArgs a) {
+__global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE && NM < 5 ? EVAL_MIN_BLOCKS_WRITE : EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, EvalArgs a) {
   constexpr int N2 = NM * NM, N3 = NM * NM * NM, NC = N3 * NM;
   constexpr int R = (N3 + 31) / 32;
   // materialise: two staging buffers per warp (dynamic shared memory, none in the other modes)
@@ -354,9 +355,9 @@ __global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE ? EVAL_MIN_BLOCKS_
       continue;
     }
 
-    // (a loop: unrolled, its registers spilled the staged path's: 2^25 points 0.191 ms instead
-    // of 0.179)
-#pragma unroll 1
+    // (materialise takes this path at the window's edges only: unrolled, it made the staged path
+    // spill, 2^25 points 0.191 ms instead of 0.179)
+#pragma unroll (MODE == MODE_WRITE ? NM : 1)
     for (int d = 0; d < NM; ++d) {
       const u64 act_d = mu_elems(digit_mode(modemap, d), ab.EA, ab.shA, ab.uA, sp.sstar_units);
       const bool d_avail = (avail >> d) & 1u, d_off = (is_o >> d) & 1u, d_notmo = (not_mo >> d) & 1u;
@@ -530,43 +531,55 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
     if (n[q] != 0.0f) atomicAdd(&cnt[q][lane], (u32)n[q]);
   __syncthreads();
 
-  if (warp == 0) {
-    // ---- the groups at the window's edges again, code by code (at most two groups)
+  // ---- the groups at the window's edges again, code by code: a warp each, from the figures
+  // that the lane owning the unit holds
+  if (warp < 2) {
     const u64 window_end = a.first + a.count;
-#pragma unroll 1
-    for (int side = 0; side < 2; ++side) {
-      const u64 g = side == 0 ? a.first / NC : (window_end - 1) / NC;
-      const u64 ug = g / sp.nvt, u = ug - a.first_unit;
-      if (u / EVAL_RUN_UNITS != blockIdx.x || (side == 1 && g == a.first / NC)) continue;
-      const u64 group_first = g * NC;
-      const u32 code_lo = a.first > group_first ? (u32)(a.first - group_first) : 0u;
-      const u32 code_hi = window_end < group_first + NC ? (u32)(window_end - group_first) : (u32)NC;
-      if (code_lo == 0 && code_hi == (u32)NC) continue;
-      const u32 vt = (u32)(g - ug * sp.nvt), v = vt / sp.nt, tau = vt - v * sp.nt;
-      const u32 em = (u32)(ug / sp.n_facts);
-      ModelRec er;
-      load_record(sp, em, er);
-      const Fact ef = sp.facts[(u32)(ug - (u64)em * sp.n_facts)];
-      const UnitBase eb = unit_of(sp, er, ef);
-      const ActBase ea = act_of(sp, er, ef, eb, v, tau);
-      const u32 width[3] = {er.wT, er.wO, er.wG};
+    const u64 g = warp == 0 ? a.first / NC : (window_end - 1) / NC;
+    const u64 ug = g / sp.nvt, u = ug - a.first_unit;
+    const u64 group_first = g * NC;
+    const u32 code_lo = a.first > group_first ? (u32)(a.first - group_first) : 0u;
+    const u32 code_hi = window_end < group_first + NC ? (u32)(window_end - group_first) : (u32)NC;
+    if (u / EVAL_RUN_UNITS == blockIdx.x && !(warp == 1 && g == a.first / NC) && (code_lo != 0 || code_hi != (u32)NC)) {
+      const int src = (int)(u % EVAL_RUN_UNITS);
+      const u32 vt = (u32)(g - ug * sp.nvt), v = vt / sp.nt, tau = vt - v * sp.nt, slot = 2 * v + tau;
+      const T E = __shfl_sync(0xffffffffu, lu.E, src), S = __shfl_sync(0xffffffffu, lu.s, src), U = __shfl_sync(0xffffffffu, lu.u, src);
+      const T W[3] = {__shfl_sync(0xffffffffu, wT, src), __shfl_sync(0xffffffffu, wO, src),
+                      __shfl_sync(0xffffffffu, as<T>(rec.wG), src)};
+      const u32 shift = __shfl_sync(0xffffffffu, lu.shift, src), counted = __shfl_sync(0xffffffffu, lu.allowed, src);
+      T bound[NM], host_bound = T(0);
+#pragma unroll
+      for (u32 q = 0; q < 4; ++q)
+        if (q == slot) {
+#pragma unroll
+          for (int d = 0; d < NM; ++d) bound[d] = __shfl_sync(0xffffffffu, lu.bound[d][q], src);
+          if (HOST_LIMITED) host_bound = __shfl_sync(0xffffffffu, lu.host_bound[q], src);
+        }
       u32 survivors = 0;
       for (u32 code = code_lo + lane; code < code_hi; code += 32) {
-        const u32 t = code % N3, d = code / N3;
+        const u32 t = code % N3, digit = code / N3;
         const u32 modes[3] = {digit_mode(modemap, t % NM), digit_mode(modemap, (t / NM) % NM), digit_mode(modemap, t / N2)};
-        const u32 ac = digit_mode(modemap, d);
-        u64 mem = mu_elems(ac, ea.EA, ea.shA, ea.uA, sp.sstar_units), host = ac == PS_MODE_O ? 2 * ea.EA * sp.accum : 0;
+        T m = T(0), h = T(0);
 #pragma unroll
         for (int st = 0; st < 3; ++st) {
-          mem += width[st] * mu_elems(modes[st], eb.E2, eb.sh, eb.u, sp.sstar_units);
-          if (modes[st] == PS_MODE_O) host += (st == 0 ? 2 * sp.accum + 1 : 2) * (u64)width[st] * eb.sh;
+          const T held = (modes[st] == PS_MODE_R ? E : in_set(SET_SHARDLIKE, modes[st]) ? S : T(0)) +
+                         (modes[st] == PS_MODE_SG ? as<T>(sp.sstar_units) * U : modes[st] == PS_MODE_M ? U : T(0));
+          m += W[st] * held;
+          if (modes[st] == PS_MODE_O) h += as<T>(st == 0 ? 2 * sp.accum + 1 : 2) * W[st] * S;
         }
-        if (((allowed_of[eb.cls][t] >> d) & 1u) && (eb.cv & req_cv) == req_cv && mem < cap_x && host < host_x) ++survivors;
+        bool fits = false;
+#pragma unroll
+        for (int d = 0; d < NM; ++d)
+          if (digit == (u32)d) fits = m < bound[d];
+        if (HOST_LIMITED) fits = fits && h < host_room && (digit_mode(modemap, digit) != PS_MODE_O || h < host_bound);
+        if (fits && ((allowed_of[shift >> 3][t] & counted) >> digit) & 1u) ++survivors;
       }
       survivors = __reduce_add_sync(0xffffffffu, survivors);
-      if (lane == 0) cnt[2 * v + tau][u % EVAL_RUN_UNITS] = survivors;
-      __syncwarp();
+      if (lane == 0) cnt[slot][src] = survivors;
     }
+  }
+  __syncthreads();
+  if (warp == 0) {
     // ---- offsets inside the run, and the list of groups with survivors
     u32 mine = 0, filled = 0, c[4];
     bool inside[4];
