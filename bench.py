@@ -555,8 +555,8 @@ def run_ours(args):
                     "h2d_bytes_per_step": int(models_pinned.numel()), "d2h_bytes_per_step": int(d2h)},
             "gpu_launches": launches_per_step * args.steps,
             # the dominant kernel of a step is the Pareto sweep (its share is in phases_ms)
-            "roofline": alu_roofline("k_sweep_pareto", "k_sweep<Pareto> ", phase_ms["pareto"]),
-            "roofline_topk": alu_roofline("k_sweep_topk", "k_sweep<top-k> ", phase_ms["topk"]),
+            "roofline": alu_roofline("k_sweep_pareto", "k_sweep<Pareto>", phase_ms["pareto"]),
+            "roofline_topk": alu_roofline("k_sweep_topk", "k_sweep<top-k>", phase_ms["topk"]),
             "roofline_hbm": {"bound": "hbm", "kernel": "k_eval<materialise>", "achieved": mat_gbs,
                              "peak": hbm_peak, "unit": "GB/s", "frac": mat_gbs / hbm_peak,
                              "traffic": (int(captured["kernels"]["k_eval_materialise"]["dram_bytes_per_point"] * count)
