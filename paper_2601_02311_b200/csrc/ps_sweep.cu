@@ -676,15 +676,16 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
         if (lane >= o) incl += up;
       }
       u32 at = incl - own;
-      for (; word; word &= word - 1) sh.heavy[at++] = (u16)(32 * lane + __ffs(word) - 1);
+      for (; word; word &= word - 1) {
+        if (!PARETO) sh.least_cell[at] = CELLS;        // (before the barrier: the first pass lowers it from any warp)
+        sh.heavy[at++] = (u16)(32 * lane + __ffs(word) - 1);
+      }
       if (lane == 31) sh.n_heavy = incl;
     }
     __syncthreads();
     const u32 n_live = sh.n_live;
     u32 n_heavy = sh.n_heavy;
     if (n_heavy == 0 || n_live == 0) continue;
-    if (!PARETO)
-      for (u32 k = tid; k < n_heavy; k += threads) sh.least_cell[k] = CELLS;
 
     // ---- the two passes.  An item is a batch of 32 listed units and a part of the triples.
     u32 parts, n_items;
