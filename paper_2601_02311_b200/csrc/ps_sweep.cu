@@ -127,6 +127,7 @@ struct BlockShared {
   u32 flags[SEG / 32];                     // units of the segment with survivors
   u16 heavy[SEG];                          // the same as a list
   u32 least_cell[SEG];                     // top-k: the lowest cell that a survivor of a listed unit falls into
+                                           // (Pareto: drop_tied's indices)
   unsigned char live[MAX_TRIPLES + 3];     // the triples the passes walk
   Rank rank[MAX_TRIPLES];
   unsigned char alive[MAX_TRIPLES + 3];
@@ -254,55 +255,22 @@ __device__ __noinline__ void sort_candidates(BlockShared& sh, int n) {
 // configuration takes 0.90 ms instead of 0.79.
 constexpr int PAIRWISE = 128;
 
-// Pareto, without regard to indices: drops the candidates that another one beats strictly;
-// returns how many are left (equal pairs all stay).
-__device__ __noinline__ int drop_dominated(BlockShared& sh, int n) {
-  const int tid = threadIdx.x, lane = tid & 31, threads = blockDim.x;
-  __syncthreads();
-  const bool pairwise = n <= PAIRWISE;
-  if (pairwise) {
-    for (int p = tid; p < n; p += threads) {
-      const u64 a = sh.cand_a[p], b = sh.cand_b[p];
-      bool keep = a != U64MAX;
-#pragma unroll 4
-      for (int q = 0; q < n; ++q) {
-        const u64 oa = sh.cand_a[q], ob = sh.cand_b[q];
-        if (oa <= a && ob <= b && (oa < a || ob < b)) keep = false;
-      }
-      sh.place[p] = keep ? 1 : 0;
-    }
-    __syncthreads();
-  } else {
-    sort_candidates(sh, n);
-  }
-  if (tid < 32) {                                        // closed up by one warp, 32 at a time
+// Closes up the candidates p < n for which `keep(p, its key)` holds, by one warp, 32 at a
+// time; returns how many are left.  (`keep` is called by all lanes; a code of NO_CODE and keys
+// of U64MAX stand for the places from n on.)
+template <typename F>
+__device__ __forceinline__ int close_up(BlockShared& sh, int n, F&& keep) {
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
     int left = 0;
-    u64 least = U64MAX, least_at = 0;                    // the least communication before these 32, and the bytes it came with
     for (int base = 0; base < n; base += 32) {
       const int p = base + lane;
-      const u64 a = p < n ? sh.cand_a[p] : U64MAX, b = p < n ? sh.cand_b[p] : U64MAX;
-      const u32 code = p < n ? sh.cand_i[p] : NO_CODE;
-      bool keep;
-      if (pairwise) {
-        keep = p < n && sh.place[p] != 0;
-      } else {
-        // in the order of (bytes, communication) a candidate stays if nothing before it has
-        // as little communication, or only its own pair
-        u64 m = b, at = a;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const u64 mu = __shfl_up_sync(0xffffffffu, m, o), au = __shfl_up_sync(0xffffffffu, at, o);
-          if (lane >= o && mu <= m) { m = mu; at = au; }
-        }
-        if (least <= m) { m = least; at = least_at; }
-        keep = a != U64MAX && m == b && at == a;         // (m: the least up to here, earliest first)
-        least = __shfl_sync(0xffffffffu, m, 31);
-        least_at = __shfl_sync(0xffffffffu, at, 31);
-      }
-      const u32 votes = __ballot_sync(0xffffffffu, keep);
-      if (keep) {
+      const Key e = p < n ? Key{sh.cand_a[p], sh.cand_b[p], sh.cand_i[p]} : Key{U64MAX, U64MAX, NO_CODE};
+      const bool stays = keep(p, e);
+      const u32 votes = __ballot_sync(0xffffffffu, stays);
+      if (stays) {
         const int to = left + __popc(votes & ((1u << lane) - 1u));
-        sh.cand_a[to] = a; sh.cand_b[to] = b; sh.cand_i[to] = code;
+        sh.cand_a[to] = e.a; sh.cand_b[to] = e.b; sh.cand_i[to] = e.i;
       }
       left += __popc(votes);
       __syncwarp();
@@ -313,8 +281,59 @@ __device__ __noinline__ int drop_dominated(BlockShared& sh, int n) {
   return sh.kept;
 }
 
+// Pareto: drops the candidates that another one beats strictly, and of those with the same
+// pair all but the smallest unit's, whose points have the smaller indices; returns how many
+// are left.  (Points that cost nothing are the same pair in every unit: kept side by side,
+// they alone would fill the buffer, 1360 of them in a model of the stress configuration.)
+// Those of one pair in one unit all stay, since the indices of their points are not known.
+__device__ __noinline__ int drop_dominated(BlockShared& sh, int n) {
+  const int tid = threadIdx.x, lane = tid & 31, threads = blockDim.x;
+  __syncthreads();
+  if (n <= PAIRWISE) {
+    for (int p = tid; p < n; p += threads) {
+      const u64 a = sh.cand_a[p], b = sh.cand_b[p];
+      const u32 unit = sh.cand_i[p] >> 8;
+      bool keep = a != U64MAX;
+#pragma unroll 4
+      for (int q = 0; q < n; ++q) {
+        const u64 oa = sh.cand_a[q], ob = sh.cand_b[q];
+        if (oa <= a && ob <= b && (oa < a || ob < b || sh.cand_i[q] >> 8 < unit)) keep = false;
+      }
+      sh.place[p] = keep ? 1 : 0;
+    }
+    __syncthreads();
+    return close_up(sh, n, [&](int p, const Key&) { return p < n && sh.place[p] != 0; });
+  }
+  sort_candidates(sh, n);
+  // In the order of (bytes, communication, unit) a candidate stays if nothing before it has as
+  // little communication, or only its own pair in its own unit.
+  u64 least = U64MAX, least_at = 0;                      // the least communication before these 32, the bytes
+  u32 least_unit = 0;                                    // and the unit that it came with first
+  return close_up(sh, n, [&](int, const Key& e) {
+    u64 m = e.b, at = e.a;
+    bool tied = least == e.b && least_at == e.a;         // with the candidate before
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u64 mu = __shfl_up_sync(0xffffffffu, m, o), au = __shfl_up_sync(0xffffffffu, at, o);
+      if (o == 1 && lane > 0) tied = mu == e.b && au == e.a;
+      if (lane >= o && mu <= m) { m = mu; at = au; }
+    }
+    if (least <= m) { m = least; at = least_at; }        // (m: the least up to here, earliest first)
+    // the unit of the pair's first candidate
+    const u32 firsts = __ballot_sync(0xffffffffu, !tied) & (0xffffffffu >> (31 - lane));
+    u32 unit = __shfl_sync(0xffffffffu, e.i >> 8, firsts ? 31 - __clz(firsts) : 0);
+    if (firsts == 0) unit = least_unit;
+    const bool keep = e.a != U64MAX && m == e.b && at == e.a && unit == e.i >> 8;
+    const u32 kept = __ballot_sync(0xffffffffu, keep);
+    if (kept) least_unit = __shfl_sync(0xffffffffu, unit, 31 - __clz(kept));
+    least = __shfl_sync(0xffffffffu, m, 31);
+    least_at = __shfl_sync(0xffffffffu, at, 31);
+    return keep;
+  });
+}
+
 // The n candidates sorted by key, without those of a pair that a smaller index has (Pareto,
-// where no strict domination is left), or the k smallest of them (top-k).  Returns how many
+// after drop_dominated and with indices), or the k smallest of them (top-k).  Returns how many
 // stay; more than KEEP_CAP are not all written.
 template <int KIND>
 __device__ __noinline__ int rank_candidates(BlockShared& sh, int n, int k_keep) {
@@ -393,21 +412,36 @@ __device__ __forceinline__ void points_of(const SpaceDev& sp, const BlockShared&
   }
 }
 
-// Pareto: the buffer's n entries get the index of their point, the smallest with the entry's
-// bytes
+// Pareto: the index of each candidate's point, the smallest with the candidate's bytes
 template <int NM>
 __device__ __noinline__ void resolve_candidates(const SpaceDev& sp, BlockShared& sh, int n, u32 modemap, u64 cap_x,
-                                                u64 host_x) {
+                                                u64 host_x, u32* index) {
   __syncthreads();
   for (int p = threadIdx.x; p < n; p += blockDim.x) {
     const u32 code = sh.cand_i[p];
     const u64 want = sh.cand_a[p];
     points_of<NM>(sp, sh, code, modemap, cap_x, host_x, [&](u64 m, u32 idx) {
-      if (m == want) sh.cand_i[p] = idx;
+      if (m == want) index[p] = idx;
       return m != want;
     });
   }
   __syncthreads();
+}
+
+// Pareto, where drop_dominated leaves too many: of the candidates of one pair in one unit only
+// the one with the smallest index stays.
+template <int NM>
+__device__ __noinline__ int drop_tied(const SpaceDev& sp, BlockShared& sh, int n, u32 modemap, u64 cap_x, u64 host_x) {
+  u32* const index = sh.least_cell;                      // (top-k's)
+  resolve_candidates<NM>(sp, sh, n, modemap, cap_x, host_x, index);
+  for (int p = threadIdx.x; p < n; p += blockDim.x) {
+    bool keep = true;
+    for (int q = 0; q < n; ++q)
+      if (sh.cand_a[q] == sh.cand_a[p] && index[q] < index[p]) keep = false;   // (same bytes: same pair)
+    sh.place[p] = keep ? 1 : 0;
+  }
+  __syncthreads();
+  return close_up(sh, n, [&](int p, const Key&) { return p < n && sh.place[p] != 0; });
 }
 
 // top-k: a hit's points below the threshold go to the buffer (the caller has made room)
@@ -799,7 +833,9 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
             if (cand[w] && bits<T>(comm[w]) < sh.cell[cell])
               atomicMin(reinterpret_cast<unsigned long long*>(&sh.cell[cell]), (unsigned long long)bits<T>(comm[w]));
           } else if (PARETO) {
-            cand[w] = cand[w] && (cell == 0 || bits<T>(comm[w]) < sh.cell[max(cell, 1) - 1]);
+            // (the first cell holds one number, zero: its own least is a bound as well)
+            const u64 least = sh.cell[max(cell, 1) - 1];
+            cand[w] = cand[w] && (cell == 0 ? bits<T>(comm[w]) <= least : bits<T>(comm[w]) < least);
           } else {
             cand[w] = cand[w] && cell <= (int)sh.limit_cell && (u64)comm[w] <= threshold.a;
           }
@@ -926,7 +962,8 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
       const bool full = sh.full != 0;
       if (PARETO) {
         if (!full) break;
-        const int n = drop_dominated(sh, min((int)sh.n_cand, CAND_CAP));
+        int n = drop_dominated(sh, min((int)sh.n_cand, CAND_CAP));
+        if (n > CAND_CAP - STEP_CAP) n = drop_tied<NM>(sp, sh, n, modemap, cap_x, host_x);
         if (n > CAND_CAP - STEP_CAP) { overflowed = true; break; }
         __syncthreads();
         if (tid == 0) sh.n_cand = (u32)n;
@@ -962,7 +999,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
   if (!overflowed) {
     if (PARETO) {
       n_list = drop_dominated(sh, (int)sh.n_cand);
-      resolve_candidates<NM>(sp, sh, n_list, modemap, cap_x, host_x);
+      resolve_candidates<NM>(sp, sh, n_list, modemap, cap_x, host_x, sh.cand_i);
       n_list = rank_candidates<KIND>(sh, n_list, 0);
     } else {
       for (int o = 16; o > 0; o >>= 1) survivors += __shfl_xor_sync(0xffffffffu, survivors, o);

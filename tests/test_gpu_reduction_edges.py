@@ -4,6 +4,7 @@ byte counts beyond a double, windows that start or end inside a group, a factori
 a run of factorisations.  Bit for bit against the oracle."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import oracle as O
 from paper_2601_02311_b200 import synth
@@ -17,6 +18,16 @@ def space_of(kind):
     if kind == "segments":              # 1.4 thousand factorisations: two segments
         return synth._space(synth.zoo(2, 21), [2520 * k for k in (1, 2, 3, 4, 5, 6, 8, 9, 10, 12, 16, 18)], t_enum_max=16,
                             k_enum_max=16, n_act=1, n_tpa=1, mode_mask=0b11111)
+    if kind == "stress":                # points that cost nothing: one pair in each of 1360 (unit, variant)
+        return synth.config("C4", n_models=2)
+    if kind == "ragged":
+        return dict(synth.config("C3", n_models=2), n_values=np.asarray([1, 7, 36, 96, 360, 1000, 1536], dtype=np.uint32),
+                    t_enum_max=12, k_enum_max=36)
+    if kind == "tied in a unit":        # 122 pairs of 460 (triple, variant) under a host budget of 6 GB
+        models = synth.zoo(1, 5)
+        models["unit_from_shape"], models["act_enabled"] = 0, 0
+        return dict(synth._space(models, list(range(1, 65)), t_enum_max=1, k_enum_max=1, n_act=2, n_tpa=2,
+                                 mode_mask=0b11111), grad_accum_steps=8)
     space = synth.config("C3", n_models=2)
     if kind == "copies":
         return dict(space, replication_k=3, grad_accum_steps=3, sstar_units=2, n_values=np.asarray([1, 6, 36, 96], dtype=np.uint32))
@@ -30,20 +41,60 @@ def space_of(kind):
 
 
 @pytest.mark.parametrize("require", [0, VALID])
-@pytest.mark.parametrize("kind", ["segments", "plain", "copies", "beyond a double", "few modes"])
+@pytest.mark.parametrize("kind", ["segments", "plain", "copies", "beyond a double", "few modes", "stress", "ragged",
+                                  "tied in a unit"])
 def test_sweeps_where_buffers_fill_and_segments_change(ctx, ps, kind, require):      # noqa: F811
     space = space_of(kind)
     gs, os_ = both(ctx, space)
     caps = [80 * GB, 1 << 61] if kind == "beyond a double" else [80 * GB, 10 ** 6 * GB]
     for comm_kind in (ps.COMM_PAPER, ps.COMM_PAPER_PLUS_EXT):
-        for host_cap in (O.NO_LIMIT, 64 * GB):
+        for host_cap in (O.NO_LIMIT, (6 if kind == "tied in a unit" else 64) * GB):
             filt = dict(require_flags=require, host_cap=host_cap, comm_kind=comm_kind)
-            for got_kind, want_kind, k in ((ps.REDUCE_PARETO, O.KIND_PARETO, 96), (ps.REDUCE_TOPK, O.KIND_TOPK, 64),
+            for got_kind, want_kind, k in ((ps.REDUCE_PARETO, O.KIND_PARETO, 128), (ps.REDUCE_TOPK, O.KIND_TOPK, 64),
                                            (ps.REDUCE_TOPK, O.KIND_TOPK, 1)):
                 want = os_.sweep(filt, caps, want_kind, k, n_threads=8)
                 assert_same_sweep(gs.sweep(filt, caps, got_kind, k), want)
                 if require:
                     assert_same_sweep(gs.sweep(dict(filt, skip_rejected=1), caps, got_kind, k), want)
+
+
+def milliseconds(call):
+    """The fastest of five, after one to warm up."""
+    times = []
+    for _ in range(6):
+        begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        begin.record()
+        call()
+        end.record()
+        end.synchronize()
+        times.append(begin.elapsed_time(end))
+    return min(times[1:])
+
+
+@pytest.mark.parametrize("kind", ["plain", "stress", "ragged", "tied in a unit"])
+def test_tied_points_do_not_send_a_model_to_the_slow_path(ctx, ps, kind):      # noqa: F811
+    """Many points of one (bytes, communication) pair are one entry of a frontier.  The path for
+    frontiers that outgrow the block's buffer evaluates every point again for each entry and takes
+    fifty times as long or more; the same table without the ties takes about as long as with them."""
+    few = space_of(kind)
+    space = dict(few, models=np.tile(few["models"], 128))
+    free = dict(require_flags=0, host_cap=O.NO_LIMIT)
+    if kind == "tied in a unit":
+        models = space["models"].copy()
+        models["unit_from_shape"] = 1
+        tied = dict(require_flags=VALID, host_cap=6 * GB, comm_kind=ps.COMM_PAPER_PLUS_EXT)
+        other, without = dict(space, models=models), tied
+    else:
+        tied = dict(free, comm_kind=ps.COMM_PAPER)
+        other, without = space, dict(free, comm_kind=ps.COMM_PAPER_PLUS_EXT)
+    took = []
+    for description, filt in ((space, tied), (other, without)):
+        gpu = ctx.space(description)
+        out, counts = gpu.alloc_sweep(1, 128)
+        took.append(milliseconds(lambda: gpu.sweep_into(filt, [10 ** 6 * GB], ps.REDUCE_PARETO, 128, out, counts)))
+        ctx.check_status()
+        assert int(counts.max()) <= 128
+    assert took[0] < 8 * took[1], took
 
 
 @pytest.mark.parametrize("kind", ["plain", "copies", "beyond a double", "few modes"])
