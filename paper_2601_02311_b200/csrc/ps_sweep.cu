@@ -18,12 +18,12 @@
 //   (atomicMin).  The prefix minimum is a staircase of strictly dominating points.
 //   Top-k: the number of survivors whose communication falls into a cell.  The first cell
 //   up to which there are k bounds the k-th smallest.
-// Second pass: appends to the block's buffers only what the staircase does not beat, or
+// Second pass: appends to the block's buffer only what the staircase does not beat, or
 // what lies within the bounding cell.  A full buffer is cut back (Pareto: to its frontier;
 // top-k: to its k smallest, the last of which is then a threshold) and the warps resume
-// where they stopped.  Nothing is inserted into a sorted list one by one.  The few points
-// that get there are resolved to indices by a thread each, in code of its own: the passes
-// stay small enough for the instruction cache.
+// where they stopped.  Nothing is inserted into a sorted list one by one.  The few that are
+// left at the end are resolved to points and indices by a thread each, in code of its own:
+// the passes stay small enough for the instruction cache.
 // The block then emits the entries, evaluating each again from its index as a self-check.
 // A frontier that outgrows the buffer takes a slow exact path.
 //
@@ -47,13 +47,14 @@ constexpr int SEG = 1024;                  // units of a segment
 constexpr int CELLS = 512;                 // cells of the histogram
 constexpr int CAND_CAP = 512;              // candidates the block's buffer holds
 constexpr int KEEP_CAP = PS_FRONTIER_FAST; // Pareto: frontier entries that can be emitted from the buffer
-constexpr int HIT_CAP = 256;               // top-k: (unit, triple, tensor-axis variant) hits the block holds
 constexpr int MAX_TRIPLES = 125;
 constexpr u32 NO_CODE = 0xffffffffu;       // an empty entry
 constexpr u32 ALL_STEPS = 0xffffffffu;
 constexpr int STEP_CAP = 128;              // entries that a step of the second pass appends at most: four a lane
-// (a hit becomes at most ten points)
-static_assert(PS_TOPK_MAX <= KEEP_CAP && HIT_CAP >= STEP_CAP && CAND_CAP - PS_TOPK_MAX >= 320,
+// (top-k: a cut leaves k candidates and what ties with the last of them in its unit, see cut_candidates;
+// a candidate becomes at most ten points)
+static_assert(PS_TOPK_MAX <= KEEP_CAP && PS_TOPK_MAX + 2 * MAX_TRIPLES <= CAND_CAP - STEP_CAP &&
+                  CAND_CAP - PS_TOPK_MAX >= 320,
               "what a step brings fits an emptied buffer");
 
 struct Key {
@@ -116,14 +117,14 @@ struct BlockShared {
   unsigned char allowed[3][MAX_TRIPLES + 3];   // allowed activation digits of a triple for the three CLS_* of a unit
   u64 state[2][5][4];                      // Theta, Omega: the coefficients of E, s, u and the host coefficient, by digit
   u64 cell[CELLS];                         // the histogram
-  u64 cand_a[CAND_CAP], cand_b[CAND_CAP];  // the buffer: Pareto (mem, comm), top-k (comm, mem)
+  u64 cand_a[CAND_CAP], cand_b[CAND_CAP];  // the buffer: Pareto (mem, comm), top-k (comm, least mem)
   u32 cand_i[CAND_CAP];
   unsigned char place[CAND_CAP];           // candidates that stay
   u64 sorted_a[KEEP_CAP], sorted_b[KEEP_CAP];
   u32 sorted_i[KEEP_CAP];
   int kept;
-  u64 hit_comm[HIT_CAP];
-  u32 hit[HIT_CAP];
+  u64 hit_a[CAND_CAP], hit_b[CAND_CAP];    // top-k: the candidates that are left, while their points fill the buffer
+  u32 hit[CAND_CAP];
   u32 flags[SEG / 32];                     // units of the segment with survivors
   u16 heavy[SEG];                          // the same as a list
   u32 least_cell[SEG];                     // top-k: the lowest cell that a survivor of a listed unit falls into
@@ -131,7 +132,7 @@ struct BlockShared {
   unsigned char live[MAX_TRIPLES + 3];     // the triples the passes walk
   Rank rank[MAX_TRIPLES];
   unsigned char alive[MAX_TRIPLES + 3];
-  u32 n_live, n_heavy, next1, next2, n_cand, n_hits, full, limit_cell, survivors;
+  u32 n_live, n_heavy, next1, next2, n_cand, full, limit_cell, survivors;
 };
 
 // the composition bits of a factorisation against the required ones (ps_filter.skip_rejected:
@@ -332,6 +333,25 @@ __device__ __noinline__ int drop_dominated(BlockShared& sh, int n) {
   });
 }
 
+// Top-k: the n candidates sorted by (communication, least bytes, unit), cut to the k smallest and
+// those that are the same in all three as the last of these (the order of points inside a unit is
+// not known here).  Each of the k stands for a point of its own, the least of its points, and the
+// points of a larger unit have larger indices: so what is dropped has none of the k smallest.
+// Returns how many stay.
+__device__ __noinline__ int cut_candidates(BlockShared& sh, int n, int k) {
+  __syncthreads();
+  if (n <= k) return n;
+  sort_candidates(sh, n);
+  const u64 a = sh.cand_a[k - 1], b = sh.cand_b[k - 1];
+  const u32 unit = sh.cand_i[k - 1] >> 8;
+  if (threadIdx.x == 0) sh.kept = k;
+  __syncthreads();
+  for (int p = k + threadIdx.x; p < n; p += blockDim.x)
+    if (sh.cand_a[p] == a && sh.cand_b[p] == b && sh.cand_i[p] >> 8 == unit) atomicAdd(&sh.kept, 1);
+  __syncthreads();
+  return sh.kept;
+}
+
 // The n candidates sorted by key, without those of a pair that a smaller index has (Pareto,
 // after drop_dominated and with indices), or the k smallest of them (top-k).  Returns how many
 // stay; more than KEEP_CAP are not all written.
@@ -444,17 +464,46 @@ __device__ __noinline__ int drop_tied(const SpaceDev& sp, BlockShared& sh, int n
   return close_up(sh, n, [&](int p, const Key&) { return p < n && sh.place[p] != 0; });
 }
 
-// top-k: a hit's points below the threshold go to the buffer (the caller has made room)
+// top-k: the points of the buffer's n candidates take their places, as many candidates at a
+// time as surely fit, the smallest first; those at or above the k-th smallest point so far are
+// left out.  Returns the number of points.
 template <int NM>
-__device__ __noinline__ void resolve_hit(const SpaceDev& sp, BlockShared& sh, u32 code, u64 comm, const Key& threshold,
-                                         u32 modemap, u64 cap_x, u64 host_x) {
-  points_of<NM>(sp, sh, code, modemap, cap_x, host_x, [&](u64 m, u32 idx) {
-    if (key_less(Key{comm, m, idx}, threshold)) {
-      const u32 at = atomicAdd(&sh.n_cand, 1u);
-      sh.cand_a[at] = comm; sh.cand_b[at] = m; sh.cand_i[at] = idx;
+__device__ __noinline__ int resolve_points(const SpaceDev& sp, BlockShared& sh, int n, int k, u32 modemap, u64 cap_x,
+                                           u64 host_x) {
+  const int tid = threadIdx.x, threads = blockDim.x;
+  const u32 per_unit = sp.nvt * NM * NM * NM * NM;
+  __syncthreads();
+  for (int p = tid; p < n; p += threads) { sh.hit_a[p] = sh.cand_a[p]; sh.hit_b[p] = sh.cand_b[p]; sh.hit[p] = sh.cand_i[p]; }
+  if (tid == 0) sh.n_cand = 0;
+  __syncthreads();
+  Key threshold{U64MAX, U64MAX, NO_CODE};
+  for (int base = 0; base < n;) {
+    int room = (CAND_CAP - (int)sh.n_cand) / (2 * NM);
+    if (room < min(n - base, 32)) {
+      const int left = rank_candidates<PS_REDUCE_TOPK>(sh, (int)sh.n_cand, k);
+      if (left == k) threshold = Key{sh.cand_a[k - 1], sh.cand_b[k - 1], sh.cand_i[k - 1]};
+      __syncthreads();
+      if (tid == 0) sh.n_cand = (u32)left;
+      room = (CAND_CAP - left) / (2 * NM);
     }
-    return true;
-  });
+    __syncthreads();
+    const int now = min(n - base, room);
+    for (int j = base + tid; j < base + now; j += threads) {
+      const u64 comm = sh.hit_a[j];
+      const u32 code = sh.hit[j];
+      if (!key_less(Key{comm, sh.hit_b[j], (code >> 8) * per_unit}, threshold)) continue;
+      points_of<NM>(sp, sh, code, modemap, cap_x, host_x, [&](u64 m, u32 idx) {
+        if (key_less(Key{comm, m, idx}, threshold)) {
+          const u32 at = atomicAdd(&sh.n_cand, 1u);
+          sh.cand_a[at] = comm; sh.cand_b[at] = m; sh.cand_i[at] = idx;
+        }
+        return true;
+      });
+    }
+    base += now;
+    __syncthreads();
+  }
+  return (int)sh.n_cand;
 }
 
 // ------------------------------------------------------------------ one point, the slow exact path
@@ -668,7 +717,9 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     if (lane == 0) sh.n_live = n;
   }
 
-  Key threshold{U64MAX, U64MAX, 0xffffffffu};        // top-k: nothing at or above it is wanted
+  // top-k: no candidate above these (communication, least bytes, unit) is wanted
+  T most_comm = T(U64MAX), most_mem = T(U64MAX);
+  u32 most_unit = NO_CODE;
   u32 survivors = 0;
   bool overflowed = false;                           // the same for every thread
   const bool skip = args.skip_rejected && req_cv != 0;
@@ -837,7 +888,9 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
             const u64 least = sh.cell[max(cell, 1) - 1];
             cand[w] = cand[w] && (cell == 0 ? bits<T>(comm[w]) <= least : bits<T>(comm[w]) < least);
           } else {
-            cand[w] = cand[w] && cell <= (int)sh.limit_cell && (u64)comm[w] <= threshold.a;
+            cand[w] = cand[w] && cell <= (int)sh.limit_cell &&
+                      (comm[w] < most_comm || (comm[w] == most_comm &&
+                                               (mem[w] < most_mem || (mem[w] == most_mem && unit <= most_unit))));
           }
         }
         if (SECOND && __any_sync(0xffffffffu, cand[0] | cand[1] | cand[2] | cand[3])) {
@@ -852,22 +905,18 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
           }
           const u32 total = __shfl_sync(0xffffffffu, incl, 31);
           u32 at = 0;
-          if (lane == 0) at = atomicAdd(PARETO ? &sh.n_cand : &sh.n_hits, total);
+          if (lane == 0) at = atomicAdd(&sh.n_cand, total);
           at = __shfl_sync(0xffffffffu, at, 0);
           // (a group that does not fit leaves empty entries where there were places)
-          const u32 limit = PARETO ? CAND_CAP : HIT_CAP;
-          const bool room = at + total <= limit;
+          const bool room = at + total <= CAND_CAP;
           at += incl - mine;
 #pragma unroll
           for (int w = 0; w < 4; ++w)
             if (cand[w]) {
-              if (at < limit) {
-                const u32 code = room ? (unit << 8) | ((u32)sh.live[min(t0 + (w >> 1), t_end - 1)] << 1) | (w & 1) : NO_CODE;
-                if (PARETO) {
-                  sh.cand_a[at] = room ? (u64)mem[w] : U64MAX; sh.cand_b[at] = room ? (u64)comm[w] : U64MAX; sh.cand_i[at] = code;
-                } else {
-                  sh.hit_comm[at] = (u64)comm[w]; sh.hit[at] = code;
-                }
+              if (at < CAND_CAP) {
+                sh.cand_a[at] = room ? (u64)(PARETO ? mem[w] : comm[w]) : U64MAX;
+                sh.cand_b[at] = room ? (u64)(PARETO ? comm[w] : mem[w]) : U64MAX;
+                sh.cand_i[at] = room ? (unit << 8) | ((u32)sh.live[min(t0 + (w >> 1), t_end - 1)] << 1) | (w & 1) : NO_CODE;
               }
               ++at;
             }
@@ -941,7 +990,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     }
     u32 item = ALL_STEPS, from = 0;                  // the warp's item in hand and the triple to resume at
     for (;;) {
-      if (tid == 0) { sh.full = 0; sh.n_hits = 0; }
+      if (tid == 0) sh.full = 0;
       __syncthreads();
       for (;;) {
         if (item == ALL_STEPS) {
@@ -959,36 +1008,19 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
         item = ALL_STEPS;
       }
       __syncthreads();
-      const bool full = sh.full != 0;
+      if (!sh.full) break;
+      int n = min((int)sh.n_cand, CAND_CAP);
       if (PARETO) {
-        if (!full) break;
-        int n = drop_dominated(sh, min((int)sh.n_cand, CAND_CAP));
+        n = drop_dominated(sh, n);
         if (n > CAND_CAP - STEP_CAP) n = drop_tied<NM>(sp, sh, n, modemap, cap_x, host_x);
         if (n > CAND_CAP - STEP_CAP) { overflowed = true; break; }
-        __syncthreads();
-        if (tid == 0) sh.n_cand = (u32)n;
       } else {
-        // the hits' points, as many hits at a time as surely fit
-        const u32 n_hits = min(sh.n_hits, (u32)HIT_CAP);
-        for (u32 base = 0; base < n_hits;) {
-          u32 room = (CAND_CAP - sh.n_cand) / (2 * NM);
-          if (room < min(n_hits - base, 32u)) {
-            const int n = rank_candidates<KIND>(sh, (int)sh.n_cand, (int)args.max_entries);
-            if (n == (int)args.max_entries) threshold = Key{sh.cand_a[n - 1], sh.cand_b[n - 1], sh.cand_i[n - 1]};
-            __syncthreads();
-            if (tid == 0) sh.n_cand = (u32)n;
-            room = (CAND_CAP - n) / (2 * NM);
-          }
-          __syncthreads();
-          const u32 now = min(n_hits - base, room);
-          for (u32 j = tid; j < now; j += threads)
-            if (sh.hit[base + j] != NO_CODE && sh.hit_comm[base + j] <= threshold.a)
-              resolve_hit<NM>(sp, sh, sh.hit[base + j], sh.hit_comm[base + j], threshold, modemap, cap_x, host_x);
-          base += now;
-          __syncthreads();
-        }
-        if (!full) break;
+        const int k = (int)args.max_entries;
+        n = cut_candidates(sh, n, k);
+        most_comm = as<T>(sh.cand_a[k - 1]); most_mem = as<T>(sh.cand_b[k - 1]); most_unit = sh.cand_i[k - 1] >> 8;
       }
+      __syncthreads();
+      if (tid == 0) sh.n_cand = (u32)n;
     }
     if (overflowed) break;
   }
@@ -1004,7 +1036,9 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     } else {
       for (int o = 16; o > 0; o >>= 1) survivors += __shfl_xor_sync(0xffffffffu, survivors, o);
       if (lane == 0 && survivors) atomicAdd(&sh.survivors, survivors);
-      n_list = rank_candidates<KIND>(sh, (int)sh.n_cand, (int)args.max_entries);
+      n_list = cut_candidates(sh, (int)sh.n_cand, (int)args.max_entries);
+      n_list = resolve_points<NM>(sp, sh, n_list, (int)args.max_entries, modemap, cap_x, host_x);
+      n_list = rank_candidates<KIND>(sh, n_list, (int)args.max_entries);
     }
     overflowed = PARETO && n_list > KEEP_CAP;
     __syncthreads();
