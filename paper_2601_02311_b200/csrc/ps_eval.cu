@@ -411,38 +411,14 @@ __global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE && NM < 5 ? EVAL_M
 }
 
 // ------------------------------------------------------------------ compaction: count
-// Survivors of the lane's unit among the four variants of one activation digit: a compare
-// per point on the fp64 pipe, masked by its input predicate, counted with predicated fp32
-// adds (small integers are exact).
-__device__ __forceinline__ void count_variants(float* n, double m, const double* b, u32 on) {
-  asm("{\n\t"
-      ".reg .pred q, p0, p1, p2, p3;\n\t"
-      "setp.ne.u32 q, %9, 0;\n\t"
-      "setp.lt.and.f64 p0, %4, %5, q;\n\t"
-      "setp.lt.and.f64 p1, %4, %6, q;\n\t"
-      "setp.lt.and.f64 p2, %4, %7, q;\n\t"
-      "setp.lt.and.f64 p3, %4, %8, q;\n\t"
-      "@p0 add.f32 %0, %0, 0f3F800000;\n\t"
-      "@p1 add.f32 %1, %1, 0f3F800000;\n\t"
-      "@p2 add.f32 %2, %2, 0f3F800000;\n\t"
-      "@p3 add.f32 %3, %3, 0f3F800000;\n\t"
-      "}"
-      : "+f"(n[0]), "+f"(n[1]), "+f"(n[2]), "+f"(n[3])
-      : "d"(m), "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]), "r"(on));
-}
-__device__ __forceinline__ void count_variants(float* n, u64 m, const u64* b, u32 on) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) n[q] += on != 0 && m < b[q] ? 1.0f : 0.0f;
-}
-
 // bytes of a state under a mode (the same for every lane) in the lane's unit
 template <int NM, typename T, bool HOST_LIMITED>
-__device__ __forceinline__ T state_bytes(const LaneUnit<NM, T, HOST_LIMITED>& lu, u32 mode, T width, u32 sstar_units) {
+__device__ __forceinline__ double state_bytes(const LaneUnit<NM, T, HOST_LIMITED>& lu, u32 mode, double width, u32 sstar_units) {
   if (mode == PS_MODE_R) return width * lu.E;
   if (mode == PS_MODE_S) return width * lu.s;
-  if (mode == PS_MODE_SG) return width * (lu.s + as<T>(sstar_units) * lu.u);
+  if (mode == PS_MODE_SG) return width * (lu.s + sstar_units * lu.u);
   if (mode == PS_MODE_M) return width * lu.u;
-  return T(0);
+  return 0.0;
 }
 
 // One block per run of 32 consecutive units; a lane owns a unit, the warps share the
@@ -495,7 +471,7 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
   LaneUnit<NM, T, HOST_LIMITED> lu;
   lu.load(sp, rec, f, ub, modemap, cap_x, host_x, have && (ub.cv & req_cv) == req_cv);
   const T host_room = as<T>(host_x);
-  const T wT = as<T>(rec.wT), wO = as<T>(rec.wO);
+  const double wT = rec.wT, wO = rec.wO, wG = rec.wG;
   const T host_T = as<T>((2 * sp.accum + 1) * rec.wT), host_O = as<T>(2 * rec.wO);
   const unsigned char* const allowed_here = allowed_of[lu.shift >> 3];
   __syncthreads();
@@ -503,11 +479,11 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
 #pragma unroll 1
   for (u32 p = warp * N2 / COUNT_WARPS; p < (warp + 1) * N2 / COUNT_WARPS; ++p) {
     const u32 th = p / NM, om = p - th * NM, th_mode = digit_mode(modemap, th), om_mode = digit_mode(modemap, om);
-    const T to_mem = state_bytes(lu, th_mode, wT, sp.sstar_units) + state_bytes(lu, om_mode, wO, sp.sstar_units);
-    const T to_host = (th_mode == PS_MODE_O ? host_T * lu.s : T(0)) + (om_mode == PS_MODE_O ? host_O * lu.s : T(0));
+    const double to_mem = state_bytes(lu, th_mode, wT, sp.sstar_units) + state_bytes(lu, om_mode, wO, sp.sstar_units);
+    const T to_host = (th_mode == PS_MODE_O ? host_T * lu.shard : T(0)) + (om_mode == PS_MODE_O ? host_O * lu.shard : T(0));
 #pragma unroll
     for (int gr = 0; gr < NM; ++gr) {
-      const T m = to_mem + lu.gr_mem[gr];
+      const double m = to_mem + lu.gr_mem[gr];
       u32 allowed = allowed_here[th + NM * om + N2 * gr] & lu.allowed;
       T h = to_host;
       if (HOST_LIMITED) {
@@ -519,9 +495,9 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
         if (HOST_LIMITED && digit_mode(modemap, d) == PS_MODE_O) {
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            n[q] += ((allowed >> d) & 1u) && m < lu.bound[d][q] && h < lu.host_bound[q] ? 1.0f : 0.0f;
+            n[q] += ((allowed >> d) & 1u) && m < lu.bounds(d)[q] && h < lu.host_bound[q] ? 1.0f : 0.0f;
         } else {
-          count_variants(n, m, lu.bound[d], allowed & (1u << d));
+          count_variants(n, m, lu.bounds(d), allowed & (1u << d));
         }
       }
     }
@@ -543,29 +519,32 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
     if (u / EVAL_RUN_UNITS == blockIdx.x && !(warp == 1 && g == a.first / NC) && (code_lo != 0 || code_hi != (u32)NC)) {
       const int src = (int)(u % EVAL_RUN_UNITS);
       const u32 vt = (u32)(g - ug * sp.nvt), v = vt / sp.nt, tau = vt - v * sp.nt, slot = 2 * v + tau;
-      const T E = __shfl_sync(0xffffffffu, lu.E, src), S = __shfl_sync(0xffffffffu, lu.s, src), U = __shfl_sync(0xffffffffu, lu.u, src);
-      const T W[3] = {__shfl_sync(0xffffffffu, wT, src), __shfl_sync(0xffffffffu, wO, src),
-                      __shfl_sync(0xffffffffu, as<T>(rec.wG), src)};
+      const double E = __shfl_sync(0xffffffffu, lu.E, src), S = __shfl_sync(0xffffffffu, lu.s, src), U = __shfl_sync(0xffffffffu, lu.u, src);
+      const double W[3] = {__shfl_sync(0xffffffffu, wT, src), __shfl_sync(0xffffffffu, wO, src),
+                           __shfl_sync(0xffffffffu, wG, src)};
+      const T shard = __shfl_sync(0xffffffffu, lu.shard, src);
       const u32 shift = __shfl_sync(0xffffffffu, lu.shift, src), counted = __shfl_sync(0xffffffffu, lu.allowed, src);
-      T bound[NM], host_bound = T(0);
+      double bound[NM];
+      T host_bound = T(0);
 #pragma unroll
       for (u32 q = 0; q < 4; ++q)
         if (q == slot) {
 #pragma unroll
-          for (int d = 0; d < NM; ++d) bound[d] = __shfl_sync(0xffffffffu, lu.bound[d][q], src);
+          for (int d = 0; d < NM; ++d) bound[d] = __shfl_sync(0xffffffffu, lu.bounds(d)[q], src);
           if (HOST_LIMITED) host_bound = __shfl_sync(0xffffffffu, lu.host_bound[q], src);
         }
       u32 survivors = 0;
       for (u32 code = code_lo + lane; code < code_hi; code += 32) {
         const u32 t = code % N3, digit = code / N3;
         const u32 modes[3] = {digit_mode(modemap, t % NM), digit_mode(modemap, (t / NM) % NM), digit_mode(modemap, t / N2)};
-        T m = T(0), h = T(0);
+        double m = 0.0;
+        T h = T(0);
 #pragma unroll
         for (int st = 0; st < 3; ++st) {
-          const T held = (modes[st] == PS_MODE_R ? E : in_set(SET_SHARDLIKE, modes[st]) ? S : T(0)) +
-                         (modes[st] == PS_MODE_SG ? as<T>(sp.sstar_units) * U : modes[st] == PS_MODE_M ? U : T(0));
+          const double held = (modes[st] == PS_MODE_R ? E : in_set(SET_SHARDLIKE, modes[st]) ? S : 0.0) +
+                              (modes[st] == PS_MODE_SG ? sp.sstar_units * U : modes[st] == PS_MODE_M ? U : 0.0);
           m += W[st] * held;
-          if (modes[st] == PS_MODE_O) h += as<T>(st == 0 ? 2 * sp.accum + 1 : 2) * W[st] * S;
+          if (modes[st] == PS_MODE_O) h += as<T>((st == 0 ? 2 * sp.accum + 1 : 2) * (u32)W[st]) * shard;
         }
         bool fits = false;
 #pragma unroll

@@ -1,6 +1,7 @@
 // A factorisation ("unit") of a model as one lane holds it, for the kernels in which the
 // lanes of a warp own units and walk the (Theta, Omega, G) triples together.
 #pragma once
+#include <type_traits>
 #include "ps_device.cuh"
 
 // ------------------------------------------------------------------ small arithmetic
@@ -17,6 +18,9 @@ __device__ __forceinline__ double mul_add(double a, double k, double acc) { retu
 template <typename T> __device__ __forceinline__ T as(u64 x);
 template <> __device__ __forceinline__ u64 as<u64>(u64 x) { return x; }
 template <> __device__ __forceinline__ double as<double>(u64 x) { return (double)(long long)x; }
+template <typename T> __device__ __forceinline__ T whole(double x);      // a whole number
+template <> __device__ __forceinline__ u64 whole<u64>(double x) { return (u64)(long long)x; }
+template <> __device__ __forceinline__ double whole<double>(double x) { return x; }
 template <typename T> __device__ __forceinline__ u64 bits(T x);
 template <> __device__ __forceinline__ u64 bits<u64>(u64 x) { return x; }
 template <> __device__ __forceinline__ u64 bits<double>(double x) { return (u64)__double_as_longlong(x); }
@@ -34,26 +38,34 @@ __device__ __forceinline__ ActBase act_of(const SpaceDev& sp, const ModelRec& re
   return act_base(rec, f, v, tau, ub.G);
 }
 
-// A unit as a lane holds it.  T = double where every byte count and volume of the space is
-// below 2^53 (exact there), else u64.  Variants are slots q = 2 v + tau; a slot that the
-// space does not have bounds everything out.
+// A unit as a lane holds it.  A triple's own device bytes are doubles: they stay below 2^52 (48
+// bytes of each of 2^46 elements and of two units of 2^36), where doubles are exact, and a bound
+// on them that is rounded, above 2^53, lies above them all the same.  T is the type of volumes,
+// host bytes and whole points' bytes: double where all of a space are below 2^53, else u64.  (With
+// the triple's bytes in 64-bit integers there too, top-k of 2048 shapes of the stress
+// configuration with 64 micro-batches a step took 2.40 ms without required flags instead of
+// 1.27.)  Variants are slots q = 2 v + tau; a slot that the space does not have bounds
+// everything out.
 template <int NM, typename T, bool HOST_LIMITED>
 struct LaneUnit {
-  T E, s, u;                 // elements of a state, of its largest shard, of a reconstruction unit
-  T gr_mem[NM], gr_host;     // G's terms; only mode O has host bytes
+  double E, s, u;            // elements of a state, of its largest shard, of a reconstruction unit
+  double gr_mem[NM];         // G's terms
+  T shard, gr_host;          // for host bytes; only mode O has any
   // a triple whose own bytes are below bound[d][q] fits the capacity with activation digit
   // d under variant q.  The offloaded digit keeps no activation bytes: its bound is the
   // capacity for every variant the space has, and its host bytes have to fit too.
   T bound[NM][4], host_bound[4];
+  double rounded[std::is_same<T, double>::value ? 1 : NM][4];              // bound as doubles, where T is not
   u32 allowed, shift;        // digits of a triple that count for this unit: (bits >> shift) & allowed
 
   __device__ __forceinline__ void load(const SpaceDev& sp, const ModelRec& rec, const Fact& f, const UnitBase& ub,
                                        u32 modemap, u64 cap_x, u64 host_x, bool live) {
-    E = as<T>(ub.E2); s = as<T>(ub.sh); u = as<T>(ub.u);
+    E = as<double>(ub.E2); s = as<double>(ub.sh); u = as<double>(ub.u);
+    shard = as<T>(ub.sh);
     gr_host = as<T>(mad_small(ub.sh, 2 * rec.wG, 0));
 #pragma unroll
     for (int d = 0; d < NM; ++d)
-      gr_mem[d] = as<T>(mad_small(mu_elems(digit_mode(modemap, d), ub.E2, ub.sh, ub.u, sp.sstar_units), rec.wG, 0));
+      gr_mem[d] = as<double>(mad_small(mu_elems(digit_mode(modemap, d), ub.E2, ub.sh, ub.u, sp.sstar_units), rec.wG, 0));
 #pragma unroll
     for (u32 q = 0; q < 4; ++q) {
       const u32 v = q >> 1, tau = q & 1;
@@ -63,6 +75,7 @@ struct LaneUnit {
       for (int d = 0; d < NM; ++d) {
         const u64 am = mu_elems(digit_mode(modemap, d), ab.EA, ab.shA, ab.uA, sp.sstar_units);
         bound[d][q] = as<T>(have && am < cap_x ? cap_x - am : 0);
+        if constexpr (!std::is_same<T, double>::value) rounded[d][q] = as<double>(bound[d][q]);
       }
       if (HOST_LIMITED) {
         const u64 ah = 2 * ab.EA * sp.accum;             // offload after fwd, reload for bwd, per micro-batch
@@ -73,4 +86,28 @@ struct LaneUnit {
     shift = 8 * ub.cls;
     allowed = live ? (1u << NM) - 1u : 0u;
   }
+  __device__ __forceinline__ const double* bounds(int d) const {
+    if constexpr (std::is_same<T, double>::value) return bound[d];
+    else return rounded[d];
+  }
 };
+
+// Survivors of the lane's unit among the four variants of one activation digit: a compare
+// per point on the fp64 pipe, masked by its input predicate, counted with predicated fp32
+// adds (small integers are exact).
+__device__ __forceinline__ void count_variants(float* n, double m, const double* b, u32 on) {
+  asm("{\n\t"
+      ".reg .pred q, p0, p1, p2, p3;\n\t"
+      "setp.ne.u32 q, %9, 0;\n\t"
+      "setp.lt.and.f64 p0, %4, %5, q;\n\t"
+      "setp.lt.and.f64 p1, %4, %6, q;\n\t"
+      "setp.lt.and.f64 p2, %4, %7, q;\n\t"
+      "setp.lt.and.f64 p3, %4, %8, q;\n\t"
+      "@p0 add.f32 %0, %0, 0f3F800000;\n\t"
+      "@p1 add.f32 %1, %1, 0f3F800000;\n\t"
+      "@p2 add.f32 %2, %2, 0f3F800000;\n\t"
+      "@p3 add.f32 %3, %3, 0f3F800000;\n\t"
+      "}"
+      : "+f"(n[0]), "+f"(n[1]), "+f"(n[2]), "+f"(n[3])
+      : "d"(m), "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]), "r"(on));
+}

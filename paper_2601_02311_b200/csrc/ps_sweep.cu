@@ -84,25 +84,21 @@ __device__ __forceinline__ Key key_shfl_xor(const Key& x, int lanes) {
 // with small integer coefficients that depend only on the triple's modes and the model's
 // byte widths.
 struct __align__(16) Triple {
-  u64 k[4];             // ka, kb, kc and kh, as the screening's type
-  u64 kx;               // kx, the same
+  double k[3];          // ka, kb, kc
+  u64 kh, kx;           // as the sweep's type
   u32 allowed;          // allowed activation digits: bits 0..4, 8..12, 16..20 for the three CLS_* of a unit;
                         // bits 24.. reductions to shards (2 bits) and all-reduces (1 bit) beyond kx * x, where
                         // shards have copies
   u32 pad;
 };
 
-// the cell of a number: its leading bit and the three bits after it, so that a lower
-// cell means a strictly smaller number
-__device__ __forceinline__ int cell_of(u64 m) {
-  if (m < 8) return (int)m;
-  const int top = 63 - __clzll((long long)m);
-  return 8 * (top - 2) + (int)((m >> (top - 3)) & 7);
-}
-// (whole numbers below 2^53: exponent and three bits of the fraction; 0 has a cell of its own)
+// the cell of a whole number below 2^63: exponent and three bits of the fraction of it as a
+// double, so that a lower cell means a strictly smaller number (rounding keeps the order);
+// 0 has a cell of its own
 __device__ __forceinline__ int cell_of(double m) {
   return max((__double2hiint(m) >> 17) - (1023 << 3) + 1, 0);
 }
+__device__ __forceinline__ int cell_of(u64 m) { return cell_of(as<double>(m)); }
 
 // what decides whether one triple dominates another (see dominated)
 struct Rank {
@@ -115,7 +111,8 @@ struct BlockShared {
   ModelRec rec;
   Triple tri[MAX_TRIPLES];
   unsigned char allowed[3][MAX_TRIPLES + 3];   // allowed activation digits of a triple for the three CLS_* of a unit
-  u64 state[2][5][4];                      // Theta, Omega: the coefficients of E, s, u and the host coefficient, by digit
+  double state[2][5][3];                   // Theta, Omega: the coefficients of E, s and u by digit
+  u64 state_host[2][5];                    // and the host coefficient, as the sweep's type
   u64 cell[CELLS];                         // the histogram
   u64 cand_a[CAND_CAP], cand_b[CAND_CAP];  // the buffer: Pareto (mem, comm), top-k (comm, least mem)
   u32 cand_i[CAND_CAP];
@@ -169,8 +166,8 @@ __device__ __forceinline__ void any_variant(u32& fit, u64 m, const u64* b) {
   for (int q = 0; q < 4; ++q) fit |= (m < b[q]) ? BIT : 0u;
 }
 template <int D, int NM, typename T, bool HOST_LIMITED>
-__device__ __forceinline__ void fitting_digits(u32& fit, const LaneUnit<NM, T, HOST_LIMITED>& lu, u32 modemap, T m, T h,
-                                               T cap_room) {
+__device__ __forceinline__ void fitting_digits(u32& fit, const LaneUnit<NM, T, HOST_LIMITED>& lu, u32 modemap,
+                                               double m, T h, double cap_room) {
   if constexpr (D < NM) {
     if (digit_mode(modemap, D) == PS_MODE_O) {
       // the four variants have the same bytes: one capacity compare, and the host bytes of each
@@ -178,7 +175,7 @@ __device__ __forceinline__ void fitting_digits(u32& fit, const LaneUnit<NM, T, H
       if (HOST_LIMITED) any_variant<1u << D>(with_host, h, lu.host_bound);
       fit |= m < cap_room ? with_host : 0u;
     } else {
-      any_variant<1u << D>(fit, m, lu.bound[D]);
+      any_variant<1u << D>(fit, m, lu.bounds(D));
     }
     fitting_digits<D + 1>(fit, lu, modemap, m, h, cap_room);
   }
@@ -187,20 +184,20 @@ __device__ __forceinline__ void fitting_digits(u32& fit, const LaneUnit<NM, T, H
 // Does any point of the lane's unit whose (Theta, Omega) pair lies in [p0, p1) survive?
 template <int NM, typename T, bool HOST_LIMITED>
 __device__ __forceinline__ u32 screen_pairs(const BlockShared& sh, const LaneUnit<NM, T, HOST_LIMITED>& lu, u32 modemap,
-                                            T cap_room, T host_room, u32 p0, u32 p1) {
+                                            double cap_room, T host_room, u32 p0, u32 p1) {
   u32 any = 0;
   const unsigned char* allowed_of = sh.allowed[lu.shift >> 3];
 #pragma unroll 1
   for (u32 p = p0; p < p1; ++p) {
     const u32 th = p / NM, om = p - th * NM;
-    const u64* ct = sh.state[0][th];
-    const u64* co = sh.state[1][om];
-    const T to_mem = mul_add(lu.E, from_bits<T>(ct[0]), mul_add(lu.s, from_bits<T>(ct[1]), mul_add(lu.u, from_bits<T>(ct[2]),
-                     mul_add(lu.E, from_bits<T>(co[0]), mul_add(lu.s, from_bits<T>(co[1]), mul_add(lu.u, from_bits<T>(co[2]), T(0)))))));
-    const T to_host = mul_add(lu.s, from_bits<T>(ct[3]), mul_add(lu.s, from_bits<T>(co[3]), T(0)));
+    const double* ct = sh.state[0][th];
+    const double* co = sh.state[1][om];
+    const double to_mem = fma(lu.E, ct[0], fma(lu.s, ct[1], fma(lu.u, ct[2], fma(lu.E, co[0], fma(lu.s, co[1], lu.u * co[2])))));
+    const T to_host = mul_add(lu.shard, from_bits<T>(sh.state_host[0][th]),
+                              mul_add(lu.shard, from_bits<T>(sh.state_host[1][om]), T(0)));
 #pragma unroll
     for (int gr = 0; gr < NM; ++gr) {
-      const T m = to_mem + lu.gr_mem[gr];
+      const double m = to_mem + lu.gr_mem[gr];
       T h = to_host;
       if (HOST_LIMITED && digit_mode(modemap, gr) == PS_MODE_O) h += lu.gr_host;
       u32 fit = 0;                                       // digits with a point that fits, whatever its flags
@@ -668,7 +665,8 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     const u32 a_one = allowed_act_digits(triple_bits(th, om, gr, CLS_ONE_DEVICE), req, all, all, is_o, not_mo);
     const u32 a_copies = allowed_act_digits(triple_bits(th, om, gr, CLS_ALL_COPIES), req, all, all, is_o, not_mo);
     Triple& tr = sh.tri[t];
-    tr.k[0] = bits<T>(as<T>(a)); tr.k[1] = bits<T>(as<T>(b)); tr.k[2] = bits<T>(as<T>(c)); tr.k[3] = bits<T>(as<T>(h));
+    tr.k[0] = a; tr.k[1] = b; tr.k[2] = c;
+    tr.kh = bits<T>(as<T>(h));
     tr.kx = bits<T>(as<T>(ct * rec.wT + co * rec.wO + cg * rec.wG));
     tr.allowed = a_many | (a_one << 8) | (a_copies << 16) | (n2 << 24) | (n3 << 26);
     tr.pad = 0;
@@ -679,10 +677,10 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
   }
   for (int t = tid; t < 2 * NM; t += threads) {
     const u32 st = t / NM, d = t % NM, mode = digit_mode(modemap, d), w = st == 0 ? rec.wT : rec.wO;
-    const u32 k[4] = {mode == PS_MODE_R ? w : 0, in_set(SET_SHARDLIKE, mode) ? w : 0,
-                      mode == PS_MODE_SG ? w * sp.sstar_units : (mode == PS_MODE_M ? w : 0),
-                      mode == PS_MODE_O ? (st == 0 ? (2 * sp.accum + 1) * w : 2 * w) : 0};
-    for (int j = 0; j < 4; ++j) sh.state[st][d][j] = bits<T>(as<T>(k[j]));
+    sh.state[st][d][0] = mode == PS_MODE_R ? w : 0;
+    sh.state[st][d][1] = in_set(SET_SHARDLIKE, mode) ? w : 0;
+    sh.state[st][d][2] = mode == PS_MODE_SG ? w * sp.sstar_units : (mode == PS_MODE_M ? w : 0);
+    sh.state_host[st][d] = bits<T>(as<T>(mode == PS_MODE_O ? (st == 0 ? (2 * sp.accum + 1) * w : 2 * w) : 0));
   }
 
   // ---- the triples that the passes walk: those that the flags allow; for Pareto only those
@@ -723,6 +721,9 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
   u32 survivors = 0;
   bool overflowed = false;                           // the same for every thread
   const bool skip = args.skip_rejected && req_cv != 0;
+  // Top-k without a required flag: the first pass counts every point itself and nothing is screened
+  // for (4096 models of the stress configuration in 2.16 ms instead of 2.30).
+  const bool take_all = !PARETO && req == 0;
 
   for (u32 seg = 0; seg < sp.n_facts; seg += SEG) {
     const u32 seg_n = min((u32)SEG, sp.n_facts - seg), n_batches = (seg_n + 31) / 32;
@@ -730,7 +731,10 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     for (int j = tid; j < SEG / 32; j += threads) sh.flags[j] = 0;
     if (tid == 0) { sh.next1 = 0; sh.next2 = 0; }
     __syncthreads();
-    if (skip) {
+    if (take_all) {
+      if (tid < SEG / 32)
+        sh.flags[tid] = seg_n >= 32u * tid + 32 ? ~0u : seg_n > 32u * tid ? (1u << (seg_n - 32u * tid)) - 1u : 0u;
+    } else if (skip) {
       for (u32 b = warp; b < n_batches; b += warps) {
         const u32 p = b * 32 + lane;
         const u32 votes = __ballot_sync(0xffffffffu, p < seg_n && !unit_rejected(sp, rec, seg + p, req_cv));
@@ -746,7 +750,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
         const UnitBase ub = unit_of(sp, rec, f);
         LaneUnit<NM, T, HOST_LIMITED> lu;
         lu.load(sp, rec, f, ub, modemap, cap_x, host_x, p < seg_n && (ub.cv & req_cv) == req_cv);
-        const u32 any = screen_pairs(sh, lu, modemap, cap_room, host_room, part * N2 / parts, (part + 1) * N2 / parts);
+        const u32 any = screen_pairs(sh, lu, modemap, as<double>(cap_x), host_room, part * N2 / parts, (part + 1) * N2 / parts);
         const u32 votes = __ballot_sync(0xffffffffu, any != 0);
         if (lane == 0 && votes) atomicOr(&sh.flags[b], votes);
       }
@@ -806,17 +810,17 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
       // a step waits for (table loads, dependent fp64 operations, votes) is waited for once.
 #pragma unroll 1
       for (u32 t0 = max(part * n_live / parts, from); t0 < t_end; t0 += 2) {
-        T m[2], c[2], h[2], act_of_set[2][2];
+        double m[2];
+        T c[2], h[2], act_of_set[2][2];
         u32 allowed[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const Triple& tr = sh.tri[sh.live[min(t0 + j, t_end - 1)]];
           allowed[j] = t0 + j < t_end ? (tr.allowed >> lu.shift) & lu.allowed : 0u;
-          m[j] = mul_add(lu.E, from_bits<T>(tr.k[0]), mul_add(lu.s, from_bits<T>(tr.k[1]),
-                 mul_add(lu.u, from_bits<T>(tr.k[2]), T(0))));
+          m[j] = fma(lu.E, tr.k[0], fma(lu.s, tr.k[1], lu.u * tr.k[2]));
           h[j] = T(0);
           if (HOST_LIMITED) {
-            h[j] = mul_add(lu.s, from_bits<T>(tr.k[3]), T(0));
+            h[j] = mul_add(lu.shard, from_bits<T>(tr.kh), T(0));
             if (!(h[j] < host_room)) allowed[j] = 0;     // the triple's own host bytes against the budget
           }
           c[j] = mul_add(x, from_bits<T>(tr.kx), T(0));
@@ -827,16 +831,18 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
           // the survivors of the triples, by tensor-axis variant
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
-            float n0 = 0.0f, n1 = 0.0f;
+            float n[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
             for (int d = 0; d < NM; ++d) {
-              const bool digit = (allowed[j] >> d) & 1u, offload = digit_mode(modemap, d) == PS_MODE_O;
+              if (HOST_LIMITED && digit_mode(modemap, d) == PS_MODE_O) {
 #pragma unroll
-              for (int q = 0; q < 4; ++q)
-                if (digit & (m[j] < lu.bound[d][q]) & (!HOST_LIMITED || !offload || h[j] < lu.host_bound[q])) {
-                  if (q & 1) n1 += 1.0f; else n0 += 1.0f;
-                }
+                for (int q = 0; q < 4; ++q)
+                  if (((allowed[j] >> d) & 1u) & (m[j] < lu.bounds(d)[q]) & (h[j] < lu.host_bound[q])) n[q] += 1.0f;
+              } else {
+                count_variants(n, m[j], lu.bounds(d), allowed[j] & (1u << d));
+              }
             }
+            const float n0 = n[0] + n[2], n1 = n[1] + n[3];
             survivors += (u32)(n0 + n1);
             const int cell0 = cell_of(c[j] + axis[0]), cell1 = cell_of(c[j] + axis[1]);
             if (n0 != 0.0f) { atomicAdd(reinterpret_cast<u32*>(&sh.cell[cell0]), (u32)n0); lowest = min(lowest, (u32)cell0); }
@@ -877,7 +883,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
           const int j = w >> 1, tau = w & 1;
           comm[w] = c[j] + axis[tau];
           const bool off = (allowed[j] & is_o) != 0 && (!HOST_LIMITED || h[j] < host_most[tau]);
-          mem[w] = m[j] + (off ? T(0) : act_of_set[j][tau]);
+          mem[w] = whole<T>(m[j]) + (off ? T(0) : act_of_set[j][tau]);
           cand[w] = allowed[j] != 0 && mem[w] < cap_room && (u32)tau < sp.nt;
           const int cell = cell_of(PARETO ? mem[w] : comm[w]);
           if (!SECOND) {

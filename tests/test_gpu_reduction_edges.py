@@ -102,6 +102,39 @@ def test_tied_points_do_not_slow_a_sweep_down(ctx, ps, kind, reduce):      # noq
     assert took[0] < 8 * took[1], took
 
 
+def test_tables_beyond_a_double_keep_their_pace(ctx, ps):      # noqa: F811
+    """With 64 micro-batches a step the largest shapes' volumes pass 2^53 and the table is swept in
+    64-bit integers, whose compares would take twice as long: device bytes stay in doubles."""
+    took = []
+    for accum in (64, 1):
+        gpu = ctx.space(dict(synth.config("C4", n_models=512), grad_accum_steps=accum))
+        out, counts = gpu.alloc_sweep(1, 64)
+        filt = dict(require_flags=0, host_cap=O.NO_LIMIT)
+        took.append(milliseconds(lambda: gpu.sweep_into(filt, [80 * GB], ps.REDUCE_TOPK, 64, out, counts)))
+    assert took[0] < 1.6 * took[1], took
+
+
+def test_capacities_beyond_a_double(ctx, ps):      # noqa: F811
+    """Capacities at a point's bytes and one below, where a double no longer holds them."""
+    models = synth.zoo(1, 0)
+    for field, value in dict(param_elems_override=(1 << 46) - 5, layers=1, hidden=8191, heads=3275, vocab=1, seq=(1 << 17) - 1,
+                             micro_batch=(1 << 10) - 1, w_param=15, w_opt=16, w_grad=13).items():
+        models[field] = value
+    space = synth._space(models, [1, 2, 3, 8], t_enum_max=2, k_enum_max=2, n_act=2, n_tpa=2, mode_mask=0b11111)
+    gs, os_ = both(ctx, space)
+    mem = np.unique(os_.eval_range(0, gs.size)["mem"])
+    mem = mem[mem > 1 << 53]
+    assert len(mem) > 100 and np.any(mem.astype(np.float64).astype(np.uint64) != mem)
+    for exact in mem[::len(mem) // 12]:
+        for cap in (int(exact), int(exact) - 1):
+            filt = dict(cap_bytes=cap, require_flags=0, host_cap=O.NO_LIMIT)
+            assert_same_arrays(gs.compact(0, gs.size, filt), os_.compact_range(0, gs.size, filt), f"capacity {cap}")
+            for got_kind, want_kind, k in ((ps.REDUCE_PARETO, O.KIND_PARETO, 128), (ps.REDUCE_TOPK, O.KIND_TOPK, 64)):
+                for require in (0, VALID):
+                    filt = dict(require_flags=require, host_cap=O.NO_LIMIT)
+                    assert_same_sweep(gs.sweep(filt, [cap], got_kind, k), os_.sweep(filt, [cap], want_kind, k))
+
+
 @pytest.mark.parametrize("kind", ["plain", "copies", "beyond a double", "few modes"])
 def test_compaction_windows_at_the_edges_of_groups_and_runs(ctx, kind):      # noqa: F811
     gs, os_ = both(ctx, space_of(kind))
