@@ -34,6 +34,7 @@ namespace {
 
 constexpr int MAX_D = 4;
 constexpr int MAX_STEPS = 16;
+constexpr int MAX_P = 8 * 32, MAX_EA = 8 * 4 * 32;   // the shape's ranges: units * h, units * b * h
 
 struct Dims {
   int units, h, b, P, EA, accum, steps, nbuf;
@@ -460,8 +461,11 @@ __global__ void __launch_bounds__(THREADS) k_verify(Dims dm, const ps_verify_cas
 template <int THREADS>
 cudaError_t launch_verify_t(const Dims& dm, const ps_verify_case* d_cases, u64 n, const double* d_data, u64 data_len,
                             double* d_theta_out, ps_verify_result* d_out, volatile u32* status, cudaStream_t stream) {
-  const int smem = make_layout(dm.P, dm.EA).total * (int)sizeof(double);      // at most 190 KB
-  cudaError_t e = cudaFuncSetAttribute(k_verify<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const int smem = make_layout(dm.P, dm.EA).total * (int)sizeof(double);
+  // (the limit belongs to the kernel, not to a launch: the same for every call, so that a small
+  // shape's call on another thread does not lower it between this one's two statements)
+  const int most = make_layout(MAX_P, MAX_EA).total * (int)sizeof(double);    // 188 KB
+  cudaError_t e = cudaFuncSetAttribute(k_verify<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)(n < (1u << 20) ? n : (1u << 20));
   k_verify<THREADS><<<blocks, THREADS, smem, stream>>>(dm, d_cases, n, d_data, data_len, d_theta_out, d_out, status);

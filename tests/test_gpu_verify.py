@@ -109,3 +109,38 @@ def test_verifier_reports_bad_cases_without_touching_memory(ctx, ps):
     with pytest.raises(ps.PsError) as e:
         ctx.verify_batch(dict(units=9, h=4, b=2), cases[:1], data)
     assert e.value.code == ps.E_RANGE
+
+
+def test_two_threads_with_shapes_of_different_size(ps):
+    """Each thread has a context of its own; the shapes take the same kernel with 24 and 188 KB of
+    shared memory a block, so the limit that one call sets must do for the other's launch."""
+    import threading
+    import torch
+    failed = []
+
+    def repeat(units):
+        stream = torch.cuda.Stream()
+        own = ps.Context(0, stream)
+        data, offsets, _ = problems(units, 32, 4, 1, seed=units)
+        with torch.cuda.stream(stream):
+            d_data = torch.from_numpy(data).cuda()
+            cases = np.array([(32, 2, offsets[2])], dtype=ps.VERIFY_CASE_DTYPE)
+            d_cases = torch.from_numpy(cases.view(np.uint8)).cuda()
+            d_out = torch.zeros(40, dtype=torch.uint8, device="cuda")
+        shape = ps._VerifyShape(units, 32, 4, 1, 1, 1, 2, 12, 2, 0, 0.05, 0.9, 0.999, 1e-8, 1e-12, 1e-14)
+        stream.synchronize()
+        for k in range(3000):
+            code = ps._lib.ps_verify_batch(own._h, ps.C.byref(shape), d_cases.data_ptr(), 1, d_data.data_ptr(),
+                                           len(data), d_out.data_ptr(), None)
+            if code != ps.OK:
+                failed.append((units, k, code))
+                break
+        if own.status() != ps.OK or d_out.cpu().numpy().view(ps.VERIFY_RESULT_DTYPE)["match"][0] != 1:
+            failed.append((units, "result"))
+
+    threads = [threading.Thread(target=repeat, args=(units,)) for units in (1, 8, 1, 8)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
