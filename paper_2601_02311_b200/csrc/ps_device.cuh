@@ -65,6 +65,11 @@ enum : u32 {
 __device__ __forceinline__ bool in_set(u32 set, u32 mode) { return (set >> mode) & 1u; }
 __device__ __forceinline__ u32 digit_mode(u32 modemap, u32 digit) { return (modemap >> (4 * digit)) & 7u; }
 
+// Host bytes of a point stay below this: offloaded activations at most 2^62 (the range of a
+// shape), the states at most (129 + 2 + 2) * 16 bytes of each of 2^46 elements.  A budget at or
+// above it limits nothing.
+constexpr u64 HOST_BYTES_END = ((u64)1 << 62) + ((u64)1 << 58);
+
 // ---------------------------------------------------------------- division
 // Divisors are degrees (< 2^24).  Powers of two, the common case, are shifts;
 // the branch is uniform wherever a warp works on one factorisation.

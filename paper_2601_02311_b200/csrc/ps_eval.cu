@@ -440,9 +440,9 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
   const u32 req = a.require_flags;
   constexpr u32 CV_BITS = PS_F_CV | PS_F_T_DIV_HEADS | PS_F_K_DIV_LAYERS | PS_F_TP_LE_MAX | PS_F_AXIS_FORM;
   const u32 req_cv = req & CV_BITS;
-  // capacities as exclusive bounds (memory and host bytes stay below 2^62)
+  // capacities as exclusive bounds (memory stays below 2^61)
   const u64 cap_x = min(a.cap_bytes, (u64)1 << 62) + 1;
-  const u64 host_x = min(a.host_cap, (u64)1 << 62) + 1;
+  const u64 host_x = min(a.host_cap, HOST_BYTES_END) + 1;
   constexpr u32 all = (1u << NM) - 1u;
   u32 own = 0, is_o = 0, not_mo = 0;
 #pragma unroll
@@ -684,7 +684,7 @@ template <int NM>
 static cudaError_t launch_count_t(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
   // every byte count exact in a double
   if (sp.all_small && a.cap_bytes < ((u64)1 << 53) - 1) {
-    if (NM < 4 || a.host_cap < ((u64)1 << 62)) k_compact_count<NM, double, true><<<a.n_runs, COUNT_WARPS * 32, 0, stream>>>(sp, a);
+    if (NM < 4 || a.host_cap < HOST_BYTES_END) k_compact_count<NM, double, true><<<a.n_runs, COUNT_WARPS * 32, 0, stream>>>(sp, a);
     else k_compact_count<NM, double, NM < 4><<<a.n_runs, COUNT_WARPS * 32, 0, stream>>>(sp, a);
   } else {
     k_compact_count<NM, u64, true><<<a.n_runs, COUNT_WARPS * 32, 0, stream>>>(sp, a);

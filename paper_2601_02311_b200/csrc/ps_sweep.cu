@@ -607,9 +607,9 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
 
   const u32 req = args.require_flags;
   const bool ext_in_objective = args.comm_kind == PS_COMM_PAPER_PLUS_EXT;
-  // capacities as exclusive bounds (memory and host bytes stay below 2^63)
+  // capacities as exclusive bounds (memory stays below 2^61)
   const u64 cap_x = min(PARETO ? args.cap_max : args.caps[blockIdx.y], (u64)1 << 62) + 1;
-  const u64 host_x = min(args.host_cap, (u64)1 << 62) + 1;
+  const u64 host_x = min(args.host_cap, HOST_BYTES_END) + 1;
   const T cap_room = as<T>(cap_x), host_room = as<T>(host_x);
   constexpr u32 CV_BITS = PS_F_CV | PS_F_T_DIV_HEADS | PS_F_K_DIV_LAYERS | PS_F_TP_LE_MAX | PS_F_AXIS_FORM;
   const u32 req_cv = req & CV_BITS;
@@ -1105,7 +1105,7 @@ template <int KIND, int NM>
 static cudaError_t launch_sweep_t(const SpaceDev& sp, const SweepArgs& a, int warps, cudaStream_t stream) {
   // every byte count exact in a double
   if (sp.all_small && a.cap_max < ((u64)1 << 53) - 1)
-    return NM < 4 || a.host_cap < ((u64)1 << 62) ? launch_sweep_p<KIND, NM, double, true>(sp, a, warps, stream)
+    return NM < 4 || a.host_cap < HOST_BYTES_END ? launch_sweep_p<KIND, NM, double, true>(sp, a, warps, stream)
                                                  : launch_sweep_p<KIND, NM, double, NM < 4>(sp, a, warps, stream);
   return launch_sweep_p<KIND, NM, u64, true>(sp, a, warps, stream);
 }

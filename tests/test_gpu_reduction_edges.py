@@ -150,3 +150,23 @@ def test_compaction_windows_at_the_edges_of_groups_and_runs(ctx, kind):      # n
                      dict(cap_bytes=1 << 61, require_flags=O.F_GI | O.F_SC, host_cap=64 * GB)):
             assert_same_arrays(gs.compact(first, last - first, filt), os_.compact_range(first, last - first, filt),
                                f"{kind} [{first}, {last})")
+
+
+@pytest.mark.parametrize("mode_mask", [0b11111, 0b11010])
+@pytest.mark.parametrize("params", [1 << 41, 1 << 46])      # byte counts in doubles and in 64-bit integers
+def test_host_bytes_at_the_end_of_their_range(ctx, ps, params, mode_mask):      # noqa: F811
+    """Offloaded activations of 2^62 - 2^48.9 bytes with offloaded states on top: more than 2^62."""
+    models = synth.zoo(1, 0)
+    for field, value in dict(param_elems_override=params, layers=1, hidden=8192, heads=3276, vocab=1, seq=1 << 17,
+                             micro_batch=1 << 10, w_param=16, w_opt=16, w_grad=16).items():
+        models[field] = value
+    space = dict(synth._space(models, [1, 2, 3, 8], t_enum_max=2, k_enum_max=2, n_act=2, n_tpa=2, mode_mask=mode_mask),
+                 grad_accum_steps=8)
+    gs, os_ = both(ctx, space)
+    assert int(os_.eval_range(0, gs.size)["host"].max()) > 1 << 62
+    for host_cap in (O.NO_LIMIT, 1 << 62, (1 << 62) + (1 << 45)):
+        for cap in (1 << 50, O.NO_LIMIT):
+            filt = dict(cap_bytes=cap, require_flags=0, host_cap=host_cap)
+            assert_same_arrays(gs.compact(0, gs.size, filt), os_.compact_range(0, gs.size, filt), f"{cap}, {host_cap}")
+            for got_kind, want_kind, k in ((ps.REDUCE_PARETO, O.KIND_PARETO, 128), (ps.REDUCE_TOPK, O.KIND_TOPK, 64)):
+                assert_same_sweep(gs.sweep(filt, [cap], got_kind, k), os_.sweep(filt, [cap], want_kind, k))
