@@ -149,7 +149,6 @@ int ps_create(ps_ctx** out, int device, void* cuda_stream) {
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { ps_destroy(ctx); return PS_E_CUDA; }
   ctx->sm_count = prop.multiProcessorCount;
-  ctx->compact_calls = 0;
   if (!ctx->check || cudaMalloc(&ctx->d_lengths, 4 * sizeof(u32)) != cudaSuccess ||
       cudaHostAlloc(reinterpret_cast<void**>(&ctx->h), sizeof(HostWords), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess ||
       cudaMemsetAsync(ctx->d_lengths, 0, 4 * sizeof(u32), ctx->stream) != cudaSuccess) {
@@ -450,11 +449,8 @@ int ps_eval_batch(ps_ctx* ctx, const ps_space* sp, uint64_t first, uint64_t coun
     a.group_offset = reinterpret_cast<u32*>(base);
     a.nonempty = reinterpret_cast<u32*>(base + group_bytes);
     a.run_offset = reinterpret_cast<u64*>(base + 2 * group_bytes);
-    // the list's length: one of the context's two counters, zero by now (the previous
-    // compaction cleared it); this call clears the other
-    a.n_nonempty = ctx->d_lengths + (ctx->compact_calls & 1u);
-    a.n_nonempty_other = ctx->d_lengths + ((ctx->compact_calls + 1) & 1u);
-    ++ctx->compact_calls;
+    a.n_nonempty = ctx->d_lengths;
+    a.n_listed = ctx->d_lengths + 1;
     a.blocks_done = ctx->d_lengths + 2;
     CUDA_OK(launch_eval_count(sp->dev, a, ctx->stream));
     CUDA_OK(launch_eval_write(sp->dev, a, ctx->stream));

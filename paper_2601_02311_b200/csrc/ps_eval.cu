@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE && NM < 5 ? EVAL_M
   // write: the groups that have survivors, from the count pass's list, dealt round-robin
   const u32 per_warp = (a.n_tiles + n_warps - 1) / n_warps;
   const u32 it_begin = MODE == MODE_WRITE ? warp_global : (u32)min((u64)warp_global * per_warp, (u64)a.n_tiles);
-  const u32 it_end = MODE == MODE_WRITE ? *a.n_nonempty : min(it_begin + per_warp, a.n_tiles);
+  const u32 it_end = MODE == MODE_WRITE ? *a.n_listed : min(it_begin + per_warp, a.n_tiles);
   const u32 it_step = MODE == MODE_WRITE ? n_warps : 1u;
   const u32 groups_per_model = sp.n_facts * sp.nvt;
 
@@ -628,7 +628,8 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
   __syncthreads();
   if (tid == 0) {
     *a.n_out = carry;
-    *a.n_nonempty_other = 0;      // the next compaction's list starts empty
+    *a.n_listed = *static_cast<volatile u32*>(a.n_nonempty);
+    *a.n_nonempty = 0;            // the next compaction's list starts empty
     *a.blocks_done = 0;
   }
 }

@@ -19,11 +19,10 @@ struct ps_ctx {
   cudaStream_t stream;
   void* scratch;
   size_t scratch_bytes;
-  u32* d_lengths;     // the compaction's two list lengths and its count of finished blocks
+  u32* d_lengths;     // the compaction's counters (EvalArgs: n_nonempty, n_listed, blocks_done)
   HostWords* h;       // pinned host memory that kernels write to (nothing has to be copied back)
   std::mutex* check;  // one ps_check_composition at a time uses h->entry
   u32 checks;
-  u32 compact_calls;  // compactions enqueued so far (picks which list length a call uses)
   int sm_count;
 };
 
@@ -93,10 +92,12 @@ struct EvalArgs {
   u32 n_units, n_runs;
   u32* group_offset;        // [n_tiles] survivors of the earlier groups of the group's run
   u32* nonempty;            // [n_tiles] the groups that have survivors, in any order
-  u32* n_nonempty;          // how many (zero before the count pass)
-  u32* n_nonempty_other;    // the next compaction's counter: cleared by the count pass, so that no
-                            // call needs a memset of its own (calls alternate between two counters)
-  u32* blocks_done;         // count pass: blocks that have finished (zero between calls)
+  // Counters of the count pass: places given out in the list and blocks that have finished.  Both
+  // are zero between calls: the last block leaves the list's length in n_listed and clears them.  So
+  // no call needs a memset of its own, and a captured call can be replayed.
+  u32* n_nonempty;
+  u32* blocks_done;
+  u32* n_listed;
   u64* run_offset;          // [n_runs] survivors of each run, then of all runs before it
   volatile u32* status;
 };

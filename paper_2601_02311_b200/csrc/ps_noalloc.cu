@@ -103,9 +103,8 @@ extern "C" int ps_eval_compact_noalloc(ps_ctx* ctx, const ps_space* sp, uint64_t
   eval_plan_runs(sp->dev, a);
   a.group_offset = reinterpret_cast<u32*>(bytes);
   a.nonempty = reinterpret_cast<u32*>(bytes + COUNT_BYTES);
-  a.n_nonempty = ctx->d_lengths + (ctx->compact_calls & 1u);          // the context's alternating list lengths
-  a.n_nonempty_other = ctx->d_lengths + ((ctx->compact_calls + 1) & 1u);
-  ++ctx->compact_calls;
+  a.n_nonempty = ctx->d_lengths;                           // the context's counters
+  a.n_listed = ctx->d_lengths + 1;
   a.blocks_done = ctx->d_lengths + 2;
   a.run_offset = reinterpret_cast<u64*>(bytes + 2 * COUNT_BYTES + LENGTH_BYTES);
   // The array still holds the previous call's numbers.  Every word this call reads is

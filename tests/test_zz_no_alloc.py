@@ -95,3 +95,43 @@ def test_noalloc_refuses_windows_beyond_its_fixed_array():
     ctx.check_status()
     gs.close()
     ctx.close()
+
+
+def test_captured_compaction_can_be_replayed():
+    """A replay finds the counters as the captured call found them, whatever ran in between."""
+    import paper_2601_02311_b200.ps as ps
+    stream = torch.cuda.Stream()
+    ctx = ps.Context(0, stream)
+    space = synth.config("C3", n_models=2)
+    gs, os_ = ctx.space(space), O.Space(space)
+    first, count, filt = 777, 600_001, dict(require_flags=ps.F_VALID, cap_bytes=192 * synth.GB)
+    want = os_.compact_range(first, count, filt)
+    with torch.cuda.stream(stream):
+        out = gs.alloc_outputs(count)
+        idx = torch.empty(count, dtype=torch.int64, device="cuda")
+        n = torch.empty(1, dtype=torch.int64, device="cuda")
+    other = dict(first=1_000_003, count=90_000, filt=dict(require_flags=0, cap_bytes=80 * synth.GB))
+
+    def check():
+        stream.synchronize()
+        k = int(n.item())
+        assert k == len(want["idx"])
+        for name in FIELDS:
+            assert np.array_equal(out[name][:k].cpu().numpy().view(want[name].dtype), want[name]), name
+        assert np.array_equal(idx[:k].cpu().numpy().view(np.uint64), want["idx"])
+
+    gs.compact_noalloc_into(first, count, out, filt, idx, n)      # (looks the array's address up)
+    check()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        gs.compact_noalloc_into(first, count, out, filt, idx, n)
+    for between in (0, 0, 1, 2):
+        with torch.cuda.stream(stream):
+            for _ in range(between):
+                assert len(gs.compact(**other)["idx"]) == len(os_.compact_range(**other)["idx"])
+            n.zero_()
+            graph.replay()
+        check()
+    del graph
+    gs.close()
+    ctx.close()
