@@ -365,7 +365,7 @@ class Space:
     # ---- ps_sweep_pareto
     def sweep_into(self, filt: dict, caps, kind: int, max_entries: int, d_out: torch.Tensor,
                    d_counts: torch.Tensor):
-        self._sweep(filt, caps, kind, max_entries, d_out.data_ptr(), d_counts.data_ptr())
+        self._sweep(filt, caps, kind, max_entries, _dptr(d_out), _dptr(d_counts))
 
     def _sweep(self, filt, caps, kind, max_entries, out_ptr, counts_ptr):
         caps = np.ascontiguousarray(caps, dtype=np.uint64)

@@ -518,3 +518,12 @@ def test_sweeps_that_skip_rejected_factorisations_give_the_same_tables(ctx, ps):
             filt = dict(require_flags=req)
             want = os_.sweep(filt, caps[1:], O.KIND_TOPK, 64, n_threads=8)
             assert_same_sweep(gs.sweep(dict(filt, skip_rejected=1), caps[1:], ps.REDUCE_TOPK, 64), want)
+
+
+def test_sweep_without_output_buffers_is_refused(ctx, ps):
+    gs = ctx.space(synth.config("C0"))
+    out, counts = gs.alloc_sweep(1, 8)
+    for d_out, d_counts in ((None, counts), (out, None)):
+        with pytest.raises(ps.PsError) as e:
+            gs.sweep_into(dict(require_flags=0), [80 * synth.GB], ps.REDUCE_TOPK, 8, d_out, d_counts)
+        assert e.value.code == ps.E_NULLPTR
