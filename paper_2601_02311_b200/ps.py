@@ -7,6 +7,7 @@ CPU fallback.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 
 import numpy as np
@@ -157,8 +158,23 @@ def _dptr(t):
     return None if t is None else C.c_void_p(t.data_ptr())
 
 
+def _on_own_stream(method):
+    """For methods that allocate: their tensors come into being, and are filled and read back, on the
+    stream that the library enqueues on.  On torch's current stream, where that is another one, a
+    buffer's zeros could land after the kernel's results, or a kernel write to memory that work
+    before it still uses."""
+    @functools.wraps(method)
+    def run(self, *args, **kwargs):
+        ctx = getattr(self, "ctx", self)
+        if ctx.on_current_stream():
+            return method(self, *args, **kwargs)
+        with torch.cuda.stream(ctx.stream if ctx.stream is not None else torch.cuda.default_stream(ctx.device)):
+            return method(self, *args, **kwargs)
+    return run
+
+
 class Context:
-    """ps_ctx: one per (device, stream)."""
+    """ps_ctx: one per (device, stream); without a stream it enqueues on the device's default stream."""
 
     def __init__(self, device: int = 0, stream: torch.cuda.Stream | None = None):
         if not torch.cuda.is_available():
@@ -217,6 +233,7 @@ class Context:
         _check(_lib.ps_select(self._h, _dptr(d_queries), n, headroom[0], headroom[1], layer[0], layer[1],
                               tp_degree, _dptr(d_out)), "ps_select")
 
+    @_on_own_stream
     def select(self, queries: np.ndarray, headroom=(7, 10), layer=(3, 10), tp_degree=8) -> np.ndarray:
         """Algorithm 1 for a structured array of SELECT_QUERY_DTYPE; returns SELECT_RESULT_DTYPE."""
         q = np.ascontiguousarray(queries)
@@ -227,6 +244,7 @@ class Context:
         self.check_status()
         return d_o.cpu().numpy()[:len(q) * 32].view(SELECT_RESULT_DTYPE)
 
+    @_on_own_stream
     def verify_batch(self, shape: dict, cases: np.ndarray, data: np.ndarray, want_theta: bool = False):
         """ps_verify_batch: `cases` a VERIFY_CASE_DTYPE array, `data` a float64 array holding every
         case's problem; returns VERIFY_RESULT_DTYPE records (and the final parameters)."""
@@ -329,6 +347,7 @@ class Space:
             out[k] = torch.empty(max(count, 1), dtype=dt, device=dev)
         return out
 
+    @_on_own_stream
     def eval_batch(self, first: int, count: int,
                    fields=("mem", "comm_paper", "comm_ext", "host", "flags")) -> dict:
         """Materialise [first, first+count) and return numpy arrays (unsigned)."""
@@ -337,6 +356,7 @@ class Space:
         self.ctx.check_status()
         return {k: _to_unsigned(v[:count]) for k, v in out.items()}
 
+    @_on_own_stream
     def compact(self, first: int, count: int, filt: dict,
                 fields=("mem", "comm_paper", "comm_ext", "host", "flags")) -> dict:
         """Filter and compact; returns numpy arrays of the survivors incl. 'idx'."""
@@ -374,6 +394,7 @@ class Space:
                                     kind, max_entries, out_ptr, counts_ptr),
                "ps_sweep_pareto")
 
+    @_on_own_stream
     def select_compare(self, n_index: int, device_bytes: int, filt: dict, d_frontier: torch.Tensor,
                        d_counts: torch.Tensor, n_caps: int, cap_index: int, max_entries: int, fast: int = 1,
                        headroom=(7, 10), layer=(3, 10), tp_degree: int = 8) -> np.ndarray:
@@ -392,14 +413,16 @@ class Space:
         d_counts = torch.empty(self.n_models * n_caps, dtype=torch.int32, device=dev)
         return d_out, d_counts
 
+    @_on_own_stream
     def sweep(self, filt: dict, caps, kind: int, max_entries: int):
-        """Returns (entries[n_models, n_caps, max_entries] structured, counts[n_models, n_caps])."""
+        """Returns (entries[n_models, n_caps, max_entries] structured, counts[n_models, n_caps]).  Both are
+        views of one buffer; up to PINNED_RESULT_BYTES it is page-locked for as long as either is kept."""
         rows = self.n_models * len(caps)
         at = rows * max_entries * 40                   # the counts lie behind the entries: one copy brings both
         d_all = torch.empty(at + rows * 4, dtype=torch.uint8, device=self.ctx.torch_device)
         base = d_all.data_ptr()
         self._sweep(filt, caps, kind, max_entries, base, base + at)
-        if d_all.numel() <= PINNED_RESULT_BYTES and self.ctx.on_current_stream():
+        if d_all.numel() <= PINNED_RESULT_BYTES:
             # a small result: the copy is enqueued behind the sweep and one wait covers both
             host = torch.empty(d_all.numel(), dtype=torch.uint8, pin_memory=True)
             host.copy_(d_all, non_blocking=True)

@@ -527,3 +527,33 @@ def test_sweep_without_output_buffers_is_refused(ctx, ps):
         with pytest.raises(ps.PsError) as e:
             gs.sweep_into(dict(require_flags=0), [80 * synth.GB], ps.REDUCE_TOPK, 8, d_out, d_counts)
         assert e.value.code == ps.E_NULLPTR
+
+
+@pytest.mark.parametrize("own_is_current", [False, True])
+def test_calls_that_allocate_with_a_stream_of_the_context(ps, own_is_current):
+    """The current stream is busy while the library works on its own: results must not wait for it,
+    nor be overwritten by what it still has to do."""
+    import torch
+    stream = torch.cuda.Stream()
+    ctx = ps.Context(0, stream)
+    space = synth.config("C3", n_models=2)
+    gs, os_ = ctx.space(space), O.Space(space)
+    filt = dict(require_flags=VALID, cap_bytes=192 * synth.GB)
+    with torch.cuda.stream(stream if own_is_current else torch.cuda.Stream()):
+        busy = torch.ones(1 << 26, dtype=torch.int64, device="cuda")
+        for _ in range(20):
+            busy.add_(1)
+        del busy                                     # its memory is free for the next allocation on this stream
+        torch.cuda._sleep(50_000_000)
+        got = gs.compact(0, 400_000, filt)
+        assert_same_arrays(got, os_.compact_range(0, 400_000, filt), "compact")
+        torch.cuda._sleep(50_000_000)
+        assert_same_sweep(gs.sweep(filt, [80 * synth.GB], ps.REDUCE_PARETO, 64), os_.sweep(filt, [80 * synth.GB], O.KIND_PARETO, 64))
+        torch.cuda._sleep(50_000_000)
+        large = gs.sweep(filt, [80 * synth.GB, 192 * synth.GB], ps.REDUCE_PARETO, 8192)     # beyond the page-locked read-back
+        assert_same_sweep(large, os_.sweep(filt, [80 * synth.GB, 192 * synth.GB], O.KIND_PARETO, 8192))
+        torch.cuda._sleep(50_000_000)
+        assert_same_arrays(gs.eval_batch(7, 3000), os_.eval_range(7, 3000), "window")
+    torch.cuda.synchronize()
+    gs.close()
+    ctx.close()
