@@ -531,29 +531,29 @@ def test_sweep_without_output_buffers_is_refused(ctx, ps):
 
 @pytest.mark.parametrize("own_is_current", [False, True])
 def test_calls_that_allocate_with_a_stream_of_the_context(ps, own_is_current):
-    """The current stream is busy while the library works on its own: results must not wait for it,
-    nor be overwritten by what it still has to do."""
+    """The current stream is busy while the library works on its own: what it still has to do, such as
+    clearing a counter, must not land on the results."""
     import torch
     stream = torch.cuda.Stream()
     ctx = ps.Context(0, stream)
     space = synth.config("C3", n_models=2)
     gs, os_ = ctx.space(space), O.Space(space)
     filt = dict(require_flags=VALID, cap_bytes=192 * synth.GB)
+    caps = [80 * synth.GB, 192 * synth.GB]
+    want_window, want_kept = os_.eval_range(7, 3000), os_.compact_range(0, 400_000, filt)
+    want_small = os_.sweep(filt, caps, O.KIND_PARETO, 64)
+    want_large = os_.sweep(filt, caps, O.KIND_PARETO, 8192)            # beyond the page-locked read-back
     with torch.cuda.stream(stream if own_is_current else torch.cuda.Stream()):
-        busy = torch.ones(1 << 26, dtype=torch.int64, device="cuda")
-        for _ in range(20):
-            busy.add_(1)
-        del busy                                     # its memory is free for the next allocation on this stream
-        torch.cuda._sleep(50_000_000)
-        got = gs.compact(0, 400_000, filt)
-        assert_same_arrays(got, os_.compact_range(0, 400_000, filt), "compact")
-        torch.cuda._sleep(50_000_000)
-        assert_same_sweep(gs.sweep(filt, [80 * synth.GB], ps.REDUCE_PARETO, 64), os_.sweep(filt, [80 * synth.GB], O.KIND_PARETO, 64))
-        torch.cuda._sleep(50_000_000)
-        large = gs.sweep(filt, [80 * synth.GB, 192 * synth.GB], ps.REDUCE_PARETO, 8192)     # beyond the page-locked read-back
-        assert_same_sweep(large, os_.sweep(filt, [80 * synth.GB, 192 * synth.GB], O.KIND_PARETO, 8192))
-        torch.cuda._sleep(50_000_000)
-        assert_same_arrays(gs.eval_batch(7, 3000), os_.eval_range(7, 3000), "window")
+        for busy in (False, True):                   # the first round brings every buffer into the allocator's pools
+            for call, check, want in (
+                    (lambda: gs.compact(0, 400_000, filt), assert_same_arrays, want_kept),
+                    (lambda: gs.sweep(filt, caps, ps.REDUCE_PARETO, 64), assert_same_sweep, want_small),
+                    (lambda: gs.sweep(filt, caps, ps.REDUCE_PARETO, 8192), assert_same_sweep, want_large),
+                    (lambda: gs.eval_batch(7, 3000), assert_same_arrays, want_window)):
+                torch.cuda.synchronize()
+                if busy:
+                    torch.cuda._sleep(100_000_000)
+                check(call(), want)
     torch.cuda.synchronize()
     gs.close()
     ctx.close()
