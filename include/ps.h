@@ -94,7 +94,7 @@ enum { PS_REDUCE_PARETO = 0, PS_REDUCE_TOPK = 1 };
 
 #define PS_NO_LIMIT UINT64_MAX
 #define PS_TOPK_MAX 64           /* largest max_entries of a top-k sweep            */
-#define PS_FRONTIER_FAST 128     /* a model whose frontier is longer (here or at a stage of its
+#define PS_FRONTIER_FAST 128     /* a model whose frontier has more entries (384 at a stage of its
                                     reduction) is reduced by a slow exact path             */
 
 /* ------------------------------------------------------------------ types */
@@ -172,9 +172,11 @@ typedef struct {
   uint32_t require_flags;
   uint32_t comm_kind;     /* objective of the sweeps: PS_COMM_PAPER or ..._PLUS_EXT */
   uint64_t cap_bytes;     /* ps_eval_batch only; the sweeps take their own list     */
-  uint32_t skip_rejected; /* sweeps only.  0: every point is evaluated (its capacity compare is
-                             executed, then masked by the flags) -- what the throughput figures
-                             are quoted on.  1: a factorisation whose composition bits (T | heads,
+  uint32_t skip_rejected; /* sweeps only.  0: every factorisation is evaluated, its points held
+                             against the capacity, then masked by the flags -- what the throughput
+                             figures are quoted on.  (Points that must have the same bytes, the up
+                             to four variants of one placement with offloaded activations, may share
+                             a compare: 17 compares for 20 points.)  1: a factorisation whose composition bits (T | heads,
                              K | layers, T <= tp_max_valid) already miss a required flag is not
                              evaluated at all; same results, less work when the filter requires
                              PS_F_CV or one of its reasons */
@@ -239,7 +241,8 @@ int ps_space_decode(const ps_space* space, uint64_t idx, ps_point* out);
  *    index order; d_idx_out (device, may be null) receives their indices,
  *    *d_n_out (device scalar, required) their number; flags carry
  *    PS_F_FEASIBLE.  Outputs need room for `count` elements in the worst case.
- * count may be 0. */
+ * count may be 0.  A captured call may be replayed while the context's scratch
+ * has not grown since (it grows with the groups of a filtered window). */
 int ps_eval_batch(ps_ctx* ctx, const ps_space* space, uint64_t first, uint64_t count,
                   const ps_filter* filter, ps_out_soa out, uint64_t* d_idx_out,
                   uint64_t* d_n_out);

@@ -431,11 +431,9 @@ int ps_eval_batch(ps_ctx* ctx, const ps_space* sp, uint64_t first, uint64_t coun
   a.out = out;
   a.idx_out = d_idx_out;
   a.n_out = d_n_out;
-  a.status = ctx->h->status;
   if (!filter) {
     CUDA_OK(launch_eval_materialise(sp->dev, a, ctx->stream));
   } else {
-    a.has_filter = 1;
     a.cap_bytes = filter->cap_bytes;
     a.host_cap = filter->host_cap;
     a.require_flags = filter->require_flags & ~(u32)PS_F_FEASIBLE;

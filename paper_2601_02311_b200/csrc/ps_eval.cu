@@ -29,13 +29,12 @@
 
 namespace {
 
-// Launch shapes (blocks of four warps per SM; four are resident at a time).  Materialise is
-// fastest with about one group per warp: short-lived blocks keep the warps of an
-// SM at different stages (set-up, staging, draining stores) and the running
-// warps write neighbouring stretches of every output array.  The write pass takes the listed groups round-robin; with
-// many short blocks the stores of neighbouring groups are in flight together
-// (every point surviving: 0.56 of the copy bandwidth with 32 warps in the grid per
-// SM, 0.62 with 256).
+// Launch shapes (blocks of four warps).  Materialise is fastest with about one group per warp:
+// short-lived blocks keep the warps of an SM at different stages (set-up, staging, draining
+// stores) and the running warps write neighbouring stretches of every output array.  The write
+// pass takes the listed groups round-robin; with many short blocks the stores of neighbouring
+// groups are in flight together (2^24 points all surviving 0.171 ms with 64 blocks per SM in the
+// grid, 0.189 with 8; 256 codes a group 0.149 and 0.164).
 #ifndef EVAL_BULK_EVICT_FIRST
 #define EVAL_BULK_EVICT_FIRST 1
 #endif
@@ -425,7 +424,7 @@ __device__ __forceinline__ double state_bytes(const LaneUnit<NM, T, HOST_LIMITED
 // (Theta, Omega) pairs.  What bounds it: the fp64 pipe (a compare per point), and for small
 // windows the chain of a unit's set-up.  As one warp per run of groups, its lanes the
 // triples, it took 21 us for 2^25 points and was followed by a scan kernel of 3 us; like
-// this it takes 15.
+// this it takes 12.
 constexpr int COUNT_WARPS = 8;
 template <int NM, typename T, bool HOST_LIMITED>
 __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev sp, EvalArgs a) {

@@ -63,10 +63,10 @@ struct SweepArgs {
 cudaError_t launch_sweep(int kind, const SpaceDev& sp, const SweepArgs& a, int sm_count, cudaStream_t stream);
 
 // ---- batch evaluation
-/* Block shape of the window kernels: four resident blocks of four warps (128 registers a thread
-   either way).  Against two blocks of eight warps: materialise -5 % (625 codes a group) to -13 %
-   (256 codes), sparse compaction -3 % to -8 %; short blocks spread the warps' set-up and store
-   phases better. */
+/* Block shape of the window kernels: blocks of four warps, four of them resident (128 registers a
+   thread; the write pass with up to four modes five, see EVAL_MIN_BLOCKS_WRITE).  Against two
+   blocks of eight warps: materialise -5 % (625 codes a group) to -13 % (256 codes); short blocks
+   spread the warps' set-up and store phases better. */
 #ifndef EVAL_THREADS
 #define EVAL_THREADS 128
 #endif
@@ -82,7 +82,6 @@ struct EvalArgs {
   // filter (compaction modes)
   u64 cap_bytes, host_cap;
   u32 require_flags;        // without PS_F_FEASIBLE
-  u32 has_filter;
   ps_out_soa out;
   u64* idx_out;
   u64* n_out;
@@ -99,7 +98,6 @@ struct EvalArgs {
   u32* blocks_done;
   u32* n_listed;
   u64* run_offset;          // [n_runs] survivors of each run, then of all runs before it
-  volatile u32* status;
 };
 
 void eval_plan_runs(const SpaceDev& sp, EvalArgs& a);   // fills first_unit, n_units, n_runs

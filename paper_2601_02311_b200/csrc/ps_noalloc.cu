@@ -94,8 +94,6 @@ extern "C" int ps_eval_compact_noalloc(ps_ctx* ctx, const ps_space* sp, uint64_t
   a.out = out;
   a.idx_out = d_idx_out;
   a.n_out = d_n_out;
-  a.status = ctx->h->status;
-  a.has_filter = 1;
   a.cap_bytes = filter->cap_bytes;
   a.host_cap = filter->host_cap;
   a.require_flags = filter->require_flags & ~(u32)PS_F_FEASIBLE;

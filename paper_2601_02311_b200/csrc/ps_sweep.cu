@@ -7,11 +7,12 @@
 // a sum of three terms, one per state, so the next triple costs one addition, and what is
 // uniform (modes, allowed digits, coefficients) comes from small tables of the block.
 //
-// Screening.  Every point of every unit: one compare against its bound, masked by the
-// flags that the placement code and the composition allow.  It leaves the list of the
-// units that have survivors (an eighth of them on the stress configuration), which the
-// next two passes walk densely.  (With ps_filter.skip_rejected the list is made from the
-// composition tests alone.)
+// Screening.  Every unit: its points are compared with their bounds (the four variants of
+// the offloaded digit have the same bytes: 17 compares for 20 points), masked by the flags
+// that the placement code and the composition allow.  It leaves the list of the units that
+// have survivors (an eighth of them on the stress configuration), which the next two
+// passes walk densely.  (With ps_filter.skip_rejected the list is made from the
+// composition tests alone; top-k without required flags lists all units.)
 //
 // First pass, over the cells of a histogram (an eighth of an octave each).
 //   Pareto: the least communication of the candidates whose bytes fall into a cell
@@ -27,12 +28,12 @@
 // The block then emits the entries, evaluating each again from its index as a self-check.
 // A frontier that outgrows the buffer takes a slow exact path.
 //
-// What bounds it: the fp64 pipe and the issue slots of the screening (a compare per point;
-// 64 a clock and SM).  4096 models of the stress configuration, 6.96e9 points: top-k 1.94 ->
-// 0.79 ms, Pareto 2.37 -> 0.85 ms against a sweep whose warps took a unit each (the set-up
-// of a unit paid by a whole warp, candidates inserted one by one into a sorted list per
-// warp, the lists merged by a second kernel); 1024 models skipping rejected factorisations
-// 0.41 -> 0.10 ms.  The screening alone takes 0.52 and 0.58 ms of the former two.
+// What bounds it: the fp64 pipe and the issue slots of the screening (64 compares a clock and
+// SM).  4096 models of the stress configuration, 6.96e9 points: top-k 1.94 -> 0.76 ms, Pareto
+// 2.37 -> 0.84 ms against a sweep whose warps took a unit each (the set-up of a unit paid by a
+// whole warp, candidates inserted one by one into a sorted list per warp, the lists merged by
+// a second kernel); 1024 models skipping rejected factorisations 0.41 -> 0.084 ms.  The
+// screening alone takes 0.52 and 0.58 ms of the former two.
 #include <type_traits>
 #include "ps_device.cuh"
 #include "ps_internal.h"
@@ -248,9 +249,9 @@ __device__ __noinline__ void sort_candidates(BlockShared& sh, int n) {
 }
 
 // Up to this many candidates every thread tests its own against all others (no barrier in
-// the loop); more are sorted, whose work grows more slowly.  With 64 instead the zoo's
-// frontiers take 0.110 ms instead of 0.100; without the sort top-k of the stress
-// configuration takes 0.90 ms instead of 0.79.
+// the loop); more are sorted, whose work grows more slowly.  Never sorted, the stress
+// configuration takes 0.826 ms for top-k instead of 0.766 and 0.887 for the frontiers instead
+// of 0.840; with 64 instead of 128 0.755 and 0.838, and the zoo's frontiers 0.6 % more.
 constexpr int PAIRWISE = 128;
 
 // Closes up the candidates p < n for which `keep(p, its key)` holds, by one warp, 32 at a

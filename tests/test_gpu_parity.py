@@ -544,7 +544,7 @@ def test_calls_that_allocate_with_a_stream_of_the_context(ps, own_is_current):
     want_small = os_.sweep(filt, caps, O.KIND_PARETO, 64)
     want_large = os_.sweep(filt, caps, O.KIND_PARETO, 8192)            # beyond the page-locked read-back
     with torch.cuda.stream(stream if own_is_current else torch.cuda.Stream()):
-        for busy in (False, True):                   # the first round brings every buffer into the allocator's pools
+        for busy in (False, True):                   # the first time brings every buffer into the allocator's pools
             for call, check, want in (
                     (lambda: gs.compact(0, 400_000, filt), assert_same_arrays, want_kept),
                     (lambda: gs.sweep(filt, caps, ps.REDUCE_PARETO, 64), assert_same_sweep, want_small),
