@@ -23,6 +23,9 @@ def space_of(kind):
     if kind == "ragged":
         return dict(synth.config("C3", n_models=2), n_values=np.asarray([1, 7, 36, 96, 360, 1000, 1536], dtype=np.uint32),
                     t_enum_max=12, k_enum_max=36)
+    if kind == "crowded cells":         # activations outweigh the rest: a quarter of the candidates pass the staircase
+        return dict(space_of("ragged"), models=synth.zoo(2, 3, max_layers=160, max_hidden_mult=128, seqs=(1 << 17,),
+                                                         max_micro_batch=64), n_act_variants=1, replication_k=3)
     if kind == "tied in a unit":        # 122 pairs of 460 (triple, variant) under a host budget of 6 GB
         models = synth.zoo(1, 5)
         models["unit_from_shape"], models["act_enabled"] = 0, 0
@@ -42,7 +45,7 @@ def space_of(kind):
 
 @pytest.mark.parametrize("require", [0, VALID])
 @pytest.mark.parametrize("kind", ["segments", "plain", "copies", "beyond a double", "few modes", "stress", "ragged",
-                                  "tied in a unit"])
+                                  "tied in a unit", "crowded cells"])
 def test_sweeps_where_buffers_fill_and_segments_change(ctx, ps, kind, require):      # noqa: F811
     space = space_of(kind)
     gs, os_ = both(ctx, space)
