@@ -29,10 +29,10 @@
 // A frontier that outgrows the buffer takes a slow exact path.
 //
 // What bounds it: the fp64 pipe and the issue slots of the screening (64 compares a clock and
-// SM).  4096 models of the stress configuration, 6.96e9 points: top-k 1.94 -> 0.76 ms, Pareto
-// 2.37 -> 0.84 ms against a sweep whose warps took a unit each (the set-up of a unit paid by a
+// SM).  4096 models of the stress configuration, 6.96e9 points: top-k 1.94 -> 0.77 ms, Pareto
+// 2.37 -> 0.83 ms against a sweep whose warps took a unit each (the set-up of a unit paid by a
 // whole warp, candidates inserted one by one into a sorted list per warp, the lists merged by
-// a second kernel); 1024 models skipping rejected factorisations 0.41 -> 0.084 ms.  The
+// a second kernel); 1024 models skipping rejected factorisations 0.41 -> 0.082 ms.  The
 // screening alone takes 0.52 and 0.58 ms of the former two.
 #include <type_traits>
 #include "ps_device.cuh"
