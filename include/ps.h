@@ -176,7 +176,8 @@ typedef struct {
                              against the capacity, then masked by the flags -- what the throughput
                              figures are quoted on.  (Points that must have the same bytes, the up
                              to four variants of one placement with offloaded activations, may share
-                             a compare: 17 compares for 20 points.)  1: a factorisation whose composition bits (T | heads,
+                             a compare: 17 compares for 20 points.  They may be held in figures rounded
+                             so that none that fits is missed; what fits there is held in whole bytes.)  1: a factorisation whose composition bits (T | heads,
                              K | layers, T <= tp_max_valid) already miss a required flag is not
                              evaluated at all; same results, less work when the filter requires
                              PS_F_CV or one of its reasons */

@@ -7,11 +7,11 @@
 // a sum of three terms, one per state, so the next triple costs one addition, and what is
 // uniform (modes, allowed digits, coefficients) comes from small tables of the block.
 //
-// Screening.  Every unit: its points are compared with their bounds (the four variants of
-// the offloaded digit have the same bytes: 17 compares for 20 points), masked by the flags
-// that the placement code and the composition allow.  It leaves the list of the units that
-// have survivors (an eighth of them on the stress configuration), which the next two
-// passes walk densely.  (With ps_filter.skip_rejected the list is made from the
+// Screening.  Every unit: its points are compared with their bounds in rounded figures, two
+// to an instruction (the four variants of the offloaded digit have the same bytes: 17
+// compares for 20 points), masked by the flags that the placement code and the composition
+// allow.  It leaves the list of the units that may have survivors (an eighth of them on the
+// stress configuration), which the next two passes walk densely and in whole bytes.  (With ps_filter.skip_rejected the list is made from the
 // composition tests alone; top-k without required flags lists all units.)
 //
 // First pass, over the cells of a histogram (an eighth of an octave each).
@@ -28,12 +28,12 @@
 // The block then emits the entries, evaluating each again from its index as a self-check.
 // A frontier that outgrows the buffer takes a slow exact path.
 //
-// What bounds it: the fp64 pipe and the issue slots of the screening (64 compares a clock and
-// SM).  4096 models of the stress configuration, 6.96e9 points: top-k 1.94 -> 0.77 ms, Pareto
-// 2.37 -> 0.83 ms against a sweep whose warps took a unit each (the set-up of a unit paid by a
-// whole warp, candidates inserted one by one into a sorted list per warp, the lists merged by
-// a second kernel); 1024 models skipping rejected factorisations 0.41 -> 0.082 ms.  The
-// screening alone takes 0.52 and 0.58 ms of the former two.
+// What bounds it: the issue slots of the screening, and the latency of a block's phases (four
+// blocks of four warps share an SM).  4096 models of the stress configuration, 6.96e9 points:
+// top-k 1.94 -> 0.62 ms, Pareto 2.37 -> 0.66 ms against a sweep whose warps took a unit each (the
+// set-up of a unit paid by a whole warp, candidates inserted one by one into a sorted list per
+// warp, the lists merged by a second kernel); 1024 models skipping rejected factorisations 0.41
+// -> 0.085 ms.  The screening takes 0.23 and 0.27 ms of the former two.
 #include <type_traits>
 #include "ps_device.cuh"
 #include "ps_internal.h"
@@ -111,9 +111,12 @@ struct Rank {
 struct BlockShared {
   ModelRec rec;
   Triple tri[MAX_TRIPLES];
-  unsigned char allowed[3][MAX_TRIPLES + 3];   // allowed activation digits of a triple for the three CLS_* of a unit
-  double state[2][5][3];                   // Theta, Omega: the coefficients of E, s and u by digit
-  u64 state_host[2][5];                    // and the host coefficient, as the sweep's type
+  float4 pair[25];                         // Theta and Omega, by NM * (Theta's digit) + Omega's: the coefficients of
+                                           // E, s and u, and that of the host bytes
+  u32 mask[3][25][10];                     // FIX_TOPS where the flags allow a point, by CLS_*, pair and G's digit: the
+                                           // activation digits that keep bytes (ScreenUnit leaves out those that they
+                                           // never allow), the offloaded one
+  u32 digits;                              // activation digits that the flags allow with any triple, a byte each CLS_*
   u64 cell[CELLS];                         // the histogram
   u64 cand_a[CAND_CAP], cand_b[CAND_CAP];  // the buffer: Pareto (mem, comm), top-k (comm, least mem)
   u32 cand_i[CAND_CAP];
@@ -135,8 +138,7 @@ struct BlockShared {
 
 // the composition bits of a factorisation against the required ones (ps_filter.skip_rejected:
 // a factorisation that misses one has no survivor, so it need not be evaluated)
-__device__ __forceinline__ bool unit_rejected(const SpaceDev& sp, const ModelRec& rec, u32 unit, u32 req_cv) {
-  const Fact f = sp.facts[unit];
+__device__ __forceinline__ bool unit_rejected(const SpaceDev& sp, const ModelRec& rec, const Fact& f, u32 req_cv) {
   const bool t_heads = rec.heads % f.T == 0, k_layers = rec.L % f.K == 0, tp_le = f.T <= sp.tp_max_valid;
   const bool whole = (u64)f.T * f.K * f.D == (u64)f.N;
   u32 cv = (t_heads ? PS_F_T_DIV_HEADS : 0) | (k_layers ? PS_F_K_DIV_LAYERS : 0) | (tp_le ? PS_F_TP_LE_MAX : 0) |
@@ -146,68 +148,143 @@ __device__ __forceinline__ bool unit_rejected(const SpaceDev& sp, const ModelRec
 }
 
 // ------------------------------------------------------------------ screening
-// Whether any of four variants of an activation digit fits: one compare per point, its
-// result chained through the next one's input predicate; BIT joins `fit` if one does.
-template <u32 BIT>
-__device__ __forceinline__ void any_variant(u32& fit, double m, const double* b) {
-  asm("{\n\t"
-      ".reg .pred p;\n\t"
-      "setp.lt.f64 p, %1, %2;\n\t"
-      "setp.lt.or.f64 p, %1, %3, p;\n\t"
-      "setp.lt.or.f64 p, %1, %4, p;\n\t"
-      "setp.lt.or.f64 p, %1, %5, p;\n\t"
-      "@p or.b32 %0, %0, %6;\n\t"
-      "}"
-      : "+r"(fit)
-      : "d"(m), "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]), "n"(BIT));
+// Bytes as 16-bit figures, two of them in a word: a unit is some fraction of the capacity (or of
+// the host budget), everything held is rounded down and everything that bounds it up.  So a point
+// that fits fits here too, and one that fits here but not in whole bytes is within a few units of
+// the capacity; what the screening lets through is tested in whole bytes by the passes.  A field
+// of a bound is 2^15 + the units that are left (-1: it cannot fit), a field held at most 2^15 - 2:
+// after one subtraction for both halves their top bits say which of the two points fit, with no
+// borrow from one half to the other.  Against a compare of doubles per point (two cycles of the
+// fp64 pipe, chained through predicates; as many instructions as points) the screening of 4096
+// models of the stress configuration takes 230 us instead of 517 (top-k) and 270 instead of 581
+// (Pareto, with a host budget), the sweeps 621 instead of 768 and 656 instead of 824.
+constexpr u32 FIX_TERM = 16383;            // a term held, at most: above every bound, and two of them below 2^15
+constexpr float FIX_CAP = 16382.0f;        // the capacity in units
+constexpr u32 FIX_NEVER = 0x7fff7fffu;     // bounds that nothing is below
+constexpr u32 FIX_TOPS = 0x80008000u;
+
+struct Scale {
+  float unit;                              // units per byte
+  float room;                              // the capacity in units, rounded up, and one
+};
+__device__ __forceinline__ Scale scale_of(u64 cap) {
+  Scale r;
+  r.unit = cap <= (u64)FIX_CAP ? 1.0f : __fdiv_rd(FIX_CAP, __ull2float_ru(cap));
+  r.room = __fadd_ru(__fmul_ru(__ull2float_ru(cap), r.unit), 1.0f);
+  return r;
 }
-template <u32 BIT>
-__device__ __forceinline__ void any_variant(u32& fit, u64 m, const u64* b) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) fit |= (m < b[q]) ? BIT : 0u;
+__device__ __forceinline__ u32 both_halves(u32 x) { return x * 0x10001u; }
+__device__ __forceinline__ u32 term_of(float x) { return __float2uint_rd(fminf(x, (float)FIX_TERM)); }
+// what is left of a capacity beside `held`, as the field of a bound less that of FIX_NEVER
+__device__ __forceinline__ u32 room_beside(const Scale& c, float held) {
+  return __float2uint_rd(fminf(fmaxf(__fsub_ru(c.room, held), 0.0f), (float)FIX_TERM));
 }
-template <int D, int NM, typename T, bool HOST_LIMITED>
-__device__ __forceinline__ void fitting_digits(u32& fit, const LaneUnit<NM, T, HOST_LIMITED>& lu, u32 modemap,
-                                               double m, T h, double cap_room) {
-  if constexpr (D < NM) {
-    if (digit_mode(modemap, D) == PS_MODE_O) {
-      // the four variants have the same bytes: one capacity compare, and the host bytes of each
-      u32 with_host = HOST_LIMITED ? 0u : 1u << D;
-      if (HOST_LIMITED) any_variant<1u << D>(with_host, h, lu.host_bound);
-      fit |= m < cap_room ? with_host : 0u;
-    } else {
-      any_variant<1u << D>(fit, m, lu.bounds(D));
-    }
-    fitting_digits<D + 1>(fit, lu, modemap, m, h, cap_room);
-  }
+// below 1 / x for a whole x below 2^24 (rcp.approx is right to one unit in the last place)
+__device__ __forceinline__ float below_reciprocal(u32 x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)x));
+  return __fmul_rd(r, 1.0f - 0x1p-22f);
 }
 
-// Does any point of the lane's unit whose (Theta, Omega) pair lies in [p0, p1) survive?
-template <int NM, typename T, bool HOST_LIMITED>
-__device__ __forceinline__ u32 screen_pairs(const BlockShared& sh, const LaneUnit<NM, T, HOST_LIMITED>& lu, u32 modemap,
-                                            double cap_room, T host_room, u32 p0, u32 p1) {
-  u32 any = 0;
-  const unsigned char* allowed_of = sh.allowed[lu.shift >> 3];
-#pragma unroll 1
-  for (u32 p = p0; p < p1; ++p) {
-    const u32 th = p / NM, om = p - th * NM;
-    const double* ct = sh.state[0][th];
-    const double* co = sh.state[1][om];
-    const double to_mem = fma(lu.E, ct[0], fma(lu.s, ct[1], fma(lu.u, ct[2], fma(lu.E, co[0], fma(lu.s, co[1], lu.u * co[2])))));
-    const T to_host = mul_add(lu.shard, from_bits<T>(sh.state_host[0][th]),
-                              mul_add(lu.shard, from_bits<T>(sh.state_host[1][om]), T(0)));
+// A unit as a lane holds it for the screening, no figure above what LaneUnit has for it.
+template <int NM, bool HOST_LIMITED>
+struct ScreenUnit {
+  float E, s, u, shard;                    // as LaneUnit's, in units
+  u32 gr_mem[NM], gr_host;                 // G's terms, in both halves
+  u32 bound[NM][2], host_bound[2];         // by activation variant; the halves are the tensor-axis variants
+  u32 room, host_room;                     // the capacity and the host budget, in both halves
+  u32 cls;
+
+  __device__ __forceinline__ void load(const SpaceDev& sp, const ModelRec& rec, const Fact& f, u32 modemap,
+                                       const Scale& cap, const Scale& host, u32 digits_of_any) {
+    const u32 G = sp.repl > 1 ? f.D / gcd_u32(sp.repl, f.D) : f.D;
+    cls = f.D == 1 ? CLS_ONE_DEVICE : (G == 1 ? CLS_ALL_COPIES : CLS_SHARDED);
+    const float over_t = below_reciprocal(f.T), over_tk = below_reciprocal(f.T * f.K), over_g = below_reciprocal(G);
+    const float P = __ull2float_rd(rec.P);
+    E = __fmul_rd(__fmul_rd(P, cap.unit), over_tk);
+    s = G == 1 ? E : __fmul_rd(E, over_g);
+    u = __fmul_rd(__fmul_rd(__ull2float_rd(rec.unit), cap.unit), over_t);
+    const float ss = (float)sp.sstar_units;
+    auto held = [&](u32 mode, float full, float part, float unit) {      // Theorem 1, as mu_elems
+      const float p = mode == PS_MODE_R ? full : (in_set(SET_SHARDLIKE, mode) ? part : 0.0f);
+      return mode == PS_MODE_SG ? __fmaf_rd(unit, ss, p) : (mode == PS_MODE_M ? unit : p);
+    };
 #pragma unroll
-    for (int gr = 0; gr < NM; ++gr) {
-      const double m = to_mem + lu.gr_mem[gr];
-      T h = to_host;
-      if (HOST_LIMITED && digit_mode(modemap, gr) == PS_MODE_O) h += lu.gr_host;
-      u32 fit = 0;                                       // digits with a point that fits, whatever its flags
-      fitting_digits<0>(fit, lu, modemap, m, h, cap_room);
-      if (HOST_LIMITED) fit = h < host_room ? fit : 0u;  // the triple's own host bytes against the budget
-      any |= fit & allowed_of[th + NM * om + NM * NM * gr];
+    for (int d = 0; d < NM; ++d)
+      gr_mem[d] = both_halves(term_of(__fmul_rd(held(digit_mode(modemap, d), E, s, u), (float)rec.wG)));
+    room = FIX_NEVER + both_halves(room_beside(cap, 0.0f));
+    if (HOST_LIMITED) {
+      shard = __fmul_rd(__fmul_rd(__fmul_rd(P, host.unit), over_tk), over_g);
+      gr_host = both_halves(term_of(__fmul_rd(shard, (float)(2 * rec.wG))));
+      host_room = FIX_NEVER + both_halves(room_beside(host, 0.0f));
+    }
+    const u32 digits = digits_of_any >> (8 * cls);       // that the flags allow in a unit of this class
+#pragma unroll
+    for (u32 v = 0; v < 2; ++v) {
+      u32 left[NM][2], host_left[2] = {0, 0};
+#pragma unroll
+      for (u32 tau = 0; tau < 2; ++tau) {
+        const bool have = v < sp.nv && tau < sp.nt;
+        const float A = __ull2float_rd(rec.A[v]), over = tau == 0 ? over_t : 1.0f;
+        const float EA = __fmul_rd(__fmul_rd(A, cap.unit), over);
+        const float uA = __fmul_rd(__fmul_rd(__ull2float_rd(rec.UA[v]), cap.unit), over);
+        const float shA = G == 1 ? EA : __fmul_rd(EA, over_g);
+#pragma unroll
+        for (int d = 0; d < NM; ++d) {
+          const u32 mode = digit_mode(modemap, d);       // (the offloaded digit's points: `room`)
+          left[d][tau] = have && mode != PS_MODE_O && ((digits >> d) & 1u) ? room_beside(cap, held(mode, EA, shA, uA)) : 0;
+        }
+        if (HOST_LIMITED && have)
+          host_left[tau] = room_beside(host, __fmul_rd(__fmul_rd(__fmul_rd(A, host.unit), over), (float)(2 * sp.accum)));
+      }
+#pragma unroll
+      for (int d = 0; d < NM; ++d) bound[d][v] = FIX_NEVER + left[d][0] + (left[d][1] << 16);
+      if (HOST_LIMITED) host_bound[v] = FIX_NEVER + host_left[0] + (host_left[1] << 16);
     }
   }
-  return any & lu.allowed;
+};
+
+// May any point of the lane's unit whose (Theta, Omega) pair lies in [p0, p1) survive?
+template <int NM, bool HOST_LIMITED>
+__device__ __forceinline__ bool screen_pairs(const BlockShared& sh, const ScreenUnit<NM, HOST_LIMITED>& su, u32 modemap,
+                                             u32 p0, u32 p1) {
+  u32 any = 0;
+#pragma unroll 1
+  for (u32 p = p0; p < p1; ++p) {
+    const float4 k = sh.pair[p];
+    const u32 to_mem = both_halves(term_of(__fmaf_rd(su.E, k.x, __fmaf_rd(su.s, k.y, __fmul_rd(su.u, k.z)))));
+    u32 fits_host[2] = {FIX_TOPS, FIX_TOPS}, fits_off[2] = {FIX_TOPS, FIX_TOPS};   // (G not offloaded, offloaded)
+    if (HOST_LIMITED) {
+      // the triple's own host bytes against the budget, and with offloaded activations beside them
+      const u32 h = both_halves(term_of(__fmul_rd(su.shard, k.w)));
+#pragma unroll
+      for (int o = 0; o < 2; ++o) {
+        const u32 with_g = o ? h + su.gr_host : h;
+        fits_host[o] = su.host_room - with_g;
+        fits_off[o] = (su.host_bound[0] - with_g) | (su.host_bound[1] - with_g);
+      }
+    }
+    u32 mask[2 * NM];                                    // by G's digit: activation digits that keep bytes, and the offloaded one
+    {
+      const uint2* row = reinterpret_cast<const uint2*>(sh.mask[su.cls][p]);
+#pragma unroll
+      for (int gr = 0; gr < NM; ++gr) { const uint2 w = row[gr]; mask[2 * gr] = w.x; mask[2 * gr + 1] = w.y; }
+    }
+#pragma unroll
+    for (int gr = 0; gr < NM; ++gr) {
+      const u32 m = to_mem + su.gr_mem[gr];
+      u32 fit = 0;
+#pragma unroll
+      for (int d = 0; d < NM; ++d)
+        if (NM < 5 || digit_mode(modemap, d) != PS_MODE_O) fit |= (su.bound[d][0] - m) | (su.bound[d][1] - m);
+      // (the variants of the offloaded digit have the same bytes: one compare)
+      const u32 off = su.room - m;
+      const bool g_off = digit_mode(modemap, gr) == PS_MODE_O;
+      any |= (fit & mask[2 * gr] & (g_off ? fits_host[1] : fits_host[0])) |
+             (off & mask[2 * gr + 1] & (g_off ? fits_off[1] : fits_off[0]));
+    }
+  }
+  return (any & FIX_TOPS) != 0;
 }
 
 // Pareto: the classes of units in which triple t can never add to a frontier because triple
@@ -624,7 +701,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
   const u32 model = sp.order[blockIdx.x];
   if (tid < (int)(sizeof(ModelRec) / 16))
     reinterpret_cast<uint4*>(&sh.rec)[tid] = reinterpret_cast<const uint4*>(&sp.recs[model])[tid];
-  if (tid == 0) { sh.survivors = 0; sh.n_cand = 0; }
+  if (tid == 0) { sh.survivors = 0; sh.n_cand = 0; sh.digits = 0; }
   for (int j = tid; j < CELLS; j += threads) sh.cell[j] = PARETO ? U64MAX : 0;
   __syncthreads();
   const ModelRec& rec = sh.rec;
@@ -647,7 +724,13 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
   for (int d = 0; d < NM; ++d)
     if (digit_mode(modemap, d) == PS_MODE_O) is_o |= 1u << d;
 
+  const bool skip = args.skip_rejected && req_cv != 0;
+  // Top-k without a required flag: the first pass counts every point itself and nothing is screened
+  // for (4096 models of the stress configuration in 2.16 ms instead of 2.30).
+  const bool take_all = !PARETO && req == 0, screened = !skip && !take_all;
+
   // ---- the block's tables of triples and of states
+  u32 digits_of_any = 0;
   for (int t = tid; t < N3; t += threads) {
     // activation-digit classes (Theorem 3: a replica needs its own activations)
     u32 own = 0, not_mo = 0;
@@ -695,16 +778,31 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     tr.allowed = a_many | (a_one << 8) | (a_copies << 16) | (n2 << 24) | (n3 << 26);
     tr.pad = 0;
     sh.rank[t] = Rank{a | ((a + b) << 8) | (c << 16), (ct * rec.wT + co * rec.wO + cg * rec.wG) | (h << 16), tr.allowed};
-    sh.allowed[CLS_SHARDED][t] = (unsigned char)a_many;
-    sh.allowed[CLS_ONE_DEVICE][t] = (unsigned char)a_one;
-    sh.allowed[CLS_ALL_COPIES][t] = (unsigned char)a_copies;
+    if (screened) {
+      const u32 pair = (t % NM) * NM + (t / NM) % NM, gr_digit = t / N2;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const u32 digits = (tr.allowed >> (8 * c)) & all;
+        *reinterpret_cast<uint2*>(&sh.mask[c][pair][2 * gr_digit]) =
+            make_uint2((digits & ~is_o) ? FIX_TOPS : 0, (digits & is_o) ? FIX_TOPS : 0);
+      }
+    }
+    digits_of_any |= tr.allowed;
   }
-  for (int t = tid; t < 2 * NM; t += threads) {
-    const u32 st = t / NM, d = t % NM, mode = digit_mode(modemap, d), w = st == 0 ? rec.wT : rec.wO;
-    sh.state[st][d][0] = mode == PS_MODE_R ? w : 0;
-    sh.state[st][d][1] = in_set(SET_SHARDLIKE, mode) ? w : 0;
-    sh.state[st][d][2] = mode == PS_MODE_SG ? w * sp.sstar_units : (mode == PS_MODE_M ? w : 0);
-    sh.state_host[st][d] = bits<T>(as<T>(mode == PS_MODE_O ? (st == 0 ? (2 * sp.accum + 1) * w : 2 * w) : 0));
+  digits_of_any = __reduce_or_sync(0xffffffffu, digits_of_any & 0x1f1f1fu);
+  if (lane == 0 && digits_of_any) atomicOr(&sh.digits, digits_of_any);
+  for (int t = tid; screened && t < N2; t += threads) {
+    const u32 modes[2] = {digit_mode(modemap, t / NM), digit_mode(modemap, t % NM)}, width[2] = {rec.wT, rec.wO};
+    u32 a = 0, b = 0, c = 0, h = 0;
+#pragma unroll
+    for (int st = 0; st < 2; ++st) {
+      if (modes[st] == PS_MODE_R) a += width[st];
+      if (in_set(SET_SHARDLIKE, modes[st])) b += width[st];
+      if (modes[st] == PS_MODE_SG) c += width[st] * sp.sstar_units;
+      if (modes[st] == PS_MODE_M) c += width[st];
+      if (modes[st] == PS_MODE_O) h += (st == 0 ? 2 * sp.accum + 1 : 2) * width[st];
+    }
+    sh.pair[t] = make_float4((float)a, (float)b, (float)c, (float)h);
   }
 
   // ---- the triples that the passes walk: those that the flags allow; for Pareto only those
@@ -745,10 +843,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
   u32 most_unit = NO_CODE;
   u32 survivors = 0;
   bool overflowed = false;                           // the same for every thread
-  const bool skip = args.skip_rejected && req_cv != 0;
-  // Top-k without a required flag: the first pass counts every point itself and nothing is screened
-  // for (4096 models of the stress configuration in 2.16 ms instead of 2.30).
-  const bool take_all = !PARETO && req == 0;
+  const Scale cap_scale = scale_of(cap_x - 1), host_scale = scale_of(host_x - 1);
 
   for (u32 seg = 0; seg < sp.n_facts; seg += SEG) {
     const u32 seg_n = min((u32)SEG, sp.n_facts - seg), n_batches = (seg_n + 31) / 32;
@@ -762,7 +857,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
     } else if (skip) {
       for (u32 b = warp; b < n_batches; b += warps) {
         const u32 p = b * 32 + lane;
-        const u32 votes = __ballot_sync(0xffffffffu, p < seg_n && !unit_rejected(sp, rec, seg + p, req_cv));
+        const u32 votes = __ballot_sync(0xffffffffu, p < seg_n && !unit_rejected(sp, rec, sp.facts[seg + min(p, seg_n - 1)], req_cv));
         if (lane == 0) sh.flags[b] = votes;
       }
     } else {
@@ -772,11 +867,10 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
       for (u32 item = warp; item < n_batches * parts; item += warps) {
         const u32 b = item / parts, part = item - b * parts, p = b * 32 + lane;
         const Fact f = sp.facts[seg + min(p, seg_n - 1)];
-        const UnitBase ub = unit_of(sp, rec, f);
-        LaneUnit<NM, T, HOST_LIMITED> lu;
-        lu.load(sp, rec, f, ub, modemap, cap_x, host_x, p < seg_n && (ub.cv & req_cv) == req_cv);
-        const u32 any = screen_pairs(sh, lu, modemap, as<double>(cap_x), host_room, part * N2 / parts, (part + 1) * N2 / parts);
-        const u32 votes = __ballot_sync(0xffffffffu, any != 0);
+        ScreenUnit<NM, HOST_LIMITED> su;
+        su.load(sp, rec, f, modemap, cap_scale, host_scale, sh.digits);
+        const bool any = screen_pairs(sh, su, modemap, part * N2 / parts, (part + 1) * N2 / parts);
+        const u32 votes = __ballot_sync(0xffffffffu, any && p < seg_n && !unit_rejected(sp, rec, f, req_cv));
         if (lane == 0 && votes) atomicOr(&sh.flags[b], votes);
       }
     }
