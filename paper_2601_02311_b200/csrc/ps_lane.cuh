@@ -92,6 +92,45 @@ struct LaneUnit {
   }
 };
 
+// A unit as a lane holds it where only the least bytes of a (triple, tensor-axis variant) count.  The flags
+// allow the digits that keep activation bytes all together or not at all: whether one of them may stand
+// beside a triple depends on the triple only for the offloaded digit (allowed_act_digits).  So their least
+// bytes are a figure of the unit, and no bound per digit and variant is held (40 registers in doubles).
+template <int NM, typename T, bool HOST_LIMITED>
+struct LeastUnit {
+  double E, s, u;
+  T shard;
+  T act[2], host_most[2];    // by tensor-axis variant: least activation bytes of `digits`, at most the capacity, and the
+                             // most that a triple's host bytes may be below, with offloaded activations beside them
+  u32 allowed, shift;
+
+  // digits: those that keep bytes and are allowed in a unit of this class
+  __device__ __forceinline__ void load(const SpaceDev& sp, const ModelRec& rec, const Fact& f, const UnitBase& ub,
+                                       u32 modemap, u64 cap_x, u64 host_x, u32 digits, bool live) {
+    E = as<double>(ub.E2); s = as<double>(ub.sh); u = as<double>(ub.u);
+    shard = as<T>(ub.sh);
+#pragma unroll
+    for (u32 tau = 0; tau < 2; ++tau) {
+      u64 least = cap_x, most = 0;
+#pragma unroll
+      for (u32 v = 0; v < 2; ++v) {
+        const bool have = v < sp.nv && tau < sp.nt;
+        const ActBase ab = act_of(sp, rec, f, ub, v, tau);
+#pragma unroll
+        for (int d = 0; d < NM; ++d)
+          if (have && ((digits >> d) & 1u))
+            least = min(least, mu_elems(digit_mode(modemap, d), ab.EA, ab.shA, ab.uA, sp.sstar_units));
+        const u64 ah = 2 * ab.EA * sp.accum;
+        if (HOST_LIMITED && have && ah < host_x) most = max(most, host_x - ah);
+      }
+      act[tau] = as<T>(least);
+      host_most[tau] = as<T>(most);
+    }
+    shift = 8 * ub.cls;
+    allowed = live ? (1u << NM) - 1u : 0u;
+  }
+};
+
 // Survivors of the lane's unit among the four variants of one activation digit: a compare
 // per point on the fp64 pipe, masked by its input predicate, counted with predicated fp32
 // adds (small integers are exact).

@@ -113,7 +113,7 @@ struct BlockShared {
   Triple tri[MAX_TRIPLES];
   float4 pair[25];                         // Theta and Omega, by NM * (Theta's digit) + Omega's: the coefficients of
                                            // E, s and u, and that of the host bytes
-  u32 mask[3][25][10];                     // FIX_TOPS where the flags allow a point, by CLS_*, pair and G's digit: the
+  alignas(8) u32 mask[3][25][10];                     // FIX_TOPS where the flags allow a point, by CLS_*, pair and G's digit: the
                                            // activation digits that keep bytes (ScreenUnit leaves out those that they
                                            // never allow), the offloaded one
   u32 digits;                              // activation digits that the flags allow with any triple, a byte each CLS_*
@@ -121,20 +121,28 @@ struct BlockShared {
   u64 cand_a[CAND_CAP], cand_b[CAND_CAP];  // the buffer: Pareto (mem, comm), top-k (comm, least mem)
   u32 cand_i[CAND_CAP];
   unsigned char place[CAND_CAP];           // candidates that stay
-  u64 sorted_a[KEEP_CAP], sorted_b[KEEP_CAP];
-  u32 sorted_i[KEEP_CAP];
   int kept;
-  u64 hit_a[CAND_CAP], hit_b[CAND_CAP];    // top-k: the candidates that are left, while their points fill the buffer
-  u32 hit[CAND_CAP];
   u32 flags[SEG / 32];                     // units of the segment with survivors
-  u16 heavy[SEG];                          // the same as a list
-  u32 least_cell[SEG];                     // top-k: the lowest cell that a survivor of a listed unit falls into
+  alignas(8) u16 heavy[SEG];               // the same as a list
+  alignas(8) u32 least_cell[SEG];                     // top-k: the lowest cell that a survivor of a listed unit falls into
                                            // (Pareto: drop_tied's indices)
   unsigned char live[MAX_TRIPLES + 3];     // the triples the passes walk
   Rank rank[MAX_TRIPLES];
   unsigned char alive[MAX_TRIPLES + 3];
   u32 n_live, n_heavy, next1, next2, n_cand, full, limit_cell, survivors;
 };
+
+// Three arrays in the place of others that are not read any more when they are written.
+struct Scratch {
+  u64* a;
+  u64* b;
+  u32* i;
+};
+// a ranking's result on its way into the buffer.  Pareto (KEEP_CAP entries): a model's last ranking, behind
+// the passes.  Top-k (PAIRWISE entries): the screening is over, and more than PAIRWISE are sorted in place.
+template <int KIND> __device__ __forceinline__ Scratch ranked_scratch(BlockShared& sh);
+// top-k: the candidates that are left, while their points fill the buffer (CAND_CAP entries, behind the passes)
+__device__ __forceinline__ Scratch hits(BlockShared& sh);
 
 // the composition bits of a factorisation against the required ones (ps_filter.skip_rejected:
 // a factorisation that misses one has no survivor, so it need not be evaluated)
@@ -331,6 +339,19 @@ __device__ __noinline__ void sort_candidates(BlockShared& sh, int n) {
 // of 0.840; with 64 instead of 128 0.755 and 0.838, and the zoo's frontiers 0.6 % more.
 constexpr int PAIRWISE = 128;
 
+static_assert(sizeof(BlockShared::cell) >= CAND_CAP * sizeof(u64) && sizeof(BlockShared::least_cell) >= CAND_CAP * sizeof(u64) &&
+                  sizeof(BlockShared::heavy) >= CAND_CAP * sizeof(u32) && CAND_CAP >= KEEP_CAP &&
+                  sizeof(BlockShared::mask) >= PAIRWISE * (2 * sizeof(u64) + sizeof(u32)),
+              "scratch in the place of others");
+__device__ __forceinline__ Scratch hits(BlockShared& sh) {
+  return Scratch{sh.cell, reinterpret_cast<u64*>(sh.least_cell), reinterpret_cast<u32*>(sh.heavy)};
+}
+template <> __device__ __forceinline__ Scratch ranked_scratch<PS_REDUCE_PARETO>(BlockShared& sh) { return hits(sh); }
+template <> __device__ __forceinline__ Scratch ranked_scratch<PS_REDUCE_TOPK>(BlockShared& sh) {
+  u64* const a = reinterpret_cast<u64*>(sh.mask);
+  return Scratch{a, a + PAIRWISE, reinterpret_cast<u32*>(a + 2 * PAIRWISE)};
+}
+
 // Closes up the candidates p < n for which `keep(p, its key)` holds, by one warp, 32 at a
 // time; returns how many are left.  (`keep` is called by all lanes; a code of NO_CODE and keys
 // of U64MAX stand for the places from n on.)
@@ -442,6 +463,7 @@ __device__ __noinline__ int rank_candidates(BlockShared& sh, int n, int k_keep) 
     sort_candidates(sh, n);
     return min(n, k_keep);
   }
+  const Scratch sorted = ranked_scratch<KIND>(sh);
   if (tid == 0) sh.kept = 0;
   if (PARETO)
     for (int p = tid; p < n; p += threads) {
@@ -463,12 +485,12 @@ __device__ __noinline__ int rank_candidates(BlockShared& sh, int n, int k_keep) 
       else rank += key_less(Key{sh.cand_a[q], sh.cand_b[q], sh.cand_i[q]}, e) ? 1 : 0;
     }
     if (PARETO) atomicAdd(&sh.kept, 1);
-    if (rank < KEEP_CAP) { sh.sorted_a[rank] = e.a; sh.sorted_b[rank] = e.b; sh.sorted_i[rank] = e.i; }
+    if (rank < KEEP_CAP) { sorted.a[rank] = e.a; sorted.b[rank] = e.b; sorted.i[rank] = e.i; }
   }
   __syncthreads();
   const int stay = PARETO ? sh.kept : min(n, k_keep);
   for (int p = tid; p < min(stay, KEEP_CAP); p += threads) {
-    sh.cand_a[p] = sh.sorted_a[p]; sh.cand_b[p] = sh.sorted_b[p]; sh.cand_i[p] = sh.sorted_i[p];
+    sh.cand_a[p] = sorted.a[p]; sh.cand_b[p] = sorted.b[p]; sh.cand_i[p] = sorted.i[p];
   }
   __syncthreads();
   return stay;
@@ -570,8 +592,9 @@ __device__ __noinline__ int resolve_points(const SpaceDev& sp, BlockShared& sh, 
                                            u64 host_x) {
   const int tid = threadIdx.x, threads = blockDim.x;
   const u32 per_unit = sp.nvt * NM * NM * NM * NM;
+  const Scratch hit = hits(sh);
   __syncthreads();
-  for (int p = tid; p < n; p += threads) { sh.hit_a[p] = sh.cand_a[p]; sh.hit_b[p] = sh.cand_b[p]; sh.hit[p] = sh.cand_i[p]; }
+  for (int p = tid; p < n; p += threads) { hit.a[p] = sh.cand_a[p]; hit.b[p] = sh.cand_b[p]; hit.i[p] = sh.cand_i[p]; }
   if (tid == 0) sh.n_cand = 0;
   __syncthreads();
   Key threshold{U64MAX, U64MAX, NO_CODE};
@@ -587,9 +610,9 @@ __device__ __noinline__ int resolve_points(const SpaceDev& sp, BlockShared& sh, 
     __syncthreads();
     const int now = min(n - base, room);
     for (int j = base + tid; j < base + now; j += threads) {
-      const u64 comm = sh.hit_a[j];
-      const u32 code = sh.hit[j];
-      if (!key_less(Key{comm, sh.hit_b[j], (code >> 8) * per_unit}, threshold)) continue;
+      const u64 comm = hit.a[j];
+      const u32 code = hit.i[j];
+      if (!key_less(Key{comm, hit.b[j], (code >> 8) * per_unit}, threshold)) continue;
       points_of<NM>(sp, sh, code, modemap, cap_x, host_x, [&](u64 m, u32 idx) {
         if (key_less(Key{comm, m, idx}, threshold)) {
           const u32 at = atomicAdd(&sh.n_cand, 1u);
@@ -911,18 +934,17 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
       const u32 unit = seg + sh.heavy[min(k, n_heavy - 1)];
       const Fact f = sp.facts[unit];
       const UnitBase ub = unit_of(sp, rec, f);
-      LaneUnit<NM, T, HOST_LIMITED> lu;
-      lu.load(sp, rec, f, ub, modemap, cap_x, host_x, k < n_heavy && (ub.cv & req_cv) == req_cv);
+      constexpr bool COUNTS = !PARETO && !SECOND;    // top-k's first pass counts points, the others want the least bytes
+      typename std::conditional<COUNTS, LaneUnit<NM, T, HOST_LIMITED>, LeastUnit<NM, T, HOST_LIMITED>>::type lu;
+      const bool live = k < n_heavy && (ub.cv & req_cv) == req_cv;
+      if constexpr (COUNTS) lu.load(sp, rec, f, ub, modemap, cap_x, host_x, live);
+      else lu.load(sp, rec, f, ub, modemap, cap_x, host_x, (sh.digits >> (8 * ub.cls)) & all & ~is_o, live);
       const T x = as<T>(ub.x);
       const T gx2 = as<T>((u64)rec.wG * ub.x2), gx3 = as<T>((u64)rec.wG * ub.x3);
-      T axis[2], host_most[2], act[2];
+      T axis[2];
 #pragma unroll
-      for (u32 tau = 0; tau < 2; ++tau) {
+      for (u32 tau = 0; tau < 2; ++tau)
         axis[tau] = as<T>(ext_in_objective ? model_axis_traffic(rec, f, ub, tau, sp.tp_coll, sp.accum) : 0);
-        host_most[tau] = HOST_LIMITED ? max(lu.host_bound[tau], lu.host_bound[2 + tau]) : T(0);
-        act[tau] = cap_room;
-      }
-      u32 set = 0;                                   // the allowed digits act[] is for
       const u32 t_end = (part + 1) * n_live / parts;
       u32 lowest = CELLS;                            // top-k, first pass: the lowest cell of a survivor
       // Two triples at a time, all four candidates side by side and one vote for them: what
@@ -930,7 +952,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
 #pragma unroll 1
       for (u32 t0 = max(part * n_live / parts, from); t0 < t_end; t0 += 2) {
         double m[2];
-        T c[2], h[2], act_of_set[2][2];
+        T c[2], h[2];
         u32 allowed[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -946,7 +968,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
           if (sp.repl > 1) c[j] += (T)((tr.allowed >> 24) & 3u) * gx2 + (T)((tr.allowed >> 26) & 1u) * gx3;
         }
         if (!__any_sync(0xffffffffu, allowed[0] | allowed[1])) continue;
-        if (!PARETO && !SECOND) {
+        if constexpr (COUNTS) {
           // the survivors of the triples, by tensor-axis variant
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
@@ -967,85 +989,63 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
             if (n0 != 0.0f) { atomicAdd(reinterpret_cast<u32*>(&sh.cell[cell0]), (u32)n0); lowest = min(lowest, (u32)cell0); }
             if (n1 != 0.0f) { atomicAdd(reinterpret_cast<u32*>(&sh.cell[cell1]), (u32)n1); lowest = min(lowest, (u32)cell1); }
           }
-          continue;
-        }
-        // For a triple and a tensor-axis variant the communication does not depend on the
-        // activation variant and digit, so of those that are allowed only the one with the
-        // least bytes can be on a frontier -- and if it does not fit, none does.  The least
-        // of the allowed set, the offloaded digit aside (it keeps no bytes):
-        auto least_act = [&](u32 digits, T* out) {
-          T most[2] = {T(0), T(0)};
-#pragma unroll
-          for (int d = 0; d < NM; ++d)
-            if (((digits & ~is_o) >> d) & 1u) {
-#pragma unroll
-              for (int q = 0; q < 4; ++q) most[q & 1] = max(most[q & 1], lu.bound[d][q]);
-            }
-          out[0] = cap_room - most[0];
-          out[1] = cap_room - most[1];
-        };
-        const bool other0 = allowed[0] != 0 && allowed[0] != set, other1 = allowed[1] != 0 && allowed[1] != set;
-        if (__any_sync(0xffffffffu, other0 | other1)) {
-          least_act(allowed[0], act_of_set[0]);
-          least_act(allowed[1], act_of_set[1]);
-          set = allowed[1];
-          act[0] = act_of_set[1][0];
-          act[1] = act_of_set[1][1];
         } else {
+          // For a triple and a tensor-axis variant the communication does not depend on the
+          // activation variant and digit, so of those that are allowed only the one with the
+          // least bytes can be on a frontier -- and if it does not fit, none does.  The offloaded
+          // digit keeps none.
+          bool cand[4];
+          T mem[4], comm[4];
 #pragma unroll
-          for (int j = 0; j < 2; ++j) { act_of_set[j][0] = act[0]; act_of_set[j][1] = act[1]; }
-        }
-        bool cand[4];
-        T mem[4], comm[4];
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          const int j = w >> 1, tau = w & 1;
-          comm[w] = c[j] + axis[tau];
-          const bool off = (allowed[j] & is_o) != 0 && (!HOST_LIMITED || h[j] < host_most[tau]);
-          mem[w] = whole<T>(m[j]) + (off ? T(0) : act_of_set[j][tau]);
-          cand[w] = allowed[j] != 0 && mem[w] < cap_room && (u32)tau < sp.nt;
-          const int cell = cell_of(PARETO ? mem[w] : comm[w]);
-          if (!SECOND) {
-            if (cand[w] && bits<T>(comm[w]) < sh.cell[cell])
-              atomicMin(reinterpret_cast<unsigned long long*>(&sh.cell[cell]), (unsigned long long)bits<T>(comm[w]));
-          } else if (PARETO) {
-            // (the first cell holds one number, zero: its own least is a bound as well)
-            const u64 least = sh.cell[max(cell, 1) - 1];
-            cand[w] = cand[w] && (cell == 0 ? bits<T>(comm[w]) <= least : bits<T>(comm[w]) < least);
-          } else {
-            cand[w] = cand[w] && cell <= (int)sh.limit_cell &&
-                      (comm[w] < most_comm || (comm[w] == most_comm &&
-                                               (mem[w] < most_mem || (mem[w] == most_mem && unit <= most_unit))));
-          }
-        }
-        if (SECOND && __any_sync(0xffffffffu, cand[0] | cand[1] | cand[2] | cand[3])) {
-          u32 mine = 0;
-#pragma unroll
-          for (int w = 0; w < 4; ++w) mine += cand[w] ? 1u : 0u;
-          u32 incl = mine;                           // inclusive prefix sum over the lanes
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const u32 up = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += up;
-          }
-          const u32 total = __shfl_sync(0xffffffffu, incl, 31);
-          u32 at = 0;
-          if (lane == 0) at = atomicAdd(&sh.n_cand, total);
-          at = __shfl_sync(0xffffffffu, at, 0);
-          // (a group that does not fit leaves empty entries where there were places)
-          const bool room = at + total <= CAND_CAP;
-          at += incl - mine;
-#pragma unroll
-          for (int w = 0; w < 4; ++w)
-            if (cand[w]) {
-              if (at < CAND_CAP) {
-                sh.cand_a[at] = room ? (u64)(PARETO ? mem[w] : comm[w]) : U64MAX;
-                sh.cand_b[at] = room ? (u64)(PARETO ? comm[w] : mem[w]) : U64MAX;
-                sh.cand_i[at] = room ? (unit << 8) | ((u32)sh.live[min(t0 + (w >> 1), t_end - 1)] << 1) | (w & 1) : NO_CODE;
-              }
-              ++at;
+          for (int w = 0; w < 4; ++w) {
+            const int j = w >> 1, tau = w & 1;
+            comm[w] = c[j] + axis[tau];
+            const bool off = (allowed[j] & is_o) != 0 && (!HOST_LIMITED || h[j] < lu.host_most[tau]);
+            mem[w] = whole<T>(m[j]) + (off ? T(0) : lu.act[tau]);
+            cand[w] = (off || (allowed[j] & ~is_o) != 0) && mem[w] < cap_room && (u32)tau < sp.nt;
+            const int cell = cell_of(PARETO ? mem[w] : comm[w]);
+            if (!SECOND) {
+              if (cand[w] && bits<T>(comm[w]) < sh.cell[cell])
+                atomicMin(reinterpret_cast<unsigned long long*>(&sh.cell[cell]), (unsigned long long)bits<T>(comm[w]));
+            } else if (PARETO) {
+              // (the first cell holds one number, zero: its own least is a bound as well)
+              const u64 least = sh.cell[max(cell, 1) - 1];
+              cand[w] = cand[w] && (cell == 0 ? bits<T>(comm[w]) <= least : bits<T>(comm[w]) < least);
+            } else {
+              cand[w] = cand[w] && cell <= (int)sh.limit_cell &&
+                        (comm[w] < most_comm || (comm[w] == most_comm &&
+                                                 (mem[w] < most_mem || (mem[w] == most_mem && unit <= most_unit))));
             }
-          if (!room) return t0;
+          }
+          if (SECOND && __any_sync(0xffffffffu, cand[0] | cand[1] | cand[2] | cand[3])) {
+            u32 mine = 0;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) mine += cand[w] ? 1u : 0u;
+            u32 incl = mine;                           // inclusive prefix sum over the lanes
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const u32 up = __shfl_up_sync(0xffffffffu, incl, o);
+              if (lane >= o) incl += up;
+            }
+            const u32 total = __shfl_sync(0xffffffffu, incl, 31);
+            u32 at = 0;
+            if (lane == 0) at = atomicAdd(&sh.n_cand, total);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            // (a group that does not fit leaves empty entries where there were places)
+            const bool room = at + total <= CAND_CAP;
+            at += incl - mine;
+#pragma unroll
+            for (int w = 0; w < 4; ++w)
+              if (cand[w]) {
+                if (at < CAND_CAP) {
+                  sh.cand_a[at] = room ? (u64)(PARETO ? mem[w] : comm[w]) : U64MAX;
+                  sh.cand_b[at] = room ? (u64)(PARETO ? comm[w] : mem[w]) : U64MAX;
+                  sh.cand_i[at] = room ? (unit << 8) | ((u32)sh.live[min(t0 + (w >> 1), t_end - 1)] << 1) | (w & 1) : NO_CODE;
+                }
+                ++at;
+              }
+            if (!room) return t0;
+          }
         }
       }
       if (!PARETO && !SECOND && lowest < CELLS) atomicMin(&sh.least_cell[k], lowest);
