@@ -117,7 +117,8 @@ struct BlockShared {
                                            // activation digits that keep bytes (ScreenUnit leaves out those that they
                                            // never allow), the offloaded one
   u32 digits;                              // activation digits that the flags allow with any triple, a byte each CLS_*
-  u64 cell[CELLS];                         // the histogram
+  alignas(16) u64 cell[CELLS];             // the histogram
+  u64 scan[4];                             // of its four quarters
   u64 cand_a[CAND_CAP], cand_b[CAND_CAP];  // the buffer: Pareto (mem, comm), top-k (comm, least mem)
   u32 cand_i[CAND_CAP];
   unsigned char place[CAND_CAP];           // candidates that stay
@@ -898,20 +899,20 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
       }
     }
     __syncthreads();
-    if (warp == 0) {                                 // the flagged units as a list
-      u32 word = sh.flags[lane];
-      const u32 own = __popc(word);
-      u32 incl = own;
-      for (int o = 1; o < 32; o <<= 1) {
-        const u32 up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
+    // the flagged units as a list, a warp for each word of flags
+    {
+      const u32 set_here = __popc(sh.flags[lane]);
+      for (u32 w = warp; w < n_batches; w += warps) {
+        const u32 word = sh.flags[w];
+        u32 at = __reduce_add_sync(0xffffffffu, (u32)lane < w ? set_here : 0u);
+        if ((word >> lane) & 1u) {
+          at += __popc(word & ((1u << lane) - 1u));
+          if (!PARETO) sh.least_cell[at] = CELLS;        // (before the barrier: the first pass lowers it from any warp)
+          sh.heavy[at] = (u16)(32 * w + lane);
+        }
       }
-      u32 at = incl - own;
-      for (; word; word &= word - 1) {
-        if (!PARETO) sh.least_cell[at] = CELLS;        // (before the barrier: the first pass lowers it from any warp)
-        sh.heavy[at++] = (u16)(32 * lane + __ffs(word) - 1);
-      }
-      if (lane == 31) sh.n_heavy = incl;
+      const u32 total = __reduce_add_sync(0xffffffffu, set_here);
+      if (tid == 0) sh.n_heavy = total;
     }
     __syncthreads();
     const u32 n_live = sh.n_live;
@@ -1060,40 +1061,60 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
       walk(std::false_type{}, item, 0);
     }
     __syncthreads();
-    if (warp == 0) {
-      constexpr int PER = CELLS / 32;
-      if (PARETO) {
-        // cell j then holds the least communication of any survivor so far in cells 0..j
-        u64 least = U64MAX;
-        for (int q = 0; q < PER; ++q) least = min(least, sh.cell[lane * PER + q]);
-        u64 incl = least;
+    // Four warps, four cells a thread.
+    constexpr int SCAN_WARPS = 4, PER = CELLS / (SCAN_WARPS * 32);
+    static_assert(PER == 4, "cells of a thread: two 16-byte accesses");
+    if (PARETO) {
+      // cell j then holds the least communication of any survivor so far in cells 0..j
+      u64 c[PER], incl = U64MAX;
+      if (warp < SCAN_WARPS) {
+        const ulonglong2* const from = reinterpret_cast<const ulonglong2*>(sh.cell + tid * PER);
+        const ulonglong2 lo = from[0], hi = from[1];
+        c[0] = lo.x; c[1] = min(c[0], (u64)lo.y); c[2] = min(c[1], (u64)hi.x); c[3] = min(c[2], (u64)hi.y);
+        incl = c[3];
         for (int o = 1; o < 32; o <<= 1) {
           const u64 up = __shfl_up_sync(0xffffffffu, incl, o);
           if (lane >= o) incl = min(incl, up);
         }
-        u64 run = __shfl_up_sync(0xffffffffu, incl, 1);
-        if (lane == 0) run = U64MAX;
-        for (int q = 0; q < PER; ++q) { run = min(run, sh.cell[lane * PER + q]); sh.cell[lane * PER + q] = run; }
-      } else {
-        // the first cell up to which there are k survivors (the last one if there are fewer)
-        u32 sum = 0;
-        for (int q = 0; q < PER; ++q) sum += (u32)sh.cell[lane * PER + q];
-        u32 incl = sum;
+        if (lane == 31) sh.scan[warp] = incl;
+      }
+      __syncthreads();
+      if (warp < SCAN_WARPS) {
+        u64 before = __shfl_up_sync(0xffffffffu, incl, 1);
+        if (lane == 0) before = U64MAX;
+        for (int w = 0; w < warp; ++w) before = min(before, sh.scan[w]);
+        ulonglong2* const to = reinterpret_cast<ulonglong2*>(sh.cell + tid * PER);
+        to[0] = make_ulonglong2(min(c[0], before), min(c[1], before));
+        to[1] = make_ulonglong2(min(c[2], before), min(c[3], before));
+      }
+    } else {
+      // the first cell up to which there are k survivors (the last one if there are fewer)
+      u32 c[PER], incl = 0;
+      if (warp < SCAN_WARPS) {
+        const ulonglong2* const from = reinterpret_cast<const ulonglong2*>(sh.cell + tid * PER);
+        const ulonglong2 lo = from[0], hi = from[1];
+        c[0] = (u32)lo.x; c[1] = c[0] + (u32)lo.y; c[2] = c[1] + (u32)hi.x; c[3] = c[2] + (u32)hi.y;
+        incl = c[3];
         for (int o = 1; o < 32; o <<= 1) {
           const u32 up = __shfl_up_sync(0xffffffffu, incl, o);
           if (lane >= o) incl += up;
         }
-        const u32 reached = __ballot_sync(0xffffffffu, incl >= args.max_entries);
-        if (reached == 0) {
-          if (lane == 0) sh.limit_cell = CELLS - 1;
-        } else if (lane == __ffs(reached) - 1) {
-          u32 run = incl - sum;
+        if (lane == 31) sh.scan[warp] = incl;
+      }
+      if (tid == 0) sh.limit_cell = CELLS - 1;
+      __syncthreads();
+      if (warp < SCAN_WARPS) {
+        u32 before = incl - c[PER - 1];
+        for (int w = 0; w < warp; ++w) before += (u32)sh.scan[w];
+        if (before < args.max_entries && before + c[PER - 1] >= args.max_entries) {
           int q = 0;
-          while ((run += (u32)sh.cell[lane * PER + q]) < args.max_entries) ++q;
-          sh.limit_cell = lane * PER + q;
+          while (before + c[q] < args.max_entries) ++q;
+          sh.limit_cell = tid * PER + q;
         }
+      }
+      __syncthreads();
+      if (warp == 0) {
         // and only the units with a survivor that low are walked again
-        __syncwarp();
         const u32 limit = sh.limit_cell;
         u32 n = 0;
         for (u32 base = 0; base < n_heavy; base += 32) {
