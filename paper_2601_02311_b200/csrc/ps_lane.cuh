@@ -28,13 +28,19 @@ template <typename T> __device__ __forceinline__ T from_bits(u64 x);
 template <> __device__ __forceinline__ u64 from_bits<u64>(u64 x) { return x; }
 template <> __device__ __forceinline__ double from_bits<double>(u64 x) { return __longlong_as_double((long long)x); }
 
+// Which degrees a kernel is compiled for: powers of two (every division a shift), any (the
+// divisions), or both with a uniform branch.  The code for the other kind is not just jumped over,
+// it takes the place of code that runs in the instruction cache.
+enum { DEGREES_ANY = 0, DEGREES_POW2 = 1, DEGREES_EITHER = 2 };
+template <int DEGREES = DEGREES_EITHER>
 __device__ __forceinline__ UnitBase unit_of(const SpaceDev& sp, const ModelRec& rec, const Fact& f) {
-  if (sp.all_pow2) return unit_base_pow2(rec, f, pow2_of(f, sp.repl), sp.tp_max_valid, true);
+  if (DEGREES == DEGREES_POW2 || (DEGREES == DEGREES_EITHER && sp.all_pow2)) return unit_base_pow2(rec, f, pow2_of(f, sp.repl), sp.tp_max_valid, true);
   return unit_base(rec, f, sp.tp_max_valid, true, sp.repl);
 }
+template <int DEGREES = DEGREES_EITHER>
 __device__ __forceinline__ ActBase act_of(const SpaceDev& sp, const ModelRec& rec, const Fact& f, const UnitBase& ub,
                                           u32 v, u32 tau) {
-  if (sp.all_pow2) return act_base_pow2(rec, pow2_of(f, sp.repl), v, tau);
+  if (DEGREES == DEGREES_POW2 || (DEGREES == DEGREES_EITHER && sp.all_pow2)) return act_base_pow2(rec, pow2_of(f, sp.repl), v, tau);
   return act_base(rec, f, v, tau, ub.G);
 }
 
@@ -46,7 +52,7 @@ __device__ __forceinline__ ActBase act_of(const SpaceDev& sp, const ModelRec& re
 // configuration with 64 micro-batches a step took 2.40 ms without required flags instead of
 // 1.27.)  Variants are slots q = 2 v + tau; a slot that the space does not have bounds
 // everything out.
-template <int NM, typename T, bool HOST_LIMITED>
+template <int NM, typename T, bool HOST_LIMITED, int DEGREES = DEGREES_EITHER>
 struct LaneUnit {
   double E, s, u;            // elements of a state, of its largest shard, of a reconstruction unit
   double gr_mem[NM];         // G's terms
@@ -70,7 +76,7 @@ struct LaneUnit {
     for (u32 q = 0; q < 4; ++q) {
       const u32 v = q >> 1, tau = q & 1;
       const bool have = v < sp.nv && tau < sp.nt;
-      const ActBase ab = act_of(sp, rec, f, ub, v, tau);
+      const ActBase ab = act_of<DEGREES>(sp, rec, f, ub, v, tau);
 #pragma unroll
       for (int d = 0; d < NM; ++d) {
         const u64 am = mu_elems(digit_mode(modemap, d), ab.EA, ab.shA, ab.uA, sp.sstar_units);
@@ -96,7 +102,7 @@ struct LaneUnit {
 // allow the digits that keep activation bytes all together or not at all: whether one of them may stand
 // beside a triple depends on the triple only for the offloaded digit (allowed_act_digits).  So their least
 // bytes are a figure of the unit, and no bound per digit and variant is held (40 registers in doubles).
-template <int NM, typename T, bool HOST_LIMITED>
+template <int NM, typename T, bool HOST_LIMITED, int DEGREES>
 struct LeastUnit {
   double E, s, u;
   T shard;
@@ -115,7 +121,7 @@ struct LeastUnit {
 #pragma unroll
       for (u32 v = 0; v < 2; ++v) {
         const bool have = v < sp.nv && tau < sp.nt;
-        const ActBase ab = act_of(sp, rec, f, ub, v, tau);
+        const ActBase ab = act_of<DEGREES>(sp, rec, f, ub, v, tau);
 #pragma unroll
         for (int d = 0; d < NM; ++d)
           if (have && ((digits >> d) & 1u))

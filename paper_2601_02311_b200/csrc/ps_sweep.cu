@@ -521,14 +521,14 @@ __device__ __noinline__ int cut_candidates(BlockShared& sh, int n, int k) {
 // A (unit, triple, tensor-axis variant) that the second pass let through: its points, in
 // index order, by one thread.  `visit(mem, idx)` sees those that the flags, the capacity
 // and the host budget allow, until it returns false.
-template <int NM, typename F>
+template <int NM, int DEGREES, typename F>
 __device__ __forceinline__ void points_of(const SpaceDev& sp, const BlockShared& sh, u32 code, u32 modemap, u64 cap_x,
                                           u64 host_x, F&& visit) {
   constexpr u32 N3 = NM * NM * NM, NC = N3 * NM;
   const ModelRec& rec = sh.rec;
   const u32 unit = code >> 8, t = (code >> 1) & 127u, tau = code & 1u;
   const Fact f = sp.facts[unit];
-  const UnitBase ub = unit_of(sp, rec, f);
+  const UnitBase ub = unit_of<DEGREES>(sp, rec, f);
   const u32 modes[3] = {digit_mode(modemap, t % NM), digit_mode(modemap, (t / NM) % NM), digit_mode(modemap, t / (NM * NM))};
   const u32 width[3] = {rec.wT, rec.wO, rec.wG};
   u64 mem = 0, host = 0;
@@ -540,7 +540,7 @@ __device__ __forceinline__ void points_of(const SpaceDev& sp, const BlockShared&
   const u32 allowed = sh.tri[t].allowed >> (8 * ub.cls);
 #pragma unroll 1
   for (u32 v = 0; v < sp.nv; ++v) {
-    const ActBase ab = act_of(sp, rec, f, ub, v, tau);
+    const ActBase ab = act_of<DEGREES>(sp, rec, f, ub, v, tau);
     const bool host_fits = host + 2 * ab.EA * sp.accum < host_x;
 #pragma unroll 1
     for (u32 d = 0; d < NM; ++d) {
@@ -554,14 +554,14 @@ __device__ __forceinline__ void points_of(const SpaceDev& sp, const BlockShared&
 }
 
 // Pareto: the index of each candidate's point, the smallest with the candidate's bytes
-template <int NM>
+template <int NM, int DEGREES>
 __device__ __noinline__ void resolve_candidates(const SpaceDev& sp, BlockShared& sh, int n, u32 modemap, u64 cap_x,
                                                 u64 host_x, u32* index) {
   __syncthreads();
   for (int p = threadIdx.x; p < n; p += blockDim.x) {
     const u32 code = sh.cand_i[p];
     const u64 want = sh.cand_a[p];
-    points_of<NM>(sp, sh, code, modemap, cap_x, host_x, [&](u64 m, u32 idx) {
+    points_of<NM, DEGREES>(sp, sh, code, modemap, cap_x, host_x, [&](u64 m, u32 idx) {
       if (m == want) index[p] = idx;
       return m != want;
     });
@@ -571,10 +571,10 @@ __device__ __noinline__ void resolve_candidates(const SpaceDev& sp, BlockShared&
 
 // Pareto, where drop_dominated leaves too many: of the candidates of one pair in one unit only
 // the one with the smallest index stays.
-template <int NM>
+template <int NM, int DEGREES>
 __device__ __noinline__ int drop_tied(const SpaceDev& sp, BlockShared& sh, int n, u32 modemap, u64 cap_x, u64 host_x) {
   u32* const index = sh.least_cell;                      // (top-k's)
-  resolve_candidates<NM>(sp, sh, n, modemap, cap_x, host_x, index);
+  resolve_candidates<NM, DEGREES>(sp, sh, n, modemap, cap_x, host_x, index);
   for (int p = threadIdx.x; p < n; p += blockDim.x) {
     bool keep = true;
     for (int q = 0; q < n; ++q)
@@ -588,7 +588,7 @@ __device__ __noinline__ int drop_tied(const SpaceDev& sp, BlockShared& sh, int n
 // top-k: the points of the buffer's n candidates take their places, as many candidates at a
 // time as surely fit, the smallest first; those at or above the k-th smallest point so far are
 // left out.  Returns the number of points.
-template <int NM>
+template <int NM, int DEGREES>
 __device__ __noinline__ int resolve_points(const SpaceDev& sp, BlockShared& sh, int n, int k, u32 modemap, u64 cap_x,
                                            u64 host_x) {
   const int tid = threadIdx.x, threads = blockDim.x;
@@ -614,7 +614,7 @@ __device__ __noinline__ int resolve_points(const SpaceDev& sp, BlockShared& sh, 
       const u64 comm = hit.a[j];
       const u32 code = hit.i[j];
       if (!key_less(Key{comm, hit.b[j], (code >> 8) * per_unit}, threshold)) continue;
-      points_of<NM>(sp, sh, code, modemap, cap_x, host_x, [&](u64 m, u32 idx) {
+      points_of<NM, DEGREES>(sp, sh, code, modemap, cap_x, host_x, [&](u64 m, u32 idx) {
         if (key_less(Key{comm, m, idx}, threshold)) {
           const u32 at = atomicAdd(&sh.n_cand, 1u);
           sh.cand_a[at] = comm; sh.cand_b[at] = m; sh.cand_i[at] = idx;
@@ -630,11 +630,12 @@ __device__ __noinline__ int resolve_points(const SpaceDev& sp, BlockShared& sh, 
 
 // ------------------------------------------------------------------ one point, the slow exact path
 // one point of a model from its index, as an output entry
+template <int DEGREES>
 __device__ __forceinline__ PointOut eval_local(const SpaceDev& sp, const ModelRec& rec, u32 lidx) {
   const LocalPoint lp = decode_local(sp, lidx);
   const Fact f = sp.facts[lp.unit];
-  const UnitBase ub = unit_of(sp, rec, f);
-  return eval_point_from(rec, f, ub, act_of(sp, rec, f, ub, lp.v, lp.tau), lp.tau, digit_mode(sp.modemap, lp.dth),
+  const UnitBase ub = unit_of<DEGREES>(sp, rec, f);
+  return eval_point_from(rec, f, ub, act_of<DEGREES>(sp, rec, f, ub, lp.v, lp.tau), lp.tau, digit_mode(sp.modemap, lp.dth),
                          digit_mode(sp.modemap, lp.dom), digit_mode(sp.modemap, lp.dgr), digit_mode(sp.modemap, lp.dac),
                          sp.tp_coll, sp.sstar_units, sp.accum);
 }
@@ -656,6 +657,7 @@ __device__ __forceinline__ void write_empty(ps_front_entry* out) {
 // more bytes and less communication than the last entry (fewest communication, then
 // smallest index, on ties).  Slow (passes = frontier length), bounded memory, any length.
 // Not inlined, so that it does not weigh on the sweep's registers.
+template <int DEGREES>
 __device__ __noinline__ void frontier_by_definition(const SpaceDev& sp, const SweepArgs& args, const ModelRec& rec,
                                                     u32 model, u64* a, u64* b, u32* ix) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, threads = blockDim.x;
@@ -667,7 +669,7 @@ __device__ __noinline__ void frontier_by_definition(const SpaceDev& sp, const Sw
   for (u32 pass = 0; pass <= ppm; ++pass) {             // a frontier has at most ppm entries
     Key best{U64MAX, U64MAX, 0xffffffffu};
     for (u64 lidx = tid; lidx < ppm; lidx += threads) {
-      const PointOut po = eval_local(sp, rec, (u32)lidx);
+      const PointOut po = eval_local<DEGREES>(sp, rec, (u32)lidx);
       const u64 comm = args.comm_kind == PS_COMM_PAPER ? po.comm_paper : po.comm_paper + po.comm_ext;
       const bool survivor = po.mem <= args.cap_max && po.host <= args.host_cap &&
                             (po.flags & args.require_flags) == args.require_flags;
@@ -693,7 +695,7 @@ __device__ __noinline__ void frontier_by_definition(const SpaceDev& sp, const Sw
       if (best.a > args.caps[ci]) continue;
       const u32 slot = found[ci]++;
       if (slot < args.max_entries && tid == 0)
-        write_entry(args.out + ((u64)model * args.n_caps + ci) * args.max_entries + slot, eval_local(sp, rec, best.i),
+        write_entry(args.out + ((u64)model * args.n_caps + ci) * args.max_entries + slot, eval_local<DEGREES>(sp, rec, best.i),
                     best.b, (u64)model * sp.ppm + best.i);
     }
     last_mem = best.a; last_comm = best.b; have_last = true;
@@ -709,11 +711,17 @@ __device__ __noinline__ void frontier_by_definition(const SpaceDev& sp, const Sw
 }
 
 // ------------------------------------------------------------------ the sweep
+// Registers of a thread: with powers of two five blocks of four warps share an SM instead of four (4096
+// models of the stress configuration 577 -> 543 us for Pareto and 611 -> 589 for top-k, 1024 models 81.0 ->
+// 82.5); the divisions of other degrees spill then (ragged counts 83 -> 102 us).  At 80 the passes spill
+// in either case (1024 models 92 us).
+constexpr int sweep_registers(int degrees) { return degrees == DEGREES_POW2 ? 96 : 128; }
+
 // KIND: the reduction; NM: allowed modes; T: the type of byte counts and volumes (see
 // LaneUnit); HOST_LIMITED: the filter has a host budget (without one the host bytes are
 // never formed).  The number of warps is the launch's (see launch_sweep).
-template <int KIND, int NM, typename T, bool HOST_LIMITED>
-__global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_constant__ SpaceDev sp,
+template <int KIND, int NM, typename T, bool HOST_LIMITED, int DEGREES>
+__global__ void __maxnreg__(sweep_registers(DEGREES)) k_sweep(const __grid_constant__ SpaceDev sp,
                                                                    const __grid_constant__ SweepArgs args) {
   constexpr int N2 = NM * NM, N3 = NM * NM * NM;
   constexpr bool PARETO = KIND == PS_REDUCE_PARETO;
@@ -934,9 +942,9 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
       const u32 b = item / parts, part = item - b * parts, k = b * 32 + lane;
       const u32 unit = seg + sh.heavy[min(k, n_heavy - 1)];
       const Fact f = sp.facts[unit];
-      const UnitBase ub = unit_of(sp, rec, f);
+      const UnitBase ub = unit_of<DEGREES>(sp, rec, f);
       constexpr bool COUNTS = !PARETO && !SECOND;    // top-k's first pass counts points, the others want the least bytes
-      typename std::conditional<COUNTS, LaneUnit<NM, T, HOST_LIMITED>, LeastUnit<NM, T, HOST_LIMITED>>::type lu;
+      typename std::conditional<COUNTS, LaneUnit<NM, T, HOST_LIMITED, DEGREES>, LeastUnit<NM, T, HOST_LIMITED, DEGREES>>::type lu;
       const bool live = k < n_heavy && (ub.cv & req_cv) == req_cv;
       if constexpr (COUNTS) lu.load(sp, rec, f, ub, modemap, cap_x, host_x, live);
       else lu.load(sp, rec, f, ub, modemap, cap_x, host_x, (sh.digits >> (8 * ub.cls)) & all & ~is_o, live);
@@ -1160,7 +1168,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
         if (front != 0) n = drop_beaten(sh, front, n);
         if (front == 0 || n > CAND_CAP / 2) {
           n = drop_dominated(sh, n);                 // (sorts: more than PAIRWISE)
-          if (n > CAND_CAP - STEP_CAP) n = drop_tied<NM>(sp, sh, n, modemap, cap_x, host_x);
+          if (n > CAND_CAP - STEP_CAP) n = drop_tied<NM, DEGREES>(sp, sh, n, modemap, cap_x, host_x);
           if (n > CAND_CAP - STEP_CAP) { overflowed = true; break; }
           front = n;
         }
@@ -1181,20 +1189,20 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
   if (!overflowed) {
     if (PARETO) {
       n_list = drop_dominated(sh, (int)sh.n_cand);
-      resolve_candidates<NM>(sp, sh, n_list, modemap, cap_x, host_x, sh.cand_i);
+      resolve_candidates<NM, DEGREES>(sp, sh, n_list, modemap, cap_x, host_x, sh.cand_i);
       n_list = rank_candidates<KIND>(sh, n_list, 0);
     } else {
       for (int o = 16; o > 0; o >>= 1) survivors += __shfl_xor_sync(0xffffffffu, survivors, o);
       if (lane == 0 && survivors) atomicAdd(&sh.survivors, survivors);
       n_list = cut_candidates(sh, (int)sh.n_cand, (int)args.max_entries);
-      n_list = resolve_points<NM>(sp, sh, n_list, (int)args.max_entries, modemap, cap_x, host_x);
+      n_list = resolve_points<NM, DEGREES>(sp, sh, n_list, (int)args.max_entries, modemap, cap_x, host_x);
       n_list = rank_candidates<KIND>(sh, n_list, (int)args.max_entries);
     }
     overflowed = PARETO && n_list > KEEP_CAP;
     __syncthreads();
   }
   if (overflowed) {
-    frontier_by_definition(sp, args, rec, model, sh.cand_a, sh.cand_b, sh.cand_i);
+    frontier_by_definition<DEGREES>(sp, args, rec, model, sh.cand_a, sh.cand_b, sh.cand_i);
     return;
   }
 
@@ -1220,7 +1228,7 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
   }
   for (int p = tid; p < n_list && (u32)p < args.max_entries; p += threads) {
     const u32 lidx = sh.cand_i[p];
-    const PointOut po = eval_local(sp, rec, lidx);
+    const PointOut po = eval_local<DEGREES>(sp, rec, lidx);
     const u64 comm = args.comm_kind == PS_COMM_PAPER ? po.comm_paper : po.comm_paper + po.comm_ext;
     const u64 list_mem = PARETO ? sh.cand_a[p] : sh.cand_b[p];
     const u64 list_comm = PARETO ? sh.cand_b[p] : sh.cand_a[p];
@@ -1234,24 +1242,30 @@ __global__ void __launch_bounds__(SWEEP_MAX_WARPS * 32, 1) k_sweep(const __grid_
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
-template <int KIND, int NM, typename T, bool HOST_LIMITED>
+template <int KIND, int NM, typename T, bool HOST_LIMITED, int DEGREES>
 static cudaError_t launch_sweep_p(const SpaceDev& sp, const SweepArgs& a, int warps, cudaStream_t stream) {
   const dim3 grid(sp.n_models, KIND == PS_REDUCE_PARETO ? 1 : a.n_caps);
   const size_t smem = sizeof(BlockShared);
-  cudaError_t e = cudaFuncSetAttribute(k_sweep<KIND, NM, T, HOST_LIMITED>,
+  cudaError_t e = cudaFuncSetAttribute(k_sweep<KIND, NM, T, HOST_LIMITED, DEGREES>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_sweep<KIND, NM, T, HOST_LIMITED><<<grid, warps * 32, smem, stream>>>(sp, a);
+  k_sweep<KIND, NM, T, HOST_LIMITED, DEGREES><<<grid, warps * 32, smem, stream>>>(sp, a);
   return cudaGetLastError();
+}
+
+template <int KIND, int NM, bool HOST_LIMITED>
+static cudaError_t launch_sweep_d(const SpaceDev& sp, const SweepArgs& a, int warps, cudaStream_t stream) {
+  return sp.all_pow2 ? launch_sweep_p<KIND, NM, double, HOST_LIMITED, DEGREES_POW2>(sp, a, warps, stream)
+                     : launch_sweep_p<KIND, NM, double, HOST_LIMITED, DEGREES_ANY>(sp, a, warps, stream);
 }
 
 template <int KIND, int NM>
 static cudaError_t launch_sweep_t(const SpaceDev& sp, const SweepArgs& a, int warps, cudaStream_t stream) {
   // every byte count exact in a double
   if (sp.all_small && a.cap_max < ((u64)1 << 53) - 1)
-    return NM < 4 || a.host_cap < HOST_BYTES_END ? launch_sweep_p<KIND, NM, double, true>(sp, a, warps, stream)
-                                                 : launch_sweep_p<KIND, NM, double, NM < 4>(sp, a, warps, stream);
-  return launch_sweep_p<KIND, NM, u64, true>(sp, a, warps, stream);
+    return NM < 4 || a.host_cap < HOST_BYTES_END ? launch_sweep_d<KIND, NM, true>(sp, a, warps, stream)
+                                                 : launch_sweep_d<KIND, NM, NM < 4>(sp, a, warps, stream);
+  return launch_sweep_p<KIND, NM, u64, true, DEGREES_EITHER>(sp, a, warps, stream);
 }
 
 template <int KIND>
