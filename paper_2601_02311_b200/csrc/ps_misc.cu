@@ -99,16 +99,24 @@ struct SelectMagic {
   double inv[SELECT_MAGIC_MAX + 1];   // 1 / t, correctly rounded
 };
 
-// floor(a / d) from a reciprocal of d that is correct to the last bit: for a < 2^52
-// the product is off by less than one, so its integer part is the quotient or a
-// neighbour of it, and the remainder says which.  One code path for every lane.
-__device__ __forceinline__ u64 div_by_reciprocal(u64 a, u32 d, double recip) {
-  if (a >= ((u64)1 << 52)) return a / d;
-  u64 q = (u64)__double2ll_rz((double)(long long)a * recip);
-  const long long rem = (long long)(a - q * d);
-  if (rem < 0) --q;
-  else if (rem >= (long long)d) ++q;
-  return q;
+// floor(a / d) for a < 2^50 from r = 1 / d within 2^-52 of it: a + 1/2 is at least 1 / (2 d) of d
+// away from any multiple, and the product is off by less than a / d * 2^-51 < 1 / (2 d).  The
+// conversions are additions: 2^52 + a has the bits of a below those of 2^52, and a sum rounded
+// down to a multiple of the 1 that is left there has the integer part of the other term.
+constexpr u64 BITS_2_52 = 0x4330000000000000ull, QUOTIENT_END = (u64)1 << 50;
+__device__ __forceinline__ u64 div_by_reciprocal(u64 a, u32 d, double r) {
+  if (a >= QUOTIENT_END) return a / d;
+  const double half_more = __longlong_as_double((long long)(BITS_2_52 | a)) - (0x1p52 - 0.5);
+  return (u64)__double_as_longlong(__dadd_rd(half_more * r, 0x1p52)) ^ BITS_2_52;
+}
+// 1 / d within 2^-52: two steps of Newton's iteration (r += r (1 - d r), the error squared each
+// time) from an approximation of 20 bits or more
+__device__ __forceinline__ double reciprocal(u32 d) {
+  const double x = __longlong_as_double((long long)(BITS_2_52 | d)) - 0x1p52;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
 }
 
 // the largest t <= tp_degree that divides n
@@ -156,22 +164,16 @@ __device__ __forceinline__ ps_select_result select_one(const ps_select_query& s,
                                                        u32 head_den, u32 layer_num, u32 layer_den,
                                                        u32 tp_degree, const SelectMagic& magic) {
   const u32 wsum = (u32)s.w_param + s.w_grad + s.w_opt;
-  const Wide m_model = wide_mul(wide_mul(s.param_elems, wsum), head_den);     // M_model * head_den
-  const Wide budget = wide_mul(s.device_bytes, head_num);                      // headroom * M_d, times head_den
-  u32 branch, T = 1, code = 32;                                // ZeRO-3 unless data parallel fits
-  if (wide_less(m_model, budget)) {
-    branch = 0; code = 0;
-  } else if (wide_less(m_model, wide_mul(budget, s.n_devices))) {
-    branch = 1;
-  } else {
-    const Wide layer = wide_mul(wide_mul(s.layer_elems, wsum), layer_den);
-    if (s.fast_interconnect && wide_less(wide_mul(s.device_bytes, layer_num), layer)) {
-      branch = 2;
-      T = largest_tensor_degree(s.n_devices, tp_degree, magic);
-    } else {
-      branch = 3;
-    }
-  }
+  // (wsum < 2^10 and the denominators are at most 2^16: one factor)
+  const Wide m_model = wide_mul(s.param_elems, wsum * head_den);              // M_model * head_den
+  const Wide budget = wide_mul(s.device_bytes, head_num);                     // headroom * M_d, times head_den
+  const Wide layer = wide_mul(s.layer_elems, wsum * layer_den);
+  u32 branch = 3, T = 1;
+  if (s.fast_interconnect && wide_less(wide_mul(s.device_bytes, layer_num), layer)) branch = 2;
+  if (wide_less(m_model, wide_mul(budget, s.n_devices))) branch = 1;
+  if (wide_less(m_model, budget)) branch = 0;
+  if (branch == 2) T = largest_tensor_degree(s.n_devices, tp_degree, magic);
+  const u32 code = branch == 0 ? 0 : 32;                       // ZeRO-3 unless data parallel fits
   // Theorem 1 and Theorem 2 for the choice, written out for the two specifications
   // the algorithm can return (no activations, no pipeline axis): with E = ceil(P / T)
   // elements per tensor rank over D = N / T replicas,
@@ -194,7 +196,7 @@ __device__ __forceinline__ ps_select_result select_one(const ps_select_query& s,
       unit_t = div_ceil(s.layer_elems, T);
     }
   }
-  const u64 quot = div_by_reciprocal(E, D, __drcp_rn((double)D));
+  const u64 quot = div_by_reciprocal(E, D, reciprocal(D));
   const u64 x = E - quot;
   u64 mem, comm;
   if (code == 0) {
@@ -211,9 +213,14 @@ __device__ __forceinline__ ps_select_result select_one(const ps_select_query& s,
   return o;
 }
 
-// SELECT_PER_THREAD queries per thread, SELECT_THREADS apart, all of their 16-byte
-// loads in flight before any arithmetic: the kernel streams 64 bytes per query, read
-// once and written once (streaming loads and stores, nothing is reused).
+// SELECT_PER_THREAD queries per thread, SELECT_THREADS apart, all of their loads in flight before
+// any arithmetic: the kernel streams 64 bytes per query, read once and written once (streaming
+// loads and stores, nothing is reused).
+// WHOLE: both arrays lie on 32-byte boundaries, and a record is one load and one store.  As two
+// 16-byte accesses each a warp's access covers every other half of 32 sectors.
+// What bounds it: issue slots (0.76 of them taken, ncu) and the HBM stream, 5.9 TB/s: 2^24 queries
+// in 183-186 us, 215 with 16-byte accesses, conversions through the slow conversion unit, a correctly
+// rounded reciprocal and a remainder test per quotient.  One query a thread takes 205.
 #ifndef SELECT_THREADS_PER_BLOCK
 #define SELECT_THREADS_PER_BLOCK 128
 #endif
@@ -227,29 +234,53 @@ __device__ __forceinline__ ps_select_result select_one(const ps_select_query& s,
 #endif
 constexpr int SELECT_THREADS = SELECT_THREADS_PER_BLOCK;
 constexpr int SELECT_PER_THREAD = SELECT_QUERIES_PER_THREAD;
+struct Words { u64 w[4]; };
+template <bool WHOLE>
+__device__ __forceinline__ Words load_words(const void* p) {
+  Words r;
+  if (WHOLE) {
+    asm volatile("ld.global.L1::no_allocate.L2::evict_first.v4.b64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(r.w[0]), "=l"(r.w[1]), "=l"(r.w[2]), "=l"(r.w[3]) : "l"(p));
+  } else {
+    const ulonglong2 a = __ldcs(static_cast<const ulonglong2*>(p)), b = __ldcs(static_cast<const ulonglong2*>(p) + 1);
+    r.w[0] = a.x; r.w[1] = a.y; r.w[2] = b.x; r.w[3] = b.y;
+  }
+  return r;
+}
+template <bool WHOLE>
+__device__ __forceinline__ void store_words(void* p, const Words& r) {
+  if (WHOLE) {
+    asm volatile("st.global.L1::no_allocate.L2::evict_first.v4.b64 [%0], {%1, %2, %3, %4};"
+                 ::"l"(p), "l"(r.w[0]), "l"(r.w[1]), "l"(r.w[2]), "l"(r.w[3]) : "memory");
+  } else {
+    __stcs(static_cast<ulonglong2*>(p), make_ulonglong2(r.w[0], r.w[1]));
+    __stcs(static_cast<ulonglong2*>(p) + 1, make_ulonglong2(r.w[2], r.w[3]));
+  }
+}
+template <bool WHOLE>
 __global__ void __launch_bounds__(SELECT_THREADS, SELECT_MIN_BLOCKS) k_select(const ps_select_query* __restrict__ q, u64 n,
                                                            u32 head_num, u32 head_den, u32 layer_num,
-                                                           u32 layer_den, u32 tp_degree, SelectMagic magic,
+                                                           u32 layer_den, u32 tp_degree, const __grid_constant__ SelectMagic magic,
                                                            ps_select_result* __restrict__ out) {
   const u64 first = (u64)blockIdx.x * (SELECT_PER_THREAD * SELECT_THREADS) + threadIdx.x;
-  ps_select_query s[SELECT_PER_THREAD];
+  Words in[SELECT_PER_THREAD];
 #pragma unroll
   for (int j = 0; j < SELECT_PER_THREAD; ++j) {
     const u64 i = first + (u64)j * SELECT_THREADS;
-    if (i < n) {
-      const uint4* src = reinterpret_cast<const uint4*>(q + i);
-      uint4* dst = reinterpret_cast<uint4*>(&s[j]);
-      dst[0] = __ldcs(src); dst[1] = __ldcs(src + 1);
-    }
+    if (i < n) in[j] = load_words<WHOLE>(q + i);
   }
 #pragma unroll
   for (int j = 0; j < SELECT_PER_THREAD; ++j) {
     const u64 i = first + (u64)j * SELECT_THREADS;
     if (i < n) {
-      const ps_select_result o = select_one(s[j], head_num, head_den, layer_num, layer_den, tp_degree, magic);
-      uint4* dst = reinterpret_cast<uint4*>(out + i);
-      const uint4* src = reinterpret_cast<const uint4*>(&o);
-      __stcs(dst, src[0]); __stcs(dst + 1, src[1]);
+      ps_select_query s;
+      s.param_elems = in[j].w[0]; s.layer_elems = in[j].w[1]; s.device_bytes = in[j].w[2];
+      const u32 last = (u32)(in[j].w[3] >> 32);
+      s.n_devices = (u32)in[j].w[3];
+      s.w_param = (uint8_t)last; s.w_grad = (uint8_t)(last >> 8); s.w_opt = (uint8_t)(last >> 16);
+      s.fast_interconnect = (uint8_t)(last >> 24);
+      const ps_select_result o = select_one(s, head_num, head_den, layer_num, layer_den, tp_degree, magic);
+      store_words<WHOLE>(out + i, Words{{o.mem, o.comm, (u64)o.branch | ((u64)o.T << 32), (u64)o.code_dp | ((u64)o.flags << 32)}});
     }
   }
 }
@@ -374,7 +405,9 @@ static SelectMagic select_magic() {
 cudaError_t launch_select(const ps_select_query* d_q, u64 n, u32 head_num, u32 head_den, u32 layer_num,
                           u32 layer_den, u32 tp_degree, ps_select_result* d_out, cudaStream_t stream) {
   const u64 per_block = (u64)SELECT_PER_THREAD * SELECT_THREADS;
-  k_select<<<(unsigned)((n + per_block - 1) / per_block), SELECT_THREADS, 0, stream>>>(
+  const unsigned blocks = (unsigned)((n + per_block - 1) / per_block);
+  const bool whole = ((reinterpret_cast<uintptr_t>(d_q) | reinterpret_cast<uintptr_t>(d_out)) & 31) == 0;
+  (whole ? k_select<true> : k_select<false>)<<<blocks, SELECT_THREADS, 0, stream>>>(
       d_q, n, head_num, head_den, layer_num, layer_den, tp_degree, select_magic(), d_out);
   return cudaGetLastError();
 }
