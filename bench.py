@@ -16,8 +16,8 @@ on the stress configuration (4096 shapes, N up to 2^14, 6 963 200 000 points):
 
 `value` counts every point each phase evaluates, per second, device-timed with
 inputs resident in HBM (the sweeps' screening holds the up to four variants of a placement with
-offloaded activations, which have the same bytes, against the capacity in one compare: 17 compares
-for 20 points); `e2e` times the same step through the C interface with
+offloaded activations, which have the same bytes, against the capacity in one compare, 17 compares
+for 20 points, in rounded figures first); `e2e` times the same step through the C interface with
 the shape table in pinned host memory and every result copied back to the host.
 Before anything is timed, sampled outputs are compared bit for bit with the CPU
 oracle; a run that is not bit-exact reports no throughput.
