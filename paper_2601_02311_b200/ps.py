@@ -35,7 +35,7 @@ COMM_PAPER, COMM_PAPER_PLUS_EXT = 0, 1
 REDUCE_PARETO, REDUCE_TOPK = 0, 1
 NO_LIMIT = (1 << 64) - 1
 TOPK_MAX = 64
-PINNED_RESULT_BYTES = 1 << 20       # a sweep's result up to this size is read back through pinned memory
+PINNED_RESULT_BYTES = 4 << 20       # a result up to this size is read back through pinned memory
 
 SELECT_QUERY_DTYPE = np.dtype([("param_elems", "<u8"), ("layer_elems", "<u8"), ("device_bytes", "<u8"),
                                ("n_devices", "<u4"), ("w_param", "u1"), ("w_grad", "u1"), ("w_opt", "u1"),
@@ -248,7 +248,8 @@ class Context:
     @_on_own_stream
     def verify_batch(self, shape: dict, cases: np.ndarray, data: np.ndarray, want_theta: bool = False):
         """ps_verify_batch: `cases` a VERIFY_CASE_DTYPE array, `data` a float64 array holding every
-        case's problem; returns VERIFY_RESULT_DTYPE records (and the final parameters)."""
+        case's problem; returns VERIFY_RESULT_DTYPE records (and the final parameters).  Both are views of
+        one buffer; up to PINNED_RESULT_BYTES it is page-locked for as long as either is kept."""
         sh = _VerifyShape(shape["units"], shape["h"], shape["b"], shape.get("accum", 1), shape.get("steps", 3),
                           shape.get("gather_buffers", 1), shape.get("w_theta", 2), shape.get("w_omega", 12),
                           shape.get("w_grad", 2), 0, shape.get("lr", 0.05), shape.get("beta1", 0.9),
@@ -258,19 +259,34 @@ class Context:
         assert cases.dtype.itemsize == 16
         data = np.ascontiguousarray(data, dtype=np.float64)
         n = len(cases)
-        dev = self.torch_device
-        d_cases = torch.from_numpy(cases.view(np.uint8).reshape(-1).copy()).to(dev)
-        d_data = torch.from_numpy(data).to(dev)
-        d_out = torch.zeros(max(n, 1) * 40, dtype=torch.uint8, device=dev)
         P = shape["units"] * shape["h"]
-        d_theta = torch.zeros(max(n, 1) * P, dtype=torch.float64, device=dev) if want_theta else None
-        _check(_lib.ps_verify_batch(self._h, C.byref(sh), _dptr(d_cases), n, _dptr(d_data), len(data),
-                                    _dptr(d_out), _dptr(d_theta)), "ps_verify_batch")
-        self.check_status()
-        res = d_out.cpu().numpy()[:n * 40].view(VERIFY_RESULT_DTYPE)
+        # the cases and their problems go up together, the parameters and records come back together
+        size = cases.nbytes + data.nbytes
+        up = torch.empty(size, dtype=torch.uint8, pin_memory=0 < size <= PINNED_RESULT_BYTES)
+        up.numpy()[:cases.nbytes] = cases.view(np.uint8).reshape(-1)
+        up.numpy()[cases.nbytes:] = data.view(np.uint8).reshape(-1)
+        d_in = up.to(self.torch_device, non_blocking=True)
+        at = n * P * 8 if want_theta else 0
+        d_all = torch.empty(max(at + n * 40, 1), dtype=torch.uint8, device=self.torch_device)
+        into, base = d_in.data_ptr(), d_all.data_ptr()
+        _check(_lib.ps_verify_batch(self._h, C.byref(sh), into, n, into + cases.nbytes if len(data) else None, len(data),
+                                    base + at, base if want_theta else None), "ps_verify_batch")
+        host, _ = self._read_back(d_all)
+        res = host[at:at + n * 40].view(VERIFY_RESULT_DTYPE)
         if want_theta:
-            return res, d_theta.cpu().numpy().reshape(-1, P)[:n]
+            return res, host[:at].view(np.float64).reshape(n, P)
         return res
+
+    def _read_back(self, d_all: torch.Tensor, allow_truncated: bool = False):
+        """A uint8 buffer's bytes on the host once the work before has been done and found in order,
+        and check_status's answer.  A small buffer is copied behind that work through pinned memory,
+        and one wait covers both."""
+        if d_all.numel() <= PINNED_RESULT_BYTES:
+            host = torch.empty(d_all.numel(), dtype=torch.uint8, pin_memory=True)
+            host.copy_(d_all, non_blocking=True)
+            return host.numpy(), self.check_status(allow_truncated)
+        status = self.check_status(allow_truncated)
+        return d_all.cpu().numpy(), status
 
     def int_peak(self, blocks: int, iters: int, sink: torch.Tensor) -> int:
         ops = C.c_uint64()
@@ -423,15 +439,7 @@ class Space:
         d_all = torch.empty(at + rows * 4, dtype=torch.uint8, device=self.ctx.torch_device)
         base = d_all.data_ptr()
         self._sweep(filt, caps, kind, max_entries, base, base + at)
-        if d_all.numel() <= PINNED_RESULT_BYTES:
-            # a small result: the copy is enqueued behind the sweep and one wait covers both
-            host = torch.empty(d_all.numel(), dtype=torch.uint8, pin_memory=True)
-            host.copy_(d_all, non_blocking=True)
-            self.last_sweep_status = self.ctx.check_status(allow_truncated=True)
-        else:
-            self.last_sweep_status = self.ctx.check_status(allow_truncated=True)
-            host = d_all.cpu()
-        flat = host.numpy()
+        flat, self.last_sweep_status = self.ctx._read_back(d_all, allow_truncated=True)
         entries = flat[:at].view(ENTRY_DTYPE).reshape(self.n_models, len(caps), max_entries)
         counts = flat[at:].view(np.uint32).reshape(self.n_models, len(caps))
         return entries, counts
