@@ -559,7 +559,7 @@ def run_ours(args):
             # the dominant kernel of a step is the Pareto sweep (its share is in phases_ms)
             "roofline": alu_roofline("k_sweep_pareto", "k_sweep<Pareto>", phase_ms["pareto"]),
             "roofline_topk": alu_roofline("k_sweep_topk", "k_sweep<top-k>", phase_ms["topk"]),
-            "roofline_hbm": {"bound": "hbm", "kernel": "k_eval<materialise>", "achieved": mat_gbs,
+            "roofline_hbm": {"bound": "hbm", "kernel": "k_eval (materialise)", "achieved": mat_gbs,
                              "peak": hbm_peak, "unit": "GB/s", "frac": mat_gbs / hbm_peak,
                              "traffic": (int(captured["kernels"]["k_eval_materialise"]["dram_bytes_per_point"] * count)
                                          if captured and "k_eval_materialise" in captured["kernels"] else None),
@@ -569,7 +569,7 @@ def run_ours(args):
         }
         dense_gbs = (BYTES_PER_POINT_MATERIALISE + 8) * dense_survivors / (dense_ms * 1e-3) / 1e9
         line["roofline_compact_dense"] = {
-            "bound": "hbm", "kernel": "k_compact_count + k_eval<write>, every point survives",
+            "bound": "hbm", "kernel": "k_compact_count + k_write, every point survives",
             "achieved": dense_gbs, "peak": hbm_peak, "unit": "GB/s", "frac": dense_gbs / hbm_peak,
             "ms": dense_ms, "survivors": dense_survivors, "bytes_per_survivor": BYTES_PER_POINT_MATERIALISE + 8,
             "traffic": None}

@@ -437,7 +437,7 @@ int ps_eval_batch(ps_ctx* ctx, const ps_space* sp, uint64_t first, uint64_t coun
     a.cap_bytes = filter->cap_bytes;
     a.host_cap = filter->host_cap;
     a.require_flags = filter->require_flags & ~(u32)PS_F_FEASIBLE;
-    // per group an offset and a place in the list of groups with survivors, per run of
+    // per group an offset and a place in the list of factorisations with survivors, per run of
     // factorisations an offset
     eval_plan_runs(sp->dev, a);
     const size_t group_bytes = (sizeof(u32) * n_groups + 15) & ~size_t(15);

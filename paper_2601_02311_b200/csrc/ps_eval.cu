@@ -19,10 +19,11 @@
 // Compaction is count -> write.  The count pass (k_compact_count) never forms a point's
 // bytes or flags: a lane owns a factorisation, and a point is one compare of a triple's own
 // bytes with a per-(variant, digit) bound, masked by the digits the required flags allow.
-// It leaves each group's offset in its run of factorisations, appends the groups that have
+// It leaves each group's offset in its run of factorisations, appends the factorisations that have
 // survivors to a list, and its last block turns the runs' totals into offsets.  The write
-// pass takes the listed groups one per warp, evaluates them and places their survivors with
-// ballot/popc prefix sums.  Output order is the index order, so the result is unique.
+// pass (k_write) takes the listed factorisations a block each, evaluates their groups from a common
+// table of triples and places their survivors with ballot/popc prefix sums.  Output order is the
+// index order, so the result is unique.
 #include "ps_device.cuh"
 #include "ps_internal.h"
 #include "ps_lane.cuh"
@@ -31,24 +32,19 @@ namespace {
 
 // Launch shapes (blocks of four warps).  Materialise is fastest with about one group per warp:
 // short-lived blocks keep the warps of an SM at different stages (set-up, staging, draining
-// stores) and the running warps write neighbouring stretches of every output array.  The write
-// pass takes the listed groups round-robin; with many short blocks the stores of neighbouring
-// groups are in flight together (2^24 points all surviving 0.171 ms with 64 blocks per SM in the
-// grid, 0.189 with 8; 256 codes a group 0.149 and 0.164).
+// stores) and the running warps write neighbouring stretches of every output array.
 #ifndef EVAL_BULK_EVICT_FIRST
 #define EVAL_BULK_EVICT_FIRST 1
 #endif
 #ifndef EVAL_GRID_PER_SM_MATERIALISE
 #define EVAL_GRID_PER_SM_MATERIALISE 128
 #endif
-// (resident blocks of the write pass with up to four modes: half of 2^23 points surviving
-// 0.067 ms with four, 0.062 with five, 0.071 with six, whose registers spill.  With five modes
-// five blocks spill as well: 2^24 points all surviving 0.204 ms against 0.175 with four.)
+// (the write pass's shape: see k_write)
 #ifndef EVAL_MIN_BLOCKS_WRITE
 #define EVAL_MIN_BLOCKS_WRITE 5
 #endif
 #ifndef EVAL_GRID_PER_SM_WRITE
-#define EVAL_GRID_PER_SM_WRITE 64
+#define EVAL_GRID_PER_SM_WRITE 16
 #endif
 constexpr int THREADS = EVAL_THREADS;
 constexpr int WARPS = THREADS / 32;
@@ -85,8 +81,6 @@ __device__ __forceinline__ u32 triple_static_all_copies(u32 th, u32 om, u32 gr) 
   const u32 st = triple_static(th, om, gr, true) & ~X_EXT0;
   return st | (in_set((1u << PS_MODE_SG) | SET_M_OR_O, gr) ? 0u : X_EXT0);
 }
-
-enum { MODE_MATERIALISE = 0, MODE_WRITE = 2 };
 
 // Staging for the materialise path.  A warp builds one output array of one
 // group (NC elements) in shared memory and hands it to the copy engine as a
@@ -154,23 +148,21 @@ __device__ __forceinline__ void load_record(const SpaceDev& sp, u32 model, Model
 }
 
 // POW2: every degree of the space is a power of two (no division is compiled in)
-template <int MODE, int NM, bool POW2>
-__global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE && NM < 5 ? EVAL_MIN_BLOCKS_WRITE : EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, EvalArgs a) {
+template <int NM, bool POW2>
+__global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, EvalArgs a) {
   constexpr int N2 = NM * NM, N3 = NM * NM * NM, NC = N3 * NM;
   constexpr int R = (N3 + 31) / 32;
-  // materialise: two staging buffers per warp (dynamic shared memory, none in the other modes)
+  // two staging buffers per warp
   extern __shared__ __align__(128) unsigned char stage_all[];
   unsigned char* const stage_warp = stage_all + (threadIdx.x >> 5) * 2 * Stage<NC>::BYTES;
   u32 stage_turn = 0;                                                     // which buffer is next
   const int lane = threadIdx.x & 31;
   const u32 warp_global = blockIdx.x * WARPS + (threadIdx.x >> 5);
   const u32 n_warps = gridDim.x * WARPS;
-  // materialise: the window's groups are dealt evenly, a contiguous stretch per warp;
-  // write: the groups that have survivors, from the count pass's list, dealt round-robin
+  // the window's groups are dealt evenly, a contiguous stretch per warp
   const u32 per_warp = (a.n_tiles + n_warps - 1) / n_warps;
-  const u32 it_begin = MODE == MODE_WRITE ? warp_global : (u32)min((u64)warp_global * per_warp, (u64)a.n_tiles);
-  const u32 it_end = MODE == MODE_WRITE ? *a.n_listed : min(it_begin + per_warp, a.n_tiles);
-  const u32 it_step = MODE == MODE_WRITE ? n_warps : 1u;
+  const u32 it_begin = (u32)min((u64)warp_global * per_warp, (u64)a.n_tiles);
+  const u32 it_end = min(it_begin + per_warp, a.n_tiles);
   const u32 groups_per_model = sp.n_facts * sp.nvt;
 
   // with all five modes allowed digit d is mode d, and the compiler knows every
@@ -205,9 +197,8 @@ __global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE && NM < 5 ? EVAL_M
   u32 st_many[R], st_one[R];                      // static description of a triple by the class of the factorisation
   u32 st_copies[POW2 ? 1 : R];                    // (the third class needs several copies of a shard)
 
-  for (u32 it = it_begin; it < it_end; it += it_step) {
-    const u32 seg = MODE == MODE_WRITE ? a.nonempty[it] : it;
-    const u64 g = a.first_group + seg;
+  for (u32 it = it_begin; it < it_end; ++it) {
+    const u64 g = a.first_group + it;
     // (a 32-bit division where the group number allows it: it is done once per group by every lane)
     const u32 model = (g >> 32) == 0 ? (u32)g / groups_per_model : (u32)(g / groups_per_model);
     const u32 gl = (u32)(g - (u64)model * groups_per_model);
@@ -295,13 +286,6 @@ __global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE && NM < 5 ? EVAL_M
     const u32 code_hi = window_end < group_first + NC ? (u32)(window_end - group_first) : (u32)NC;
     const u64 out_base = group_first - a.first;          // (wraps when the group starts before the window; only used with code >= code_lo)
 
-    u32 n_kept = 0;
-    u64 write_base = 0;
-    if (MODE == MODE_WRITE) {
-      // survivors before this group: those of the runs before its run, and of the run's earlier groups
-      write_base = a.run_offset[(u32)(g / sp.nvt - a.first_unit) / EVAL_RUN_UNITS] + a.group_offset[seg];
-    }
-
     // flags of a point = what the triple fixes | what the digit fixes | what needs both:
     //   gradient integrity needs the triple's two availability bits and the digit's,
     //   "paper priced" needs a triple without M/O and unpriced traffic and a digit without M/O
@@ -316,7 +300,7 @@ __global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE && NM < 5 ? EVAL_M
     const bool whole = code_lo == 0 && code_hi == (u32)NC;      // the window covers the group
     const bool all_out = a.out.mem && a.out.comm_paper && a.out.comm_ext && a.out.host && a.out.flags;
 
-    if (MODE == MODE_MATERIALISE && whole && all_out) {
+    if (whole && all_out) {
       // one output array at a time: stage the group's NC values, hand them to the copy engine
 #pragma unroll
       for (int which = 0; which < 5; ++which) {
@@ -354,9 +338,9 @@ __global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE && NM < 5 ? EVAL_M
       continue;
     }
 
-    // (materialise takes this path at the window's edges only: unrolled, it made the staged path
-    // spill, 2^25 points 0.191 ms instead of 0.179)
-#pragma unroll (MODE == MODE_WRITE ? NM : 1)
+    // (at the window's edges only: unrolled, it made the staged path spill, 2^25 points 0.191 ms
+    // instead of 0.179)
+#pragma unroll 1
     for (int d = 0; d < NM; ++d) {
       const u64 act_d = mu_elems(digit_mode(modemap, d), ab.EA, ab.shA, ab.uA, sp.sstar_units);
       const bool d_avail = (avail >> d) & 1u, d_off = (is_o >> d) & 1u, d_notmo = (not_mo >> d) & 1u;
@@ -366,47 +350,167 @@ __global__ void __launch_bounds__(THREADS, MODE == MODE_WRITE && NM < 5 ? EVAL_M
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const u32 code = lane + 32 * r + d * N3;
-        const bool inside = live[r] && (whole || (code >= code_lo && code < code_hi));
+        if (!(live[r] && (whole || (code >= code_lo && code < code_hi)))) continue;
         const u64 mem = mem3[r] + act_d;
         const u64 host = host3[r] + host_add;
         const u32 fl = fl_base[r] | fl_digit | (fl_gi[r] & gi_mask) | (fl_priced[r] & priced_mask);
-        if (MODE == MODE_MATERIALISE) {
-          if (inside) {
-            const u64 o = out_base + code;
-            if (all_out) {
-              a.out.mem[o] = mem;
-              a.out.comm_paper[o] = paper3[r];
-              a.out.comm_ext[o] = ext3[r] + c_axis;
-              a.out.host[o] = host;
-              a.out.flags[o] = fl;
-            } else {
-              if (a.out.mem) a.out.mem[o] = mem;
-              if (a.out.comm_paper) a.out.comm_paper[o] = paper3[r];
-              if (a.out.comm_ext) a.out.comm_ext[o] = ext3[r] + c_axis;
-              if (a.out.host) a.out.host[o] = host;
-              if (a.out.flags) a.out.flags[o] = fl;
-            }
-          }
+        const u64 o = out_base + code;
+        if (all_out) {
+          a.out.mem[o] = mem;
+          a.out.comm_paper[o] = paper3[r];
+          a.out.comm_ext[o] = ext3[r] + c_axis;
+          a.out.host[o] = host;
+          a.out.flags[o] = fl;
         } else {
-          const bool pass = inside && mem <= a.cap_bytes && host <= a.host_cap &&
-                            (fl & a.require_flags) == a.require_flags;
-          const u32 votes = __ballot_sync(0xffffffffu, pass);
-          if (MODE == MODE_WRITE && pass) {
-            const u64 o = write_base + n_kept + __popc(votes & ((1u << lane) - 1u));
-            if (a.idx_out) a.idx_out[o] = group_first + code;
-            if (a.out.mem) a.out.mem[o] = mem;
-            if (a.out.comm_paper) a.out.comm_paper[o] = paper3[r];
-            if (a.out.comm_ext) a.out.comm_ext[o] = ext3[r] + c_axis;
-            if (a.out.host) a.out.host[o] = host;
-            if (a.out.flags) a.out.flags[o] = fl | PS_F_FEASIBLE;
-          }
-          n_kept += __popc(votes);
+          if (a.out.mem) a.out.mem[o] = mem;
+          if (a.out.comm_paper) a.out.comm_paper[o] = paper3[r];
+          if (a.out.comm_ext) a.out.comm_ext[o] = ext3[r] + c_axis;
+          if (a.out.host) a.out.host[o] = host;
+          if (a.out.flags) a.out.flags[o] = fl;
         }
       }
     }
   }
   // the staging buffers must outlive the bulk stores that read them
-  if (MODE == MODE_MATERIALISE && lane == 0) bulk_wait_all();
+  if (lane == 0) bulk_wait_all();
+}
+
+// ------------------------------------------------------------------ compaction: write
+// A unit's triples as its groups share them: bytes, traffic on the data axis, host bytes and flags.
+template <int NM>
+struct UnitTable {
+  static constexpr int N3 = NM * NM * NM;
+  u64 mem[N3], paper[N3], ext[N3], host[N3];
+  u32 flags[N3];              // high half: the bits that need the triple and the digit
+};
+
+// A block takes the listed units in turns of as many as give each of its warps a group: the warps
+// of a unit make its table of triples together, a thread a triple, and then each evaluates its
+// group (activation and tensor-axis variant) from that table and places its survivors by ballot and
+// popc.  What bounds it: the set-up of a group and its stores.  With the triples' coefficients and
+// figures formed by every warp for itself, four triples a lane, 2^23 points with half of them
+// surviving took 74 us and 2^25 with one in two thousand 32, with the count pass; like this 68 and 28,
+// launched before the count pass has ended 67 and 26.5, with 16 blocks per SM in the grid instead of 64 (most
+// of which found nothing left to do) 64.6 and 25; with 6 blocks 80 and 24.
+template <int NM, bool POW2>
+__global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS_WRITE) k_write(const __grid_constant__ SpaceDev sp,
+                                                                         const __grid_constant__ EvalArgs a) {
+  constexpr int N2 = NM * NM, N3 = NM * NM * NM, NC = N3 * NM, R = (N3 + 31) / 32;
+  __shared__ UnitTable<NM> tables[WARPS];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const u32 nvt = sp.nvt, teams = WARPS / nvt, team = warp / nvt, vt = warp - team * nvt;   // nvt: 1, 2 or 4
+  const u32 v = vt / sp.nt, tau = vt - v * sp.nt;
+  UnitTable<NM>& table = tables[team];
+  const u32 modemap = (NM == 5) ? 0x43210u : sp.modemap;
+  u32 own = 0;                                             // Theorem 3: a replica needs its own activations
+#pragma unroll
+  for (int d = 0; d < NM; ++d)
+    if (in_set(SET_ACT_OWN, digit_mode(modemap, d))) own |= 1u << d;
+  asm volatile("griddepcontrol.wait;" ::: "memory");      // the count pass has ended, nothing of it is read before
+  const u32 n_listed = *a.n_listed;
+  for (u64 first = (u64)blockIdx.x * teams; first < n_listed; first += (u64)gridDim.x * teams) {
+    const bool have = first + team < n_listed;
+    const u32 place = a.nonempty[have ? first + team : first];
+    const u64 ug = a.first_unit + place;
+    const u32 model = (ug >> 32) == 0 ? (u32)ug / sp.n_facts : (u32)(ug / sp.n_facts);
+    ModelRec rec;
+    load_record(sp, model, rec);
+    if (v) { rec.A[0] = rec.A[1]; rec.UA[0] = rec.UA[1]; }  // (the warp's variant; an index known here keeps the record in registers)
+    const Fact f = sp.facts[(u32)(ug - (u64)model * sp.n_facts)];
+    const u32 repl = POW2 ? 1u : sp.repl;
+    const Pow2 p2 = POW2 ? pow2_of(f) : pow2_of(f, repl);
+    const UnitBase ub = POW2 ? unit_base_pow2_one_copy(rec, f, p2, sp.tp_max_valid, true)
+                        : p2.all ? unit_base_pow2(rec, f, p2, sp.tp_max_valid, true)
+                                 : unit_base(rec, f, sp.tp_max_valid, true, repl);
+    __syncthreads();                                       // (the tables of the turn before have been read)
+    for (u32 t = tid - team * 32 * nvt; t < (u32)N3; t += 32 * nvt) {
+      const u32 th = digit_mode(modemap, t % NM), om = digit_mode(modemap, (t / NM) % NM), gr = digit_mode(modemap, t / N2);
+      const u32 modes[3] = {th, om, gr}, width[3] = {rec.wT, rec.wO, rec.wG};
+      const bool on_shard = in_set(SET_UPDATE_ON_SHARD, om);
+      u32 ca = 0, cb = 0, cc = 0;
+#pragma unroll
+      for (int st = 0; st < 3; ++st) {        // Theorem 1: R holds E, S and S* a shard, S* and M a unit
+        if (modes[st] == PS_MODE_R) ca += width[st];
+        if (in_set(SET_SHARDLIKE, modes[st])) cb += width[st];
+        if (modes[st] == PS_MODE_SG) cc += width[st] * sp.sstar_units;
+        if (modes[st] == PS_MODE_M) cc += width[st];
+      }
+      // Theorem 2, and what the execution model moves beyond it (as in k_eval)
+      const u32 kp = (th == PS_MODE_SG ? 2 * sp.accum * rec.wT : 0) +
+                     (gr == PS_MODE_R ? 2 * rec.wG : (gr == PS_MODE_S ? rec.wG : 0));
+      u32 ke = 0;
+      if (th == PS_MODE_O) ke += 2 * sp.accum * rec.wT;
+      if (th == PS_MODE_R && on_shard) ke += rec.wT;
+      if (om == PS_MODE_SG) ke += rec.wO;
+      if (gr == PS_MODE_SG) ke += 2 * rec.wG;
+      if (gr == PS_MODE_M) ke += (on_shard ? 1 : 2) * rec.wG;
+      if (gr == PS_MODE_O) ke += rec.wG;
+      const u32 kh = (th == PS_MODE_O ? (2 * sp.accum + 1) * rec.wT : 0) + (om == PS_MODE_O ? 2 * rec.wO : 0) +
+                     (gr == PS_MODE_O ? 2 * rec.wG : 0);
+      u64 paper = mad_small(ub.x, kp, 0), ext = mad_small(ub.x, ke, 0);
+      if (repl > 1) {
+        paper += (u64)rec.wG * ((gr == PS_MODE_S ? ub.x2 : 0) + (gr == PS_MODE_R ? ub.x3 : 0));
+        ext += (u64)rec.wG * (((gr == PS_MODE_SG || gr == PS_MODE_O || (gr == PS_MODE_M && on_shard)) ? ub.x2 : 0) +
+                              ((gr == PS_MODE_M && !on_shard) ? ub.x3 : 0));
+      }
+      table.mem[t] = mad_small(ub.E2, ca, mad_small(ub.sh, cb, mad_small(ub.u, cc, 0)));
+      table.paper[t] = paper;
+      table.ext[t] = ext;
+      table.host[t] = mad_small(ub.sh, kh, 0);
+      const u32 st = !POW2 && ub.cls == CLS_ALL_COPIES ? triple_static_all_copies(th, om, gr) : triple_static(th, om, gr, ub.d1);
+      constexpr u32 both = PS_F_THETA_AVAIL | PS_F_GRAD_COVER;
+      table.flags[t] = ub.cv | PS_F_FEASIBLE | (st & (both | PS_F_SC)) | ((st & X_HOST3) ? PS_F_USES_HOST : 0) |
+                       ((st & both) == both ? PS_F_GI << 16 : 0) |
+                       ((st & (X_EXT0 | X_MO3)) == X_EXT0 ? PS_F_PAPER_PRICED << 16 : 0);
+    }
+    __syncthreads();
+    const u64 g = ug * nvt + vt, tile = g - a.first_group;               // (wraps before the window)
+    if (!have || tile >= a.n_tiles) continue;
+    // ---- the warp's group: what its variant and the digits add
+    const ActBase ab = POW2 ? act_base_pow2_one_copy(rec, p2, 0, tau)
+                       : p2.all ? act_base_pow2(rec, p2, 0, tau) : act_base(rec, f, 0, tau, ub.G);
+    const u64 c_axis = model_axis_traffic(rec, f, ub, tau, sp.tp_coll, sp.accum);
+    const u64 act_host = 2 * ab.EA * sp.accum;
+    const u32 avail = ub.d1 ? ((1u << NM) - 1u) : own;                    // digits with PS_F_ACT_AVAIL
+    const u64 group_first = g * NC, window_end = a.first + a.count;
+    const u32 code_lo = a.first > group_first ? (u32)(a.first - group_first) : 0u;
+    const u32 code_hi = window_end < group_first + NC ? (u32)(window_end - group_first) : (u32)NC;
+    // survivors before this group: those of the runs before its run, and of the run's earlier groups
+    u64 at = a.run_offset[place / EVAL_RUN_UNITS] + a.group_offset[tile];
+    u64 mem3[R], host3[R];
+    u32 flags3[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int t = min(lane + 32 * r, N3 - 1);
+      mem3[r] = table.mem[t]; host3[r] = table.host[t]; flags3[r] = table.flags[t];
+    }
+#pragma unroll
+    for (int d = 0; d < NM; ++d) {
+      const u32 mode = digit_mode(modemap, d);
+      const u64 act = mu_elems(mode, ab.EA, ab.shA, ab.uA, sp.sstar_units), host_add = mode == PS_MODE_O ? act_host : 0;
+      const u32 with = (((avail >> d) & 1u) ? PS_F_GI : 0) | (!in_set(SET_M_OR_O, mode) ? PS_F_PAPER_PRICED : 0);
+      const u32 alone = (((avail >> d) & 1u) ? PS_F_ACT_AVAIL : 0) | (mode == PS_MODE_O ? PS_F_USES_HOST : 0);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const u32 t = lane + 32 * r, code = t + d * N3;
+        const u64 mem = mem3[r] + act, host = host3[r] + host_add;
+        const u32 fl = (flags3[r] & 0xffffu) | alone | ((flags3[r] >> 16) & with);
+        const bool pass = t < (u32)N3 && code >= code_lo && code < code_hi && mem <= a.cap_bytes && host <= a.host_cap &&
+                          (fl & a.require_flags) == a.require_flags;
+        const u32 votes = __ballot_sync(0xffffffffu, pass);
+        if (pass) {
+          const u64 o = at + __popc(votes & ((1u << lane) - 1u));
+          if (a.idx_out) a.idx_out[o] = group_first + code;
+          if (a.out.mem) a.out.mem[o] = mem;
+          if (a.out.comm_paper) a.out.comm_paper[o] = table.paper[t];
+          if (a.out.comm_ext) a.out.comm_ext[o] = table.ext[t] + c_axis;
+          if (a.out.host) a.out.host[o] = host;
+          if (a.out.flags) a.out.flags[o] = fl;
+        }
+        at += __popc(votes);
+      }
+    }
+  }
 }
 
 // ------------------------------------------------------------------ compaction: count
@@ -435,6 +539,7 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
   __shared__ u64 carry;
   __shared__ u32 last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  asm volatile("griddepcontrol.launch_dependents;");     // the write pass waits for this grid's end itself
   const u32 modemap = (NM == 5) ? 0x43210u : sp.modemap;
   const u32 req = a.require_flags;
   constexpr u32 CV_BITS = PS_F_CV | PS_F_T_DIV_HEADS | PS_F_K_DIV_LAYERS | PS_F_TP_LE_MAX | PS_F_AXIS_FORM;
@@ -475,8 +580,9 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
   const unsigned char* const allowed_here = allowed_of[lu.shift >> 3];
   __syncthreads();
   float n[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  const u32 pairs = __any_sync(0xffffffffu, lu.allowed != 0) ? N2 : 0;     // (a run without a unit that can pass is not walked)
 #pragma unroll 1
-  for (u32 p = warp * N2 / COUNT_WARPS; p < (warp + 1) * N2 / COUNT_WARPS; ++p) {
+  for (u32 p = warp * pairs / COUNT_WARPS; p < (warp + 1) * pairs / COUNT_WARPS; ++p) {
     const u32 th = p / NM, om = p - th * NM, th_mode = digit_mode(modemap, th), om_mode = digit_mode(modemap, om);
     const double to_mem = state_bytes(lu, th_mode, wT, sp.sstar_units) + state_bytes(lu, om_mode, wO, sp.sstar_units);
     const T to_host = (th_mode == PS_MODE_O ? host_T * lu.shard : T(0)) + (om_mode == PS_MODE_O ? host_O * lu.shard : T(0));
@@ -558,7 +664,7 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
   }
   __syncthreads();
   if (warp == 0) {
-    // ---- offsets inside the run, and the list of groups with survivors
+    // ---- offsets inside the run, and the list of units with survivors
     u32 mine = 0, filled = 0, c[4];
     bool inside[4];
     u64 at[4];
@@ -569,8 +675,8 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
       inside[q] = have && v < sp.nv && tau < sp.nt && at[q] < a.n_tiles;
       c[q] = inside[q] ? cnt[q][lane] : 0;
       mine += c[q];
-      filled += c[q] ? 1u : 0u;
     }
+    filled = mine ? 1u : 0u;
     u32 incl = mine, listed = filled;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -584,9 +690,9 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
 #pragma unroll
     for (u32 q = 0; q < 4; ++q) {
       if (inside[q]) a.group_offset[at[q]] = before;
-      if (c[q]) a.nonempty[base++] = (u32)at[q];
       before += c[q];
     }
+    if (filled) a.nonempty[base] = k;
     if (lane == 31) a.run_offset[blockIdx.x] = incl;
     // ---- the block that finishes last turns the runs' totals into offsets
     __threadfence();
@@ -633,40 +739,51 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
   }
 }
 
-template <int MODE, int NM, bool POW2>
-cudaError_t launch_eval_p(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
-  // one warp per run of groups; enough blocks to fill the GPU, no more than groups
+int multiprocessors() {
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+template <int NM, bool POW2>
+cudaError_t launch_eval_p(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
+  // one warp per run of groups; enough blocks to fill the GPU, no more than groups
   const unsigned needed = (a.n_tiles + WARPS - 1) / WARPS;
-  const unsigned most = (unsigned)sms * (MODE == MODE_MATERIALISE ? EVAL_GRID_PER_SM_MATERIALISE
-                                                                  : EVAL_GRID_PER_SM_WRITE);
+  const unsigned most = (unsigned)multiprocessors() * EVAL_GRID_PER_SM_MATERIALISE;
   const unsigned blocks = needed < most ? needed : most;
-  constexpr int NC = NM * NM * NM * NM;
-  const size_t smem = MODE == MODE_MATERIALISE ? (size_t)WARPS * 2 * Stage<NC>::BYTES : 0;
+  const size_t smem = (size_t)WARPS * 2 * Stage<NM * NM * NM * NM>::BYTES;
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_eval<MODE, NM, POW2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_eval<NM, POW2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_eval<MODE, NM, POW2><<<blocks, THREADS, smem, stream>>>(sp, a);
+  k_eval<NM, POW2><<<blocks, THREADS, smem, stream>>>(sp, a);
   return cudaGetLastError();
 }
 
-template <int MODE, int NM>
-cudaError_t launch_eval_t(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
-  return (sp.all_pow2 && sp.repl == 1) ? launch_eval_p<MODE, NM, true>(sp, a, stream)
-                                       : launch_eval_p<MODE, NM, false>(sp, a, stream);
+template <int NM, bool POW2>
+cudaError_t launch_write_p(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
+  const unsigned teams = WARPS / sp.nvt, needed = (a.n_units + teams - 1) / teams;
+  const unsigned most = (unsigned)multiprocessors() * EVAL_GRID_PER_SM_WRITE;
+  // enqueued so that its blocks are there when the count pass's last ones end
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t config = {};
+  config.gridDim = dim3(needed < most ? needed : most);
+  config.blockDim = dim3(THREADS);
+  config.stream = stream;
+  config.attrs = &early;
+  config.numAttrs = 1;
+  return cudaLaunchKernelEx(&config, k_write<NM, POW2>, sp, a);
 }
 
-template <int MODE>
-cudaError_t launch_eval_m(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
-  switch (sp.nm) {
-    case 1: return launch_eval_t<MODE, 1>(sp, a, stream);
-    case 2: return launch_eval_t<MODE, 2>(sp, a, stream);
-    case 3: return launch_eval_t<MODE, 3>(sp, a, stream);
-    case 4: return launch_eval_t<MODE, 4>(sp, a, stream);
-    default: return launch_eval_t<MODE, 5>(sp, a, stream);
-  }
+template <int NM>
+cudaError_t launch_materialise_t(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
+  return (sp.all_pow2 && sp.repl == 1) ? launch_eval_p<NM, true>(sp, a, stream) : launch_eval_p<NM, false>(sp, a, stream);
+}
+template <int NM>
+cudaError_t launch_write_t(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
+  return (sp.all_pow2 && sp.repl == 1) ? launch_write_p<NM, true>(sp, a, stream) : launch_write_p<NM, false>(sp, a, stream);
 }
 
 }  // namespace
@@ -678,7 +795,13 @@ void eval_plan_runs(const SpaceDev& sp, EvalArgs& a) {
 }
 
 cudaError_t launch_eval_materialise(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
-  return launch_eval_m<MODE_MATERIALISE>(sp, a, stream);
+  switch (sp.nm) {
+    case 1: return launch_materialise_t<1>(sp, a, stream);
+    case 2: return launch_materialise_t<2>(sp, a, stream);
+    case 3: return launch_materialise_t<3>(sp, a, stream);
+    case 4: return launch_materialise_t<4>(sp, a, stream);
+    default: return launch_materialise_t<5>(sp, a, stream);
+  }
 }
 template <int NM>
 static cudaError_t launch_count_t(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
@@ -701,5 +824,11 @@ cudaError_t launch_eval_count(const SpaceDev& sp, const EvalArgs& a, cudaStream_
   }
 }
 cudaError_t launch_eval_write(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
-  return launch_eval_m<MODE_WRITE>(sp, a, stream);
+  switch (sp.nm) {
+    case 1: return launch_write_t<1>(sp, a, stream);
+    case 2: return launch_write_t<2>(sp, a, stream);
+    case 3: return launch_write_t<3>(sp, a, stream);
+    case 4: return launch_write_t<4>(sp, a, stream);
+    default: return launch_write_t<5>(sp, a, stream);
+  }
 }

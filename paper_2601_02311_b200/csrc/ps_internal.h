@@ -64,7 +64,7 @@ cudaError_t launch_sweep(int kind, const SpaceDev& sp, const SweepArgs& a, int s
 
 // ---- batch evaluation
 /* Block shape of the window kernels: blocks of four warps, four of them resident (128 registers a
-   thread; the write pass with up to four modes five, see EVAL_MIN_BLOCKS_WRITE).  Against two
+   thread; the write pass five, see EVAL_MIN_BLOCKS_WRITE).  Against two
    blocks of eight warps: materialise -5 % (625 codes a group) to -13 % (256 codes); short blocks
    spread the warps' set-up and store phases better. */
 #ifndef EVAL_THREADS
@@ -90,7 +90,7 @@ struct EvalArgs {
   u64 first_unit;
   u32 n_units, n_runs;
   u32* group_offset;        // [n_tiles] survivors of the earlier groups of the group's run
-  u32* nonempty;            // [n_tiles] the groups that have survivors, in any order
+  u32* nonempty;            // [n_units] the units that have survivors, counted from first_unit, in any order
   // Counters of the count pass: places given out in the list and blocks that have finished.  Both
   // are zero between calls: the last block leaves the list's length in n_listed and clears them.  So
   // no call needs a memset of its own, and a captured call can be replayed.
