@@ -93,7 +93,11 @@ __device__ __forceinline__ u32 triple_static_all_copies(u32 th, u32 om, u32 gr) 
 // size): the shared and global addresses of every element then agree modulo 16,
 // the elements before the first 16-byte boundary and after the last one (at
 // most 16 / element size - 1 each) are written with plain stores, and everything
-// between goes out as one bulk store.
+// between goes out as one bulk store.  Of a group at an edge of the window the part
+// inside goes out the same way: a loop of its own for such groups, with its code fetched
+// where a window is short and nothing hides that, took a window of 700 points (625 codes
+// a group) 4.9 us with predicated stores and 5.9 with branches around them; staged it takes
+// 3.9 (256 codes: 3.3 and 3.6), and 2^25 points 171 us instead of 179 and 176.
 template <int NC>
 struct Stage {
   static constexpr int SLOTS = NC + 4;                                   // u64 slots, room for the skew
@@ -109,18 +113,21 @@ __device__ __forceinline__ void bulk_wait_read() {
 }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// All lanes have written `n` elements of type T to buf[skew ...]; store them to dst[0 .. n).
+// All lanes have written element c of a group to buf[c + skew]; store those from lo to hi to dst[lo .. hi).
 template <typename T>
-__device__ __forceinline__ void warp_bulk_store(T* __restrict__ dst, const T* buf, int skew, int n, int lane) {
+__device__ __forceinline__ void warp_bulk_store(T* __restrict__ dst, const T* buf, int skew, int lo, int hi, int lane) {
   constexpr int PER16 = 16 / (int)sizeof(T);
   // make the lanes' shared-memory writes visible to the copy engine
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncwarp();
-  const int head = min((PER16 - skew) & (PER16 - 1), n);                 // elements before the first boundary
+  dst += lo;
+  buf += lo + skew;
+  const int n = hi - lo;
+  const int head = min(-(lo + skew) & (PER16 - 1), n);                   // elements before the first boundary
   const int body = ((n - head) / PER16) * PER16;
-  if (lane < head) dst[lane] = buf[skew + lane];
+  if (lane < head) dst[lane] = buf[lane];
   const int tail = n - head - body;
-  if (lane < tail) dst[head + body + lane] = buf[skew + head + body + lane];
+  if (lane < tail) dst[head + body + lane] = buf[head + body + lane];
   if (lane == 0 && body > 0) {
 #if EVAL_BULK_EVICT_FIRST
     // The output is written once and not read back by this kernel: with the evict-first
@@ -129,11 +136,11 @@ __device__ __forceinline__ void warp_bulk_store(T* __restrict__ dst, const T* bu
     unsigned long long policy;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;"
-                 ::"l"(dst + head), "r"(smem_addr(buf + skew + head)), "r"(body * (int)sizeof(T)), "l"(policy)
+                 ::"l"(dst + head), "r"(smem_addr(buf + head)), "r"(body * (int)sizeof(T)), "l"(policy)
                  : "memory");
 #else
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                 ::"l"(dst + head), "r"(smem_addr(buf + skew + head)), "r"(body * (int)sizeof(T))
+                 ::"l"(dst + head), "r"(smem_addr(buf + head)), "r"(body * (int)sizeof(T))
                  : "memory");
 #endif
   }
@@ -249,8 +256,10 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
     const UnitBase ub = POW2 ? unit_base_pow2_one_copy(rec, f, p2, sp.tp_max_valid, true)
                         : p2.all ? unit_base_pow2(rec, f, p2, sp.tp_max_valid, true)
                                  : unit_base(rec, f, sp.tp_max_valid, true, repl);
-    const ActBase ab = POW2 ? act_base_pow2_one_copy(rec, p2, v, tau)
-                       : p2.all ? act_base_pow2(rec, p2, v, tau) : act_base(rec, f, v, tau, ub.G);
+    ModelRec variant = rec;                      // (an index into the record would put all of it into local memory)
+    variant.A[0] = __ldg(&sp.recs[model].A[v]); variant.UA[0] = __ldg(&sp.recs[model].UA[v]);
+    const ActBase ab = POW2 ? act_base_pow2_one_copy(variant, p2, 0, tau)
+                       : p2.all ? act_base_pow2(variant, p2, 0, tau) : act_base(variant, f, 0, tau, ub.G);
     const u64 c_axis = model_axis_traffic(rec, f, ub, tau, sp.tp_coll, sp.accum);
     u64 act[NM];
 #pragma unroll
@@ -297,10 +306,9 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
       fl_gi[r] = ((st[r] & both) == both) ? PS_F_GI : 0;
       fl_priced[r] = ((st[r] & (X_EXT0 | X_MO3)) == X_EXT0) ? PS_F_PAPER_PRICED : 0;
     }
-    const bool whole = code_lo == 0 && code_hi == (u32)NC;      // the window covers the group
     const bool all_out = a.out.mem && a.out.comm_paper && a.out.comm_ext && a.out.host && a.out.flags;
 
-    if (whole && all_out) {
+    if (all_out) {
       // one output array at a time: stage the group's NC values, hand them to the copy engine
 #pragma unroll
       for (int which = 0; which < 5; ++which) {
@@ -332,14 +340,13 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
             else stage32[slot] = fl_base[r] | fl_digit | (fl_gi[r] & gi_mask) | (fl_priced[r] & priced_mask);
           }
         }
-        if (which < 4) warp_bulk_store(dst64, stage, skew, NC, lane);
-        else warp_bulk_store(dst32, stage32, skew, NC, lane);
+        if (which < 4) warp_bulk_store(dst64, stage, skew, code_lo, code_hi, lane);
+        else warp_bulk_store(dst32, stage32, skew, code_lo, code_hi, lane);
       }
       continue;
     }
 
-    // (at the window's edges only: unrolled, it made the staged path spill, 2^25 points 0.191 ms
-    // instead of 0.179)
+    // (some of the outputs only)
 #pragma unroll 1
     for (int d = 0; d < NM; ++d) {
       const u64 act_d = mu_elems(digit_mode(modemap, d), ab.EA, ab.shA, ab.uA, sp.sstar_units);
@@ -350,24 +357,13 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const u32 code = lane + 32 * r + d * N3;
-        if (!(live[r] && (whole || (code >= code_lo && code < code_hi)))) continue;
-        const u64 mem = mem3[r] + act_d;
-        const u64 host = host3[r] + host_add;
-        const u32 fl = fl_base[r] | fl_digit | (fl_gi[r] & gi_mask) | (fl_priced[r] & priced_mask);
+        if (!(live[r] && code >= code_lo && code < code_hi)) continue;
         const u64 o = out_base + code;
-        if (all_out) {
-          a.out.mem[o] = mem;
-          a.out.comm_paper[o] = paper3[r];
-          a.out.comm_ext[o] = ext3[r] + c_axis;
-          a.out.host[o] = host;
-          a.out.flags[o] = fl;
-        } else {
-          if (a.out.mem) a.out.mem[o] = mem;
-          if (a.out.comm_paper) a.out.comm_paper[o] = paper3[r];
-          if (a.out.comm_ext) a.out.comm_ext[o] = ext3[r] + c_axis;
-          if (a.out.host) a.out.host[o] = host;
-          if (a.out.flags) a.out.flags[o] = fl;
-        }
+        if (a.out.mem) a.out.mem[o] = mem3[r] + act_d;
+        if (a.out.comm_paper) a.out.comm_paper[o] = paper3[r];
+        if (a.out.comm_ext) a.out.comm_ext[o] = ext3[r] + c_axis;
+        if (a.out.host) a.out.host[o] = host3[r] + host_add;
+        if (a.out.flags) a.out.flags[o] = fl_base[r] | fl_digit | (fl_gi[r] & gi_mask) | (fl_priced[r] & priced_mask);
       }
     }
   }
