@@ -1002,7 +1002,9 @@ __global__ void __maxnreg__(sweep_registers(DEGREES)) k_sweep(const __grid_const
           // For a triple and a tensor-axis variant the communication does not depend on the
           // activation variant and digit, so of those that are allowed only the one with the
           // least bytes can be on a frontier -- and if it does not fit, none does.  The offloaded
-          // digit keeps none.
+          // digit keeps none.  (Where it is the only one allowed and the host budget keeps it out, the
+          // capacity stands for the activations' bytes: with a test of its own for that in `cand` the
+          // passes lose 5 to 12 %, 1024 models skipping rejected factorisations 83 us instead of 74.)
           bool cand[4];
           T mem[4], comm[4];
 #pragma unroll
@@ -1010,8 +1012,9 @@ __global__ void __maxnreg__(sweep_registers(DEGREES)) k_sweep(const __grid_const
             const int j = w >> 1, tau = w & 1;
             comm[w] = c[j] + axis[tau];
             const bool off = (allowed[j] & is_o) != 0 && (!HOST_LIMITED || h[j] < lu.host_most[tau]);
-            mem[w] = whole<T>(m[j]) + (off ? T(0) : lu.act[tau]);
-            cand[w] = (off || (allowed[j] & ~is_o) != 0) && mem[w] < cap_room && (u32)tau < sp.nt;
+            const bool keeps = !HOST_LIMITED || (allowed[j] & ~is_o) != 0;
+            mem[w] = whole<T>(m[j]) + (off ? T(0) : keeps ? lu.act[tau] : cap_room);
+            cand[w] = allowed[j] != 0 && mem[w] < cap_room && (u32)tau < sp.nt;
             const int cell = cell_of(PARETO ? mem[w] : comm[w]);
             if (!SECOND) {
               if (cand[w] && bits<T>(comm[w]) < sh.cell[cell])
