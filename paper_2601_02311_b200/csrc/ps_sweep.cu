@@ -711,18 +711,17 @@ __device__ __noinline__ void frontier_by_definition(const SpaceDev& sp, const Sw
 }
 
 // ------------------------------------------------------------------ the sweep
-// Registers of a thread: with powers of two five blocks of four warps share an SM instead of four (4096
-// models of the stress configuration 577 -> 543 us for Pareto and 611 -> 589 for top-k, 1024 models 81.0 ->
-// 82.5); the divisions of other degrees spill then (ragged counts 83 -> 102 us).  At 80 the passes spill
-// in either case (1024 models 92 us).
-constexpr int sweep_registers(int degrees) { return degrees == DEGREES_POW2 ? 96 : 128; }
+// Registers of a thread.  With powers of two the frontier passes fit 96, and five blocks of four warps
+// share an SM instead of four (4096 models of the stress configuration 577 -> 543 us); the divisions of other
+// degrees spill then (ragged counts 83 -> 102 us).  The first pass of top-k holds twenty bounds and spills
+// at 96, so it is compiled for both, and launch_sweep_d chooses.  At 80 the passes spill in any case.
+constexpr int FEW_REGISTERS = 96, ALL_REGISTERS = 128;
 
 // KIND: the reduction; NM: allowed modes; T: the type of byte counts and volumes (see
 // LaneUnit); HOST_LIMITED: the filter has a host budget (without one the host bytes are
 // never formed).  The number of warps is the launch's (see launch_sweep).
-template <int KIND, int NM, typename T, bool HOST_LIMITED, int DEGREES>
-__global__ void __maxnreg__(sweep_registers(DEGREES)) k_sweep(const __grid_constant__ SpaceDev sp,
-                                                                   const __grid_constant__ SweepArgs args) {
+template <int KIND, int NM, typename T, bool HOST_LIMITED, int DEGREES, int REGISTERS>
+__global__ void __maxnreg__(REGISTERS) k_sweep(const __grid_constant__ SpaceDev sp, const __grid_constant__ SweepArgs args) {
   constexpr int N2 = NM * NM, N3 = NM * NM * NM;
   constexpr bool PARETO = KIND == PS_REDUCE_PARETO;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1245,40 +1244,55 @@ __global__ void __maxnreg__(sweep_registers(DEGREES)) k_sweep(const __grid_const
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
-template <int KIND, int NM, typename T, bool HOST_LIMITED, int DEGREES>
+template <int KIND, int NM, typename T, bool HOST_LIMITED, int DEGREES, int REGISTERS = ALL_REGISTERS>
 static cudaError_t launch_sweep_p(const SpaceDev& sp, const SweepArgs& a, int warps, cudaStream_t stream) {
   const dim3 grid(sp.n_models, KIND == PS_REDUCE_PARETO ? 1 : a.n_caps);
   const size_t smem = sizeof(BlockShared);
-  cudaError_t e = cudaFuncSetAttribute(k_sweep<KIND, NM, T, HOST_LIMITED, DEGREES>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const auto kernel = k_sweep<KIND, NM, T, HOST_LIMITED, DEGREES, REGISTERS>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_sweep<KIND, NM, T, HOST_LIMITED, DEGREES><<<grid, warps * 32, smem, stream>>>(sp, a);
+  kernel<<<grid, warps * 32, smem, stream>>>(sp, a);
   return cudaGetLastError();
 }
 
+// Top-k with powers of two: 96 registers where five blocks an SM instead of four outweigh the spills.  That
+// is a table of more than two rounds of blocks (2000 models of a data axis 163 -> 151 us, 4096 of the stress
+// configuration 587 -> 566, 1500 skipping 105 -> 97.5), or one that is a single round then and two
+// otherwise, unless rejected factorisations are skipped, whose blocks end at very different times (700
+// models 154 -> 151 us, without required flags 448 -> 374; skipping 73 -> 82).  Else 128 (400 models 117 us
+// instead of 123, skipping 71 instead of 77, with a host budget 125 instead of 138; 1000 of the pareto
+// configuration with a host budget 141 instead of 148).
+static bool few_registers(const SpaceDev& sp, const SweepArgs& a, int sm_count) {
+  const u64 blocks = (u64)sp.n_models * a.n_caps, sms = (u64)sm_count;
+  return blocks > 8 * sms || (blocks > 4 * sms && blocks <= 5 * sms && !a.skip_rejected);
+}
+
 template <int KIND, int NM, bool HOST_LIMITED>
-static cudaError_t launch_sweep_d(const SpaceDev& sp, const SweepArgs& a, int warps, cudaStream_t stream) {
-  return sp.all_pow2 ? launch_sweep_p<KIND, NM, double, HOST_LIMITED, DEGREES_POW2>(sp, a, warps, stream)
-                     : launch_sweep_p<KIND, NM, double, HOST_LIMITED, DEGREES_ANY>(sp, a, warps, stream);
+static cudaError_t launch_sweep_d(const SpaceDev& sp, const SweepArgs& a, int sm_count, int warps, cudaStream_t stream) {
+  if (!sp.all_pow2) return launch_sweep_p<KIND, NM, double, HOST_LIMITED, DEGREES_ANY>(sp, a, warps, stream);
+  constexpr int MANY = KIND == PS_REDUCE_PARETO ? FEW_REGISTERS : ALL_REGISTERS;
+  return few_registers(sp, a, sm_count)
+             ? launch_sweep_p<KIND, NM, double, HOST_LIMITED, DEGREES_POW2, FEW_REGISTERS>(sp, a, warps, stream)
+             : launch_sweep_p<KIND, NM, double, HOST_LIMITED, DEGREES_POW2, MANY>(sp, a, warps, stream);
 }
 
 template <int KIND, int NM>
-static cudaError_t launch_sweep_t(const SpaceDev& sp, const SweepArgs& a, int warps, cudaStream_t stream) {
+static cudaError_t launch_sweep_t(const SpaceDev& sp, const SweepArgs& a, int sm_count, int warps, cudaStream_t stream) {
   // every byte count exact in a double
   if (sp.all_small && a.cap_max < ((u64)1 << 53) - 1)
-    return NM < 4 || a.host_cap < HOST_BYTES_END ? launch_sweep_d<KIND, NM, true>(sp, a, warps, stream)
-                                                 : launch_sweep_d<KIND, NM, NM < 4>(sp, a, warps, stream);
+    return NM < 4 || a.host_cap < HOST_BYTES_END ? launch_sweep_d<KIND, NM, true>(sp, a, sm_count, warps, stream)
+                                                 : launch_sweep_d<KIND, NM, NM < 4>(sp, a, sm_count, warps, stream);
   return launch_sweep_p<KIND, NM, u64, true, DEGREES_EITHER>(sp, a, warps, stream);
 }
 
 template <int KIND>
-static cudaError_t launch_sweep_k(const SpaceDev& sp, const SweepArgs& a, int warps, cudaStream_t stream) {
+static cudaError_t launch_sweep_k(const SpaceDev& sp, const SweepArgs& a, int sm_count, int warps, cudaStream_t stream) {
   switch (sp.nm) {
-    case 1: return launch_sweep_t<KIND, 1>(sp, a, warps, stream);
-    case 2: return launch_sweep_t<KIND, 2>(sp, a, warps, stream);
-    case 3: return launch_sweep_t<KIND, 3>(sp, a, warps, stream);
-    case 4: return launch_sweep_t<KIND, 4>(sp, a, warps, stream);
-    default: return launch_sweep_t<KIND, 5>(sp, a, warps, stream);
+    case 1: return launch_sweep_t<KIND, 1>(sp, a, sm_count, warps, stream);
+    case 2: return launch_sweep_t<KIND, 2>(sp, a, sm_count, warps, stream);
+    case 3: return launch_sweep_t<KIND, 3>(sp, a, sm_count, warps, stream);
+    case 4: return launch_sweep_t<KIND, 4>(sp, a, sm_count, warps, stream);
+    default: return launch_sweep_t<KIND, 5>(sp, a, sm_count, warps, stream);
   }
 }
 
@@ -1288,6 +1302,6 @@ cudaError_t launch_sweep(int kind, const SpaceDev& sp, const SweepArgs& a, int s
   const u64 blocks = (u64)sp.n_models * (kind == PS_REDUCE_PARETO ? 1 : a.n_caps);
   int warps = 4;
   while (warps < SWEEP_MAX_WARPS && blocks * warps * 2 <= (u64)sm_count * 16) warps *= 2;
-  return kind == PS_REDUCE_PARETO ? launch_sweep_k<PS_REDUCE_PARETO>(sp, a, warps, stream)
-                                  : launch_sweep_k<PS_REDUCE_TOPK>(sp, a, warps, stream);
+  return kind == PS_REDUCE_PARETO ? launch_sweep_k<PS_REDUCE_PARETO>(sp, a, sm_count, warps, stream)
+                                  : launch_sweep_k<PS_REDUCE_TOPK>(sp, a, sm_count, warps, stream);
 }
