@@ -44,10 +44,13 @@ namespace {
 #define EVAL_MIN_BLOCKS_WRITE 5
 #endif
 #ifndef EVAL_GRID_PER_SM_WRITE
-#define EVAL_GRID_PER_SM_WRITE 16
+#define EVAL_GRID_PER_SM_WRITE 32
 #endif
 constexpr int THREADS = EVAL_THREADS;
 constexpr int WARPS = THREADS / 32;
+
+// the flags that a composition has or has not, whatever its placements
+constexpr u32 CV_BITS = PS_F_CV | PS_F_T_DIV_HEADS | PS_F_K_DIV_LAYERS | PS_F_TP_LE_MAX | PS_F_AXIS_FORM;
 
 // internal bits of a triple's static description (above the public flag bits)
 enum : u32 {
@@ -386,8 +389,9 @@ struct UnitTable {
 // popc.  What bounds it: the set-up of a group and its stores.  With the triples' coefficients and
 // figures formed by every warp for itself, four triples a lane, 2^23 points with half of them
 // surviving took 74 us and 2^25 with one in two thousand 32, with the count pass; like this 68 and 28,
-// launched before the count pass has ended 67 and 26.5, with 16 blocks per SM in the grid instead of 64 (most
-// of which found nothing left to do) 64.6 and 25; with 6 blocks 80 and 24.
+// launched before the count pass has ended 67 and 26.5.  Five blocks are resident: with four 2^25 points that
+// all survive take 305 us instead of 316, half of 2^23 67.7 instead of 61.2 (256 codes a group) and 48.4 instead of
+// 45.1 (625).  The grid: see launch_write_p.
 template <int NM, bool POW2>
 __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS_WRITE) k_write(const __grid_constant__ SpaceDev sp,
                                                                          const __grid_constant__ EvalArgs a) {
@@ -538,7 +542,6 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 2) k_compact_count(SpaceDev 
   asm volatile("griddepcontrol.launch_dependents;");     // the write pass waits for this grid's end itself
   const u32 modemap = (NM == 5) ? 0x43210u : sp.modemap;
   const u32 req = a.require_flags;
-  constexpr u32 CV_BITS = PS_F_CV | PS_F_T_DIV_HEADS | PS_F_K_DIV_LAYERS | PS_F_TP_LE_MAX | PS_F_AXIS_FORM;
   const u32 req_cv = req & CV_BITS;
   // capacities as exclusive bounds (memory stays below 2^61)
   const u64 cap_x = min(a.cap_bytes, (u64)1 << 62) + 1;
@@ -758,8 +761,14 @@ cudaError_t launch_eval_p(const SpaceDev& sp, const EvalArgs& a, cudaStream_t st
 
 template <int NM, bool POW2>
 cudaError_t launch_write_p(const SpaceDev& sp, const EvalArgs& a, cudaStream_t stream) {
+  // 32 blocks an SM, not more than there are units; 64 where there are more units than that and the filter requires
+  // nothing of the composition, so that most of them may be listed.  Short blocks keep the warps at
+  // different stages, but those that find nothing left to do cost a launch.  With 16, 32 and 64: 2^25 points that all
+  // survive 337, 324 and 316 us (five modes; 2^24 in four modes 196, 184 and 177), half of 2^23 59.9, 58.4 and
+  // 61.2, one of 2^25 in two thousand (valid placements) 25.1, 25.1 and 27.1.
   const unsigned teams = WARPS / sp.nvt, needed = (a.n_units + teams - 1) / teams;
-  const unsigned most = (unsigned)multiprocessors() * EVAL_GRID_PER_SM_WRITE;
+  const unsigned per_sm = (unsigned)multiprocessors() * EVAL_GRID_PER_SM_WRITE;
+  const unsigned most = needed > 2 * per_sm && (a.require_flags & CV_BITS) == 0 ? 2 * per_sm : per_sm;
   // enqueued so that its blocks are there when the count pass's last ones end
   cudaLaunchAttribute early;
   early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
