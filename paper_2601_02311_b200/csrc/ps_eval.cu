@@ -48,6 +48,7 @@ namespace {
 #endif
 constexpr int THREADS = EVAL_THREADS;
 constexpr int WARPS = THREADS / 32;
+static_assert(THREADS % 128 == 0, "k_write gives every variant of a unit a warp: one, two or four");
 
 // the flags that a composition has or has not, whatever its placements
 constexpr u32 CV_BITS = PS_F_CV | PS_F_T_DIV_HEADS | PS_F_K_DIV_LAYERS | PS_F_TP_LE_MAX | PS_F_AXIS_FORM;
