@@ -140,7 +140,8 @@ struct Scratch {
   u32* i;
 };
 // a ranking's result on its way into the buffer.  Pareto (KEEP_CAP entries): a model's last ranking, behind
-// the passes.  Top-k (PAIRWISE entries): the screening is over, and more than PAIRWISE are sorted in place.
+// the passes.  Top-k (PAIRWISE entries, in the place of the screening's masks): also behind the passes, since a cut
+// inside them sorts in place -- the buffer is full then, and a later segment is screened with the masks.
 template <int KIND> __device__ __forceinline__ Scratch ranked_scratch(BlockShared& sh);
 // top-k: the candidates that are left, while their points fill the buffer (CAND_CAP entries, behind the passes)
 __device__ __forceinline__ Scratch hits(BlockShared& sh);
@@ -340,6 +341,7 @@ __device__ __noinline__ void sort_candidates(BlockShared& sh, int n) {
 // of 0.840; with 64 instead of 128 0.755 and 0.838, and the zoo's frontiers 0.6 % more.
 constexpr int PAIRWISE = 128;
 
+static_assert(CAND_CAP > PAIRWISE, "a full buffer is sorted in place: a ranking would overwrite the masks of later segments");
 static_assert(sizeof(BlockShared::cell) >= CAND_CAP * sizeof(u64) && sizeof(BlockShared::least_cell) >= CAND_CAP * sizeof(u64) &&
                   sizeof(BlockShared::heavy) >= CAND_CAP * sizeof(u32) && CAND_CAP >= KEEP_CAP &&
                   sizeof(BlockShared::mask) >= PAIRWISE * (2 * sizeof(u64) + sizeof(u32)),
