@@ -28,8 +28,10 @@ on a bounded sample of the same workload.
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import os
+import re
 import subprocess
 import sys
 import tempfile
@@ -49,14 +51,32 @@ UNIT = "evals/s"
 BYTES_PER_POINT_MATERIALISE = 36
 
 
+# what a kernel is compiled from
+HEADERS = ("ps_lane.cuh", "ps_device.cuh", "ps_internal.h")
+KERNEL_SOURCES = {"k_sweep": ("ps_sweep.cu",) + HEADERS, "k_eval": ("ps_eval.cu",) + HEADERS}
+
+
+def source_digest(kernel):
+    """A digest of the code that `kernel` is compiled from, comments and spacing aside."""
+    digest = hashlib.sha256()
+    for name in KERNEL_SOURCES[kernel]:
+        text = open(os.path.join(ROOT, "paper_2601_02311_b200", "csrc", name)).read()
+        text = re.sub(r"//[^\n]*|/\*.*?\*/", " ", text, flags=re.S)
+        digest.update(" ".join(text.split()).encode())
+    return digest.hexdigest()[:16]
+
+
 def ncu_counters():
     """Figures only a profiler can give (executed instructions per point, pipe
-    utilisation, DRAM traffic), from the tracked summary of the last capture.
-    They describe the kernels of the commit named there, on the stress
-    configuration; the bench prints that commit and uses them on that workload
-    only."""
+    utilisation, DRAM traffic), from the tracked summary of the last capture, on the
+    workloads that it names.  A kernel whose code has changed since has none: its
+    instructions per point times today's rate would say nothing."""
     try:
-        return json.load(open(os.path.join(ROOT, "profiles", "ncu_counters.json")))
+        ncu = json.load(open(os.path.join(ROOT, "profiles", "ncu_counters.json")))
+        current = {k for k in KERNEL_SOURCES if ncu["source_digests"].get(k) == source_digest(k)}
+        for w in ncu["workloads"].values():
+            w["kernels"] = {k: v for k, v in w["kernels"].items() if any(k.startswith(c + "_") for c in current)}
+        return ncu
     except Exception:
         return None
 
