@@ -98,10 +98,12 @@ __device__ __forceinline__ u32 triple_static_all_copies(u32 th, u32 om, u32 gr) 
 // the elements before the first 16-byte boundary and after the last one (at
 // most 16 / element size - 1 each) are written with plain stores, and everything
 // between goes out as one bulk store.  Of a group at an edge of the window the part
-// inside goes out the same way: a loop of its own for such groups, with its code fetched
-// where a window is short and nothing hides that, took a window of 700 points (625 codes
-// a group) 4.9 us with predicated stores and 5.9 with branches around them; staged it takes
-// 3.9 (256 codes: 3.3 and 3.6), and 2^25 points 171 us instead of 179 and 176.
+// inside goes out the same way with 625 codes a group: a loop of its own for such groups, with its
+// code fetched where a window is short and nothing hides that, took a window of 700 points
+// 4.9 us with predicated stores and 5.9 with branches around them; staged it takes 3.9, and 2^25
+// points 171 us instead of 179 and 176.  With up to 256 codes such groups take the plain loop: short
+// windows 3.3 us instead of 3.6 (one behind the other 4.2 instead of 5.0 to 6.2), 2^24 points 99
+// instead of 109, since the staged path knows its bounds when it is compiled.
 template <int NC>
 struct Stage {
   static constexpr int SLOTS = NC + 4;                                   // u64 slots, room for the skew
@@ -312,7 +314,7 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
     }
     const bool all_out = a.out.mem && a.out.comm_paper && a.out.comm_ext && a.out.host && a.out.flags;
 
-    if (all_out) {
+    if (all_out && (NM == 5 || (code_lo == 0 && code_hi == (u32)NC))) {
       // one output array at a time: stage the group's NC values, hand them to the copy engine
 #pragma unroll
       for (int which = 0; which < 5; ++which) {
@@ -350,7 +352,7 @@ __global__ void __launch_bounds__(THREADS, EVAL_MIN_BLOCKS) k_eval(SpaceDev sp, 
       continue;
     }
 
-    // (some of the outputs only)
+    // (some of the outputs only; with up to four modes the groups at the window's edges)
 #pragma unroll 1
     for (int d = 0; d < NM; ++d) {
       const u64 act_d = mu_elems(digit_mode(modemap, d), ab.EA, ab.shA, ab.uA, sp.sstar_units);
