@@ -14,9 +14,10 @@ GB = synth.GB
 
 @pytest.mark.parametrize("per_sm,over", [(4, 0), (4, 1), (5, 0), (5, 1), (8, 0), (8, 1)])
 @pytest.mark.parametrize("mode_mask", [0b11111, 0b10110])
-def test_topk_where_blocks_fill_the_gpu(ctx, ps, mode_mask, per_sm, over):      # noqa: F811
+@pytest.mark.parametrize("name", ["C1", "C3"])            # (22 factorisations, 290)
+def test_topk_where_blocks_fill_the_gpu(ctx, ps, name, mode_mask, per_sm, over):      # noqa: F811
     n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + over
-    space = dict(synth.config("C1", n_models=n), mode_mask=mode_mask)
+    space = dict(synth.config(name, n_models=n), mode_mask=mode_mask)
     few = np.arange(0, n, 37)
     gs, os_ = ctx.space(space), O.Space(dict(space, models=space["models"][few]))
     ppm = gs.points_per_model
