@@ -156,3 +156,31 @@ __device__ __forceinline__ void count_variants(float* n, double m, const double*
       : "+f"(n[0]), "+f"(n[1]), "+f"(n[2]), "+f"(n[3])
       : "d"(m), "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]), "r"(on));
 }
+// The same for the offloaded digit under a host budget: a bound for the triple's host bytes each as well.  Left
+// to the compiler as conditions, a top-k sweep with a host budget waited for the additions one after the other:
+// 300 models of the stress configuration without required flags 323 -> 282 us, 500 skipping 115 -> 99.
+__device__ __forceinline__ void count_offloaded(float* n, double m, const double* b, double h, const double* hb, u32 on) {
+  asm("{\n\t"
+      ".reg .pred q, p0, p1, p2, p3;\n\t"
+      "setp.ne.u32 q, %9, 0;\n\t"
+      "setp.lt.and.f64 p0, %10, %11, q;\n\t"
+      "setp.lt.and.f64 p1, %10, %12, q;\n\t"
+      "setp.lt.and.f64 p2, %10, %13, q;\n\t"
+      "setp.lt.and.f64 p3, %10, %14, q;\n\t"
+      "setp.lt.and.f64 p0, %4, %5, p0;\n\t"
+      "setp.lt.and.f64 p1, %4, %6, p1;\n\t"
+      "setp.lt.and.f64 p2, %4, %7, p2;\n\t"
+      "setp.lt.and.f64 p3, %4, %8, p3;\n\t"
+      "@p0 add.f32 %0, %0, 0f3F800000;\n\t"
+      "@p1 add.f32 %1, %1, 0f3F800000;\n\t"
+      "@p2 add.f32 %2, %2, 0f3F800000;\n\t"
+      "@p3 add.f32 %3, %3, 0f3F800000;\n\t"
+      "}"
+      : "+f"(n[0]), "+f"(n[1]), "+f"(n[2]), "+f"(n[3])
+      : "d"(m), "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]), "r"(on), "d"(h), "d"(hb[0]), "d"(hb[1]), "d"(hb[2]), "d"(hb[3]));
+}
+__device__ __forceinline__ void count_offloaded(float* n, double m, const double* b, u64 h, const u64* hb, u32 on) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if ((on != 0) & (m < b[q]) & (h < hb[q])) n[q] += 1.0f;
+}

@@ -986,9 +986,7 @@ __global__ void __maxnreg__(REGISTERS) k_sweep(const __grid_constant__ SpaceDev 
 #pragma unroll
             for (int d = 0; d < NM; ++d) {
               if (HOST_LIMITED && digit_mode(modemap, d) == PS_MODE_O) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                  if (((allowed[j] >> d) & 1u) & (m[j] < lu.bounds(d)[q]) & (h[j] < lu.host_bound[q])) n[q] += 1.0f;
+                count_offloaded(n, m[j], lu.bounds(d), h[j], lu.host_bound, allowed[j] & (1u << d));
               } else {
                 count_variants(n, m[j], lu.bounds(d), allowed[j] & (1u << d));
               }
