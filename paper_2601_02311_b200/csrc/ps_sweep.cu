@@ -1256,20 +1256,19 @@ static cudaError_t launch_sweep_p(const SpaceDev& sp, const SweepArgs& a, int wa
 }
 
 // Top-k with powers of two: 96 registers where five blocks an SM instead of four outweigh the spills.  A table
-// of one round of blocks never gains (300 models of the stress configuration 138 -> 144 us, with a host budget 154 -> 172).
+// of one round of blocks never gains (300 models of the stress configuration 138 -> 144 us, with a host budget 139 -> 156).
 // Beyond it, with 128 -> 96 registers:
 //   up to 32 factorisations, blocks that last alike: 700 models of a data axis 78 -> 64 us, skipping rejected
 //     factorisations 73 -> 61, 1100 105 -> 92 (900 76.5 -> 78.6, the worst);
 //   four modes, 8 bytes of spills: up to five blocks an SM 128 is better (700 models of a grid 87 -> 97), beyond
-//     96 (900: 111 -> 98, with a host budget 118 -> 113; 1180 skipping 107 -> 95);
+//     96 (900: 111 -> 98, with a host budget 119 -> 113; 1180 skipping 107 -> 95);
 //   five modes, 48 bytes of spills, 104 with a host budget: up to eight blocks an SM 128 is better (700 models of the
-//     stress configuration 148 -> 163, 1000 skipping 115 -> 121, with a host budget as well 130 -> 147), beyond 96
-//     (1350: 232 -> 220, 2400: 375 -> 356, skipping 206 -> 192); with a host budget and skipping up to nine (330
-//     models and four capacities, two copies of every shard 184 -> 206, but 1200 of the pareto configuration 141 -> 136);
+//     stress configuration 148 -> 163, 1000 skipping 115 -> 121, with a host budget as well 116 -> 133), beyond 96
+//     (1350: 232 -> 220, 2400: 375 -> 356, skipping 206 -> 192);
 //   without required flags the blocks last alike and long: where 96 make it a single round, 700 models 448 -> 374.
 static bool few_registers(const SpaceDev& sp, const SweepArgs& a, int sm_count) {
   const u64 blocks = (u64)sp.n_models * a.n_caps, sms = (u64)sm_count;
-  const u64 most = sp.n_facts <= 32 ? 4 : sp.nm <= 4 ? 5 : a.skip_rejected && a.host_cap < HOST_BYTES_END ? 9 : 8;
+  const u64 most = sp.n_facts <= 32 ? 4 : sp.nm <= 4 ? 5 : 8;
   return blocks > most * sms || (a.require_flags == 0 && blocks > 4 * sms && blocks <= 5 * sms);
 }
 
