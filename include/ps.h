@@ -365,9 +365,9 @@ int ps_select_compare(ps_ctx* ctx, const ps_space* space, uint32_t n_index, uint
  * device-wide synchronisation of cudaFree/cudaMalloc.  ps_eval_batch may do
  * both when its scratch has to grow.  This function never calls cudaMalloc,
  * cudaFree or any allocating routine: its scratch tables (a survivor count per
- * group of |mode_mask|^4 consecutive points, the list of groups that have
- * survivors, and a prefix sum per run of up to 32 groups) sit in a fixed 2 MiB
- * array inside the library image, which every GPU that loads the library holds
+ * group of |mode_mask|^4 consecutive points, the list of factorisations that
+ * have survivors, and a prefix sum per run of up to 32 factorisations) sit in a
+ * fixed 2 MiB array inside the library image, which every GPU that loads the library holds
  * until the process ends.
  *
  * Arguments, outputs, order of the survivors and error behaviour are those of

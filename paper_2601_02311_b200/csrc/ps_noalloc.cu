@@ -1,5 +1,5 @@
 // ps_eval_compact_noalloc: the filter-and-compact path of ps_eval_batch for
-// callers that must not allocate device memory.  The groups' offsets, the list of groups
+// callers that must not allocate device memory.  The groups' offsets, the list of factorisations
 // with survivors and the prefix sums over runs of factorisations live in a fixed array that
 // is part of the library image instead of in the context's growable scratch.
 #include <cuda_runtime.h>
@@ -17,7 +17,7 @@ constexpr size_t LENGTH_BYTES = 256;
 constexpr size_t OFFSET_BYTES = sizeof(u64) * (size_t)PS_NOALLOC_MAX_GROUPS;
 
 // 2 MiB on every GPU that loads the library, for the life of the process:
-// [0, COUNT_BYTES) offset of each group in its run, then the list of groups that have
+// [0, COUNT_BYTES) offset of each group in its run, then the list of factorisations that have
 // survivors and the exclusive prefix sums (one per run of factorisations, so at most one
 // per group).
 static __device__ __align__(256) unsigned char g_fixed_scratch[2 * COUNT_BYTES + LENGTH_BYTES + OFFSET_BYTES];

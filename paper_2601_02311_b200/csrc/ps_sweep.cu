@@ -1,18 +1,20 @@
 // Fused sweep: enumerate -> evaluate -> filter -> reduce -> emit, nothing materialised,
 // one launch and one block per model (top-k: per model and capacity).  A block walks the
 // model's factorisations ("units") in segments, and everywhere a lane owns a unit: it
-// forms the unit's shard quantities (all divisions) and the bounds that a (Theta, Omega,
-// G) triple's own bytes must stay below to fit with an activation variant and digit, all
-// in registers; then the lanes of a warp walk the triples together.  A triple's bytes are
-// a sum of three terms, one per state, so the next triple costs one addition, and what is
-// uniform (modes, allowed digits, coefficients) comes from small tables of the block.
+// forms the unit's shard quantities, and what a (Theta, Omega, G) triple's own bytes are held
+// against, in registers (the screening: bounds in rounded figures, without a division; top-k's first
+// pass, which counts points: a bound per activation variant and digit, LaneUnit; the other passes: the
+// least activation bytes, LeastUnit); then the lanes of a warp walk the triples together.  A
+// triple's bytes are a sum of three terms, one per state, and what is uniform (modes, allowed
+// digits, coefficients) comes from small tables of the block.
 //
 // Screening.  Every unit: its points are compared with their bounds in rounded figures, two
 // to an instruction (the four variants of the offloaded digit have the same bytes: 17
 // compares for 20 points), masked by the flags that the placement code and the composition
 // allow.  It leaves the list of the units that may have survivors (an eighth of them on the
-// stress configuration), which the next two passes walk densely and in whole bytes.  (With ps_filter.skip_rejected the list is made from the
-// composition tests alone; top-k without required flags lists all units.)
+// stress configuration), which the next two passes walk densely and in whole bytes.  (With
+// ps_filter.skip_rejected the list is made from the composition tests alone; top-k without
+// required flags lists all units.)
 //
 // First pass, over the cells of a histogram (an eighth of an octave each).
 //   Pareto: the least communication of the candidates whose bytes fall into a cell
@@ -336,9 +338,9 @@ __device__ __noinline__ void sort_candidates(BlockShared& sh, int n) {
 }
 
 // Up to this many candidates every thread tests its own against all others (no barrier in
-// the loop); more are sorted, whose work grows more slowly.  Never sorted, the stress
-// configuration takes 0.826 ms for top-k instead of 0.766 and 0.887 for the frontiers instead
-// of 0.840; with 64 instead of 128 0.755 and 0.838, and the zoo's frontiers 0.6 % more.
+// the loop); more are sorted, whose work grows more slowly.  With 64 instead of 128 the stress
+// configuration takes 586 us for top-k instead of 591, but the frontiers 555 instead of 546 and
+// those of 1024 models 86 instead of 83.
 constexpr int PAIRWISE = 128;
 
 static_assert(CAND_CAP > PAIRWISE, "a full buffer is sorted in place: a ranking would overwrite the masks of later segments");
