@@ -32,10 +32,10 @@
 //
 // What bounds it: the issue slots of the screening, and the latency of a block's phases (five
 // blocks of four warps share an SM).  4096 models of the stress configuration, 6.96e9 points:
-// top-k 1.94 -> 0.59 ms, Pareto 2.37 -> 0.55 ms against a sweep whose warps took a unit each (the
+// top-k 1.94 -> 0.57 ms, Pareto 2.37 -> 0.54 ms against a sweep whose warps took a unit each (the
 // set-up of a unit paid by a whole warp, candidates inserted one by one into a sorted list per
 // warp, the lists merged by a second kernel); 1024 models skipping rejected factorisations 0.41
-// -> 0.083 ms.  The screening takes 0.23 and 0.27 ms of the former two.
+// -> 0.072 ms.  The screening takes 0.23 and 0.27 ms of the former two.
 #include <type_traits>
 #include "ps_device.cuh"
 #include "ps_internal.h"
